@@ -204,19 +204,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   pdl_launch_dependents();
 
   if (warp == 0) {
-    if (lane == 0) {
-      uint32_t kbg = 0, s = 0, ph = 0;                       // k-block counter across tiles, ring position
-      bool ok = true;
-      uint32_t pit = 0;
-      const uint32_t full0 = PAIR ? ptx::mapa(ptx::smem_u32(full), 0) : 0u;     // the even CTA's `full` barriers
-      for (uint32_t t = cta_first; t < total_tiles && ok; t += cta_step, ++pit) {
-        const TileIdx ti_ = split_tile(t, g.fd_tiles_n, g.fd_tiles_m);
-        const uint32_t tile_n = ti_.tile_n, tile_m = PAIR ? 2 * ti_.tile_m + rank : ti_.tile_m, batch = ti_.batch;
-        const TileCoord ta = op_coords(g.ca, tile_m, batch, BM), tb = op_coords(g.cb, tile_n, batch, BN);
-        const int brow0 = tb.row0 + (int)rank * BN_CTA;
-        for (int kb = 0; kb < nkb; ++kb, ++kbg) {
-          ok = ptx::mbar_wait(&empty[s], ph ^ 1, abort_flag, g.status);
-          if (!ok) break;
+    // The whole warp walks the loop and one elected lane issues (as for the products below): under a branch on one lane every
+    // operand of a copy is moved to a uniform register in front of it, about 210 ns per copy instead of 120 -- and a k-block's
+    // two copies have less than 270 ns if the products are not to wait for them.
+    uint32_t kbg = 0, s = 0, ph = 0;                         // k-block counter across tiles, ring position
+    bool ok = true;
+    const uint32_t full0 = PAIR ? ptx::mapa(ptx::smem_u32(full), 0) : 0u;     // the even CTA's `full` barriers
+    for (uint32_t t = cta_first; t < total_tiles && ok; t += cta_step) {
+      const TileIdx ti_ = split_tile(t, g.fd_tiles_n, g.fd_tiles_m);
+      const uint32_t tile_n = ti_.tile_n, tile_m = PAIR ? 2 * ti_.tile_m + rank : ti_.tile_m, batch = ti_.batch;
+      const TileCoord ta = op_coords(g.ca, tile_m, batch, BM), tb = op_coords(g.cb, tile_n, batch, BN);
+      const int brow0 = tb.row0 + (int)rank * BN_CTA;
+      for (int kb = 0; kb < nkb; ++kb, ++kbg) {
+        ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(&empty[s], ph ^ 1, abort_flag, g.status) ? 1 : 0) != 0;
+        if (!ok) break;
+        if (ptx::elect_one()) {
           if constexpr (PAIR) {
             if (leader) ptx::mbar_expect_tx(&full[s], 2 * (two_producers ? A_STAGE_BYTES : A_STAGE_BYTES + B_STAGE_BYTES));
             tma_load_op_pair(g.ca, sA + s * A_STAGE_BYTES, &tmA, full0 + s * 8, kb * BK, ta.row0, ta);
@@ -227,16 +229,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             if (A_MN) tma_load_op(g.ca, sA + s * A_STAGE_BYTES + A_STAGE_BYTES / 2, &tmA, &full[s], kb * BK, ta.row0 + 64, ta);
             if (!two_producers) tma_load_op(g.cb, sB + s * B_STAGE_BYTES, &tmB, &full[s], kb * BK, tb.row0, tb);
           }
-          if (++s == STAGES) { s = 0; ph ^= 1; }
         }
+        __syncwarp();
+        if (++s == STAGES) { s = 0; ph ^= 1; }
       }
-      if (*abort_flag && PAIR) {
+    }
+    if (lane == 0 && *abort_flag) {
+      if (PAIR) {
         // unwinding a pair: the copies of the odd CTA are counted on the even CTA's barriers, so each side just gives
         // whatever is in flight a fixed time to land
         const unsigned long long t0 = ptx::globaltimer();
         while (ptx::globaltimer() - t0 < 100000ull) {
         }
-      } else if (*abort_flag) {
+      } else {
         // unwinding: give copies already in flight a bounded chance to land before the CTA leaves
         for (uint32_t k = (kbg > (uint32_t)STAGES ? kbg - STAGES : 0); k < kbg; ++k) {
           const unsigned long long t0 = ptx::globaltimer();
@@ -245,6 +250,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
       }
     }
+    __syncwarp();
   } else if (warp == 1) {
     // The whole warp walks the loop and one elected lane issues: with warp-uniform control flow the descriptors
     // stay in uniform registers (under a branch on lane 0 each operand is moved there in front of every product).
@@ -299,7 +305,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   } else if (warp >= 2 + kEpiWarps) {
     // second producer: the B operand (long reductions only; a short one is
     // cheaper to feed from one thread)
-    if (lane == 0 && two_producers) {
+    if (two_producers) {
       uint32_t s = 0, ph = 1;
       bool ok = true;
       const uint32_t full0 = PAIR ? ptx::mapa(ptx::smem_u32(full), 0) : 0u;
@@ -309,15 +315,18 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const TileCoord tb = op_coords(g.cb, tile_n, batch, BN);
         const int brow0 = tb.row0 + (int)rank * BN_CTA;
         for (int kb = 0; kb < nkb; ++kb) {
-          ok = ptx::mbar_wait(&empty[s], ph, abort_flag, g.status);
+          ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(&empty[s], ph, abort_flag, g.status) ? 1 : 0) != 0;
           if (!ok) break;
-          if constexpr (PAIR) {
-            if (leader) ptx::mbar_expect_tx(&full[s], 2 * B_STAGE_BYTES);
-            tma_load_op_pair(g.cb, sB + s * B_STAGE_BYTES, &tmB, full0 + s * 8, kb * BK, brow0, tb);
-          } else {
-            ptx::mbar_expect_tx(&full[s], B_STAGE_BYTES);
-            tma_load_op(g.cb, sB + s * B_STAGE_BYTES, &tmB, &full[s], kb * BK, tb.row0, tb);
+          if (ptx::elect_one()) {
+            if constexpr (PAIR) {
+              if (leader) ptx::mbar_expect_tx(&full[s], 2 * B_STAGE_BYTES);
+              tma_load_op_pair(g.cb, sB + s * B_STAGE_BYTES, &tmB, full0 + s * 8, kb * BK, brow0, tb);
+            } else {
+              ptx::mbar_expect_tx(&full[s], B_STAGE_BYTES);
+              tma_load_op(g.cb, sB + s * B_STAGE_BYTES, &tmB, &full[s], kb * BK, tb.row0, tb);
+            }
           }
+          __syncwarp();
           if (++s == STAGES) { s = 0; ph ^= 1; }
         }
       }
