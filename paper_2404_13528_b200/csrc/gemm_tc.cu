@@ -104,20 +104,6 @@ __device__ __forceinline__ TileIdx split_tile(uint32_t t, const FastDiv& fn, con
   return {t - r * fn.d, r - b * fm.d, b};
 }
 
-// GELU in the bf16 epilogue: u * Phi(u) with Phi evaluated through the hyperbolic-tangent form
-// 0.5 (1 + tanh(sqrt(2/pi) (u + 0.044715 u^3))) and the hardware tanh.  It differs from the erf
-// form by at most 5e-4 in absolute value, i.e. by less than an eighth of a bf16 ulp wherever the
-// result exceeds 1 and by less than 1e-4 |u| near zero, at a third of the instruction count (the
-// epilogue of the fc1 GEMM is issue-bound).  The fp32 kernels use erff.
-__device__ __forceinline__ float gelu_fast(float u) {
-  const float u2 = u * u;
-  const float inner = u * fmaf(0.0356774081f, u2, 0.7978845608f);
-  float t;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(inner));
-  const float h = 0.5f * u;
-  return fmaf(h, t, h);
-}
-
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = 64 + 32 * kEpiWarps + 32;      // + a second TMA producer warp (B operand)
 
@@ -527,7 +513,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         if (g.gelu) {
 #pragma unroll
-          for (int j = 0; j < RC; ++j) acc[j] = gelu_fast(acc[j]);
+          for (int j = 0; j < RC; ++j) acc[j] = gelu_tanh(acc[j]);
         }
         if (rrow) {
 #pragma unroll
@@ -706,7 +692,8 @@ int encode_cached(const void* ptr, int rank, const uint64_t* dims, const uint64_
     if (i < rank - 1) s[i] = strides_b[i];
   }
   CUresult r = enc(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void*>(ptr), d, s, b, es,
-                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                   CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_bytes == 0 ? CU_TENSOR_MAP_SWIZZLE_NONE :
+                   swizzle_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return SMARTMEM_ERR_CUDA;
@@ -835,6 +822,15 @@ int tc_encode_2d_sw64(const void* ptr, long long inner, long long outer, long lo
   return encode_cached(ptr, 2, dims, strides, box, out, 64);
 }
 
+int tc_encode_2d_plain(const void* ptr, long long inner, long long outer, long long pitch_elems, int box_inner, int box_outer,
+                       CUtensorMap* out) {
+  if (((uintptr_t)ptr & 15) || (pitch_elems * 2) % 16) return SMARTMEM_ERR_ALIGNMENT;
+  const uint64_t dims[2] = {(uint64_t)inner, (uint64_t)outer};
+  const uint64_t strides[1] = {(uint64_t)pitch_elems * 2};
+  const uint32_t box[2] = {(uint32_t)box_inner, (uint32_t)box_outer};
+  return encode_cached(ptr, 2, dims, strides, box, out, 0);
+}
+
 int tc_encode_nd_sw64(const void* ptr, int rank, const long long* dims, const long long* strides_elems, const int* box,
                       CUtensorMap* out) {
   if (rank < 2 || rank > 5 || ((uintptr_t)ptr & 15) || box[0] * 2 != 64) return SMARTMEM_ERR_ALIGNMENT;
@@ -852,6 +848,12 @@ int tc_encode_nd_sw64(const void* ptr, int rank, const long long* dims, const lo
 }
 
 int tc_sm_count() { return sm_count(); }
+
+int tc_cluster_ctas(int size) {
+  // of 148 SMs: cudaOccupancyMaxActiveClusters, one CTA per SM
+  static const int ctas[9] = {0, 148, 148, 135, 132, 130, 132, 105, 120};
+  return ctas[size] * sm_count() / 148;
+}
 
 int tc_operand_from_map(const smartmem_index_map_t& m, int n_batch_atoms, int n_row_atoms, const void* ptr,
                         TcOperand* op) {
@@ -898,6 +900,9 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
   if (N % 8) return SMARTMEM_ERR_UNSUPPORTED;
   const bool a_mn = A.k_stride != 1;
   if (B.k_stride != 1) return SMARTMEM_ERR_UNSUPPORTED;
+  if (gemm_splitk_supported(A, B, ep, batch, M, N, K) && (ep.rms_gamma || gemm_splitk_wins(M, N, K)))
+    return launch_gemm_splitk(A, B, ep, M, N, K, st);
+  if (ep.rms_gamma) return SMARTMEM_ERR_UNSUPPORTED;
   // tile width: the widest of {256, 128, 96, 64} that divides N (fewest wasted columns), else 128
   int bn = 128;
   if (ep.rope_cols > 0) bn = (M <= BM && batch == 1 && N / 256 < tc_sm_count()) ? 128 : 256;   // one head or two per tile

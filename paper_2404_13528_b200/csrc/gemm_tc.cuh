@@ -42,6 +42,9 @@ struct TcEpilogue {
   // batch == 1, M a multiple of out2_S.
   void* out2;
   long long out2_S;
+  // RMSNorm of A's rows inside the GEMM (null: none): gamma [K].  Few rows only (gemm_splitk.cu).
+  const void* rms_gamma;
+  float rms_eps;
 };
 
 int tc_operand_from_map(const smartmem_index_map_t& m, int n_batch_atoms, int n_row_atoms, const void* ptr,
@@ -49,6 +52,13 @@ int tc_operand_from_map(const smartmem_index_map_t& m, int n_batch_atoms, int n_
 TcOperand tc_operand_plain(const void* ptr, long long rows, long long K, long long ld);
 int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep, long long batch, long long M,
                    long long N, long long K, cudaStream_t st);
+
+// GEMM for few rows, split along the reduction over the CTAs of a cluster (gemm_splitk.cu): plain row-major operands, every
+// epilogue but the second copy.  launch_gemm_tc hands over where gemm_splitk_wins.
+bool gemm_splitk_supported(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep, long long batch, long long M, long long N,
+                           long long K);
+bool gemm_splitk_wins(long long M, long long N, long long K);
+int launch_gemm_splitk(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep, long long M, long long N, long long K, cudaStream_t st);
 
 // bf16 row-major [outer, inner] matrix as a 2-D tensor map with 128-byte swizzle (box_inner = 64).
 int tc_encode_2d(const void* ptr, long long inner, long long outer, long long pitch_elems, int box_inner, int box_outer,
@@ -60,7 +70,12 @@ int tc_encode_2d_sw64(const void* ptr, long long inner, long long outer, long lo
 // of 32 innermost elements.
 int tc_encode_nd_sw64(const void* ptr, int rank, const long long* dims, const long long* strides_elems, const int* box,
                       CUtensorMap* out);
+// Same without swizzle.
+int tc_encode_2d_plain(const void* ptr, long long inner, long long outer, long long pitch_elems, int box_inner, int box_outer,
+                       CUtensorMap* out);
 int tc_sm_count();
+// SMs that clusters of `size` (1..8) CTAs, one per SM, fill: a cluster must find its CTAs inside one GPC.
+int tc_cluster_ctas(int size);
 
 // Fused MLP half of a block: out = A + GELU(LN(A) W1^T + b1) W2^T + b2 with the hidden activation and the
 // normalised rows kept on chip.  A [M, C], W1 [hidden, C], W2 [C, hidden], C in {64, 96}, hidden a multiple
