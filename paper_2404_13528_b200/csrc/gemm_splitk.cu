@@ -361,9 +361,13 @@ bool gemm_splitk_supported(const TcOperand& X, const TcOperand& W, const TcEpilo
          (ep.seg_cols == 0 || ep.seg_cols % BN_W == 0);
 }
 
-// One row tile of the tiled kernel: there the stream of W through 64-96 CTAs is the bound (M = 64, K = 4096: N = 12288 31 us
-// against 22 here, N = 4096 15.9 against 11.0; two rows, 19 and 8.4 us).
-bool gemm_splitk_wins(long long M, long long N, long long K) { return M <= 128; }
+// Microseconds, fitted to measurements: a fixed part, the exchange of the partial sums (distributed shared memory moves about
+// 14 bytes per clock and SM, which is what ends the range at 128 rows), and the stream of W.  Below 32 rows always: the tiled
+// kernel's copies of a mostly empty A tile are slower than full ones (two rows, N = 12288, K = 4096: 31 us against 19).
+double gemm_splitk_us(long long M, long long N, long long K) {
+  const double nb = (double)((M + 15) / 16 * 16);
+  return M > 128 ? 1e30 : M < 32 ? 0.0 : 3.0 + 0.018 * nb + (double)N * (double)K * 2.0 / 6.2e6 * (1.0 + nb / 260.0);
+}
 
 int launch_gemm_splitk(const TcOperand& X, const TcOperand& W, const TcEpilogue& ep, long long M, long long N, long long K, cudaStream_t st) {
   SplitArgs g;

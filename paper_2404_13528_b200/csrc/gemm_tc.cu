@@ -15,10 +15,9 @@
 // the epilogue of the previous tile meanwhile (TMEM -> registers -> bias / GELU / RoPE / residual ->
 // bf16 -> staged whole-row stores, optionally scattering rows through an index map: window reverse +
 // reverse cyclic shift folded into the store).
+#include <cstring>
 #include <mutex>
 #include <unordered_map>
-#include <string>
-#include <vector>
 
 #include "gemm_tc.cuh"
 #include "ptx.cuh"
@@ -558,7 +557,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
               if (v == VPR - 1) {
                 ptx::fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) {
+                if (lane == 0 && (int)tile_m * BM + q * 32 < g.M) {
                   ptx::tma_store_2d(&tmC, cstage + e * CBOX_BYTES, n0 + c0, (int)tile_m * BM + q * 32);
                   ptx::bulk_commit_group();
                 }
@@ -662,17 +661,33 @@ EncodeTiledFn get_encode() {
   return fn;
 }
 
+// Encoded maps by what they were encoded from; a call looks up three to seven of them, so the key is a flat array of words
+// compared and hashed without an allocation.
+struct TmKey {
+  uint64_t w[12];
+  bool operator==(const TmKey& o) const { return memcmp(w, o.w, sizeof(w)) == 0; }
+};
+struct TmHash {
+  size_t operator()(const TmKey& k) const {
+    uint64_t h = 0x9E3779B97F4A7C15ull;
+    for (uint64_t v : k.w) h = (h ^ v) * 0xBF58476D1CE4E5B9ull, h ^= h >> 29;
+    return (size_t)h;
+  }
+};
 std::mutex g_tm_mu;
-std::unordered_map<std::string, CUtensorMap> g_tm_cache;
+std::unordered_map<TmKey, CUtensorMap, TmHash> g_tm_cache;
 
 int encode_cached(const void* ptr, int rank, const uint64_t* dims, const uint64_t* strides_b, const uint32_t* box,
                   CUtensorMap* out, int swizzle_bytes = 128) {
-  std::string key((const char*)&ptr, sizeof(ptr));
-  key.append((const char*)&rank, sizeof(rank));
-  key.append((const char*)dims, sizeof(uint64_t) * rank);
-  key.append((const char*)strides_b, sizeof(uint64_t) * (rank - 1));
-  key.append((const char*)box, sizeof(uint32_t) * rank);
-  key.append((const char*)&swizzle_bytes, sizeof(int));
+  TmKey key;
+  memset(&key, 0, sizeof(key));
+  key.w[0] = (uint64_t)(uintptr_t)ptr;
+  key.w[1] = ((uint64_t)rank << 16) | (uint64_t)swizzle_bytes;
+  for (int i = 0; i < rank; ++i) {
+    key.w[2 + i] = dims[i];
+    if (i < rank - 1) key.w[7 + i] = strides_b[i];
+    key.w[11] = key.w[11] << 10 | box[i];            // (a box has at most 256 elements a side)
+  }
   {
     std::lock_guard<std::mutex> lk(g_tm_mu);
     auto it = g_tm_cache.find(key);
@@ -900,26 +915,8 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
   if (N % 8) return SMARTMEM_ERR_UNSUPPORTED;
   const bool a_mn = A.k_stride != 1;
   if (B.k_stride != 1) return SMARTMEM_ERR_UNSUPPORTED;
-  if (gemm_splitk_supported(A, B, ep, batch, M, N, K) && (ep.rms_gamma || gemm_splitk_wins(M, N, K)))
-    return launch_gemm_splitk(A, B, ep, M, N, K, st);
-  if (ep.rms_gamma) return SMARTMEM_ERR_UNSUPPORTED;
-  // tile width: the widest of {256, 128, 96, 64} that divides N (fewest wasted columns), else 128
-  int bn = 128;
-  if (ep.rope_cols > 0) bn = (M <= BM && batch == 1 && N / 256 < tc_sm_count()) ? 128 : 256;   // one head or two per tile
-  else if (N % 256 == 0) {
-    // 256 or 128 wide: whichever leaves fewer idle SMs in the last wave (time of a wave ~ tile width plus a fixed part).
-    // Only for short reductions: a 128-wide tile reads as many operand bytes per product as shared memory delivers,
-    // so over a long K the wider tile wins even with a ragged last wave (measured at K = 2048).
-    const long long tm = (M + BM - 1) / BM * batch, sms = tc_sm_count();
-    const long long w256 = (tm * (N / 256) + sms - 1) / sms, w128 = (tm * (N / 128) + sms - 1) / sms;
-    bn = (K <= 1024 && w128 * (128 + 48) < w256 * (256 + 48)) ? 128 : 256;
-  } else if (N % 128 == 0) bn = 128;
-  else if (N % 96 == 0) bn = 96;
-  else if (N % 64 == 0) bn = 64;
-  // One row tile only (a decode step: M <= 128) and few wide column tiles: the GEMM streams the weight
-  // once and is bound by how many SMs pull on it, so take the narrowest tile that divides N.
-  if (ep.rope_cols == 0 && batch == 1 && M <= BM && !a_mn && N % 64 == 0 && N / bn < tc_sm_count()) bn = 64;
-  if (a_mn && bn < 128) bn = 128;                         // MN-major A operands come with 128- and 256-wide tiles only
+  const bool splitk_ok = gemm_splitk_supported(A, B, ep, batch, M, N, K);
+  if (ep.rms_gamma) return splitk_ok ? launch_gemm_splitk(A, B, ep, M, N, K, st) : SMARTMEM_ERR_UNSUPPORTED;
   if (ep.rope_cols > 0 && (N % 256 || ep.rope_cols % 256 || ep.rope_S < 1)) return SMARTMEM_ERR_UNSUPPORTED;
   if (ep.rope_cols > 0 && ep.rope_dim != 0 && ep.rope_dim != 32 && ep.rope_dim != 64 && ep.rope_dim != 128) return SMARTMEM_ERR_UNSUPPORTED;
   if (ep.seg_cols > 0) {
@@ -928,26 +925,61 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
       if (!ep.seg_out[i] || ((uintptr_t)ep.seg_out[i] & 15) || ep.seg_ld[i] % 8) return SMARTMEM_ERR_ALIGNMENT;
   }
   const int nkb = (int)((K + BK - 1) / BK);
-  // 256 wide, short K: wider store rounds instead of a 4th stage.  Narrow tiles: their stages are
-  // small, and a tile is consumed faster than a load's latency, so the ring runs several tiles ahead.
-  const int stages = bn == 256 ? (nkb <= 4 ? 3 : 4) : (bn <= 96 ? 6 : 4);
-  // CTA pairs (two SMs on one 256 x 256 tile) where the row tiles pair up and there is more than one wave of work for
-  // the single-CTA kernel: below that the operand feed is not what bounds the GEMM.
+  const long long tiles_m1 = (M + BM - 1) / BM;
+  // CTA pairs (two SMs on one tile of 256 rows): their epilogue writes 32-byte vectors.
   // SMARTMEM_GEMM_PAIR=0 keeps every GEMM on single CTAs (for measuring what pairing buys).
   static const int allow_pair = [] { const char* e = getenv("SMARTMEM_GEMM_PAIR"); return (e && e[0] == '0') ? 0 : 1; }();
-  const long long tiles_m1 = (M + BM - 1) / BM;
-  const bool pair = allow_pair && (bn == 256 || bn == 128) && !a_mn && tiles_m1 % 2 == 0 && nkb > 4 && N % 256 == 0 &&
-              tiles_m1 * (N / 256) * batch > tc_sm_count() &&
-              (!ep.rowmap || devmap_offsets_multiple_of(*ep.rowmap, 16)) && ep.seg_cols == 0 && !ep.out2 && ep.ldc % 16 == 0 &&
-              ep.out_batch_stride % 16 == 0 && ((uintptr_t)ep.out & 31) == 0;   // (its epilogue writes 32-byte vectors)
-  if (pair) {
-    // width of a pair's tile: 256 unless the last wave of 256-wide tiles is so ragged that the waves of half the width
-    // are shorter.  Microseconds per tile, fitted to measurements: per k-block a 256-wide tile costs its products and a
-    // 128-wide one its operand feed (about 2/3 of that), plus a fixed part for the epilogue the ring cannot hide.
-    const long long pairs = tc_sm_count() / 2, t256 = tiles_m1 / 2 * (N / 256) * batch;
-    const long long w256 = (t256 + pairs - 1) / pairs, w128 = (2 * t256 + pairs - 1) / pairs;
-    bn = (ep.rope_cols == 0 && w128 * (nkb * 0.21 + 1.2) < w256 * (nkb * 0.33 + 2.2)) ? 128 : 256;
+  const bool pair_ok = allow_pair && !a_mn && tiles_m1 > 1 && nkb > 4 && N % 256 == 0 && A.n_row_atoms == 1 &&
+                       (!ep.rowmap || devmap_offsets_multiple_of(*ep.rowmap, 16)) && ep.seg_cols == 0 && !ep.out2 && ep.ldc % 16 == 0 &&
+                       ep.out_batch_stride % 16 == 0 && ((uintptr_t)ep.out & 31) == 0;
+  int bn = 128;
+  bool pair = false;
+  if (batch == 1) {
+    // Tile width, and single CTAs or pairs: the smallest of the times fitted to measurements (us): a fixed part, the k-blocks of
+    // the first tile, and for every further wave its k-blocks or, where the reduction is short, its epilogue.  A narrow tile
+    // costs more per column but splits the columns over more SMs: M = 666, N = K = 2048 (48 tiles of 128 x 256, 96 of half
+    // that) 16.1 us on 256-wide single tiles, 9.6 on 128-wide pairs; M = 196, N = 512, K = 2048 14.1 -> 8.8 us on 64-wide ones.
+    struct Option { int bn; bool pair; double fixed, per_kb, wave, wave_min; };
+    static const Option options[] = {{64, false, 2.4, 0.185, 0.3, 1.9}, {96, false, 2.4, 0.25, 0.3, 2.0}, {128, false, 2.6, 0.27, 0.4, 2.8},
+                                     {256, false, 4.4, 0.36, 0.5, 4.0}, {128, true, 3.0, 0.185, 0.2, 2.2}, {256, true, 4.6, 0.33, 0.4, 3.0}};
+    double best = 0.0;
+    for (const Option& o : options) {
+      if (o.pair && !pair_ok) continue;
+      if (ep.rope_cols > 0 && o.bn < 128) continue;          // rotary pairs stay inside a tile
+      if (a_mn && o.bn < 128) continue;                      // MN-major A operands come with 128- and 256-wide tiles only
+      if (ep.seg_cols > 0 && ep.seg_cols % o.bn) continue;
+      if (B.n_row_atoms > 1 && B.row_extent[B.n_row_atoms - 1] % o.bn) continue;
+      const long long tiles = (o.pair ? (tiles_m1 + 1) / 2 : tiles_m1) * ((N + o.bn - 1) / o.bn), slots = tc_sm_count() / (o.pair ? 2 : 1);
+      const double kbs = nkb * o.per_kb, wave = kbs + o.wave > o.wave_min ? kbs + o.wave : o.wave_min;
+      const double t = o.fixed + kbs + (double)((tiles + slots - 1) / slots - 1) * wave;
+      if (best == 0.0 || t < best) { best = t; bn = o.bn; pair = o.pair; }
+    }
+    if (splitk_ok && gemm_splitk_us(M, N, K) < best) return launch_gemm_splitk(A, B, ep, M, N, K, st);
+  } else {
+    // batched: the widest of {256, 128, 96, 64} that divides N (fewest wasted columns), else 128; 256 or 128, whichever leaves
+    // fewer idle SMs in the last wave (time of a wave ~ tile width plus a fixed part), for short reductions only: a 128-wide tile
+    // reads as many operand bytes per product as shared memory delivers, so over a long K the wider tile wins even with a
+    // ragged last wave (measured at K = 2048)
+    if (ep.rope_cols > 0) bn = 256;
+    else if (N % 256 == 0) {
+      const long long tm = tiles_m1 * batch, sms = tc_sm_count();
+      const long long w256 = (tm * (N / 256) + sms - 1) / sms, w128 = (tm * (N / 128) + sms - 1) / sms;
+      bn = (K <= 1024 && w128 * (128 + 48) < w256 * (256 + 48)) ? 128 : 256;
+    } else if (N % 128 == 0) bn = 128;
+    else if (N % 96 == 0) bn = 96;
+    else if (N % 64 == 0) bn = 64;
+    if (a_mn && bn < 128) bn = 128;
+    // pairs where the row tiles pair up and there is more than one wave of work for the single-CTA kernel
+    pair = pair_ok && bn >= 128 && tiles_m1 % 2 == 0 && tiles_m1 * (N / 256) * batch > tc_sm_count();
+    if (pair) {
+      const long long pairs = tc_sm_count() / 2, t256 = tiles_m1 / 2 * (N / 256) * batch;
+      const long long w256 = (t256 + pairs - 1) / pairs, w128 = (2 * t256 + pairs - 1) / pairs;
+      bn = (ep.rope_cols == 0 && w128 * (nkb * 0.21 + 1.2) < w256 * (nkb * 0.33 + 2.2)) ? 128 : 256;
+    }
   }
+  // single CTAs: 256 wide, short K: wider store rounds instead of a 4th stage.  Narrow tiles: their stages are
+  // small, and a tile is consumed faster than a load's latency, so the ring runs several tiles ahead.
+  const int stages = bn == 256 ? (nkb <= 4 ? 3 : 4) : bn == 64 ? 8 : bn == 96 ? 7 : 5;
   GemmArgs g;
   memset(&g, 0, sizeof(g));
   CUtensorMap ta, tb;
@@ -980,7 +1012,7 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
   g.status = device_status_ptr();
   if (!g.status) return SMARTMEM_ERR_CUDA;
   g.tiles_n = (int)((N + bn - 1) / bn);
-  g.tiles_m = (int)(pair ? tiles_m1 / 2 : tiles_m1);       // pairs walk over tiles of 256 rows
+  g.tiles_m = (int)(pair ? (tiles_m1 + 1) / 2 : tiles_m1); // pairs walk over tiles of 256 rows
   g.fd_tiles_n = make_fastdiv((uint32_t)g.tiles_n);
   g.fd_tiles_m = make_fastdiv((uint32_t)g.tiles_m);
   g.batch = (int)batch;
@@ -999,8 +1031,8 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
   if (pair) return launch_t<128, 8, false, true>(ta, tb, tc, g, st);
 #define SM_CASE(BN_, ST_, MN_)                                                                  \
   if (bn == BN_ && stages == ST_ && a_mn == MN_) return launch_t<BN_, ST_, MN_>(ta, tb, tc, g, st);
-  SM_CASE(256, 3, false) SM_CASE(256, 4, false) SM_CASE(128, 4, false) SM_CASE(96, 6, false) SM_CASE(64, 6, false)
-  SM_CASE(256, 3, true) SM_CASE(256, 4, true) SM_CASE(128, 4, true)
+  SM_CASE(256, 3, false) SM_CASE(256, 4, false) SM_CASE(128, 5, false) SM_CASE(96, 7, false) SM_CASE(64, 8, false)
+  SM_CASE(256, 3, true) SM_CASE(256, 4, true) SM_CASE(128, 5, true)
 #undef SM_CASE
   return SMARTMEM_ERR_UNSUPPORTED;
 }

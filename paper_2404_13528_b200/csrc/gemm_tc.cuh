@@ -54,10 +54,10 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
                    long long N, long long K, cudaStream_t st);
 
 // GEMM for few rows, split along the reduction over the CTAs of a cluster (gemm_splitk.cu): plain row-major operands, every
-// epilogue but the second copy.  launch_gemm_tc hands over where gemm_splitk_wins.
+// epilogue but the second copy.  launch_gemm_tc hands over where gemm_splitk_us is below its own estimate.
 bool gemm_splitk_supported(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep, long long batch, long long M, long long N,
                            long long K);
-bool gemm_splitk_wins(long long M, long long N, long long K);
+double gemm_splitk_us(long long M, long long N, long long K);
 int launch_gemm_splitk(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep, long long M, long long N, long long K, cudaStream_t st);
 
 // bf16 row-major [outer, inner] matrix as a 2-D tensor map with 128-byte swizzle (box_inner = 64).
