@@ -59,7 +59,7 @@ constexpr int N_BARS = 18;
 constexpr int RSTD_RING = 4;                       // tiles whose rstd may be live at once (statistics run up to two tiles ahead of GELU)
 
 struct MlpArgs {
-  int M, C, hidden, n_chunks, tiles;
+  int M, C, hidden, n_chunks, tiles, w1_rows;
   uint32_t smem_bytes;
   const __nv_bfloat16 *b1, *b2, *ln_gamma, *ln_beta;
   float ln_eps;
@@ -154,15 +154,28 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     ptx::prefetch_tensormap(&tmA);
     ptx::prefetch_tensormap(&tmW1);
     ptx::prefetch_tensormap(&tmW2);
-    // the weights: parameters, not produced by the kernel before this one, so they are requested before the dependency wait
-    ptx::mbar_expect_tx(w1_full, (uint32_t)g.hidden * (uint32_t)C * 2u);
+  }
+  if (warp == 0) {
+    __syncwarp();
+    // The weights: parameters, not produced by the kernel before this one, so they are requested before the dependency wait, in
+    // few boxes issued by an elected lane (a box per chunk or k-block under a branch on thread 0 took 21 issues of about 0.2 us)
+    if (ptx::elect_one()) {
+      ptx::mbar_expect_tx(w1_full, (uint32_t)g.hidden * (uint32_t)C * 2u);
+      ptx::mbar_expect_tx(w2_full, (uint32_t)g.hidden * (uint32_t)C * 2u);
+    }
+    __syncwarp();
 #pragma unroll 1
     for (int kb = 0; kb < NKB; ++kb)
 #pragma unroll 1
-      for (int c = 0; c < NC; ++c) ptx::tma_load_2d(sW1 + kb * W1_KB + c * KBT, &tmW1, w1_full, kb * KB, c * HC);
-    ptx::mbar_expect_tx(w2_full, (uint32_t)g.hidden * (uint32_t)C * 2u);
+      for (int r = 0; r < g.hidden; r += g.w1_rows) {
+        if (ptx::elect_one()) ptx::tma_load_2d(sW1 + kb * W1_KB + r * 64, &tmW1, w1_full, kb * KB, r);
+        __syncwarp();
+      }
 #pragma unroll 1
-    for (int kb = 0; kb < g.hidden / KB; ++kb) ptx::tma_load_2d(sW2 + kb * W2_KB, &tmW2, w2_full, kb * KB, 0);
+    for (int kb = 0; kb < g.hidden / KB; kb += 4) {    // four k-blocks of 32 columns per box
+      if (ptx::elect_one()) ptx::tma_load_3d(sW2 + kb * W2_KB, &tmW2, w2_full, 0, 0, kb);
+      __syncwarp();
+    }
   }
 #pragma unroll 1
   for (int i = tid; i < C; i += kThreads) {
@@ -239,17 +252,20 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
   if (warp == 0) {
     // producer: the raw rows of the CTA's tiles, one tile ahead
-    if (lane == 0) {
+    {
       bool ok = true;
 #pragma unroll 1
       for (int ti = 0; ti < my_tiles && ok; ++ti) {
         const int b = ti & 1;
-        ok = ptx::mbar_wait_relaxed(&a_empty[b], ((ti >> 1) & 1) ^ 1, abort_flag, g.status);
+        ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait_relaxed(&a_empty[b], ((ti >> 1) & 1) ^ 1, abort_flag, g.status) ? 1 : 0) != 0;
         if (!ok) break;
         const int t = (int)blockIdx.x + ti * (int)gridDim.x;
-        ptx::mbar_expect_tx(&a_full[b], (uint32_t)A_BYTES);
-#pragma unroll 1
-        for (int kb = 0; kb < NKB; ++kb) ptx::tma_load_2d(sA + b * A_BYTES + kb * KBT, &tmA, &a_full[b], kb * KB, t * BM);
+        if (ptx::elect_one()) {
+          ptx::mbar_expect_tx(&a_full[b], (uint32_t)A_BYTES);
+#pragma unroll
+          for (int kb = 0; kb < NKB; ++kb) ptx::tma_load_2d(sA + b * A_BYTES + kb * KBT, &tmA, &a_full[b], kb * KB, t * BM);
+        }
+        __syncwarp();
       }
     }
   } else if (warp == 1) {
@@ -523,6 +539,7 @@ int launch_mlp_fused(const void* A, const void* ln_gamma, const void* ln_beta, f
   }
   CUtensorMap ta, tw1, tw2;
   int rc;
+  const int w1_rows = (int)(hidden <= 256 ? hidden : hidden / 2);                     // (a box has at most 256 rows)
   {
     const long long dims[2] = {C, M}, strides[1] = {C};
     const int box[2] = {KB, BM};
@@ -530,17 +547,17 @@ int launch_mlp_fused(const void* A, const void* ln_gamma, const void* ln_beta, f
   }
   {
     const long long dims[2] = {C, hidden}, strides[1] = {C};
-    const int box[2] = {KB, HC};
+    const int box[2] = {KB, w1_rows};
     if ((rc = tc_encode_nd_sw64(W1, 2, dims, strides, box, &tw1)) != SMARTMEM_OK) return rc;
   }
   {
-    const long long dims[2] = {hidden, C}, strides[1] = {hidden};
-    const int box[2] = {KB, (int)C};
-    if ((rc = tc_encode_nd_sw64(W2, 2, dims, strides, box, &tw2)) != SMARTMEM_OK) return rc;
+    const long long dims[3] = {KB, C, hidden / KB}, strides[2] = {hidden, KB};      // (column, row, k-block)
+    const int box[3] = {KB, (int)C, 4};
+    if ((rc = tc_encode_nd_sw64(W2, 3, dims, strides, box, &tw2)) != SMARTMEM_OK) return rc;
   }
   MlpArgs g;
   memset(&g, 0, sizeof(g));
-  g.M = (int)M; g.C = (int)C; g.hidden = (int)hidden; g.n_chunks = (int)(hidden / HC);
+  g.M = (int)M; g.C = (int)C; g.hidden = (int)hidden; g.n_chunks = (int)(hidden / HC); g.w1_rows = w1_rows;
   g.tiles = (int)((M + BM - 1) / BM);
   g.b1 = (const __nv_bfloat16*)b1; g.b2 = (const __nv_bfloat16*)b2;
   g.out = (__nv_bfloat16*)out;

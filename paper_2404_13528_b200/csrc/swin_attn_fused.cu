@@ -180,20 +180,24 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
     *abort_flag = 0;
     ptx::fence_barrier_init();
     ptx::fence_proxy_async();
-    // the weights do not depend on the kernel before this one: fetch them right away
-    ptx::prefetch_tensormap(&tmWq);
-    ptx::prefetch_tensormap(&tmWp);
     ptx::prefetch_tensormap(&tmX);
-    ptx::mbar_expect_tx(w_full, (uint32_t)(NH * NH * WQ_TILE + NH * WP_TILE));
+  }
+  if (warp == 0) {
+    __syncwarp();
+    // The weights do not depend on the kernel before this one: fetch them right away, in few boxes issued by an elected lane (a
+    // box per head, k-block and q / k / v under a branch on thread 0 took 30 issues of about 0.2 us)
+    if (ptx::elect_one()) ptx::mbar_expect_tx(w_full, (uint32_t)(NH * NH * WQ_TILE + NH * WP_TILE));
+    __syncwarp();
 #pragma unroll 1
-    for (int h = 0; h < NH; ++h)                       // (head, k-block, q / k / v): a box of 32 weight rows x 32 columns
+    for (int h = 0; h < NH; ++h) {
 #pragma unroll 1
-      for (int kb = 0; kb < NH; ++kb)
-#pragma unroll
-        for (int which = 0; which < 3; ++which)
-          ptx::tma_load_2d(sWq + (h * NH + kb) * WQ_TILE + which * (D * 64), &tmWq, w_full, kb * D, which * C + h * D);
-#pragma unroll 1
-    for (int h = 0; h < NH; ++h) ptx::tma_load_2d(sWp + h * WP_TILE, &tmWp, w_full, h * D, 0);
+      for (int kb = 0; kb < NH; ++kb) {                // (head, k-block): 32 columns x 32 weight rows each of q, k and v
+        if (ptx::elect_one()) ptx::tma_load_3d(sWq + (h * NH + kb) * WQ_TILE, &tmWq, w_full, kb * D, h * D, 0);
+        __syncwarp();
+      }
+      if (ptx::elect_one()) ptx::tma_load_2d(sWp + h * WP_TILE, &tmWp, w_full, h * D, 0);
+      __syncwarp();
+    }
   }
   if (warp == 0) ptx::tmem_alloc(tmem_slot, TMEM_COLS);
   // parameter-only tables
@@ -856,7 +860,9 @@ int launch_swin_attn_fused(const smartmem_swin_params_t& p, const DevMap& rowmap
   if (!p.rel_bias_table) return SMARTMEM_ERR_INVALID_ARG;
   CUtensorMap twq, twp, tx;
   int rc;
-  if ((rc = tc_encode_2d_sw64(p.w_qkv, C, 3 * C, C, D, D, &twq)) != SMARTMEM_OK) return rc;
+  const long long wq_dims[3] = {C, C, 3}, wq_strides[2] = {C, (long long)C * C};
+  const int wq_box[3] = {D, D, 3};
+  if ((rc = tc_encode_nd_sw64(p.w_qkv, 3, wq_dims, wq_strides, wq_box, &twq)) != SMARTMEM_OK) return rc;
   if ((rc = tc_encode_2d_sw64(p.w_proj, C, C, C, D, C, &twp)) != SMARTMEM_OK) return rc;
   memset(&tx, 0, sizeof(tx));
   const long long dims[4] = {C, p.W, p.H, p.B}, strides[3] = {C, (long long)p.W * C, (long long)p.H * p.W * C};
