@@ -1,9 +1,8 @@
 // Map-driven copy kernels: the consumer is the identity, so the kernel is exactly the
 // composed index map of an eliminated layout run (Section 3.2.1) applied on the load side.
 // They serve the copy-only chains and every materialised layout operator of EXPLICIT mode.
-#include <vector>
-
 #include "common.cuh"
+#include "gemm_tc.cuh"
 
 namespace smartmem {
 
@@ -133,7 +132,8 @@ struct TransposeArgs {
   FastDiv outer_ext[kMaxDevAtoms];
   long long outer_src[kMaxDevAtoms], outer_dst[kMaxDevAtoms];
   long long src_stride_i, dst_stride_j, base;
-  int tiles_i, tiles_j;
+  int tiles_i, tiles_j, ext_i, ext_j;
+  FastDiv fd_tiles_i, fd_tiles_j;
 };
 
 __global__ void __launch_bounds__(256) copy_transpose16_kernel(const __grid_constant__ TransposeArgs a,
@@ -180,6 +180,81 @@ __global__ void __launch_bounds__(256) copy_transpose16_kernel(const __grid_cons
   }
 }
 
+// The same for any extents: tiles at the edges are ragged, loads are LV and stores SV elements wide (the widest vectors that
+// divide the extents and every stride and offset of their side).  [4,256,57,57] -> channels last: 2-byte gathers through the
+// map took 34 us, the tiles (2-byte loads, 16-byte stores) take 8.
+template <int LV, int SV>
+__global__ void __launch_bounds__(256) copy_transpose_any_kernel(const __grid_constant__ TransposeArgs a, const uint16_t* __restrict__ src,
+                                                                 uint16_t* __restrict__ dst) {
+  constexpr int P = 66;                       // pitch of a tile row [j][i]: an odd number of words
+  __shared__ __align__(16) uint16_t tile[64 * P];
+  uint32_t b = blockIdx.x, q = fd_div(b, a.fd_tiles_j);
+  const int j0 = (int)(b - q * a.fd_tiles_j.d) * 64;
+  b = q;
+  q = fd_div(b, a.fd_tiles_i);
+  const int i0 = (int)(b - q * a.fd_tiles_i.d) * 64;
+  b = q;
+  long long so = a.base, dof = 0;
+  for (int k = a.n_outer - 1; k >= 0; --k) {
+    q = fd_div(b, a.outer_ext[k]);
+    const uint32_t digit = b - q * a.outer_ext[k].d;
+    b = q;
+    so += (long long)digit * a.outer_src[k];
+    dof += (long long)digit * a.outer_dst[k];
+  }
+  const int ni = min(64, a.ext_i - i0), nj = min(64, a.ext_j - j0);
+  pdl_wait();
+  pdl_launch_dependents();
+  using LT = typename VecT<2 * LV>::type;
+  {
+    constexpr int VPR = 64 / LV, RPP = 256 / VPR, PASSES = 64 / RPP;
+    const int jv = threadIdx.x % VPR * LV, ir = threadIdx.x / VPR;
+    LT v[PASSES];
+#pragma unroll
+    for (int p = 0; p < PASSES; ++p) {
+      const int i = ir + p * RPP;
+      if (i < ni && jv < nj) v[p] = *reinterpret_cast<const LT*>(src + so + (long long)(i0 + i) * a.src_stride_i + j0 + jv);
+    }
+#pragma unroll
+    for (int p = 0; p < PASSES; ++p) {
+      const int i = ir + p * RPP;
+      if (i < ni && jv < nj) {
+        const uint16_t* e = reinterpret_cast<const uint16_t*>(&v[p]);
+#pragma unroll
+        for (int k = 0; k < LV; ++k) tile[(jv + k) * P + i] = e[k];
+      }
+    }
+  }
+  __syncthreads();
+  {
+    using ST = typename VecT<2 * SV>::type;
+    constexpr int VPR = 64 / SV, RPP = 256 / VPR, PASSES = 64 / RPP;
+    const int iv = threadIdx.x % VPR * SV, jr = threadIdx.x / VPR;
+#pragma unroll
+    for (int p = 0; p < PASSES; ++p) {
+      const int j = jr + p * RPP;
+      if (j < nj && iv < ni) {
+        ST v;
+        if constexpr (SV == 1) {
+          v = tile[j * P + iv];
+        } else {
+          uint32_t* w = reinterpret_cast<uint32_t*>(&v);
+#pragma unroll
+          for (int k = 0; k < SV / 2; ++k) w[k] = *reinterpret_cast<const uint32_t*>(tile + j * P + iv + 2 * k);
+        }
+        *reinterpret_cast<ST*>(dst + dof + (long long)(j0 + j) * a.dst_stride_j + i0 + iv) = v;
+      }
+    }
+  }
+}
+
+template <int LV>
+void launch_transpose_any(int sv, dim3 grid, cudaStream_t st, const TransposeArgs& t, const uint16_t* src, uint16_t* dst) {
+  if (sv == 8) launch_pdl(copy_transpose_any_kernel<LV, 8>, grid, dim3(256), 0, st, t, src, dst);
+  else if (sv == 4) launch_pdl(copy_transpose_any_kernel<LV, 4>, grid, dim3(256), 0, st, t, src, dst);
+  else if (sv == 2) launch_pdl(copy_transpose_any_kernel<LV, 2>, grid, dim3(256), 0, st, t, src, dst);
+  else launch_pdl(copy_transpose_any_kernel<LV, 1>, grid, dim3(256), 0, st, t, src, dst);
+}
 
 // Batched transpose of small contiguous blocks: the last two consumer atoms are (J, I) of a
 // source block [I][J] that is contiguous (stride of I == extent of J), e.g. a materialised K^T of
@@ -293,7 +368,8 @@ int launch_copy_map(const smartmem_index_map_t& map, int elem_size, const void* 
     if (make_devmap(map, 0, n - 2, 1, true, &outer) && blocks < (1ll << 31)) {
       const int EI = (int)map.extent[n - 1], EJ = (int)map.extent[n - 2];
       const size_t smem = (size_t)EI * (EJ + 2) * 2;
-      if (smem <= 40000) {
+      // (a CTA per block: with few blocks the tiles below spread the work wider)
+      if (smem <= 40000 && blocks >= tc_sm_count()) {
       launch_pdl(copy_block_transpose16_kernel, dim3((unsigned)blocks), dim3(256), smem, st, outer, (const uint16_t*)src, (uint16_t*)dst, EI, EJ);
       count_launch();
       return cudaGetLastError() == cudaSuccess ? SMARTMEM_OK : SMARTMEM_ERR_CUDA;
@@ -325,34 +401,54 @@ int launch_copy_map(const smartmem_index_map_t& map, int elem_size, const void* 
     int J = -1;
     for (int a = 0; a < n - 1; ++a)
       if (map.src_stride[a] == 1) J = a;
-    if (J >= 0 && map.extent[n - 1] % 64 == 0 && map.extent[J] % 64 == 0 && n - 2 <= kMaxDevAtoms) {
+    if (J >= 0 && map.extent[n - 1] >= 8 && map.extent[J] >= 8 && n - 2 <= kMaxDevAtoms && map.extent[n - 1] < (1ll << 30) &&
+        map.extent[J] < (1ll << 30)) {
       TransposeArgs t;
       memset(&t, 0, sizeof(t));
-      std::vector<long long> cstride(n);
+      long long cstride[SMARTMEM_MAX_ATOMS];
       long long run = 1;
       for (int a = n - 1; a >= 0; --a) {
         cstride[a] = run;
         run *= map.extent[a];
       }
-      bool ok = map.base % 8 == 0 && map.src_stride[n - 1] % 8 == 0 && cstride[J] % 8 == 0;
+      // low bits set in any extent, stride or offset of a side limit the width of its vectors
+      unsigned long long src_bits = (unsigned long long)(map.base | map.src_stride[n - 1] | map.extent[J]);
+      unsigned long long dst_bits = (unsigned long long)(cstride[J] | map.extent[n - 1]);
+      bool ok = true;
       long long outer = 1;
       for (int a = 0; a < n - 1; ++a) {
         if (a == J) continue;
-        ok = ok && map.src_stride[a] % 8 == 0 && cstride[a] % 8 == 0 && map.extent[a] < (1ll << 31);
+        src_bits |= (unsigned long long)map.src_stride[a];
+        dst_bits |= (unsigned long long)cstride[a];
+        ok = ok && map.extent[a] < (1ll << 31);
         t.outer_ext[t.n_outer] = make_fastdiv((uint32_t)map.extent[a]);
         t.outer_src[t.n_outer] = map.src_stride[a];
         t.outer_dst[t.n_outer] = cstride[a];
         ++t.n_outer;
         outer *= map.extent[a];
       }
+      const int lv = src_bits % 8 == 0 ? 8 : src_bits % 4 == 0 ? 4 : src_bits % 2 == 0 ? 2 : 1;
+      const int sv = dst_bits % 8 == 0 ? 8 : dst_bits % 4 == 0 ? 4 : dst_bits % 2 == 0 ? 2 : 1;
       t.src_stride_i = map.src_stride[n - 1];
       t.dst_stride_j = cstride[J];
       t.base = map.base;
-      t.tiles_i = (int)(map.extent[n - 1] / 64);
-      t.tiles_j = (int)(map.extent[J] / 64);
-      long long blocks = outer * t.tiles_i * t.tiles_j;
+      t.ext_i = (int)map.extent[n - 1];
+      t.ext_j = (int)map.extent[J];
+      t.tiles_i = (t.ext_i + 63) / 64;
+      t.tiles_j = (t.ext_j + 63) / 64;
+      t.fd_tiles_i = make_fastdiv((uint32_t)t.tiles_i);
+      t.fd_tiles_j = make_fastdiv((uint32_t)t.tiles_j);
+      const long long blocks = outer * t.tiles_i * t.tiles_j;
       if (ok && blocks < (1ll << 31)) {
-        launch_pdl(copy_transpose16_kernel, dim3((unsigned)blocks), dim3(256), 0, st, t, (const uint16_t*)src, (uint16_t*)dst);
+        const dim3 grid((unsigned)blocks);
+        const uint16_t* s16 = (const uint16_t*)src;
+        uint16_t* d16 = (uint16_t*)dst;
+        if (lv == 8 && sv == 8 && t.ext_i % 64 == 0 && t.ext_j % 64 == 0)
+          launch_pdl(copy_transpose16_kernel, grid, dim3(256), 0, st, t, s16, d16);
+        else if (lv == 8) launch_transpose_any<8>(sv, grid, st, t, s16, d16);
+        else if (lv == 4) launch_transpose_any<4>(sv, grid, st, t, s16, d16);
+        else if (lv == 2) launch_transpose_any<2>(sv, grid, st, t, s16, d16);
+        else launch_transpose_any<1>(sv, grid, st, t, s16, d16);
         count_launch();
         return cudaGetLastError() == cudaSuccess ? SMARTMEM_OK : SMARTMEM_ERR_CUDA;
       }
