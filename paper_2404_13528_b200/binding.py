@@ -1,7 +1,8 @@
 """ctypes binding of the C ABI in include/smartmem.h.
 
 Argument marshalling only: every step of the hot path runs inside the CUDA library.  The
-functions keep the C names.  Device buffers are passed as integers (``tensor.data_ptr()``),
+functions keep the C names.  The calls a program makes per step go through a small CPython extension
+(csrc/fastcall.c) that converts their arguments without ctypes.  Device buffers are passed as integers (``tensor.data_ptr()``),
 streams as ``torch.cuda.current_stream().cuda_stream``.  If the shared library is missing
 the import of any entry point raises -- there is no fallback.
 """
@@ -75,6 +76,7 @@ EXPORTED = [
 ]
 
 _lib = None
+_fast = None                              # the CPython entry to the per-step calls, bound to the library's functions
 
 
 def lib() -> C.CDLL:
@@ -127,6 +129,17 @@ def lib() -> C.CDLL:
         f.restype, f.argtypes = res, args
     _lib = L
     return L
+
+
+def _bind_fast():
+    """Loads _fastcall.so (built next to the library) and hands it the addresses of the per-step calls."""
+    global _fast
+    L = lib()
+    from . import _fastcall
+    _fastcall.bind(*(C.cast(getattr(L, n), C.c_void_p).value for n in
+                     ("smartmem_swin_block", "smartmem_attn_layer", "smartmem_attn_decode", "smartmem_run_chain")))
+    _fast = _fastcall
+    return _fast
 
 
 class SmartmemError(RuntimeError):
@@ -248,9 +261,9 @@ def smartmem_plan_eval_sequential(plan: int, step: int, operand: int, i: int) ->
 
 def smartmem_run_chain(plan: int, inputs, outputs, workspace: int, workspace_bytes: int, stream: int):
     """inputs / outputs: lists of device pointers (ints)."""
-    ai = (C.c_void_p * len(inputs))(*inputs)
-    ao = (C.c_void_p * len(outputs))(*outputs)
-    _check(lib().smartmem_run_chain(plan, ai, ao, workspace, workspace_bytes, stream), "smartmem_run_chain")
+    rc = (_fast or _bind_fast()).run_chain(plan, inputs, outputs, workspace, workspace_bytes, stream)
+    if rc:
+        raise SmartmemError(rc, "smartmem_run_chain")
 
 
 def smartmem_swin_block_workspace_bytes(p: SwinParams, mode: int) -> int:
@@ -260,7 +273,9 @@ def smartmem_swin_block_workspace_bytes(p: SwinParams, mode: int) -> int:
 
 
 def smartmem_swin_block(p: SwinParams, x: int, y: int, workspace: int, workspace_bytes: int, mode: int, stream: int):
-    _check(lib().smartmem_swin_block(C.byref(p), x, y, workspace, workspace_bytes, mode, stream), "smartmem_swin_block")
+    rc = (_fast or _bind_fast()).swin_block(p, x, y, workspace, workspace_bytes, mode, stream)
+    if rc:
+        raise SmartmemError(rc, "smartmem_swin_block")
 
 
 def smartmem_swin_block_half(p: SwinParams, x: int, y: int, workspace: int, workspace_bytes: int, mode: int, half: int, stream: int):
@@ -299,7 +314,9 @@ def smartmem_attn_layer_workspace_bytes(p: AttnParams, mode: int) -> int:
 
 
 def smartmem_attn_layer(p: AttnParams, x: int, y: int, workspace: int, workspace_bytes: int, mode: int, stream: int):
-    _check(lib().smartmem_attn_layer(C.byref(p), x, y, workspace, workspace_bytes, mode, stream), "smartmem_attn_layer")
+    rc = (_fast or _bind_fast()).attn_layer(p, x, y, workspace, workspace_bytes, mode, stream)
+    if rc:
+        raise SmartmemError(rc, "smartmem_attn_layer")
 
 
 def smartmem_attn_decode_workspace_bytes(p: AttnParams, mode: int) -> int:
@@ -310,8 +327,9 @@ def smartmem_attn_decode_workspace_bytes(p: AttnParams, mode: int) -> int:
 
 def smartmem_attn_decode(p: AttnParams, pos: int, x: int, k_cache: int, v_cache: int, y: int, workspace: int,
                          workspace_bytes: int, mode: int, stream: int):
-    _check(lib().smartmem_attn_decode(C.byref(p), pos, x, k_cache, v_cache, y, workspace, workspace_bytes, mode, stream),
-           "smartmem_attn_decode")
+    rc = (_fast or _bind_fast()).attn_decode(p, pos, x, k_cache, v_cache, y, workspace, workspace_bytes, mode, stream)
+    if rc:
+        raise SmartmemError(rc, "smartmem_attn_decode")
 
 
 def smartmem_profile_begin():

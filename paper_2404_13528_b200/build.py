@@ -4,15 +4,17 @@ from __future__ import annotations
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libsmartmem.so")
+FASTCALL = os.path.join(HERE, "_fastcall.so")            # CPython entry to the per-step calls (csrc/fastcall.c)
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
-    "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC", 
+    "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC",
     "-cudart", "static",
 ]
 
@@ -22,11 +24,19 @@ def _sources():
 
 
 def _stale() -> bool:
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(FASTCALL):
         return True
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(FASTCALL))
     deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [os.path.join(ROOT, "include", "smartmem.h")]
     return any(os.path.getmtime(d) > t for d in deps)
+
+
+def build_fastcall() -> None:
+    cmd = [os.environ.get("CC", "gcc"), "-O2", "-shared", "-fPIC", "-Wall", "-I", sysconfig.get_paths()["include"], "-o", FASTCALL,
+           os.path.join(CSRC, "fastcall.c")]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("the C compiler failed:\n" + " ".join(cmd) + "\n" + r.stdout + r.stderr)
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
@@ -42,6 +52,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("nvcc failed:\n" + " ".join(cmd) + "\n" + r.stdout + r.stderr)
+    build_fastcall()
     if verbose:
         sys.stderr.write(r.stderr)
     return LIB
