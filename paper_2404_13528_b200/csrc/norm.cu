@@ -7,6 +7,7 @@
 
 #include "common.cuh"
 #include "gemm_tc.cuh"
+#include "ptx.cuh"
 
 namespace smartmem {
 namespace {
@@ -31,10 +32,8 @@ __device__ __forceinline__ void unpack8_bf16(const uint4& u, float (&f)[8]) {
 // lane l is vector l + k * LPR of the row, so a warp-wide load covers 32 / LPR rows with runs of
 // LPR * 16 contiguous bytes).  RPG rows per lane group are in flight together.  GENERIC: any row
 // length; the row is re-read from L1/L2 for each pass instead of being kept.
-// 16-bit elements stay packed in registers (16 instead of 32 per row slice) and are unpacked for each pass: with six CTAs
-// per SM the 12 544 rows of a 14 x 14 x 64 activation are all in flight in a single wave (four CTAs made it 1.3 waves).
 template <typename T, int LPR, bool RMS, int RPG, bool GENERIC>
-__global__ void __launch_bounds__(256, (!GENERIC && sizeof(T) == 2 && RPG == 1) ? 6 : 1) norm_kernel(const T* __restrict__ src, T* __restrict__ dst,
+__global__ void __launch_bounds__(256) norm_kernel(const T* __restrict__ src, T* __restrict__ dst,
                                                    const T* __restrict__ gamma, const T* __restrict__ beta, float eps,
                                                    long long rows, int C, int vpl, const __grid_constant__ DevMap rowmap,
                                                    int has_map) {
@@ -46,17 +45,7 @@ __global__ void __launch_bounds__(256, (!GENERIC && sizeof(T) == 2 && RPG == 1) 
   const long long row0 = (long long)blockIdx.x * (GPB * RPG) + grp;
   const int nvec = C / KV;
   const float invC = 1.0f / (float)C;
-  constexpr bool PACKED = !GENERIC && sizeof(T) == 2;       // (KV == 8: one 16-byte vector)
-  float v[PACKED ? 1 : RPG][PACKED ? 1 : NV][KV];
-  uint4 pv[PACKED ? RPG : 1][PACKED ? NV : 1];
-  auto slice = [&](int r, int k, float (&f)[KV]) {           // values of (row r, vector k) as fp32
-    if constexpr (PACKED) {
-      unpack8_bf16(pv[r][k], reinterpret_cast<float(&)[8]>(f));
-    } else {
-#pragma unroll
-      for (int e = 0; e < KV; ++e) f[e] = v[r][k][e];
-    }
-  };
+  float v[RPG][NV][KV];
   const T* s[RPG];
   bool active[RPG];
   float sum[RPG];
@@ -82,10 +71,7 @@ __global__ void __launch_bounds__(256, (!GENERIC && sizeof(T) == 2 && RPG == 1) 
 #pragma unroll
       for (int k = 0; k < NV; ++k) {
         const int vi = sub + k * LPR;
-        if constexpr (PACKED) {
-          pv[r][k] = make_uint4(0, 0, 0, 0);
-          if (k < vpl && active[r] && vi < nvec) pv[r][k] = *reinterpret_cast<const uint4*>(s[r] + vi * KV);
-        } else if (k < vpl && active[r] && vi < nvec) {
+        if (k < vpl && active[r] && vi < nvec) {
           ElemIO<T>::load(s[r] + vi * KV, v[r][k]);
         } else {
 #pragma unroll
@@ -100,10 +86,8 @@ __global__ void __launch_bounds__(256, (!GENERIC && sizeof(T) == 2 && RPG == 1) 
 #pragma unroll
       for (int k = 0; k < NV; ++k)
         if (k < vpl) {
-          float f[KV];
-          slice(r, k, f);
 #pragma unroll
-          for (int e = 0; e < KV; ++e) sum[r] += RMS ? f[e] * f[e] : f[e];
+          for (int e = 0; e < KV; ++e) sum[r] += RMS ? v[r][k][e] * v[r][k][e] : v[r][k][e];
         }
     } else {
       for (int vi = sub; vi < nvec && active[r]; vi += LPR) {
@@ -128,10 +112,8 @@ __global__ void __launch_bounds__(256, (!GENERIC && sizeof(T) == 2 && RPG == 1) 
         for (int k = 0; k < NV; ++k) {
           const int vi = sub + k * LPR;
           if (k < vpl && active[r] && vi < nvec) {
-            float f[KV];
-            slice(r, k, f);
 #pragma unroll
-            for (int e = 0; e < KV; ++e) sq += (f[e] - mean[r]) * (f[e] - mean[r]);
+            for (int e = 0; e < KV; ++e) sq += (v[r][k][e] - mean[r]) * (v[r][k][e] - mean[r]);
           }
         }
       } else {
@@ -163,11 +145,7 @@ __global__ void __launch_bounds__(256, (!GENERIC && sizeof(T) == 2 && RPG == 1) 
         if constexpr (!RMS) ElemIO<T>::load(beta + vi * KV, b);
 #pragma unroll
         for (int r = 0; r < RPG; ++r)
-          if (active[r]) {
-            float f[KV];
-            slice(r, k, f);
-            emit(r, vi, f, g, b);
-          }
+          if (active[r]) emit(r, vi, v[r][k], g, b);
       }
     }
   } else {
@@ -183,6 +161,146 @@ __global__ void __launch_bounds__(256, (!GENERIC && sizeof(T) == 2 && RPG == 1) 
         }
     }
   }
+}
+
+// bf16 rows of up to 1024 elements (LayerNorm and RMSNorm of the wide blocks and of the chains), read at one of three kinds of
+// offset: contiguous rows, whole rows through a row map (cyclic shift + window partition), or 16-byte vectors through a map
+// whose row boundary falls between two atoms -- there a vector's offset is the sum of a part that depends on the row
+// (evaluated once per row by one lane) and a part that depends on its place in the row (once per lane, before the loop).
+// What bounds it is instruction issue: packed fp32 pairs for all the arithmetic, LPR lanes
+// per row with NV vectors each so that no lane idles; a warp walks over several groups of rows and has the next group's
+// vectors in flight.
+__device__ __forceinline__ ptx::f32x2 widen2(uint32_t w) { return ptx::pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
+__device__ __forceinline__ float hsum2(ptx::f32x2 v) {
+  float lo, hi;
+  ptx::unpack2(v, lo, hi);
+  return lo + hi;
+}
+enum RowSource { ROWS_CONTIGUOUS = 0, ROWS_MAPPED = 1, VECTORS_MAPPED = 2 };
+
+template <bool RMS, int LPR, int NV, int SRC>
+__global__ void __launch_bounds__(256, NV <= 3 ? 3 : 2) norm_rows_kernel(const __nv_bfloat16* __restrict__ src, __nv_bfloat16* __restrict__ dst,
+                                                                         const __nv_bfloat16* __restrict__ gamma,
+                                                                         const __nv_bfloat16* __restrict__ beta, float eps, int rows, int C,
+                                                                         const __grid_constant__ DevMap map, int split) {
+  constexpr int RPW = 32 / LPR;                          // rows of a warp at a time
+  const int lane = threadIdx.x & 31, sub = lane % LPR;
+  const int nvec = C / 8;
+  const float invC = 1.0f / (float)C;
+  const int step = (int)gridDim.x * (8 * RPW);
+  const int row0 = ((int)blockIdx.x * 8 + (int)(threadIdx.x >> 5)) * RPW + lane / LPR;
+  // gamma and beta in shared memory, read anew for every row (in registers, and widened there by the compiler, they leave no
+  // room for the rows in flight)
+  __shared__ __align__(16) __nv_bfloat16 par[RMS ? 1 : 2][LPR * NV * 8];
+  for (int i = threadIdx.x; i < nvec; i += 256) {
+    *reinterpret_cast<uint4*>(&par[0][i * 8]) = *reinterpret_cast<const uint4*>(gamma + i * 8);
+    if constexpr (!RMS) *reinterpret_cast<uint4*>(&par[1][i * 8]) = *reinterpret_cast<const uint4*>(beta + i * 8);
+  }
+  int col[NV];                                           // element offset of vector k inside its row
+#pragma unroll
+  for (int k = 0; k < NV; ++k) {
+    const int vi = sub + k * LPR;
+    col[k] = vi * 8;
+    if (SRC == VECTORS_MAPPED && vi < nvec) col[k] = (int)devmap_part_rolled(map, split, map.n_atoms, (uint32_t)vi).off;
+  }
+  __syncthreads();
+  auto request = [&](int row, uint4 (&v)[NV]) {
+    long long off = (long long)row * C;
+    if constexpr (SRC != ROWS_CONTIGUOUS) {
+      off = 0;
+      if (sub == 0 && row < rows)
+        off = SRC == ROWS_MAPPED ? devmap_eval_unrolled(map, (uint32_t)row) : map.base + devmap_part_rolled(map, 0, split, (uint32_t)row).off;
+      off = __shfl_sync(0xFFFFFFFFu, off, lane - sub);
+    }
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      v[k] = make_uint4(0, 0, 0, 0);
+      if (sub + k * LPR < nvec && row < rows) v[k] = *reinterpret_cast<const uint4*>(src + off + col[k]);
+    }
+  };
+  pdl_wait();
+  pdl_launch_dependents();
+  uint4 x[NV], nx[NV];
+  request(row0, nx);
+  // (trip count uniform over the warp: the shuffles below)
+  for (int row = row0; row - lane / LPR < rows; row += step) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) x[k] = nx[k];
+    if (row - lane / LPR + step < rows) request(row + step, nx);
+    ptx::f32x2 s2[2] = {ptx::pack2(0.f, 0.f), ptx::pack2(0.f, 0.f)};
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const uint32_t w[4] = {x[k].x, x[k].y, x[k].z, x[k].w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s2[i & 1] = RMS ? ptx::fma2(widen2(w[i]), widen2(w[i]), s2[i & 1]) : ptx::add2(widen2(w[i]), s2[i & 1]);
+    }
+    const float sum = group_sum<LPR>(hsum2(ptx::add2(s2[0], s2[1])));
+    float mean = 0.f, rstd;
+    if constexpr (RMS) {
+      rstd = rsqrtf(sum * invC + eps);
+    } else {
+      mean = sum * invC;
+      const ptx::f32x2 nm = ptx::pack2(-mean, -mean);
+      s2[0] = s2[1] = ptx::pack2(0.f, 0.f);
+#pragma unroll
+      for (int k = 0; k < NV; ++k)
+        if (sub + k * LPR < nvec) {
+          const uint32_t w[4] = {x[k].x, x[k].y, x[k].z, x[k].w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const ptx::f32x2 d = ptx::add2(widen2(w[i]), nm);
+            s2[i & 1] = ptx::fma2(d, d, s2[i & 1]);
+          }
+        }
+      rstd = rsqrtf(group_sum<LPR>(hsum2(ptx::add2(s2[0], s2[1]))) * invC + eps);
+    }
+    // y = (x rstd - mean rstd) g + b in fp32, rounded once
+    const float ms = -mean * rstd;
+    const ptx::f32x2 rs2 = ptx::pack2(rstd, rstd), ms2 = ptx::pack2(ms, ms);
+    __nv_bfloat16* d = dst + (long long)row * C;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const int vi = sub + k * LPR;
+      if (vi < nvec && row < rows) {
+        const uint4 g = ptx::ld_shared_v4(&par[0][vi * 8]), b = RMS ? g : ptx::ld_shared_v4(&par[RMS ? 0 : 1][vi * 8]);
+        const uint32_t w[4] = {x[k].x, x[k].y, x[k].z, x[k].w}, gw[4] = {g.x, g.y, g.z, g.w}, bw[4] = {b.x, b.y, b.z, b.w};
+        uint32_t o[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          float lo, hi;
+          ptx::unpack2(RMS ? ptx::mul2(ptx::mul2(widen2(w[i]), rs2), widen2(gw[i])) : ptx::fma2(ptx::fma2(widen2(w[i]), rs2, ms2), widen2(gw[i]), widen2(bw[i])), lo, hi);
+          o[i] = float2_to_bf16x2(lo, hi);
+        }
+        *reinterpret_cast<uint4*>(d + vi * 8) = make_uint4(o[0], o[1], o[2], o[3]);
+      }
+    }
+  }
+}
+
+// LPR and NV by the number of vectors of a row; the grid is what is resident at once.
+template <bool RMS, int SRC>
+int launch_norm_rows(const void* src, void* dst, const void* gamma, const void* beta, float eps, long long rows, int C, const DevMap& map,
+                     int split, cudaStream_t st) {
+  const int nvec = C / 8;
+#define SM_ROWS(LPR, NV)                                                                                                       \
+  {                                                                                                                            \
+    constexpr int rpb = 8 * (32 / LPR);                                                                                        \
+    const long long blocks = (rows + rpb - 1) / rpb, slots = (NV <= 3 ? 3ll : 2ll) * tc_sm_count();                            \
+    launch_pdl(norm_rows_kernel<RMS, LPR, NV, SRC>, dim3((unsigned)(blocks < slots ? blocks : slots)), dim3(256), 0, st,       \
+               (const __nv_bfloat16*)src, (__nv_bfloat16*)dst, (const __nv_bfloat16*)gamma, (const __nv_bfloat16*)beta, eps,   \
+               (int)rows, C, map, split);                                                                                      \
+  }
+  if (nvec <= 8) SM_ROWS(8, 1)
+  else if (nvec <= 16) SM_ROWS(8, 2)
+  else if (nvec <= 24) SM_ROWS(8, 3)
+  else if (nvec <= 32) SM_ROWS(16, 2)
+  else if (nvec <= 48) SM_ROWS(16, 3)
+  else if (nvec <= 64) SM_ROWS(32, 2)
+  else if (nvec <= 96) SM_ROWS(32, 3)
+  else SM_ROWS(32, 4)
+#undef SM_ROWS
+  count_launch();
+  return cudaGetLastError() == cudaSuccess ? SMARTMEM_OK : SMARTMEM_ERR_CUDA;
 }
 
 // Wide rows (more than 128 vectors): one CTA per row, every thread keeps up to 4 of the row's 16-byte
@@ -357,6 +475,14 @@ int launch_norm_t(const void* src, void* dst, const void* gamma, const void* bet
     unsigned grid = (unsigned)((rows + rpb - 1) / rpb);                                                   \
     launch_pdl(norm_kernel<T, LPR, RMS, RPG, GEN>, dim3(grid), dim3(256), 0, st, s, d, g, b, eps, rows, C, vpl, dm, has);     \
   }
+  if constexpr (sizeof(T) == 2) {
+    if (nvec <= 128)
+      return rowmap ? launch_norm_rows<RMS, ROWS_MAPPED>(src, dst, gamma, beta, eps, rows, C, dm, 0, st)
+                    : launch_norm_rows<RMS, ROWS_CONTIGUOUS>(src, dst, gamma, beta, eps, rows, C, dm, 0, st);
+    if (!rowmap && nvec <= 1024)
+      launch_pdl(norm_wide_kernel<T, RMS>, dim3((unsigned)rows), dim3(256), 0, st, s, d, g, b, eps, C);
+    else SM_LAUNCH(32, 1, true)
+  } else {
   if (nvec <= 16) SM_LAUNCH(4, 1, false)
   else if (nvec <= 32) SM_LAUNCH(8, 2, false)
   else if (nvec <= 64) SM_LAUNCH(16, 1, false)
@@ -364,6 +490,7 @@ int launch_norm_t(const void* src, void* dst, const void* gamma, const void* bet
   else if (!rowmap && nvec <= 1024)
     launch_pdl(norm_wide_kernel<T, RMS>, dim3((unsigned)rows), dim3(256), 0, st, s, d, g, b, eps, C);
   else SM_LAUNCH(32, 1, true)
+  }
 #undef SM_LAUNCH
   count_launch();
   return cudaGetLastError() == cudaSuccess ? SMARTMEM_OK : SMARTMEM_ERR_CUDA;
@@ -555,6 +682,13 @@ int launch_norm_map_t(const void* src, void* dst, const void* gamma, const void*
   DevMap dm;
   if (!make_devmap(map, 0, map.n_atoms, KV, true, &dm)) return SMARTMEM_ERR_UNSUPPORTED;
   const int nvec = C / KV;
+  if constexpr (sizeof(T) == 2) {
+    const int split = devmap_split(dm, nvec);             // (C <= 1024: a row is at most 128 vectors)
+    long long reach = 0;                                  // the largest offset inside a row
+    for (int a = split; split >= 0 && a < dm.n_atoms; ++a) reach += (long long)(dm.ext[a].d - 1) * (dm.stride[a] < 0 ? -dm.stride[a] : dm.stride[a]);
+    if (split >= 0 && dm.n_rolls == 0 && reach < (1ll << 31))
+      return launch_norm_rows<false, VECTORS_MAPPED>(src, dst, gamma, beta, eps, rows, C, dm, split, st);
+  }
 #define SM_NG(NV_, RPW_)                                                                                             \
   launch_pdl(norm_gather_kernel<T, false, NV_, RPW_>, dim3((unsigned)((rows + 8 * RPW_ - 1) / (8 * RPW_))), dim3(256), 0, st, \
              (const T*)src, (T*)dst, (const T*)gamma, (const T*)beta, eps, rows, C, dm);
