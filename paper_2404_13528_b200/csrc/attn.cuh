@@ -33,6 +33,13 @@ __device__ __forceinline__ int region_label2(int ty, int tx, int ws, int wy, int
 }
 #endif
 
+// The halves of an fp32 block in one kernel each (swin_f32.cu).  The attention half gathers and scatters its rows through
+// `rowmap` (windowed row -> element offset of the token in x and y).
+bool swin_attn_f32_supported(int C, int heads, int window);
+bool swin_mlp_f32_supported(int C, long long hidden);
+int launch_swin_attn_f32(const smartmem_swin_params_t& p, const DevMap& rowmap, const void* x, void* y, cudaStream_t st);
+int launch_swin_mlp_f32(const smartmem_swin_params_t& p, const void* x, void* y, long long M, cudaStream_t st);
+
 // Causal attention over [S] positions for `heads` heads of dimension 128 (bf16).
 struct CausalAttnArgs {
   AttnOperand q, k, v, o;   // n = batch, h = head

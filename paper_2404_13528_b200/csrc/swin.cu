@@ -93,9 +93,11 @@ struct Path {
 Path choose_path(const smartmem_swin_params_t& p, int mode) {
   const bool bf16 = p.dtype == SMARTMEM_BF16;
   Path t;
-  t.fuse_attn = mode == SMARTMEM_ELIMINATE && swin_attn_fused_supported(p.dtype, p.C, p.heads, p.window);
+  t.fuse_attn = mode == SMARTMEM_ELIMINATE && (bf16 ? swin_attn_fused_supported(p.dtype, p.C, p.heads, p.window)
+                                                    : swin_attn_f32_supported(p.C, p.heads, p.window));
   t.fuse_ln1 = bf16 && gemm_ln_supported(3 * (long long)p.C, p.C);
-  t.fuse_mlp = bf16 && p.mlp_ratio > 0 && mlp_fused_supported(p.C, (long long)p.C * p.mlp_ratio);
+  t.fuse_mlp = p.mlp_ratio > 0 && (bf16 ? mlp_fused_supported(p.C, (long long)p.C * p.mlp_ratio)
+                                        : swin_mlp_f32_supported(p.C, (long long)p.C * p.mlp_ratio));
   return t;
 }
 
@@ -242,7 +244,7 @@ int run_block(const smartmem_swin_params_t* pp, const void* x, void* y, void* wo
     // MLP half only
   } else if (path.fuse_attn) {
     // narrow blocks: the whole attention half in one kernel (rows gathered and scattered through the composed map)
-    SM_TRY("attn_half_fused", launch_swin_attn_fused(p, m.e1_rows, x, y1, st));
+    SM_TRY("attn_half_fused", f32 ? launch_swin_attn_f32(p, m.e1_rows, x, y1, st) : launch_swin_attn_fused(p, m.e1_rows, x, y1, st));
   } else if (elim) {
     if (fuse_ln1) {
       // narrow blocks: LN1, the shift o partition gather and the QKV projection in one kernel
@@ -299,7 +301,7 @@ int run_block(const smartmem_swin_params_t* pp, const void* x, void* y, void* wo
       // narrow blocks: LN2 + fc1 + GELU + fc2 + residual in one kernel; neither the normalised rows
       // nor the hidden activation leave the chip
       SM_TRY("mlp_fused_ln2_fc1_gelu_fc2_residual",
-             launch_mlp_fused(y1, p.ln2_g, p.ln2_b, p.ln_eps, p.w_fc1, p.b_fc1, p.w_fc2, p.b_fc2, y, M, C, hid, st));
+             f32 ? launch_swin_mlp_f32(p, y1, y, M, st) : launch_mlp_fused(y1, p.ln2_g, p.ln2_b, p.ln_eps, p.w_fc1, p.b_fc1, p.w_fc2, p.b_fc2, y, M, C, hid, st));
     } else {
       SM_TRY("ln2", launch_norm(p.dtype, false, y1, at(L.yn), p.ln2_g, p.ln2_b, p.ln_eps, M, (int)C, nullptr, st));
       SM_TRY("fc1_gemm_gelu", linear(at(L.yn), p.w_fc1, p.b_fc1, at(L.hid), hid, C, 1, nullptr, nullptr));
