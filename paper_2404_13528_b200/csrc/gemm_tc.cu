@@ -137,7 +137,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   // lean epilogue: a 32 x 32 output box per epilogue warp (64-byte rows, 64-byte swizzle), right behind the ring
   constexpr int CBOX_BYTES = 32 * 64;
   uint8_t* cstage = sB + STAGES * B_STAGE_BYTES;
-  uint64_t* full = reinterpret_cast<uint64_t*>(cstage + (LEAN ? kEpiWarps * CBOX_BYTES : 0));
+  // two-stage kernel: two staging tiles of 128 x 256, each four lane quadrants of four 32 x 64 boxes (128-byte rows and swizzle)
+  constexpr bool QTMA = STAGES == 2;
+  constexpr int QTILE_BYTES = 4 * 32 * 512;
+  uint64_t* full = reinterpret_cast<uint64_t*>(cstage + (LEAN ? kEpiWarps * CBOX_BYTES : QTMA ? 2 * QTILE_BYTES : 0));
   uint64_t* empty = full + STAGES;
   uint64_t* tmem_full = empty + STAGES;                      // [2]
   uint64_t* tmem_empty = tmem_full + 2;                      // [2]
@@ -170,7 +173,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   if (warp == 0 && lane == 0) {
     ptx::prefetch_tensormap(&tmA);
     ptx::prefetch_tensormap(&tmB);
-    if (LEAN && g.tma_out) ptx::prefetch_tensormap(&tmC);
+    if (QTMA || (LEAN && g.tma_out)) ptx::prefetch_tensormap(&tmC);
   }
   if (warp == 1) {
     if constexpr (PAIR) ptx::tmem_alloc_pair(tmem_slot, TMEM_COLS);
@@ -334,7 +337,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int q = warp & 3;                                  // TMEM lane quadrant this warp may read
     const int grp = e >> 2;
     constexpr bool QSTAGE = !DIRECT && !(BN == 256 && STAGES == 4);  // per-quadrant staging of whole rows
-    constexpr bool QBULK = BN == 256 && !A_MN;               // staged rows leave as bulk copies (512-byte rows; not the MN-major-A kernel: 13.1 vs 12.1 us)
+    constexpr bool QBULK = BN == 256 && !A_MN && !QTMA;      // staged rows leave as bulk copies (512-byte rows; not the MN-major-A kernel: 13.1 vs 12.1 us)
     constexpr int QROW = BN * 2 + 16;                        // bytes; the pad keeps phase 1 conflict-free
     uint8_t* stage = stage_base + e * (32 * STG_ROW);
     uint8_t* qstage = stage_base + q * (32 * QROW);
@@ -427,6 +430,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if (!ok) break;
       ptx::tc_fence_after();
       const uint32_t taddr = tmem_base + buf * ACC_COLS + ((uint32_t)(q * 32) << 16);
+      uint8_t* qtile = cstage + (it & 1) * QTILE_BYTES + q * (QTILE_BYTES / 4);
+      if constexpr (QTMA) {
+        // the boxes that left this staging tile two tiles ago have been read
+        if (lane == 0) ptx::bulk_wait_group_read<1>();
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory");
+      }
       if constexpr (QSTAGE && QBULK) {
         // the previous tile's row copies have read the staging rows before anyone overwrites them
         if (lane < 8) ptx::bulk_wait_group_read<0>();
@@ -567,6 +576,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             } else {
               pk_prev = pk;
             }
+          } else if constexpr (QTMA) {
+            const int c = c0 + v * 8;
+            *reinterpret_cast<uint4*>(qtile + (c >> 6) * 4096 + lane * 128 + ((((c & 63) >> 3) ^ (lane & 7)) << 4)) = pk;
           } else if constexpr (QSTAGE) *reinterpret_cast<uint4*>(qstage + lane * QROW + (c0 + v * 8) * 2) = pk;
           else *reinterpret_cast<uint4*>(stage + lane * STG_ROW + v * 16) = pk;
         }
@@ -593,7 +605,18 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           else ptx::mbar_arrive(&tmem_empty[buf]);
         }
       }
-      if constexpr (QSTAGE && QBULK) {
+      if constexpr (QTMA) {
+        // Very short reductions (batched q k^T): the tile's store is all there is, and with one staging tile the store path
+        // idled while the next tile was converted.  Two tiles, and a warp sends one 32 x 64 box of its quadrant (rows and
+        // columns past the edge are clipped): 8 x 16 heads, 1024 x 1024 scores of 64: 70.5 -> 52 us.
+        ptx::fence_proxy_async();
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory");
+        if (lane == 0) {
+          if ((int)tile_m * BM + q * 32 < g.M && n0 + grp * 64 < g.N)
+            ptx::tma_store_3d(&tmC, qtile + grp * 4096, n0 + grp * 64, (int)tile_m * BM + q * 32, (int)batch);
+          ptx::bulk_commit_group();
+        }
+      } else if constexpr (QSTAGE && QBULK) {
         // the four warps of the quadrant have filled a 32 x 256 staging tile: every 512-byte row leaves as one bulk copy
         // (shared memory -> global), eight rows per warp, so no thread spends instructions on moving the tile.  Measured:
         // the batched q k^T GEMM 78.4 -> 72.6 us; on 192-byte rows (the 96-wide scatter GEMM) the same was slower, 22.3 vs
@@ -800,7 +823,7 @@ int launch_t(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc
   constexpr bool QST = !PAIR && !(BN == 256 && STAGES == 4);
   constexpr int RCc = !QST ? 16 : ((BN / 4) > 32 ? 32 : (BN / 4));
   constexpr size_t smem = 1024 + STAGES * (A_STAGE_BYTES + (PAIR ? BN / 2 : BN) * BK * 2) + (2 * STAGES + 4) * 8 + 16 +
-                          (LEAN ? kEpiWarps * 32 * 64 : PAIR ? 0 : !QST ? kEpiWarps * 32 * (RCc * 2 + 16) : 4 * 32 * (BN * 2 + 16));   // pairs store from registers
+                          (LEAN ? kEpiWarps * 32 * 64 : PAIR ? 0 : STAGES == 2 ? 2 * 4 * 32 * 512 : !QST ? kEpiWarps * 32 * (RCc * 2 + 16) : 4 * 32 * (BN * 2 + 16));   // pairs store from registers
   if (ensure_max_dynamic_smem((const void*)gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN>, (int)smem) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   profile_tick("gemm_tc", st);
   const long long tiles = (long long)g.tiles_n * g.tiles_m * g.batch;
@@ -961,6 +984,7 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
     // reads as many operand bytes per product as shared memory delivers, so over a long K the wider tile wins even with a
     // ragged last wave (measured at K = 2048)
     if (ep.rope_cols > 0) bn = 256;
+    else if (nkb <= 2 && N >= 192 && !a_mn && tiles_m1 * batch * ((N + 255) / 256) >= tc_sm_count()) bn = 256;   // bound by its stores
     else if (N % 256 == 0) {
       const long long tm = tiles_m1 * batch, sms = tc_sm_count();
       const long long w256 = (tm * (N / 256) + sms - 1) / sms, w128 = (tm * (N / 128) + sms - 1) / sms;
@@ -979,7 +1003,8 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
   }
   // single CTAs: 256 wide, short K: wider store rounds instead of a 4th stage.  Narrow tiles: their stages are
   // small, and a tile is consumed faster than a load's latency, so the ring runs several tiles ahead.
-  const int stages = bn == 256 ? (nkb <= 4 ? 3 : 4) : bn == 64 ? 8 : bn == 96 ? 7 : 5;
+  const bool plain_out = !pair && !a_mn && !ep.rowmap && ep.seg_cols == 0 && !ep.out2;
+  int stages = bn == 256 ? (nkb <= 2 && plain_out ? 2 : nkb <= 4 ? 3 : 4) : bn == 64 ? 8 : bn == 96 ? 7 : 5;
   GemmArgs g;
   memset(&g, 0, sizeof(g));
   CUtensorMap ta, tb;
@@ -1029,6 +1054,13 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
   }
   if (pair && bn == 256) return launch_t<256, 6, false, true>(ta, tb, tc, g, st);
   if (pair) return launch_t<128, 8, false, true>(ta, tb, tc, g, st);
+  if (stages == 2) {
+    const uint64_t dims[3] = {(uint64_t)N, (uint64_t)M, (uint64_t)batch};
+    const uint64_t strides[2] = {(uint64_t)ep.ldc * 2, (uint64_t)(batch > 1 ? ep.out_batch_stride : ep.ldc * M) * 2};
+    const uint32_t box[3] = {64, 32, 1};
+    if (encode_cached(ep.out, 3, dims, strides, box, &tc) == SMARTMEM_OK) return launch_t<256, 2, false>(ta, tb, tc, g, st);
+    stages = 3;
+  }
 #define SM_CASE(BN_, ST_, MN_)                                                                  \
   if (bn == BN_ && stages == ST_ && a_mn == MN_) return launch_t<BN_, ST_, MN_>(ta, tb, tc, g, st);
   SM_CASE(256, 3, false) SM_CASE(256, 4, false) SM_CASE(128, 5, false) SM_CASE(96, 7, false) SM_CASE(64, 8, false)

@@ -1,0 +1,59 @@
+"""GPU parity of the row-norm, ragged-transpose, batched-score and fp32 block kernels at the edges of their tiles."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import chains
+from paper_2404_13528_b200 import binding as sm
+from paper_2404_13528_b200 import synth
+from tests.gpu_util import assert_close_bf16, to_dev, to_host_bits, to_host_f64
+from tests.test_gpu_chains import CH2A, CH2B, patch_merging_case, run_plan
+from tests.test_gpu_swin import case
+from tests.test_planner import _ops_from_chain
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,C,H,W", [
+    (3, 9, 5, 13),            # odd on both sides: 2-byte loads and stores
+    (2, 66, 8, 9),            # 16-byte loads, 4-byte stores, two tiles each way
+    (1, 136, 7, 10),          # 4-byte loads, 16-byte stores; one image
+    (2, 100, 3, 4),           # a tile shorter than a pass
+    (4, 64, 8, 8), (1, 8, 1, 8),
+])
+def test_ragged_channels_last_copies_bit_exact(B, C, H, W):
+    x = synth.normal(501, 0, (B, C, H, W), dtype="bf16")
+    chain = CH2B(B, C, H, W)
+    out = run_plan(_ops_from_chain(chain) + [sm.make_op(sm.OP_COPY)], [sm.make_desc((B, C, H, W))], sm.ELIMINATE, [to_dev(x)], (B, H * W, C))
+    assert np.array_equal(to_host_bits(out), chains.apply_layout_chain(x, chain))
+
+
+@pytest.mark.parametrize("B,S,H,D", [
+    (20, 200, 8, 64),         # one 256-wide tile per 128 rows, clipped at row and column 200
+    (40, 136, 4, 32), (10, 264, 16, 128),   # the shortest reduction; two k-blocks, eight columns in the second tile
+])
+def test_batched_scores_clipped_tiles(B, S, H, D):
+    q = synth.normal(502, 0, (B, S, H * D), dtype="bf16")
+    k = synth.normal(502, 1, (B, S, H * D), dtype="bf16")
+    ops = _ops_from_chain(CH2A(B, S, H, D)) + [sm.make_op(sm.OP_BMM_NT, side_input=(1, 0))]
+    out = run_plan(ops, [sm.make_desc((B, S, H * D))] * 2, sm.ELIMINATE, [to_dev(q), to_dev(k)], (B, H, S, S))
+    ref = chains.chain_2a_scores(synth.to_f64(q), synth.to_f64(k), H)
+    assert_close_bf16(to_host_f64(out), ref, f"{B} x {S}")
+
+
+@pytest.mark.parametrize("C", [8, 24, 40, 64, 72, 136, 192, 256])
+def test_row_norm_widths(C):
+    """4 C from 32 to 1024 elements: every split of a row over lanes, with and without idle ones."""
+    patch_merging_case(2, 6, 10, C)
+
+
+@pytest.mark.parametrize("cfg", [
+    dict(B=2, H=14, W=21, C=96, heads=3, window=7, shift=3, mlp_ratio=4),     # three CTAs per window, ragged last 16 rows
+    dict(B=1, H=8, W=16, C=64, heads=2, window=8, shift=4, mlp_ratio=2),      # T = 64
+    dict(B=1, H=7, W=7, C=32, heads=1, window=7, shift=0, mlp_ratio=1),       # no cluster in the attention half
+    dict(B=1, H=6, W=4, C=128, heads=8, window=2, shift=1, mlp_ratio=4),      # T = 4, eight heads
+    dict(B=1, H=4, W=4, C=192, heads=6, window=4, shift=2, mlp_ratio=4),      # hidden features over eight CTAs
+    dict(B=1, H=4, W=4, C=320, heads=10, window=4, shift=0, mlp_ratio=4),     # beyond both kernels: kernel by kernel
+])
+def test_fp32_blocks(cfg):
+    case(503, dtype="f32", **cfg)
