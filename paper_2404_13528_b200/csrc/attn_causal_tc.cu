@@ -1,7 +1,7 @@
 // Causal attention (prefill, head dimension 128) on the tcgen05 tensor cores.
 //
 // One CTA = 128 query positions of one head.  K and V stream through shared memory in tiles of
-// 64 keys (TMA, double buffered); S = Q K^T and O += P V are tcgen05.mma with the accumulators in
+// 64 keys (TMA, three stages of keys, two of values); S = Q K^T and O += P V are tcgen05.mma with the accumulators in
 // TMEM (two S buffers, one O: 256 columns); four softmax warps own one query row per thread (the TMEM lane),
 // so row maxima and sums need no shuffles.  P goes back to the tensor core through tensor memory: it is
 // written as bf16 pairs over the S buffer it was computed from and read by the second MMA as its A
@@ -10,7 +10,7 @@
 // refreshed when it grows by more than 2^8 (then O and the running sum are rescaled), which keeps
 // the TMEM read-modify-write of O off the common path.
 //
-// The 64-key tiles keep a CTA at 96 KB of shared memory and 256 TMEM columns, so TWO CTAs share an
+// The 64-key tiles keep a CTA at 112 KB of shared memory and 256 TMEM columns, so TWO CTAs share an
 // SM: while one is in its softmax (which is bound by the exponential unit) the other one's MMAs
 // run, which a single CTA with one softmax group could not overlap.
 //
@@ -29,6 +29,8 @@ constexpr int BQ = 128, BKV = 64, D = 128;
 constexpr int KB = 128 * 64 * 2;                      // one 128 x 64 bf16 block (Q, P)
 constexpr int KBK = BKV * 64 * 2;                     // one 64 x 64 bf16 block (K, V)
 constexpr uint32_t TM_S = 0, TM_O = 128, TMEM_COLS = 256;   // two S buffers of 64 columns, O of 128: two CTAs share an SM's 512
+constexpr int KSTAGES = 3, N_BARS = 1 + 2 * KSTAGES + 4 + 4 + 3;
+constexpr uint32_t SMEM_BYTES = 2 * KB + (2 * KSTAGES + 4) * KBK + N_BARS * 8 + 16;
 constexpr int kThreads = 192;
 constexpr float kRescaleThreshold = 8.0f;             // log2 units
 
@@ -49,6 +51,12 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float y;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+  return y;
+}
+
 __global__ void __launch_bounds__(kThreads, 2)
 causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                       const __grid_constant__ CUtensorMap tmV, const __grid_constant__ TcAttnArgs g) {
@@ -56,15 +64,15 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   const uint32_t pad = (1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u;
   uint8_t* smem = smem_raw + pad;
   uint8_t* sQ = smem;                                  // [2 k-blocks][16 KB]
-  uint8_t* sK = sQ + 2 * KB;                           // [2 stages][2 k-blocks][8 KB]
-  uint8_t* sV = sK + 4 * KBK;                          // [2 stages][2 d-chunks][8 KB]
+  uint8_t* sK = sQ + 2 * KB;                           // [3 stages][2 k-blocks][8 KB]
+  uint8_t* sV = sK + 2 * KSTAGES * KBK;                // [2 stages][2 d-chunks][8 KB]
   uint64_t* bars = reinterpret_cast<uint64_t*>(sV + 4 * KBK);
-  uint64_t *q_full = bars, *k_full = bars + 1, *k_empty = bars + 3, *v_full = bars + 5, *v_empty = bars + 7;
-  uint64_t *s_full = bars + 9, *s_empty = bars + 11, *p_full = bars + 13, *p_empty = bars + 14, *o_done = bars + 15;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
+  uint64_t *q_full = bars, *k_full = bars + 1, *k_empty = k_full + KSTAGES, *v_full = k_empty + KSTAGES, *v_empty = v_full + 2;
+  uint64_t *s_full = v_empty + 2, *s_empty = s_full + 2, *p_full = s_empty + 2, *p_empty = p_full + 1, *o_done = p_empty + 1;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + N_BARS);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
 
-  if (pad + 2 * KB + 8 * KBK + 16 * 8 + 16 > g.smem_bytes) {
+  if (pad + SMEM_BYTES > g.smem_bytes) {
     if (threadIdx.x == 0) atomicExch(g.status, (int)SMARTMEM_ERR_UNSUPPORTED);
     return;
   }
@@ -79,9 +87,11 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
 
   if (threadIdx.x == 0) {
     ptx::mbar_init(q_full, 1);
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < KSTAGES; ++i) {
       ptx::mbar_init(&k_full[i], 1);
       ptx::mbar_init(&k_empty[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
       ptx::mbar_init(&v_full[i], 1);
       ptx::mbar_init(&v_empty[i], 1);
       ptx::mbar_init(&s_full[i], 1);
@@ -108,23 +118,37 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   pdl_launch_dependents();
 
   if (warp == 0) {
-    if (lane == 0) {
-      const int qc = g.q_col0 + h * g.col_per_head, kc = g.k_col0 + h * g.col_per_head, vc = g.v_col0 + h * g.col_per_head;
+    // Keys run a tile ahead of the values, one copy per tile of each, issued by an elected lane of a warp-uniform loop: with two
+    // stages of both, four copies a tile issued under a branch on one lane and K(j + 1) behind the wait for V(j), a tile's keys
+    // arrived 1.9 us after the products that freed their stage -- the period of a tile (S = 2048, 32 heads: 53 us).
+    const int qc = (g.q_col0 + h * g.col_per_head) / 64, kc = (g.k_col0 + h * g.col_per_head) / 64, vc = (g.v_col0 + h * g.col_per_head) / 64;
+    if (ptx::elect_one()) {
       ptx::mbar_expect_tx(q_full, 2 * KB);
-      for (int kb = 0; kb < 2; ++kb) ptx::tma_load_2d(sQ + kb * KB, &tmQ, q_full, qc + kb * 64, (int)(row_base + qt * BQ));
-      bool ok = true;
-      for (int j = 0; j < n_kv && ok; ++j) {
-        const int s = j & 1;
-        const uint32_t ph = (j >> 1) & 1;
-        const int krow = (int)(row_base + (long long)j * BKV);
-        ok = ptx::mbar_wait(&k_empty[s], ph ^ 1, abort_flag, g.status);
+      ptx::tma_load_3d(sQ, &tmQ, q_full, 0, (int)(row_base + qt * BQ), qc);
+    }
+    __syncwarp();
+    bool ok = true;
+    uint32_t ks = 0, kph = 1;
+    for (int i = -1; i < n_kv && ok; ++i) {
+      if (i + 1 < n_kv) {
+        ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(&k_empty[ks], kph, abort_flag, g.status) ? 1 : 0) != 0;
         if (!ok) break;
-        ptx::mbar_expect_tx(&k_full[s], 2 * KBK);
-        for (int kb = 0; kb < 2; ++kb) ptx::tma_load_2d(sK + (s * 2 + kb) * KBK, &tmK, &k_full[s], kc + kb * 64, krow);
-        ok = ptx::mbar_wait(&v_empty[s], ph ^ 1, abort_flag, g.status);
+        if (ptx::elect_one()) {
+          ptx::mbar_expect_tx(&k_full[ks], 2 * KBK);
+          ptx::tma_load_3d(sK + ks * 2 * KBK, &tmK, &k_full[ks], 0, (int)(row_base + (long long)(i + 1) * BKV), kc);
+        }
+        __syncwarp();
+        if (++ks == KSTAGES) { ks = 0; kph ^= 1; }
+      }
+      if (i >= 0) {
+        const int s = i & 1;
+        ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(&v_empty[s], ((i >> 1) & 1) ^ 1, abort_flag, g.status) ? 1 : 0) != 0;
         if (!ok) break;
-        ptx::mbar_expect_tx(&v_full[s], 2 * KBK);
-        for (int dc = 0; dc < 2; ++dc) ptx::tma_load_2d(sV + (s * 2 + dc) * KBK, &tmV, &v_full[s], vc + dc * 64, krow);
+        if (ptx::elect_one()) {
+          ptx::mbar_expect_tx(&v_full[s], 2 * KBK);
+          ptx::tma_load_3d(sV + s * 2 * KBK, &tmV, &v_full[s], 0, (int)(row_base + (long long)i * BKV), vc);
+        }
+        __syncwarp();
       }
     }
   } else if (warp == 1) {
@@ -134,11 +158,12 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       const uint32_t idesc_s = ptx::make_idesc_bf16(BQ, BKV, false, false);
       const uint32_t idesc_pv = ptx::make_idesc_bf16(BQ, D, false, true);      // V: MN-major B operand
       bool ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(q_full, 0, abort_flag, g.status) ? 1 : 0) != 0;
+      uint32_t kst = 0, kph = 0;
       auto issue_s = [&](int j) {
         const int s = j & 1;
         const uint32_t ph = (j >> 1) & 1;
         ok = ok && ptx::mbar_wait(&s_empty[s], ph ^ 1, abort_flag, g.status);
-        ok = ok && ptx::mbar_wait(&k_full[s], ph, abort_flag, g.status);
+        ok = ok && ptx::mbar_wait(&k_full[kst], kph, abort_flag, g.status);
         ok = __all_sync(0xFFFFFFFFu, ok ? 1 : 0) != 0;
         if (!ok) return;
         ptx::tc_fence_after();
@@ -146,15 +171,16 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
 #pragma unroll
           for (int kb = 0; kb < 2; ++kb) {
             const uint64_t ad = ptx::make_smem_desc(ptx::smem_u32(sQ + kb * KB), 16, 1024);
-            const uint64_t bd = ptx::make_smem_desc(ptx::smem_u32(sK + (s * 2 + kb) * KBK), 16, 1024);
+            const uint64_t bd = ptx::make_smem_desc(ptx::smem_u32(sK + (kst * 2 + kb) * KBK), 16, 1024);
 #pragma unroll
             for (int k = 0; k < 4; ++k)                 // a k16 step moves both start addresses by 32 bytes
               ptx::tc_mma_bf16(tmem_base + TM_S + s * BKV, ad + 2 * k, bd + 2 * k, idesc_s, (kb | k) ? 1u : 0u);
           }
-          ptx::tc_commit(&k_empty[s]);
+          ptx::tc_commit(&k_empty[kst]);
           ptx::tc_commit(&s_full[s]);
         }
         __syncwarp();
+        if (++kst == KSTAGES) { kst = 0; kph ^= 1; }
       };
       auto issue_pv = [&](int j) {
         const int s = j & 1;
@@ -203,15 +229,16 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
 #pragma unroll
       for (int ch = 0; ch < BKV / 32; ++ch) ptx::tmem_ld32(ts + ch * 32, rv + ch * 32);
       ptx::tmem_ld_wait();
-      float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};   // row maximum (log2 domain), four independent chains
-      if (diag) {
+      if (diag) {                                      // keys beyond the row's position
 #pragma unroll
         for (int c = 0; c < BKV; ++c)
-          if (kj0 + c <= qi) mx4[c & 3] = fmaxf(mx4[c & 3], __uint_as_float(rv[c]));
-      } else {
-#pragma unroll
-        for (int c = 0; c < BKV; ++c) mx4[c & 3] = fmaxf(mx4[c & 3], __uint_as_float(rv[c]));
+          if (kj0 + c > qi) rv[c] = 0xFF800000u;       // -inf
       }
+      float mx4[4];                                    // row maximum, four independent chains of three-way maxima
+#pragma unroll
+      for (int k = 0; k < 4; ++k) mx4[k] = __uint_as_float(rv[k]);
+#pragma unroll
+      for (int c = 4; c < BKV; c += 2) mx4[(c >> 1) & 3] = max3(mx4[(c >> 1) & 3], __uint_as_float(rv[c]), __uint_as_float(rv[c + 1]));
       float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * g.scale_log2;   // the scale is positive
       float corr = 1.f;
       bool rescale = false;
@@ -223,20 +250,21 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       }
       // p = 2^(s - m), packed to bf16 for the second MMA
       uint32_t pk[BKV / 2];
-      float l0 = 0.f, l1 = 0.f;
+      const ptx::f32x2 sc2 = ptx::pack2(g.scale_log2, g.scale_log2), nm2 = ptx::pack2(-m_used, -m_used);
+      ptx::f32x2 l2[2] = {ptx::pack2(0.f, 0.f), ptx::pack2(0.f, 0.f)};
 #pragma unroll
       for (int c = 0; c < BKV; c += 2) {
-        float p0 = ex2(fmaf(__uint_as_float(rv[c]), g.scale_log2, -m_used));
-        float p1 = ex2(fmaf(__uint_as_float(rv[c + 1]), g.scale_log2, -m_used));
-        if (diag) {
-          if (kj0 + c > qi) p0 = 0.f;
-          if (kj0 + c + 1 > qi) p1 = 0.f;
-        }
-        l0 += p0;
-        l1 += p1;
+        float e0, e1;
+        ptx::unpack2(ptx::fma2(ptx::pack2(__uint_as_float(rv[c]), __uint_as_float(rv[c + 1])), sc2, nm2), e0, e1);
+        const float p0 = ex2(e0), p1 = ex2(e1);
+        l2[(c >> 1) & 1] = ptx::add2(l2[(c >> 1) & 1], ptx::pack2(p0, p1));
         pk[c / 2] = float2_to_bf16x2(p0, p1);
       }
-      l += l0 + l1;
+      {
+        float l0, l1;
+        ptx::unpack2(ptx::add2(l2[0], l2[1]), l0, l1);
+        l += l0 + l1;
+      }
       if (__any_sync(0xFFFFFFFFu, rescale)) {
         // O is rescaled in place: the previous P V, which accumulates into it, must have completed
         ok = ptx::mbar_wait(p_empty, (j & 1) ^ 1, abort_flag, g.status);
@@ -326,15 +354,21 @@ int launch_causal_attention_tc(const CausalAttnArgs& a, cudaStream_t st) {
     // one [B*S, row pitch] matrix holds q, k and v side by side; columns are offsets from q
     const long long kcol = ((const char*)a.k.ptr - (const char*)a.q.ptr) / 2, vcol = ((const char*)a.v.ptr - (const char*)a.q.ptr) / 2;
     if (kcol < 0 || vcol < 0 || kcol + H * D > st_ || vcol + H * D > st_) return SMARTMEM_ERR_UNSUPPORTED;
-    if ((rc = tc_encode_2d(a.q.ptr, st_, B * S, st_, 64, BQ, &tq)) != SMARTMEM_OK) return rc;
-    if ((rc = tc_encode_2d(a.q.ptr, st_, B * S, st_, 64, BKV, &tk)) != SMARTMEM_OK) return rc;   // same buffer, 64-row boxes
+    if (kcol % 64 || vcol % 64) return SMARTMEM_ERR_UNSUPPORTED;
+    // [64 columns][row][chunk of 64 columns]: both chunks of a head in one copy
+    const long long dims[3] = {64, B * S, st_ / 64}, strides[2] = {st_, 64};
+    const int qbox[3] = {64, BQ, 2}, kbox[3] = {64, BKV, 2};
+    if ((rc = tc_encode_nd_sw128(a.q.ptr, 3, dims, strides, qbox, &tq)) != SMARTMEM_OK) return rc;
+    if ((rc = tc_encode_nd_sw128(a.q.ptr, 3, dims, strides, kbox, &tk)) != SMARTMEM_OK) return rc;   // same buffer, 64-row boxes
     tv = tk;
     g.q_col0 = 0; g.k_col0 = (int)kcol; g.v_col0 = (int)vcol; g.col_per_head = D;
     g.row_per_batch = S; g.row_per_head = 0;
   } else if (head_major) {
-    if ((rc = tc_encode_2d(a.q.ptr, D, B * H * S, D, 64, 128, &tq)) != SMARTMEM_OK) return rc;
-    if ((rc = tc_encode_2d(a.k.ptr, D, B * H * S, D, 64, BKV, &tk)) != SMARTMEM_OK) return rc;
-    if ((rc = tc_encode_2d(a.v.ptr, D, B * H * S, D, 64, BKV, &tv)) != SMARTMEM_OK) return rc;
+    const long long dims[3] = {64, B * H * S, 2}, strides[2] = {D, 64};
+    const int qbox[3] = {64, BQ, 2}, kbox[3] = {64, BKV, 2};
+    if ((rc = tc_encode_nd_sw128(a.q.ptr, 3, dims, strides, qbox, &tq)) != SMARTMEM_OK) return rc;
+    if ((rc = tc_encode_nd_sw128(a.k.ptr, 3, dims, strides, kbox, &tk)) != SMARTMEM_OK) return rc;
+    if ((rc = tc_encode_nd_sw128(a.v.ptr, 3, dims, strides, kbox, &tv)) != SMARTMEM_OK) return rc;
     g.col_per_head = 0;
     g.row_per_batch = H * S; g.row_per_head = S;
   } else {
@@ -350,7 +384,7 @@ int launch_causal_attention_tc(const CausalAttnArgs& a, cudaStream_t st) {
   if (!g.status) return SMARTMEM_ERR_CUDA;
   // 112 KB of tiles: two CTAs per SM only fit without a spare kilobyte of alignment slack (the kernel
   // reports a misaligned base instead of overrunning)
-  const size_t smem = 2 * KB + 8 * KBK + 16 * 8 + 16;
+  const size_t smem = SMEM_BYTES;
   g.smem_bytes = (uint32_t)smem;
   if (ensure_max_dynamic_smem((const void*)causal_attn_tc_kernel, (int)smem, 100) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   const long long ctas = (long long)g.n_qt * B * H;

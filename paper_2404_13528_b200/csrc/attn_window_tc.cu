@@ -8,7 +8,7 @@
 // fragment bookkeeping and no shared-memory fragment loads, which is what bounded the warp-MMA
 // version (it was instruction-issue bound).
 //
-// q, k, v are TMA boxes of 64 rows x 32 columns inside the [M, 3C] buffer of the QKV GEMM (head
+// q, k, v are TMA boxes of 64 tokens x 32 features x 2 windows inside the [M, 3C] buffer of the QKV GEMM (head
 // split, K transpose eliminated); operands that TMA cannot address (the materialised K^T of the
 // explicit variant) are loaded by four helper warps into the same swizzled layout.  V is used as it
 // lies ([key, d] rows) through the MN-major operand mode.  Results are stored as whole 64-byte rows
@@ -47,9 +47,8 @@ constexpr int kThreads = 32 * (3 + kGroups * kSoftmaxWarps + kLoaderWarps);   //
 struct WinTcArgs {
   WinAttnArgs a;
   int n_pairs, tma_mask;                               // bit m set: operand m (q, k, v) comes through TMA
+  int merged;                                          // q, k and v of a pair in one copy (tm0 has a fifth dimension)
   FastDiv fd_T;
-  int col0[3], col_per_head[3];                        // TMA column of (operand, head)
-  long long row_per_window[3], row_per_head[3];        // TMA row of (window, head): n * rpw + h * rph
   int* status;
 };
 
@@ -170,31 +169,33 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
   const uint32_t tmem_base = *tmem_slot;
   pdl_wait();                       // the tables above depend on parameters only: they overlapped the previous kernel's tail
   pdl_launch_dependents();
-  const CUtensorMap* tms[3] = {&tm0, &tm1, &tm2};
   const AttnOperand* ops[3] = {&a.q, &a.k, &a.v};
 
   if (warp == 0) {
     // ---- TMA producer ------------------------------------------------------------------------
-    if (lane == 0) {
-      int n_tma = 0;
-      for (int m = 0; m < 3; ++m) n_tma += (g.tma_mask >> m) & 1;
-      bool ok = true;
-      uint32_t it = 0;
-      for (int p = cidx; p < g.n_pairs && ok; p += cstride, ++it) {
-        const int s = it % NSTAGE;
-        ok = ptx::mbar_wait(&in_empty[s], ((it / NSTAGE) & 1) ^ 1, abort_flag, g.status);
-        if (!ok) break;
-        const int nwin = (2 * p + 1 < a.n_windows) ? 2 : 1;
-        ptx::mbar_expect_tx(&in_full[s], (uint32_t)(n_tma * nwin * TP * 64));
-        for (int m = 0; m < 3; ++m) {
-          if (!((g.tma_mask >> m) & 1)) continue;
-          for (int w = 0; w < nwin; ++w) {
-            const long long n = 2 * p + w;
-            ptx::tma_load_2d(sIn + s * STAGE_BYTES + m * OP_BYTES + w * (TP * 64), tms[m], &in_full[s],
-                             g.col0[m] + h * g.col_per_head[m], (int)(n * g.row_per_window[m] + h * g.row_per_head[m]));
-          }
+    // A pair's operand is one box {32 features, 64 tokens, head, 2 windows}: tokens past T and a missing second window are
+    // filled with zeros.  Where q, k and v lie at equal distances (the QKV buffer) one copy brings all three.  (Six boxes a
+    // pair, issued under a branch on one lane at about 0.2 us each, were the kernel's period.)
+    int n_tma = 0;
+    for (int m = 0; m < 3; ++m) n_tma += (g.tma_mask >> m) & 1;
+    bool ok = true;
+    uint32_t s = 0, ph = 1;
+    for (int p = cidx; p < g.n_pairs && ok; p += cstride) {
+      ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(&in_empty[s], ph, abort_flag, g.status) ? 1 : 0) != 0;
+      if (!ok) break;
+      if (ptx::elect_one()) {
+        uint8_t* dst = sIn + s * STAGE_BYTES;
+        ptx::mbar_expect_tx(&in_full[s], (uint32_t)(n_tma * OP_BYTES));
+        if (g.merged) {
+          ptx::tma_load_5d(dst, &tm0, &in_full[s], 0, 0, h, 2 * p, 0);
+        } else {
+          if (g.tma_mask & 1) ptx::tma_load_4d(dst, &tm0, &in_full[s], 0, 0, h, 2 * p);
+          if (g.tma_mask & 2) ptx::tma_load_4d(dst + OP_BYTES, &tm1, &in_full[s], 0, 0, h, 2 * p);
+          if (g.tma_mask & 4) ptx::tma_load_4d(dst + 2 * OP_BYTES, &tm2, &in_full[s], 0, 0, h, 2 * p);
         }
       }
+      __syncwarp();
+      if (++s == NSTAGE) { s = 0; ph ^= 1; }
     }
   } else if (warp == 1) {
     // ---- P V issuer (and owner of the tensor memory): the whole warp walks the loop, an elected lane issues ----
@@ -492,16 +493,21 @@ int launch_window_attention_tc(const WinAttnArgs& a_in, long long n_windows, cud
   const long long T = a.T, H = a.heads;
   for (int m = 0; m < 3; ++m) {
     const AttnOperand& o = *ops[m];
-    // rows of 32 contiguous elements, 16-byte aligned pitch; two addressing patterns
-    const bool rows_ok = o.se == 1 && o.st % 8 == 0 && ((uintptr_t)o.ptr & 15) == 0;
-    if (rows_ok && o.sh == D && o.sn == T * o.st) {                 // [M, pitch] with heads side by side
-      if (tc_encode_2d_sw64(o.ptr, H * D, n_windows * T, o.st, D, TP, &tm[m]) != SMARTMEM_OK) continue;
-      g.col0[m] = 0; g.col_per_head[m] = D; g.row_per_window[m] = T; g.row_per_head[m] = 0;
-      g.tma_mask |= 1 << m;
-    } else if (rows_ok && o.st == D && o.sh == T * D && o.sn == H * T * D) {     // [nW, nH, T, d]
-      if (tc_encode_2d_sw64(o.ptr, D, n_windows * H * T, D, D, TP, &tm[m]) != SMARTMEM_OK) continue;
-      g.col0[m] = 0; g.col_per_head[m] = 0; g.row_per_window[m] = H * T; g.row_per_head[m] = T;
-      g.tma_mask |= 1 << m;
+    // rows of 32 contiguous elements; token, head and window strides of whole 16-byte vectors
+    if (o.se != 1 || o.st % 8 || o.sh % 8 || o.sn % 8 || o.st <= 0 || o.sh <= 0 || o.sn <= 0 || ((uintptr_t)o.ptr & 15)) continue;
+    const long long dims[4] = {D, T, H, n_windows}, strides[3] = {o.st, o.sh, o.sn};
+    const int box[4] = {D, TP, 1, 2};
+    if (tc_encode_nd_sw64(o.ptr, 4, dims, strides, box, &tm[m]) == SMARTMEM_OK) g.tma_mask |= 1 << m;
+  }
+  const long long dk = ((const char*)a.k.ptr - (const char*)a.q.ptr) / 2, dv = ((const char*)a.v.ptr - (const char*)a.k.ptr) / 2;
+  if (g.tma_mask == 7 && dk > 0 && dk == dv && dk % 8 == 0 && a.k.st == a.q.st && a.v.st == a.q.st && a.k.sh == a.q.sh && a.v.sh == a.q.sh &&
+      a.k.sn == a.q.sn && a.v.sn == a.q.sn) {
+    const long long dims[5] = {D, T, H, n_windows, 3}, strides[4] = {a.q.st, a.q.sh, a.q.sn, dk};
+    const int box[5] = {D, TP, 1, 2, 3};
+    CUtensorMap t;
+    if (tc_encode_nd_sw64(a.q.ptr, 5, dims, strides, box, &t) == SMARTMEM_OK) {
+      tm[0] = t;
+      g.merged = 1;
     }
   }
   const size_t smem = 1024 + NSTAGE * STAGE_BYTES + TP * BIAS_ROW * 4 + (2 * kGroups + 1) * TP * 4 +

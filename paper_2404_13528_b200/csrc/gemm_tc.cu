@@ -869,9 +869,9 @@ int tc_encode_2d_plain(const void* ptr, long long inner, long long outer, long l
   return encode_cached(ptr, 2, dims, strides, box, out, 0);
 }
 
-int tc_encode_nd_sw64(const void* ptr, int rank, const long long* dims, const long long* strides_elems, const int* box,
-                      CUtensorMap* out) {
-  if (rank < 2 || rank > 5 || ((uintptr_t)ptr & 15) || box[0] * 2 != 64) return SMARTMEM_ERR_ALIGNMENT;
+static int encode_nd(const void* ptr, int rank, const long long* dims, const long long* strides_elems, const int* box, int swizzle_bytes,
+                     CUtensorMap* out) {
+  if (rank < 2 || rank > 5 || ((uintptr_t)ptr & 15) || box[0] * 2 != swizzle_bytes) return SMARTMEM_ERR_ALIGNMENT;
   uint64_t d[5], sb[4];
   uint32_t b[5];
   for (int i = 0; i < rank; ++i) {
@@ -882,7 +882,15 @@ int tc_encode_nd_sw64(const void* ptr, int rank, const long long* dims, const lo
       if (sb[i - 1] % 16) return SMARTMEM_ERR_ALIGNMENT;
     }
   }
-  return encode_cached(ptr, rank, d, sb, b, out, 64);
+  return encode_cached(ptr, rank, d, sb, b, out, swizzle_bytes);
+}
+int tc_encode_nd_sw64(const void* ptr, int rank, const long long* dims, const long long* strides_elems, const int* box,
+                      CUtensorMap* out) {
+  return encode_nd(ptr, rank, dims, strides_elems, box, 64, out);
+}
+int tc_encode_nd_sw128(const void* ptr, int rank, const long long* dims, const long long* strides_elems, const int* box,
+                       CUtensorMap* out) {
+  return encode_nd(ptr, rank, dims, strides_elems, box, 128, out);
 }
 
 int tc_sm_count() { return sm_count(); }

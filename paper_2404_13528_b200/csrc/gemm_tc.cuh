@@ -70,6 +70,9 @@ int tc_encode_2d_sw64(const void* ptr, long long inner, long long outer, long lo
 // of 32 innermost elements.
 int tc_encode_nd_sw64(const void* ptr, int rank, const long long* dims, const long long* strides_elems, const int* box,
                       CUtensorMap* out);
+// Same with 128-byte swizzle and a box of 64 innermost elements.
+int tc_encode_nd_sw128(const void* ptr, int rank, const long long* dims, const long long* strides_elems, const int* box,
+                       CUtensorMap* out);
 // Same without swizzle.
 int tc_encode_2d_plain(const void* ptr, long long inner, long long outer, long long pitch_elems, int box_inner, int box_outer,
                        CUtensorMap* out);
