@@ -115,15 +115,18 @@ constexpr int kThreads = 64 + 32 * kEpiWarps + 32;      // + a second TMA produc
 // 128 x 256 tile (48 KB per k-block against the ~64 bytes per clock an SM takes in) -- and keeps its own 128 rows of the
 // accumulator, which it drains itself.  The even CTA counts both CTAs' bytes on its `full` barriers, issues the products
 // and signals `empty` / `tmem_full` in both CTAs; both CTAs' epilogue warps arrive on its `tmem_empty`.
-// LEAN (pairs only): the epilogue knows bias and GELU only (no rotary embedding, residual or second copy), which leaves it
-// the registers to pull its whole accumulator slice out of tensor memory at once and hand the buffer back before any
-// arithmetic -- for short reductions, where a tile's products take no longer than its epilogue.
+// LEAN: the epilogue knows bias and GELU only (no rotary embedding or second copy; a residual and a row map only on 128-wide
+// tiles), which leaves it the registers to pull its whole accumulator slice out of tensor memory at once and hand the buffer
+// back before any arithmetic -- for short reductions, where a tile's products take no longer than its epilogue -- and its rows
+// leave as 32 x 32 TMA boxes, or as 32-byte vectors through the row map, without staging a tile.  On single CTAs (us):
+// M = 50 176, N = 384, K = 128 16.4 -> 11.1, M = 12 544, N = 768, K = 192 9.5 -> 7.1.
 template <int BN, int STAGES, bool A_MN, bool PAIR, bool LEAN>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmC, const __grid_constant__ GemmArgs g) {
   static_assert(!PAIR || ((BN == 256 || BN == 128) && !A_MN), "CTA pairs: 256- or 128-wide tiles, K-major A");
-  static_assert(!LEAN || PAIR, "the lean epilogue comes with CTA pairs");
+  static_assert(!LEAN || BN % 128 == 0, "the lean epilogue's boxes are 32 columns wide");
+  constexpr bool RES = !LEAN || BN == 128;                 // the epilogue can add a residual
   constexpr int BN_CTA = PAIR ? BN / 2 : BN;               // rows of B this CTA loads
   constexpr int B_STAGE_BYTES = BN_CTA * BK * 2;
   constexpr uint32_t ACC_COLS = BN <= 32 ? 32 : BN <= 64 ? 64 : BN <= 128 ? 128 : 256;   // one accumulator buffer
@@ -326,9 +329,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     //   phase 2 (threads spread along the row): 16-byte stores, RC*2 contiguous bytes per row,
     // so a store instruction writes whole 32-byte sectors and several sectors of one line at once.
     constexpr int CG = BN / 4;
-    constexpr bool DIRECT = PAIR;                            // rows leave the registers as 32-byte stores: no staging at all
+    constexpr bool DIRECT = PAIR || LEAN;                            // rows leave the registers as 32-byte stores: no staging at all
     constexpr bool EARLY = DIRECT && LEAN;                   // accumulator slice to registers first, buffer released at once
-    constexpr int RC = (BN == 256 && STAGES == 4 && !PAIR) ? 16 : (CG > 32 ? 32 : CG);   // 4 stages leave less staging room
+    constexpr int RC = (BN == 256 && STAGES == 4 && !PAIR && !LEAN) ? 16 : (CG > 32 ? 32 : CG);   // 4 stages leave less staging room
     constexpr int ROUNDS = CG / RC;
     constexpr int RH = ROUNDS > 1 ? ROUNDS / 2 : 1;          // BN == 256: rounds [0, RH) hold the first halves of rotary pairs
     constexpr int VPR = RC / 8;                              // 16-byte vectors per row per round
@@ -381,7 +384,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (row_ok) off = g.has_rowmap ? devmap_eval_unrolled(g.rowmap, (uint32_t)row) : (long long)row * ld_t;
         off += (long long)batch * g.out_batch_stride;
       }
-      const __nv_bfloat16* __restrict__ rrow = (!LEAN && g.residual) ? g.residual + off : nullptr;
+      const __nv_bfloat16* __restrict__ rrow = (RES && g.residual) ? g.residual + off : nullptr;
       const bool rope_tile = !LEAN && (BN == 256 || BN == 128) && g.rope_cols > 0 && n0 < g.rope_cols;
       auto col_of = [&](int rd) {
         return BN == 256 ? 128 * (grp >> 1) + 32 * (grp & 1) + RC * (rd % RH) + 64 * (rd / RH) : grp * CG;
@@ -389,10 +392,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
       uint4 res[VPR];
       auto fetch_res = [&](int c0) {
-        if constexpr (DIRECT) {                              // (pairs: full tiles, 32-byte aligned rows) whole sectors per load
+        if constexpr (DIRECT) {                              // (32-byte aligned rows, N a multiple of 16) whole sectors per load
           if (rrow && row_ok && res_wide) {
 #pragma unroll
-            for (int v = 0; v < VPR; v += 2) ptx::ld_global_v8(rrow + n0 + c0 + v * 8, res[v], res[v + 1]);
+            for (int v = 0; v < VPR; v += 2) {
+              res[v] = res[v + 1] = make_uint4(0, 0, 0, 0);
+              if (n0 + c0 + v * 8 < g.N) ptx::ld_global_v8(rrow + n0 + c0 + v * 8, res[v], res[v + 1]);
+            }
             return;
           }
         }
@@ -451,7 +457,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         ptx::tmem_ld_wait();
         ptx::tc_fence_before();
         __syncwarp();
-        if (lane == 0) ptx::mbar_arrive_cluster(tmem_empty0 + buf * 8);
+        if (lane == 0) {
+          if constexpr (PAIR) ptx::mbar_arrive_cluster(tmem_empty0 + buf * 8);
+          else ptx::mbar_arrive(&tmem_empty[buf]);
+        }
       }
 #pragma unroll
       for (int rd = 0; rd < ROUNDS; ++rd) {
@@ -572,7 +581,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 }
               }
             } else if (v & 1) {
-              if (row_ok) ptx::st_global_v8(out_t + off + n0 + c0 + (v - 1) * 8, pk_prev, pk);
+              if (row_ok && n0 + c0 + v * 8 < g.N) ptx::st_global_v8(out_t + off + n0 + c0 + (v - 1) * 8, pk_prev, pk);
             } else {
               pk_prev = pk;
             }
@@ -963,19 +972,27 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
   const bool pair_ok = allow_pair && !a_mn && tiles_m1 > 1 && nkb > 4 && N % 256 == 0 && A.n_row_atoms == 1 &&
                        (!ep.rowmap || devmap_offsets_multiple_of(*ep.rowmap, 16)) && ep.seg_cols == 0 && !ep.out2 && ep.ldc % 16 == 0 &&
                        ep.out_batch_stride % 16 == 0 && ((uintptr_t)ep.out & 31) == 0;
+  // the lean epilogue on single CTAs: whole rows as TMA boxes, or (128 wide) 32-byte vectors through the row map
+  const bool lean_ok = !a_mn && batch == 1 && ep.rope_cols == 0 && ep.seg_cols == 0 && !ep.out2;
+  const bool lean256_ok = lean_ok && !ep.rowmap && !ep.residual;
+  const bool lean128_ok = lean_ok && (lean256_ok || (N % 16 == 0 && ep.ldc % 16 == 0 && ((uintptr_t)ep.out & 31) == 0 && ((uintptr_t)ep.residual & 31) == 0 &&
+                                                      (!ep.rowmap || devmap_offsets_multiple_of(*ep.rowmap, 16))));
   int bn = 128;
-  bool pair = false;
+  bool pair = false, lean = false;
   if (batch == 1) {
     // Tile width, and single CTAs or pairs: the smallest of the times fitted to measurements (us): a fixed part, the k-blocks of
     // the first tile, and for every further wave its k-blocks or, where the reduction is short, its epilogue.  A narrow tile
     // costs more per column but splits the columns over more SMs: M = 666, N = K = 2048 (48 tiles of 128 x 256, 96 of half
     // that) 16.1 us on 256-wide single tiles, 9.6 on 128-wide pairs; M = 196, N = 512, K = 2048 14.1 -> 8.8 us on 64-wide ones.
-    struct Option { int bn; bool pair; double fixed, per_kb, wave, wave_min; };
-    static const Option options[] = {{64, false, 2.4, 0.185, 0.3, 1.9}, {96, false, 2.4, 0.25, 0.3, 2.0}, {128, false, 2.6, 0.27, 0.4, 2.8},
-                                     {256, false, 4.4, 0.36, 0.5, 4.0}, {128, true, 3.0, 0.185, 0.2, 2.2}, {256, true, 4.6, 0.33, 0.4, 3.0}};
+    struct Option { int bn; bool pair, lean; double fixed, per_kb, wave, wave_min; };
+    static const Option options[] = {{64, false, false, 2.4, 0.185, 0.55, 0.95}, {96, false, false, 2.9, 0.22, 0.8, 1.2},
+                                     {128, false, true, 2.6, 0.26, 0.7, 1.15},   {256, false, true, 3.9, 0.5, -0.2, 1.65},
+                                     {128, false, false, 2.6, 0.27, 0.4, 2.8},   {256, false, false, 4.4, 0.36, 0.5, 4.0},
+                                     {128, true, false, 3.0, 0.185, 0.2, 2.2},   {256, true, false, 4.6, 0.33, 0.4, 3.0}};
     double best = 0.0;
     for (const Option& o : options) {
       if (o.pair && !pair_ok) continue;
+      if (o.lean && !(o.bn == 128 ? lean128_ok : lean256_ok)) continue;
       if (ep.rope_cols > 0 && o.bn < 128) continue;          // rotary pairs stay inside a tile
       if (a_mn && o.bn < 128) continue;                      // MN-major A operands come with 128- and 256-wide tiles only
       if (ep.seg_cols > 0 && ep.seg_cols % o.bn) continue;
@@ -983,7 +1000,7 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
       const long long tiles = (o.pair ? (tiles_m1 + 1) / 2 : tiles_m1) * ((N + o.bn - 1) / o.bn), slots = tc_sm_count() / (o.pair ? 2 : 1);
       const double kbs = nkb * o.per_kb, wave = kbs + o.wave > o.wave_min ? kbs + o.wave : o.wave_min;
       const double t = o.fixed + kbs + (double)((tiles + slots - 1) / slots - 1) * wave;
-      if (best == 0.0 || t < best) { best = t; bn = o.bn; pair = o.pair; }
+      if (best == 0.0 || t < best) { best = t; bn = o.bn; pair = o.pair; lean = o.lean; }
     }
     if (splitk_ok && gemm_splitk_us(M, N, K) < best) return launch_gemm_splitk(A, B, ep, M, N, K, st);
   } else {
@@ -1051,15 +1068,16 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
   g.batch = (int)batch;
   if ((long long)g.tiles_n * g.tiles_m * g.batch >= (1ll << 31)) return SMARTMEM_ERR_UNSUPPORTED;
   CUtensorMap tc = ta;                                     // (a valid map for the kernels that store without TMA)
-  if (pair && bn == 256 && nkb <= 16 && ep.rope_cols == 0 && !ep.residual) {
-    if (batch == 1 && !ep.rowmap) {                        // output as 32 x 32 boxes of [M, N] with pitch ldc
-      const uint64_t dims[2] = {(uint64_t)N, (uint64_t)M}, strides[1] = {(uint64_t)ep.ldc * 2};
-      const uint32_t box[2] = {32, 32};
-      if (encode_cached(ep.out, 2, dims, strides, box, &tc, 64) == SMARTMEM_OK) g.tma_out = 1;
-      else tc = ta;
-    }
-    return launch_t<256, 6, false, true, true>(ta, tb, tc, g, st);
+  const bool pair_lean = pair && bn == 256 && nkb <= 16 && ep.rope_cols == 0 && !ep.residual;
+  if ((pair_lean || lean) && batch == 1 && !ep.rowmap) {     // output as 32 x 32 boxes of [M, N] with pitch ldc
+    const uint64_t dims[2] = {(uint64_t)N, (uint64_t)M}, strides[1] = {(uint64_t)ep.ldc * 2};
+    const uint32_t box[2] = {32, 32};
+    if (encode_cached(ep.out, 2, dims, strides, box, &tc, 64) == SMARTMEM_OK) g.tma_out = 1;
+    else if (lean) return SMARTMEM_ERR_CUDA;
+    else tc = ta;
   }
+  if (pair_lean) return launch_t<256, 6, false, true, true>(ta, tb, tc, g, st);
+  if (lean) return bn == 128 ? launch_t<128, 5, false, false, true>(ta, tb, tc, g, st) : launch_t<256, 4, false, false, true>(ta, tb, tc, g, st);
   if (pair && bn == 256) return launch_t<256, 6, false, true>(ta, tb, tc, g, st);
   if (pair) return launch_t<128, 8, false, true>(ta, tb, tc, g, st);
   if (stages == 2) {
