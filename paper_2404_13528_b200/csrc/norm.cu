@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(256) norm_kernel(const T* __restrict__ src, T*
 // bf16 rows of up to 1024 elements (LayerNorm and RMSNorm of the wide blocks and of the chains), read at one of three kinds of
 // offset: contiguous rows, whole rows through a row map (cyclic shift + window partition), or 16-byte vectors through a map
 // whose row boundary falls between two atoms -- there a vector's offset is the sum of a part that depends on the row
-// (evaluated once per row by one lane) and a part that depends on its place in the row (once per lane, before the loop).
+// (evaluated for a warp's next 32 rows by its lanes) and a part that depends on its place in the row (once per lane, before the loop).
 // What bounds it is instruction issue: packed fp32 pairs for all the arithmetic, LPR lanes
 // per row with NV vectors each so that no lane idles; a warp walks over several groups of rows and has the next group's
 // vectors in flight.
@@ -204,29 +204,44 @@ __global__ void __launch_bounds__(256, NV <= 3 ? 3 : 2) norm_rows_kernel(const _
     if (SRC == VECTORS_MAPPED && vi < nvec) col[k] = (int)devmap_part_rolled(map, split, map.n_atoms, (uint32_t)vi).off;
   }
   __syncthreads();
-  auto request = [&](int row, uint4 (&v)[NV]) {
-    long long off = (long long)row * C;
+  // Row part of the map: a warp's next 32 rows, one per lane, in one go (one lane evaluating the map of each row as it came
+  // put the whole evaluation, about 300 cycles, between two rows).  Row r of group i is lane i * RPW + r's.
+  constexpr int GROUPS = 32 / RPW;                       // groups of rows per evaluation
+  long long row_off = 0;
+  auto offsets = [&](int first) {                        // first: the first row of the warp's next group
     if constexpr (SRC != ROWS_CONTIGUOUS) {
-      off = 0;
-      if (sub == 0 && row < rows)
-        off = SRC == ROWS_MAPPED ? devmap_eval_unrolled(map, (uint32_t)row) : map.base + devmap_part_rolled(map, 0, split, (uint32_t)row).off;
-      off = __shfl_sync(0xFFFFFFFFu, off, lane - sub);
+      const int row = first + (lane / RPW) * step + lane % RPW;
+      row_off = 0;
+      if (row < rows)
+        row_off = SRC == ROWS_MAPPED ? devmap_eval_unrolled(map, (uint32_t)row) : map.base + devmap_part_rolled(map, 0, split, (uint32_t)row).off;
     }
+  };
+  auto request = [&](int row, int group, uint4 (&v)[NV]) {
+    long long off = (long long)row * C;
+    if constexpr (SRC != ROWS_CONTIGUOUS) off = __shfl_sync(0xFFFFFFFFu, row_off, group * RPW + lane / LPR);
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
       v[k] = make_uint4(0, 0, 0, 0);
       if (sub + k * LPR < nvec && row < rows) v[k] = *reinterpret_cast<const uint4*>(src + off + col[k]);
     }
   };
+  offsets(row0 - lane / LPR);
   pdl_wait();
   pdl_launch_dependents();
   uint4 x[NV], nx[NV];
-  request(row0, nx);
+  request(row0, 0, nx);
+  int group = 0;
   // (trip count uniform over the warp: the shuffles below)
   for (int row = row0; row - lane / LPR < rows; row += step) {
 #pragma unroll
     for (int k = 0; k < NV; ++k) x[k] = nx[k];
-    if (row - lane / LPR + step < rows) request(row + step, nx);
+    if (row - lane / LPR + step < rows) {
+      if (SRC != ROWS_CONTIGUOUS && ++group == GROUPS) {
+        offsets(row - lane / LPR + step);
+        group = 0;
+      }
+      request(row + step, group, nx);
+    }
     ptx::f32x2 s2[2] = {ptx::pack2(0.f, 0.f), ptx::pack2(0.f, 0.f)};
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
