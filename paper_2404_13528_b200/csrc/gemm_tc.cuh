@@ -89,6 +89,12 @@ int launch_mlp_fused(const void* A, const void* ln_gamma, const void* ln_beta, f
                      const void* W2, const void* b2, void* out, long long M, long long C, long long hidden,
                      cudaStream_t st);
 
+// The same for few rows where the weights do not fit one SM: the hidden features split over a cluster (gemm_mlp_cluster.cu).
+// mlp_cluster_wins: it covers the shape and beats the separate kernels.
+bool mlp_cluster_wins(long long M, long long C, long long hidden);
+int launch_mlp_cluster(const void* x, const void* ln_g, const void* ln_b, float eps, const void* W1, const void* b1, const void* W2,
+                       const void* b2, void* out, long long M, long long C, long long hidden, cudaStream_t st);
+
 // LayerNorm o row-gather o linear for narrow rows: out[m, :] = LN(X[src(m), :]) W^T + bias, with X rows of
 // K in {64, 96} elements, W [N, K], N a multiple of 96 (at most 288).  `rowmap` (null: identity) gives
 // the element offset of consumer row m in X; gamma/beta null: no normalisation (plain gather).

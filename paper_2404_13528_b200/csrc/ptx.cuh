@@ -223,6 +223,8 @@ __device__ __forceinline__ float2 ld_cluster_f32x2(uint32_t addr) {
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }   // (need not be converged)
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync() {      // every thread of every CTA of the cluster, converged
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -332,6 +334,13 @@ __device__ __forceinline__ void ld_global_v8(const void* p, uint4& a, uint4& b) 
 // Untiled bulk store: `bytes` (a multiple of 16) contiguous bytes, both addresses 16-byte aligned.
 __device__ __forceinline__ void bulk_store(void* gdst, const void* src, uint32_t bytes) {
   asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(gdst), "r"(smem_u32(src)), "r"(bytes)
+               : "memory");
+}
+// Bulk copy between the shared memories of two CTAs of a cluster, counted on a barrier of the destination (both shared::cluster
+// addresses; a multiple of 16 bytes).
+__device__ __forceinline__ void bulk_copy_cluster(uint32_t dst_cluster, const void* src, uint32_t bytes, uint32_t bar_cluster) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst_cluster),
+               "r"(smem_u32(src)), "r"(bytes), "r"(bar_cluster)
                : "memory");
 }
 __device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }

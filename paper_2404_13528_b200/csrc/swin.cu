@@ -89,6 +89,7 @@ size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
 // Which fused kernels a block takes (they decide which intermediates exist at all).
 struct Path {
   bool fuse_attn, fuse_ln1, fuse_mlp;
+  bool mlp_cluster;                // (fuse_mlp) the hidden features split over a cluster
 };
 Path choose_path(const smartmem_swin_params_t& p, int mode) {
   const bool bf16 = p.dtype == SMARTMEM_BF16;
@@ -98,6 +99,8 @@ Path choose_path(const smartmem_swin_params_t& p, int mode) {
   t.fuse_ln1 = bf16 && gemm_ln_supported(3 * (long long)p.C, p.C);
   t.fuse_mlp = p.mlp_ratio > 0 && (bf16 ? mlp_fused_supported(p.C, (long long)p.C * p.mlp_ratio)
                                         : swin_mlp_f32_supported(p.C, (long long)p.C * p.mlp_ratio));
+  t.mlp_cluster = bf16 && p.mlp_ratio > 0 && !t.fuse_mlp && mlp_cluster_wins((long long)p.B * p.H * p.W, p.C, (long long)p.C * p.mlp_ratio);
+  t.fuse_mlp = t.fuse_mlp || t.mlp_cluster;
   return t;
 }
 
@@ -301,7 +304,9 @@ int run_block(const smartmem_swin_params_t* pp, const void* x, void* y, void* wo
       // narrow blocks: LN2 + fc1 + GELU + fc2 + residual in one kernel; neither the normalised rows
       // nor the hidden activation leave the chip
       SM_TRY("mlp_fused_ln2_fc1_gelu_fc2_residual",
-             f32 ? launch_swin_mlp_f32(p, y1, y, M, st) : launch_mlp_fused(y1, p.ln2_g, p.ln2_b, p.ln_eps, p.w_fc1, p.b_fc1, p.w_fc2, p.b_fc2, y, M, C, hid, st));
+             f32 ? launch_swin_mlp_f32(p, y1, y, M, st)
+             : path.mlp_cluster ? launch_mlp_cluster(y1, p.ln2_g, p.ln2_b, p.ln_eps, p.w_fc1, p.b_fc1, p.w_fc2, p.b_fc2, y, M, C, hid, st)
+                                : launch_mlp_fused(y1, p.ln2_g, p.ln2_b, p.ln_eps, p.w_fc1, p.b_fc1, p.w_fc2, p.b_fc2, y, M, C, hid, st));
     } else {
       SM_TRY("ln2", launch_norm(p.dtype, false, y1, at(L.yn), p.ln2_g, p.ln2_b, p.ln_eps, M, (int)C, nullptr, st));
       SM_TRY("fc1_gemm_gelu", linear(at(L.yn), p.w_fc1, p.b_fc1, at(L.hid), hid, C, 1, nullptr, nullptr));

@@ -57,3 +57,14 @@ def test_row_norm_widths(C):
 ])
 def test_fp32_blocks(cfg):
     case(503, dtype="f32", **cfg)
+
+
+@pytest.mark.parametrize("cfg", [
+    dict(B=1, H=7, W=7, C=192, heads=6, window=7, shift=0, mlp_ratio=4),      # one tile of 49 rows, hidden features over four CTAs
+    dict(B=3, H=14, W=14, C=192, heads=6, window=7, shift=3, mlp_ratio=2),    # over two CTAs, ragged last 76 rows
+    dict(B=1, H=16, W=8, C=128, heads=4, window=4, shift=2, mlp_ratio=4),     # exactly one tile, the widest slice (256)
+    dict(B=2, H=14, W=14, C=128, heads=4, window=7, shift=3, mlp_ratio=1),    # one CTA per tile
+    dict(B=1, H=14, W=14, C=192, heads=6, window=7, shift=3, mlp_ratio=3),    # 576 does not split into whole blocks: kernel by kernel
+])
+def test_mlp_over_a_cluster(cfg):
+    case(504, dtype="bf16", **cfg)
