@@ -178,8 +178,12 @@ __device__ __forceinline__ float hsum2(ptx::f32x2 v) {
 }
 enum RowSource { ROWS_CONTIGUOUS = 0, ROWS_MAPPED = 1, VECTORS_MAPPED = 2 };
 
+// CTAs an SM holds: as many as leave the rows in flight in registers.  Four with a warp per row of two vectors (12544 x 512: 6.49 us
+// with three, 6.08 with four); the narrower rows lose with four (their lanes carry more rows at a time).
+constexpr int norm_ctas(int LPR, int NV) { return LPR == 32 && NV == 2 ? 4 : NV <= 3 ? 3 : 2; }
+
 template <bool RMS, int LPR, int NV, int SRC>
-__global__ void __launch_bounds__(256, NV <= 3 ? 3 : 2) norm_rows_kernel(const __nv_bfloat16* __restrict__ src, __nv_bfloat16* __restrict__ dst,
+__global__ void __launch_bounds__(256, norm_ctas(LPR, NV)) norm_rows_kernel(const __nv_bfloat16* __restrict__ src, __nv_bfloat16* __restrict__ dst,
                                                                          const __nv_bfloat16* __restrict__ gamma,
                                                                          const __nv_bfloat16* __restrict__ beta, float eps, int rows, int C,
                                                                          const __grid_constant__ DevMap map, int split) {
@@ -300,7 +304,7 @@ int launch_norm_rows(const void* src, void* dst, const void* gamma, const void* 
 #define SM_ROWS(LPR, NV)                                                                                                       \
   {                                                                                                                            \
     constexpr int rpb = 8 * (32 / LPR);                                                                                        \
-    const long long blocks = (rows + rpb - 1) / rpb, slots = (NV <= 3 ? 3ll : 2ll) * tc_sm_count();                            \
+    const long long blocks = (rows + rpb - 1) / rpb, slots = (long long)norm_ctas(LPR, NV) * tc_sm_count();                       \
     launch_pdl(norm_rows_kernel<RMS, LPR, NV, SRC>, dim3((unsigned)(blocks < slots ? blocks : slots)), dim3(256), 0, st,       \
                (const __nv_bfloat16*)src, (__nv_bfloat16*)dst, (const __nv_bfloat16*)gamma, (const __nv_bfloat16*)beta, eps,   \
                (int)rows, C, map, split);                                                                                      \
