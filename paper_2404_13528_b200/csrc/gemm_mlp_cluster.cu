@@ -20,13 +20,13 @@
 #include <cstring>
 
 #include "gemm_tc.cuh"
+#include "ln_operand.cuh"
 #include "ptx.cuh"
 
 namespace smartmem {
 namespace {
 
 constexpr int BM = 128, BK = 64;
-constexpr int KB_BYTES = BM * BK * 2;              // one 128 x 64 operand block: 16 KB
 constexpr int kWorkers = 16, kThreads = 32 * (kWorkers + 1);
 constexpr int kMaxSplits = 4;
 constexpr uint32_t TM_D1 = 0, TM_D2 = 256, TMEM_COLS = 512;
@@ -39,27 +39,6 @@ struct MlpClusterArgs {
   __nv_bfloat16* out;
   int* status;
 };
-
-__device__ __forceinline__ ptx::f32x2 widen(uint32_t w) { return ptx::pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
-__device__ __forceinline__ float hsum(ptx::f32x2 v) {
-  float lo, hi;
-  ptx::unpack2(v, lo, hi);
-  return lo + hi;
-}
-// eight bf16 values: their sum, the sum of (x + nm)^2, and (x rs + ms) g + b in fp32, rounded once
-__device__ __forceinline__ float sum8(const uint4& u) {
-  return hsum(ptx::add2(ptx::add2(widen(u.x), widen(u.y)), ptx::add2(widen(u.z), widen(u.w))));
-}
-__device__ __forceinline__ float sq8(const uint4& u, float nm) {
-  const ptx::f32x2 m = ptx::pack2(nm, nm), a = ptx::add2(widen(u.x), m), b = ptx::add2(widen(u.y), m), c = ptx::add2(widen(u.z), m),
-                   d = ptx::add2(widen(u.w), m);
-  return hsum(ptx::add2(ptx::fma2(a, a, ptx::mul2(b, b)), ptx::fma2(c, c, ptx::mul2(d, d))));
-}
-__device__ __forceinline__ uint32_t affine2(uint32_t w, ptx::f32x2 rs, ptx::f32x2 ms, uint32_t g, uint32_t b) {
-  float lo, hi;
-  ptx::unpack2(ptx::fma2(ptx::fma2(widen(w), rs, ms), widen(g), widen(b)), lo, hi);
-  return float2_to_bf16x2(lo, hi);
-}
 
 template <int NV, int N16>                         // C / 64, hs / 64
 __global__ void __launch_bounds__(kThreads, 1)
@@ -130,7 +109,7 @@ mlp_cluster_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_consta
       if (ptx::elect_one()) {
 #pragma unroll
         for (int kb = 0; kb < NV; ++kb) {
-          const uint64_t ad = ptx::make_smem_desc(a0 + kb * KB_BYTES, 16, 1024), bd = ptx::make_smem_desc(w1 + kb * g.hs * 128, 16, 1024);
+          const uint64_t ad = ptx::make_smem_desc(a0 + kb * kLnBlockBytes, 16, 1024), bd = ptx::make_smem_desc(w1 + kb * g.hs * 128, 16, 1024);
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k) ptx::tc_mma_bf16(tmem_base + TM_D1, ad + 2 * k, bd + 2 * k, idesc, (kb | k) ? 1u : 0u);
         }
@@ -144,7 +123,7 @@ mlp_cluster_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_consta
       const uint32_t idesc = ptx::make_idesc_bf16(BM, C, false, false);
       if (ptx::elect_one()) {
         for (int kb = 0; kb < g.hs / BK; ++kb) {
-          const uint64_t ad = ptx::make_smem_desc(a0 + kb * KB_BYTES, 16, 1024), bd = ptx::make_smem_desc(w2 + kb * C * 128, 16, 1024);
+          const uint64_t ad = ptx::make_smem_desc(a0 + kb * kLnBlockBytes, 16, 1024), bd = ptx::make_smem_desc(w2 + kb * C * 128, 16, 1024);
 #pragma unroll
           for (int k = 0; k < BK / 16; ++k) ptx::tc_mma_bf16(tmem_base + TM_D2, ad + 2 * k, bd + 2 * k, idesc, (kb | k) ? 1u : 0u);
         }
@@ -172,40 +151,7 @@ mlp_cluster_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_consta
         x[j][k] = make_uint4(0, 0, 0, 0);
         if (m < g.M) x[j][k] = *reinterpret_cast<const uint4*>(g.x + (size_t)m * C + (sub + 8 * k) * 8);
       }
-    float mean[2], rstd[2];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      mean[j] = 0.f;
-#pragma unroll
-      for (int k = 0; k < NV; ++k) mean[j] += sum8(x[j][k]);
-    }
-#pragma unroll
-    for (int d = 4; d > 0; d >>= 1)
-#pragma unroll
-      for (int j = 0; j < 2; ++j) mean[j] += __shfl_xor_sync(0xFFFFFFFFu, mean[j], d);
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      mean[j] *= 1.0f / (float)C;
-      rstd[j] = 0.f;
-#pragma unroll
-      for (int k = 0; k < NV; ++k) rstd[j] += sq8(x[j][k], -mean[j]);
-    }
-#pragma unroll
-    for (int d = 4; d > 0; d >>= 1)
-#pragma unroll
-      for (int j = 0; j < 2; ++j) rstd[j] += __shfl_xor_sync(0xFFFFFFFFu, rstd[j], d);
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int r = warp * 8 + j * 4 + rsub;
-      rstd[j] = rsqrtf(rstd[j] * (1.0f / (float)C) + g.eps);
-      const float ms = -mean[j] * rstd[j];
-      const ptx::f32x2 r2 = ptx::pack2(rstd[j], rstd[j]), m2 = ptx::pack2(ms, ms);
-#pragma unroll
-      for (int k = 0; k < NV; ++k)                   // vector sub + 8 k is chunk `sub` of k-block k
-        *reinterpret_cast<uint4*>(sA + k * KB_BYTES + r * 128 + ((sub ^ (r & 7)) << 4)) =
-            make_uint4(affine2(x[j][k].x, r2, m2, ga[k].x, be[k].x), affine2(x[j][k].y, r2, m2, ga[k].y, be[k].y),
-                       affine2(x[j][k].z, r2, m2, ga[k].z, be[k].z), affine2(x[j][k].w, r2, m2, ga[k].w, be[k].w));
-    }
+    ln_rows_to_operand<NV>(x, ga, be, g.eps, sA, warp, lane);
     ptx::fence_proxy_async();
     __syncwarp();
     if (lane == 0) ptx::mbar_arrive(a_ready);
@@ -231,7 +177,7 @@ mlp_cluster_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_consta
           const float2 f = bf16x2_to_float2(bw[e]);
           o[e] = float2_to_bf16x2(gelu_tanh(__uint_as_float(v[p][2 * e]) + f.x), gelu_tanh(__uint_as_float(v[p][2 * e + 1]) + f.y));
         }
-        uint8_t* h = sA + (c >> 6) * KB_BYTES + r * 128;
+        uint8_t* h = sA + (c >> 6) * kLnBlockBytes + r * 128;
         const int ch = (c & 63) >> 3;
         *reinterpret_cast<uint4*>(h + ((ch ^ (r & 7)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
         *reinterpret_cast<uint4*>(h + (((ch + 1) ^ (r & 7)) << 4)) = make_uint4(o[4], o[5], o[6], o[7]);
@@ -331,7 +277,7 @@ struct Sizes {
 };
 Sizes sizes_of(int C, int hs, int S) {
   Sizes z;
-  const int rows = (C > hs ? C : hs) / BK * KB_BYTES;              // the rows, later the hidden slice
+  const int rows = (C > hs ? C : hs) / BK * kLnBlockBytes;              // the rows, later the hidden slice
   z.w1_off = rows;
   z.w2_off = rows + C / BK * hs * 128;
   const int operands = z.w2_off + hs / BK * C * 128, partial = BM * C * 4, recv = (S - 1) * (BM / S) * C * 4;

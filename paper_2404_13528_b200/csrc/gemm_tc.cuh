@@ -101,6 +101,11 @@ int launch_mlp_cluster(const void* x, const void* ln_g, const void* ln_b, float 
 bool gemm_ln_supported(long long N, long long K);
 int launch_gemm_ln(const void* X, const DevMap* rowmap, const void* gamma, const void* beta, float eps, const void* W,
                    const void* bias, void* out, long long M, long long N, long long K, cudaStream_t st);
+// The same, with an optional GELU, for few rows of 128, 192 or 256 elements (gemm_ln_wave.cu).  gemm_ln_wave_wins: it covers the shape and
+// beats the separate kernels.
+bool gemm_ln_wave_wins(long long M, long long N, long long K);
+int launch_gemm_ln_wave(const void* X, const DevMap* rowmap, const void* gamma, const void* beta, float eps, const void* W, const void* bias,
+                        int gelu, void* out, long long M, long long N, long long K, cudaStream_t st);
 
 // Attention half of a narrow Swin block (bf16, head dimension 32, 2 or 3 heads, window^2 <= 64) in one kernel:
 // y = x + unshift(unpartition(proj(window_attention(qkv(LN1(partition(shift(x)))))))), every layout operator folded into the

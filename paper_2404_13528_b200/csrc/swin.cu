@@ -89,18 +89,22 @@ size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
 // Which fused kernels a block takes (they decide which intermediates exist at all).
 struct Path {
   bool fuse_attn, fuse_ln1, fuse_mlp;
+  bool ln1_wave;                   // (fuse_ln1) a slice of the columns per CTA
   bool mlp_cluster;                // (fuse_mlp) the hidden features split over a cluster
+  bool ln2_wave;                   // LN2 + fc1 + GELU in one kernel
 };
 Path choose_path(const smartmem_swin_params_t& p, int mode) {
   const bool bf16 = p.dtype == SMARTMEM_BF16;
   Path t;
   t.fuse_attn = mode == SMARTMEM_ELIMINATE && (bf16 ? swin_attn_fused_supported(p.dtype, p.C, p.heads, p.window)
                                                     : swin_attn_f32_supported(p.C, p.heads, p.window));
-  t.fuse_ln1 = bf16 && gemm_ln_supported(3 * (long long)p.C, p.C);
+  t.ln1_wave = bf16 && gemm_ln_wave_wins((long long)p.B * p.H * p.W, 3 * (long long)p.C, p.C);
+  t.fuse_ln1 = t.ln1_wave || (bf16 && gemm_ln_supported(3 * (long long)p.C, p.C));
   t.fuse_mlp = p.mlp_ratio > 0 && (bf16 ? mlp_fused_supported(p.C, (long long)p.C * p.mlp_ratio)
                                         : swin_mlp_f32_supported(p.C, (long long)p.C * p.mlp_ratio));
   t.mlp_cluster = bf16 && p.mlp_ratio > 0 && !t.fuse_mlp && mlp_cluster_wins((long long)p.B * p.H * p.W, p.C, (long long)p.C * p.mlp_ratio);
   t.fuse_mlp = t.fuse_mlp || t.mlp_cluster;
+  t.ln2_wave = bf16 && p.mlp_ratio > 0 && !t.fuse_mlp && gemm_ln_wave_wins((long long)p.B * p.H * p.W, (long long)p.C * p.mlp_ratio, p.C);
   return t;
 }
 
@@ -242,6 +246,10 @@ int run_block(const smartmem_swin_params_t* pp, const void* x, void* y, void* wo
   a.scale = 1.0f / sqrtf((float)d);
 
   const bool fuse_ln1 = path.fuse_ln1;
+  auto ln1_qkv = [&](const void* rows, const DevMap* map) {
+    return path.ln1_wave ? launch_gemm_ln_wave(rows, map, p.ln1_g, p.ln1_b, p.ln_eps, p.w_qkv, p.b_qkv, 0, at(L.qkv), M, 3 * C, C, st)
+                         : launch_gemm_ln(rows, map, p.ln1_g, p.ln1_b, p.ln_eps, p.w_qkv, p.b_qkv, at(L.qkv), M, 3 * C, C, st);
+  };
 #define SM_TRY(label, expr) do { if (tm) tm->tick(label); rc = (expr); if (rc != SMARTMEM_OK) return rc; } while (0)
   if (half == 1) {
     // MLP half only
@@ -251,7 +259,7 @@ int run_block(const smartmem_swin_params_t* pp, const void* x, void* y, void* wo
   } else if (elim) {
     if (fuse_ln1) {
       // narrow blocks: LN1, the shift o partition gather and the QKV projection in one kernel
-      SM_TRY("ln1_gather_qkv_gemm", launch_gemm_ln(x, &m.e1_rows, p.ln1_g, p.ln1_b, p.ln_eps, p.w_qkv, p.b_qkv, at(L.qkv), M, 3 * C, C, st));
+      SM_TRY("ln1_gather_qkv_gemm", ln1_qkv(x, &m.e1_rows));
     } else {
       SM_TRY("ln1_gather", launch_norm(p.dtype, false, x, at(L.xn), p.ln1_g, p.ln1_b, p.ln_eps, M, (int)C, &m.e1_rows, st));
       SM_TRY("qkv_gemm", linear(at(L.xn), p.w_qkv, p.b_qkv, at(L.qkv), 3 * C, C, 0, nullptr, nullptr));
@@ -278,7 +286,7 @@ int run_block(const smartmem_swin_params_t* pp, const void* x, void* y, void* wo
     }
     SM_TRY("copy_partition", launch_copy_map(m.part, esz, xs, at(L.xw), st));
     if (fuse_ln1) {
-      SM_TRY("ln1_qkv_gemm", launch_gemm_ln(at(L.xw), nullptr, p.ln1_g, p.ln1_b, p.ln_eps, p.w_qkv, p.b_qkv, at(L.qkv), M, 3 * C, C, st));
+      SM_TRY("ln1_qkv_gemm", ln1_qkv(at(L.xw), nullptr));
     } else {
       SM_TRY("qkv_gemm", linear(at(L.xw), p.w_qkv, p.b_qkv, at(L.qkv), 3 * C, C, 0, nullptr, nullptr));
     }
@@ -308,8 +316,12 @@ int run_block(const smartmem_swin_params_t* pp, const void* x, void* y, void* wo
              : path.mlp_cluster ? launch_mlp_cluster(y1, p.ln2_g, p.ln2_b, p.ln_eps, p.w_fc1, p.b_fc1, p.w_fc2, p.b_fc2, y, M, C, hid, st)
                                 : launch_mlp_fused(y1, p.ln2_g, p.ln2_b, p.ln_eps, p.w_fc1, p.b_fc1, p.w_fc2, p.b_fc2, y, M, C, hid, st));
     } else {
-      SM_TRY("ln2", launch_norm(p.dtype, false, y1, at(L.yn), p.ln2_g, p.ln2_b, p.ln_eps, M, (int)C, nullptr, st));
-      SM_TRY("fc1_gemm_gelu", linear(at(L.yn), p.w_fc1, p.b_fc1, at(L.hid), hid, C, 1, nullptr, nullptr));
+      if (path.ln2_wave) {
+        SM_TRY("ln2_fc1_gemm_gelu", launch_gemm_ln_wave(y1, nullptr, p.ln2_g, p.ln2_b, p.ln_eps, p.w_fc1, p.b_fc1, 1, at(L.hid), M, hid, C, st));
+      } else {
+        SM_TRY("ln2", launch_norm(p.dtype, false, y1, at(L.yn), p.ln2_g, p.ln2_b, p.ln_eps, M, (int)C, nullptr, st));
+        SM_TRY("fc1_gemm_gelu", linear(at(L.yn), p.w_fc1, p.b_fc1, at(L.hid), hid, C, 1, nullptr, nullptr));
+      }
       SM_TRY("fc2_gemm_residual", linear(at(L.hid), p.w_fc2, p.b_fc2, y, C, hid, 0, y1, nullptr));
     }
   }

@@ -68,3 +68,15 @@ def test_fp32_blocks(cfg):
 ])
 def test_mlp_over_a_cluster(cfg):
     case(504, dtype="bf16", **cfg)
+
+
+@pytest.mark.parametrize("cfg", [
+    dict(B=1, H=7, W=7, C=256, heads=8, window=7, shift=3, mlp_ratio=4),      # one tile of 49 rows, slices of 64 columns, GELU
+    dict(B=7, H=14, W=14, C=256, heads=8, window=7, shift=3, mlp_ratio=4),    # slices of 128, ragged last 92 rows
+    dict(B=17, H=16, W=8, C=256, heads=8, window=8, shift=0, mlp_ratio=3),    # slices of 128 (QKV and fc1)
+    dict(B=37, H=16, W=8, C=256, heads=8, window=8, shift=4, mlp_ratio=4),    # a full wave: slices of 192 and 256
+    dict(B=38, H=16, W=8, C=256, heads=8, window=8, shift=4, mlp_ratio=4),    # one tile more: kernel by kernel
+    dict(B=5, H=14, W=14, C=128, heads=4, window=7, shift=3, mlp_ratio=0),    # the narrowest rows
+])
+def test_norm_linear_in_one_wave(cfg):
+    case(505, dtype="bf16", **cfg)
