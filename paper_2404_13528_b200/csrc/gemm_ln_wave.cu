@@ -4,12 +4,11 @@
 // thousand rows there is nothing to stream: a launch, a dependency and a drain cost the normalisation and the product each more
 // than their work.  A CTA takes 128 rows and a slice of the output columns, normalises the rows (again in every slice: they come
 // from L2) straight into the operand, and multiplies them with its slice of W, fetched before the dependency wait.  Bound by that
-// chain (1.5 us rows, 0.9 product, 0.8 output and the dependency).  Measured, a block's attention half with norm + QKV linear
-// before -> with this: 3920 x 192 17.4 -> 15.7 us (93 CTAs), 7840 x 128 19.1 -> 16.3 (124), 1568 x 256 16.6 -> 15.4 (78), 4704 x 256
-// 20.5 -> 19.1 (148); an MLP half with norm + fc1 + GELU: 1568 x 256 13.1 -> 12.0.
+// chain (1.5 us rows, 0.9 product, 0.6 output and the dependency).  Measured, a block's attention half with norm + QKV linear
+// before -> with this: 3920 x 192 17.4 -> 15.4 us (93 CTAs), 7840 x 128 19.1 -> 16.3 (124), 1568 x 256 16.6 -> 14.8 (78), 4704 x 256
+// 20.5 -> 18.4 (148); an MLP half with norm + fc1 + GELU: 1568 x 256 13.1 -> 11.3.
 //
-// Warp roles: 0-15 rows, then bias and output through shared memory as 32 x 64 boxes; 16 fetches W, owns the tensor memory and issues
-// the product.
+// Warp roles: 0-15 rows, then bias and output; 16 fetches W, owns the tensor memory and issues the product.
 #include <cstring>
 
 #include "gemm_tc.cuh"
@@ -23,27 +22,26 @@ constexpr int BM = 128, BK = 64;
 constexpr int kWorkers = 16, kThreads = 32 * (kWorkers + 1);
 
 struct LnWaveArgs {
-  int M, slices, has_map, gelu;
+  int M, N, slices, has_map, gelu, wide;
   float eps;
   const __nv_bfloat16 *x, *ln_g, *ln_b, *bias;
+  __nv_bfloat16* out;
   DevMap rowmap;
   int* status;
 };
 
 template <int NV, int NB>
-constexpr int wave_out_bytes() { return (NV > NB ? NV : NB) * kLnBlockBytes; }       // the rows, later the output
-template <int NV, int NB>
-constexpr int wave_smem_bytes() { return 1024 + wave_out_bytes<NV, NB>() + NV * NB * 64 * 128 + NB * 64 * 2 + 4 * 8; }
+constexpr int wave_smem_bytes() { return 1024 + NV * kLnBlockBytes + NV * NB * 64 * 128 + NB * 64 * 2 + 4 * 8; }
 
 template <int NV, int NB>                          // K / 64, columns of a slice / 64
 __global__ void __launch_bounds__(kThreads, 1)
-ln_wave_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmO, const __grid_constant__ LnWaveArgs g) {
+ln_wave_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ LnWaveArgs g) {
   constexpr int K = 64 * NV, NS = 64 * NB;
   constexpr uint32_t TMEM_COLS = NB > 2 ? 256 : NS;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
   uint8_t* sA = smem;
-  uint8_t* sW = smem + wave_out_bytes<NV, NB>();   // [NV][NS x 128 B]
+  uint8_t* sW = smem + NV * kLnBlockBytes;   // [NV][NS x 128 B]
   __nv_bfloat16* bias_s = reinterpret_cast<__nv_bfloat16*>(sW + NV * NS * 128);
   uint64_t* w_full = reinterpret_cast<uint64_t*>(bias_s + NS);
   uint64_t *a_ready = w_full + 1, *d_full = w_full + 2;
@@ -62,15 +60,12 @@ ln_wave_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       ptx::fence_barrier_init();
       ptx::fence_proxy_async();
       ptx::prefetch_tensormap(&tmW);
-      ptx::prefetch_tensormap(&tmO);
       ptx::mbar_expect_tx(w_full, (uint32_t)(NS * K * 2));
     }
     __syncwarp();
-#pragma unroll
-    for (int kb = 0; kb < NV; ++kb) {              // a parameter: fetched before the dependency wait
-      if (ptx::elect_one()) ptx::tma_load_2d(sW + kb * NS * 128, &tmW, w_full, kb * BK, n0);
-      __syncwarp();
-    }
+    // a parameter: fetched before the dependency wait, all k-blocks in one copy
+    if (ptx::elect_one()) ptx::tma_load_3d(sW, &tmW, w_full, 0, n0, 0);
+    __syncwarp();
     ptx::tmem_alloc(tmem_slot, TMEM_COLS);
   }
   if (tid < NS / 8)
@@ -123,49 +118,33 @@ ln_wave_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         if (m0 + warp * 8 + r < g.M) x[j][k] = *reinterpret_cast<const uint4*>(g.x + off + (sub + L * k) * 8);
       }
     }
-    ln_rows_to_operand<NV>(x, ga, be, g.eps, sA, warp, lane);
+    ln_rows_to_operand<NV>(x, ga, be, g.eps, sA, warp * 8, lane);
     ptx::fence_proxy_async();
     __syncwarp();
     if (lane == 0) ptx::mbar_arrive(a_ready);
 
-    // ---- output: a thread per row and quarter of the columns, through the rows' memory ------------------------------------
-    const int q = warp & 3, grp = warp >> 2, r = q * 32 + lane;
+    // ---- output: a thread per row and quarter of the columns, rows leave the registers as whole sectors ---------------------
+    const int q = warp & 3, grp = warp >> 2, m = m0 + q * 32 + lane;
     const bool ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(d_full, 0, abort_flag, g.status) ? 1 : 0) != 0;
     if (ok) {
       ptx::tc_fence_after();
-      uint32_t v[NB][16];
-#pragma unroll
-      for (int p = 0; p < NB; ++p) ptx::tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (grp * NB + p) * 16, v[p]);
-      ptx::tmem_ld_wait();
 #pragma unroll
       for (int p = 0; p < NB; ++p) {
         const int c = (grp * NB + p) * 16;
+        uint32_t v[16], o[8];
+        ptx::tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + c, v);
         const uint4 b0 = *reinterpret_cast<const uint4*>(bias_s + c), b1 = *reinterpret_cast<const uint4*>(bias_s + c + 8);
         const uint32_t bw[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-        uint32_t o[8];
+        ptx::tmem_ld_wait();
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           float2 f = bf16x2_to_float2(bw[e]);
-          f = make_float2(__uint_as_float(v[p][2 * e]) + f.x, __uint_as_float(v[p][2 * e + 1]) + f.y);
+          f = make_float2(__uint_as_float(v[2 * e]) + f.x, __uint_as_float(v[2 * e + 1]) + f.y);
           if (g.gelu) f = make_float2(gelu_tanh(f.x), gelu_tanh(f.y));
           o[e] = float2_to_bf16x2(f.x, f.y);
         }
-        uint8_t* h = sA + (c >> 6) * kLnBlockBytes + r * 128;
-        const int ch = (c & 63) >> 3;
-        *reinterpret_cast<uint4*>(h + ((ch ^ (r & 7)) << 4)) = make_uint4(o[0], o[1], o[2], o[3]);
-        *reinterpret_cast<uint4*>(h + (((ch + 1) ^ (r & 7)) << 4)) = make_uint4(o[4], o[5], o[6], o[7]);
+        if (m < g.M) ln_store16(g.out + (size_t)m * g.N + n0 + c, o, g.wide);
       }
-      ptx::fence_proxy_async();
-    }
-    asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory");        // the four warps of these 32 rows
-    if (ok && grp == 0 && m0 + q * 32 < g.M) {                          // (rows past M are clipped by the tensor map)
-      if (ptx::elect_one()) {
-#pragma unroll
-        for (int b = 0; b < NB; ++b) ptx::tma_store_2d(&tmO, sA + b * kLnBlockBytes + q * 4096, n0 + b * 64, m0 + q * 32);
-        ptx::bulk_commit_group();
-        ptx::bulk_wait_group<0>();                   // the CTA's shared memory must outlive its stores
-      }
-      __syncwarp();
     }
   }
   ptx::tc_fence_before();
@@ -177,18 +156,18 @@ ln_wave_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 }
 
 template <int NV, int NB>
-int launch_wave(const CUtensorMap& tw, const CUtensorMap& to, const LnWaveArgs& g, cudaStream_t st) {
+int launch_wave(const CUtensorMap& tw, const LnWaveArgs& g, cudaStream_t st) {
   if (ensure_max_dynamic_smem((const void*)ln_wave_kernel<NV, NB>, wave_smem_bytes<NV, NB>()) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   profile_tick("gemm_ln_wave", st);
   const unsigned grid = (unsigned)((g.M + BM - 1) / BM * g.slices);
-  if (launch_pdl(ln_wave_kernel<NV, NB>, dim3(grid), dim3(kThreads), wave_smem_bytes<NV, NB>(), st, tw, to, g) != cudaSuccess) return SMARTMEM_ERR_CUDA;
+  if (launch_pdl(ln_wave_kernel<NV, NB>, dim3(grid), dim3(kThreads), wave_smem_bytes<NV, NB>(), st, tw, g) != cudaSuccess) return SMARTMEM_ERR_CUDA;
   count_launch();
   return SMARTMEM_OK;
 }
 
-int launch_blocks(int nv, int nb, const CUtensorMap& tw, const CUtensorMap& to, const LnWaveArgs& g, cudaStream_t st) {
+int launch_blocks(int nv, int nb, const CUtensorMap& tw, const LnWaveArgs& g, cudaStream_t st) {
   switch (nv * 8 + nb) {
-#define SM_WAVE(NV, NB) case NV * 8 + NB: return launch_wave<NV, NB>(tw, to, g, st);
+#define SM_WAVE(NV, NB) case NV * 8 + NB: return launch_wave<NV, NB>(tw, g, st);
     SM_WAVE(2, 1) SM_WAVE(2, 2) SM_WAVE(2, 3) SM_WAVE(2, 4)
     SM_WAVE(3, 1) SM_WAVE(3, 2) SM_WAVE(3, 3) SM_WAVE(3, 4)
     SM_WAVE(4, 1) SM_WAVE(4, 2) SM_WAVE(4, 3) SM_WAVE(4, 4)
@@ -222,16 +201,16 @@ int launch_gemm_ln_wave(const void* X, const DevMap* rowmap, const void* gamma, 
   if ((uintptr_t)bias & 15) return SMARTMEM_ERR_ALIGNMENT;
   LnWaveArgs g;
   memset(&g, 0, sizeof(g));
-  g.M = (int)M; g.slices = (int)(N / ns); g.has_map = rowmap ? 1 : 0; g.gelu = gelu;
+  g.M = (int)M; g.N = (int)N; g.slices = (int)(N / ns); g.has_map = rowmap ? 1 : 0; g.gelu = gelu;
   if (rowmap) g.rowmap = *rowmap;
   g.eps = eps;
-  g.x = (const __nv_bfloat16*)X; g.ln_g = (const __nv_bfloat16*)gamma; g.ln_b = (const __nv_bfloat16*)beta; g.bias = (const __nv_bfloat16*)bias;
+  g.x = (const __nv_bfloat16*)X; g.ln_g = (const __nv_bfloat16*)gamma; g.ln_b = (const __nv_bfloat16*)beta; g.bias = (const __nv_bfloat16*)bias; g.out = (__nv_bfloat16*)out;
+  g.wide = ((uintptr_t)out & 31) == 0;
   g.status = device_status_ptr();
   if (!g.status) return SMARTMEM_ERR_CUDA;
-  CUtensorMap tw, to;
-  int rc = tc_encode_2d(W, K, N, K, BK, ns, &tw);
-  if (rc == SMARTMEM_OK) rc = tc_encode_2d(out, N, M, N, 64, 32, &to);
-  return rc == SMARTMEM_OK ? launch_blocks((int)(K / 64), nb, tw, to, g, st) : rc;
+  CUtensorMap tw;
+  int rc = tc_encode_2d_blocks(W, K, N, K / BK, ns, &tw);
+  return rc == SMARTMEM_OK ? launch_blocks((int)(K / 64), nb, tw, g, st) : rc;
 }
 
 }  // namespace smartmem

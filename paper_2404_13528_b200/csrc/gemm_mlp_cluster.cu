@@ -82,15 +82,11 @@ mlp_cluster_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_consta
       if (S > 1) ptx::mbar_expect_tx(recv_full, (uint32_t)(S - 1) * slice_bytes);
     }
     __syncwarp();
-    // the weight slices are parameters: fetched before the dependency wait
-    for (int kb = 0; kb < NV; ++kb) {
-      if (ptx::elect_one()) ptx::tma_load_2d(sW1 + kb * g.hs * 128, &tmW1, w1_full, kb * BK, rank * g.hs);
-      __syncwarp();
-    }
-    for (int kb = 0; kb < g.hs / BK; ++kb) {
-      if (ptx::elect_one()) ptx::tma_load_2d(sW2 + kb * C * 128, &tmW2, w2_full, rank * g.hs + kb * BK, 0);
-      __syncwarp();
-    }
+    // the weight slices are parameters: fetched before the dependency wait, all k-blocks of one in a copy
+    if (ptx::elect_one()) ptx::tma_load_3d(sW1, &tmW1, w1_full, 0, rank * g.hs, 0);
+    __syncwarp();
+    if (ptx::elect_one()) ptx::tma_load_3d(sW2, &tmW2, w2_full, 0, 0, rank * (g.hs / BK));
+    __syncwarp();
     ptx::tmem_alloc(tmem_slot, TMEM_COLS);
   }
   if (tid < HS / 8) reinterpret_cast<uint4*>(b1_s)[tid] = *reinterpret_cast<const uint4*>(g.b1 + rank * HS + tid * 8);
@@ -151,7 +147,7 @@ mlp_cluster_kernel(const __grid_constant__ CUtensorMap tmW1, const __grid_consta
         x[j][k] = make_uint4(0, 0, 0, 0);
         if (m < g.M) x[j][k] = *reinterpret_cast<const uint4*>(g.x + (size_t)m * C + (sub + 8 * k) * 8);
       }
-    ln_rows_to_operand<NV>(x, ga, be, g.eps, sA, warp, lane);
+    ln_rows_to_operand<NV>(x, ga, be, g.eps, sA, warp * 8, lane);
     ptx::fence_proxy_async();
     __syncwarp();
     if (lane == 0) ptx::mbar_arrive(a_ready);
@@ -321,8 +317,8 @@ int launch_mlp_cluster(const void* x, const void* ln_g, const void* ln_b, float 
   g.status = device_status_ptr();
   if (!g.status) return SMARTMEM_ERR_CUDA;
   CUtensorMap t1, t2;
-  int rc = tc_encode_2d(W1, C, hidden, C, BK, g.hs, &t1);
-  if (rc == SMARTMEM_OK) rc = tc_encode_2d(W2, hidden, C, hidden, BK, (int)C, &t2);
+  int rc = tc_encode_2d_blocks(W1, C, hidden, C / BK, g.hs, &t1);
+  if (rc == SMARTMEM_OK) rc = tc_encode_2d_blocks(W2, hidden, C, g.hs / BK, C, &t2);
   if (rc != SMARTMEM_OK) return rc;
   static constexpr decltype(&mlp_cluster_kernel<1, 1>) kernels[3][4] = {
       {mlp_cluster_kernel<1, 1>, mlp_cluster_kernel<1, 2>, mlp_cluster_kernel<1, 3>, mlp_cluster_kernel<1, 4>},

@@ -902,6 +902,12 @@ int tc_encode_nd_sw128(const void* ptr, int rank, const long long* dims, const l
   return encode_nd(ptr, rank, dims, strides_elems, box, 128, out);
 }
 
+int tc_encode_2d_blocks(const void* ptr, long long inner, long long outer, long long blocks, long long rows, CUtensorMap* out) {
+  const long long dims[3] = {BK, outer, inner / BK}, strides[2] = {inner, BK};
+  const int box[3] = {BK, (int)rows, (int)blocks};
+  return tc_encode_nd_sw128(ptr, 3, dims, strides, box, out);
+}
+
 int tc_sm_count() { return sm_count(); }
 
 int tc_cluster_ctas(int size) {

@@ -73,6 +73,9 @@ int tc_encode_nd_sw64(const void* ptr, int rank, const long long* dims, const lo
 // Same with 128-byte swizzle and a box of 64 innermost elements.
 int tc_encode_nd_sw128(const void* ptr, int rank, const long long* dims, const long long* strides_elems, const int* box,
                        CUtensorMap* out);
+// A contiguous matrix [outer, inner] (inner a multiple of 64) as blocks of 64 columns: coordinates (0, row, block); a box of `rows` rows
+// and `blocks` blocks arrives as one K-major operand block of rows x 128 bytes after the other.
+int tc_encode_2d_blocks(const void* ptr, long long inner, long long outer, long long blocks, long long rows, CUtensorMap* out);
 // Same without swizzle.
 int tc_encode_2d_plain(const void* ptr, long long inner, long long outer, long long pitch_elems, int box_inner, int box_outer,
                        CUtensorMap* out);
@@ -106,6 +109,11 @@ int launch_gemm_ln(const void* X, const DevMap* rowmap, const void* gamma, const
 bool gemm_ln_wave_wins(long long M, long long N, long long K);
 int launch_gemm_ln_wave(const void* X, const DevMap* rowmap, const void* gamma, const void* beta, float eps, const void* W, const void* bias,
                         int gelu, void* out, long long M, long long N, long long K, cudaStream_t st);
+// LayerNorm o gather o linear without bias for rows of 256 or 384 elements, gathered in 16-byte vectors through a map over
+// [M, K] without rolls (gemm_ln_pair.cu; SMARTMEM_ERR_UNSUPPORTED where the map does not split into rows).  out may not overlap X.
+bool gemm_ln_pair_supported(const smartmem_index_map_t& map, long long M, long long N, long long K);
+int launch_gemm_ln_pair(const void* X, const smartmem_index_map_t& map, const void* gamma, const void* beta, float eps, const void* W,
+                        void* out, long long M, long long N, long long K, cudaStream_t st);
 
 // Attention half of a narrow Swin block (bf16, head dimension 32, 2 or 3 heads, window^2 <= 64) in one kernel:
 // y = x + unshift(unpartition(proj(window_attention(qkv(LN1(partition(shift(x)))))))), every layout operator folded into the
