@@ -204,7 +204,24 @@ EXPORT int smartmem_run_chain(const smartmem_plan_t* plan, const void* const* in
     if (ref == -1) return outputs[0];
     return (char*)workspace + plan->slot_offset[-2 - ref];
   };
-  for (const Step& s : plan->steps) {
+  // LayerNorm whose rows only the linear after it reads: one kernel, the normalised rows never leave the chip
+  auto norm_linear = [&](const Step& n, const Step& l) {
+    if (n.kind != STEP_NORM || l.kind != STEP_LINEAR || n.dtype != SMARTMEM_BF16 || l.dtype != SMARTMEM_BF16 ||
+        n.dst > -2 || l.src[0] != n.dst || l.map[0].klass != 0 || l.batch != 1 || l.M != n.M || l.K != n.K ||
+        !gemm_ln_pair_wins(n.map[0], n.M, l.N, n.K))
+      return (int)SMARTMEM_ERR_UNSUPPORTED;
+    const char *x = (const char*)buf(n.src[0]), *y = (const char*)buf(l.dst);
+    if (x < y + l.M * l.N * 2 && y < x + n.M * n.K * 2) return (int)SMARTMEM_ERR_UNSUPPORTED;      // in place: the rows must be read first
+    return launch_gemm_ln_pair(x, n.map[0], inputs[n.weight], inputs[n.weight2], n.eps, inputs[l.weight], buf(l.dst), l.M, l.N, l.K, st);
+  };
+  for (size_t i = 0; i < plan->steps.size(); ++i) {
+    const Step& s = plan->steps[i];
+    if (s.kind == STEP_NORM && i + 1 < plan->steps.size()) {
+      const int rc = norm_linear(s, plan->steps[i + 1]);
+      if (rc == SMARTMEM_OK) ++i;
+      if (rc == SMARTMEM_OK) continue;
+      if (rc != SMARTMEM_ERR_UNSUPPORTED) return rc;
+    }
     const int esz = s.dtype == SMARTMEM_F32 ? 4 : 2;
     int rc = SMARTMEM_OK;
     if (s.kind == STEP_COPY) {

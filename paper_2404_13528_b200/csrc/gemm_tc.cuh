@@ -109,9 +109,9 @@ int launch_gemm_ln(const void* X, const DevMap* rowmap, const void* gamma, const
 bool gemm_ln_wave_wins(long long M, long long N, long long K);
 int launch_gemm_ln_wave(const void* X, const DevMap* rowmap, const void* gamma, const void* beta, float eps, const void* W, const void* bias,
                         int gelu, void* out, long long M, long long N, long long K, cudaStream_t st);
-// LayerNorm o gather o linear without bias for rows of 256 or 384 elements, gathered in 16-byte vectors through a map over
+// LayerNorm o gather o linear without bias for rows of 256, 384 or 512 elements, gathered in 16-byte vectors through a map over
 // [M, K] without rolls (gemm_ln_pair.cu; SMARTMEM_ERR_UNSUPPORTED where the map does not split into rows).  out may not overlap X.
-bool gemm_ln_pair_supported(const smartmem_index_map_t& map, long long M, long long N, long long K);
+bool gemm_ln_pair_wins(const smartmem_index_map_t& map, long long M, long long N, long long K);
 int launch_gemm_ln_pair(const void* X, const smartmem_index_map_t& map, const void* gamma, const void* beta, float eps, const void* W,
                         void* out, long long M, long long N, long long K, cudaStream_t st);
 

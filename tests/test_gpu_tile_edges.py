@@ -80,3 +80,16 @@ def test_mlp_over_a_cluster(cfg):
 ])
 def test_norm_linear_in_one_wave(cfg):
     case(505, dtype="bf16", **cfg)
+
+
+@pytest.mark.parametrize("B,H,W,C", [
+    (1, 2, 2, 64), (1, 2, 2, 96),             # one row
+    (3, 26, 22, 64),                          # 429 rows of 256: three tiles of 192, ragged last 45
+    (20, 64, 62, 64),                         # 19840 rows: two rounds of 192-row tiles
+    (15, 62, 62, 96),                         # 14415 rows of 384: one round of 256-row tiles, ragged last 79
+    (5, 124, 124, 96),                        # 19220 rows: two rounds of 192-row tiles, ragged last 20
+    (1, 2, 2, 128), (3, 26, 22, 128),         # rows of 512, two slices of the columns
+    (9, 62, 64, 128), (10, 62, 64, 128),      # 8928 rows in one round; 9920 are two: kernel by kernel
+])
+def test_merge_in_one_kernel(B, H, W, C):
+    patch_merging_case(B, H, W, C)
