@@ -118,7 +118,8 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + N_BARS);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
-  float* ln_s = reinterpret_cast<float*>(tmem_slot + 4);     // [2][C]: gamma, beta
+  float* ln_s = reinterpret_cast<float*>(tmem_slot + 4);     // [C] beta, [C] gamma as bf16 (+ spare)
+  __nv_bfloat16* lng_s = reinterpret_cast<__nv_bfloat16*>(ln_s + C);
   float* rstd_s = ln_s + 2 * C;                              // [RSTD_RING][128]
 
   // The tiles fill the 227 KB almost completely, so the launch cannot afford a spare kilobyte of
@@ -177,17 +178,18 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
       __syncwarp();
     }
   }
+  // (warp 0 is busy with the copies)
 #pragma unroll 1
-  for (int i = tid; i < C; i += kThreads) {
-    ln_s[i] = __bfloat162float(g.ln_gamma[i]);
-    ln_s[C + i] = __bfloat162float(g.ln_beta[i]);
+  for (int i = tid - 32; warp != 0 && i < C; i += kThreads - 32) {
+    lng_s[i] = g.ln_gamma[i];
+    ln_s[i] = __bfloat162float(g.ln_beta[i]);
     uint4 k0, k1;
     bias_col(2.0f * __bfloat162float(g.b2[i]), k0, k1);     // (the output accumulator holds twice the result)
     *reinterpret_cast<uint4*>(sB2x + plain_off(i, 0)) = k0;
     *reinterpret_cast<uint4*>(sB2x + plain_off(i, 1)) = k1;
   }
 #pragma unroll 1
-  for (int i = tid; i < (2 * AX_BYTES + ID_BYTES) / 16; i += kThreads) {
+  for (int i = tid - 32; warp != 0 && i < (2 * AX_BYTES + ID_BYTES) / 16; i += kThreads - 32) {
     uint8_t* p = i < 2 * AX_BYTES / 16 ? sAx + i * 16 : sId + (i - 2 * AX_BYTES / 16) * 16;
     *reinterpret_cast<uint4*>(p) = make_uint4(0, 0, 0, 0);
   }
@@ -206,34 +208,16 @@ mlp_fused_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
   if (warp != 0) {
     w_ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(w1_full, 0, abort_flag, g.status) ? 1 : 0) != 0;
     if (w_ok) {
-      const int nch = C / 8;
+      constexpr int nch = C / 8;
 #pragma unroll 1
       for (int t2 = tid - 32; t2 < 2 * g.hidden; t2 += kThreads - 32) {
         const int row = t2 >> 1, half = t2 & 1;
-        float csum = 0.f, bsum = half ? 0.f : __bfloat162float(g.b1[row]);
-        float bsum2 = 0.f;
-#pragma unroll 2
-        for (int ci = half * (nch / 2); ci < (half + 1) * (nch / 2); ++ci) {     // chunk ci of the row: k-block ci / 4, chunk ci % 4
-          uint4* p = reinterpret_cast<uint4*>(sW1 + (ci >> 2) * W1_KB + sw64_off(row, ci & 3));
-          const uint4 wv = *p;
-          const uint32_t w4[4] = {wv.x, wv.y, wv.z, wv.w};
-          const float4 ga0 = *reinterpret_cast<const float4*>(ln_s + ci * 8), ga1 = *reinterpret_cast<const float4*>(ln_s + ci * 8 + 4);
-          const float4 be0 = *reinterpret_cast<const float4*>(ln_s + C + ci * 8), be1 = *reinterpret_cast<const float4*>(ln_s + C + ci * 8 + 4);
-          const float ga[8] = {ga0.x, ga0.y, ga0.z, ga0.w, ga1.x, ga1.y, ga1.z, ga1.w};
-          const float be[8] = {be0.x, be0.y, be0.z, be0.w, be1.x, be1.y, be1.z, be1.w};
-          uint32_t o4[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const float2 f = bf16x2_to_float2(w4[e]);
-            bsum = fmaf(be[2 * e], f.x, bsum);
-            bsum2 = fmaf(be[2 * e + 1], f.y, bsum2);
-            o4[e] = float2_to_bf16x2(ga[2 * e] * f.x, ga[2 * e + 1] * f.y);
-            const float2 r2 = bf16x2_to_float2(o4[e]);
-            csum += r2.x + r2.y;
-          }
-          *p = make_uint4(o4[0], o4[1], o4[2], o4[3]);
-        }
-        bsum += bsum2;
+        const float b0 = half ? 0.f : __bfloat162float(g.b1[row]);
+        FoldSums f;
+#pragma unroll 1
+        for (int ci = half * (nch / 2); ci < (half + 1) * (nch / 2); ++ci)      // chunk ci of the row: k-block ci / 4, chunk ci % 4
+          fold_chunk(sW1 + (ci >> 2) * W1_KB + sw64_off(row, ci & 3), lng_s + ci * 8, ln_s + ci * 8, f);
+        float csum = f.c(), bsum = b0 + f.b();
         csum += __shfl_xor_sync(0xFFFFFFFFu, csum, 1);
         bsum += __shfl_xor_sync(0xFFFFFFFFu, bsum, 1);
         if (half == 0) {

@@ -81,7 +81,7 @@ constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t TM_Y = NBUF * BUF_COLS;          // the projection's accumulator (C columns) after the item buffers
 constexpr uint32_t ROW_INVALID = 0xFFFFFFFFu;       // no such row (a padding row of the tile, or a window past the end)
 constexpr int WIN_MISSING = 0, WIN_GATHER = 1, WIN_BOX = 2;
-constexpr int N_BARS = 26;
+constexpr int N_BARS = 29;
 
 struct FusedArgs {
   int n_windows, n_pairs, T, ws, shift, H, W;
@@ -128,15 +128,16 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
   float* bp_s = reinterpret_cast<float*>(bias_s + NH * T * BR);    // [C]
   float* rstd_s = bp_s + C;                                        // [na][128]
   uint32_t* rowoff_s = reinterpret_cast<uint32_t*>(rstd_s + na * BM);   // [NRING][128]: row offset in 16-byte units
-  float* ln_s = reinterpret_cast<float*>(rowoff_s + NRING * BM);   // [2][C]: gamma, beta
+  float* ln_s = reinterpret_cast<float*>(rowoff_s + NRING * BM);   // [C] beta, [C] gamma as bf16 (+ spare)
+  __nv_bfloat16* lng_s = reinterpret_cast<__nv_bfloat16*>(ln_s + C);
   int* tyx_s = reinterpret_cast<int*>(ln_s + 2 * C);               // [64]: ty << 8 | tx
   uint32_t* kmask_s = reinterpret_cast<uint32_t*>(tyx_s + TP);     // [4]
   int4* tok_s = reinterpret_cast<int4*>(kmask_s + 4);              // [64]: the map's contribution of token t: (offset, u0, u1, -)
   int4* win_s = tok_s + TP;                                        // [2 units][2 windows]: the contribution of window n: (offset lo, hi, u0, u1)
   int* wkind_s = reinterpret_cast<int*>(win_s + 4);                // [na][2 windows] (+ pad): how the window's rows come in
   uint64_t* bars = reinterpret_cast<uint64_t*>(wkind_s + 8);
-  uint64_t* w_full = bars;
-  uint64_t *a_full = bars + 1, *a_free = a_full + 3, *landed = a_free + 3;     // [3] each: per slot of the row ring
+  uint64_t* w_full = bars;                                         // [NH] QKV weights of a head, then the projection's
+  uint64_t *a_full = bars + 4, *a_free = a_full + 3, *landed = a_free + 3;     // [3] each: per slot of the row ring
   uint64_t *s_full = landed + 3, *o_full = s_full + 3;             // [3] each: per group (the group issues these products itself)
   uint64_t *acc_full = o_full + 3, *ob_full = acc_full + NBUF;     // [NBUF] each: per item buffer (items 4 apart share one)
   uint64_t *y_full = ob_full + NBUF, *y_empty = y_full + 1;
@@ -160,76 +161,107 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
   const int total = U * NH;                                                         // items
   const float LOG2E = 1.4426950408889634f;
 
-  if (tid == 0) {
-    ptx::mbar_init(w_full, 1);
-#pragma unroll 1
-    for (int i = 0; i < 3; ++i) {
-      ptx::mbar_init(&a_full[i], 4);
-      ptx::mbar_init(&a_free[i], NH + 1);
-      ptx::mbar_init(&landed[i], 4);
-      ptx::mbar_init(&s_full[i], 1);
-      ptx::mbar_init(&o_full[i], 1);
-    }
-#pragma unroll 1
-    for (int i = 0; i < NBUF; ++i) {
-      ptx::mbar_init(&acc_full[i], 1);
-      ptx::mbar_init(&ob_full[i], 4);
-    }
-    ptx::mbar_init(y_full, 1);
-    ptx::mbar_init(y_empty, 4);
-    *abort_flag = 0;
-    ptx::fence_barrier_init();
-    ptx::fence_proxy_async();
-    ptx::prefetch_tensormap(&tmX);
-  }
+  // The prologue is a tenth of the kernel at the benchmark's batch (a CTA cannot start beside one of the kernel before it: shared
+  // memory), so it is kept short: the weight copies leave before anything else is set up, every global load is requested before the
+  // first is used, and what does not need the weights is done by warps that do not fold them (10300 -> 5000 cycles).
   if (warp == 0) {
-    __syncwarp();
-    // The weights do not depend on the kernel before this one: fetch them right away, in few boxes issued by an elected lane (a
-    // box per head, k-block and q / k / v under a branch on thread 0 took 30 issues of about 0.2 us)
-    if (ptx::elect_one()) ptx::mbar_expect_tx(w_full, (uint32_t)(NH * NH * WQ_TILE + NH * WP_TILE));
+    // The weights do not depend on the kernel before this one: fetch them right away, in one box per head and one for the
+    // projection, issued by an elected lane (a copy takes about 130 ns to issue)
+    if (ptx::elect_one()) {
+#pragma unroll
+      for (int h = 0; h <= NH; ++h) ptx::mbar_init(&w_full[h], 1);
+      ptx::fence_barrier_init();
+      ptx::fence_proxy_async();
+#pragma unroll
+      for (int h = 0; h <= NH; ++h) ptx::mbar_expect_tx(&w_full[h], (uint32_t)(NH * (h < NH ? WQ_TILE : WP_TILE)));
+    }
     __syncwarp();
 #pragma unroll 1
-    for (int h = 0; h < NH; ++h) {
-#pragma unroll 1
-      for (int kb = 0; kb < NH; ++kb) {                // (head, k-block): 32 columns x 32 weight rows each of q, k and v
-        if (ptx::elect_one()) ptx::tma_load_3d(sWq + (h * NH + kb) * WQ_TILE, &tmWq, w_full, kb * D, h * D, 0);
-        __syncwarp();
-      }
-      if (ptx::elect_one()) ptx::tma_load_2d(sWp + h * WP_TILE, &tmWp, w_full, h * D, 0);
+    for (int i = 0, h = (int)blockIdx.x % NH; i < NH; ++i, h = h + 1 == NH ? 0 : h + 1) {    // (not every CTA asks L2 for the same head first)
+      // 32 weight rows each of q, k and v, every k-block of 32 columns
+      if (ptx::elect_one()) ptx::tma_load_4d(sWq + h * NH * WQ_TILE, &tmWq, &w_full[h], 0, h * D, 0, 0);
       __syncwarp();
     }
-  }
-  if (warp == 0) ptx::tmem_alloc(tmem_slot, TMEM_COLS);
-  // parameter-only tables
-  const int n_table = (2 * ws - 1) * (2 * ws - 1);
-  for (int i = tid; i < NH * 256; i += kThreads) {
-    const int h = i >> 8, e = i & 255;
-    raw_s[i] = e < n_table ? reinterpret_cast<const uint16_t*>(g.table)[e * NH + h] : (uint16_t)0;
-  }
-  if (tid < TP) {
-    tyx_s[tid] = ((tid / ws) << 8) | (tid % ws);
-    int4 tk = make_int4(0, 0, 0, 0);
-    if (g.split >= 0 && tid < T) {
-      const DevMapPart pt = devmap_part_rolled(g.rowmap, g.split, g.rowmap.n_atoms, (uint32_t)tid);
-      tk = make_int4((int)pt.off, pt.u0, pt.u1, 0);
+    if (ptx::elect_one()) ptx::tma_load_3d(sWp, &tmWp, &w_full[NH], 0, 0, 0);
+    __syncwarp();
+  } else if (warp == 1) {
+    if (ptx::elect_one()) {
+#pragma unroll 1
+      for (int i = 0; i < 3; ++i) {
+        ptx::mbar_init(&a_full[i], 4);
+        ptx::mbar_init(&a_free[i], NH + 1);
+        ptx::mbar_init(&landed[i], 4);
+        ptx::mbar_init(&s_full[i], 1);
+        ptx::mbar_init(&o_full[i], 1);
+      }
+#pragma unroll 1
+      for (int i = 0; i < NBUF; ++i) {
+        ptx::mbar_init(&acc_full[i], 1);
+        ptx::mbar_init(&ob_full[i], 4);
+      }
+      ptx::mbar_init(y_full, 1);
+      ptx::mbar_init(y_empty, 4);
+      *abort_flag = 0;
+      ptx::fence_barrier_init();
+      ptx::fence_proxy_async();
+      ptx::prefetch_tensormap(&tmX);
     }
-    tok_s[tid] = tk;
+    __syncwarp();
+  } else if (warp == 2) {
+    ptx::tmem_alloc(tmem_slot, TMEM_COLS);
   }
-  for (int i = tid; i < C; i += kThreads) {
-    ln_s[i] = __bfloat162float(g.ln_g[i]);
-    ln_s[C + i] = __bfloat162float(g.ln_b[i]);
-    bp_s[i] = __bfloat162float(g.b_proj[i]);
+  // parameter-only tables: requested here, stored below
+  static_assert(NH * 256 <= 2 * kThreads && C <= kThreads, "two table entries and one channel per thread");
+  const int n_table = (2 * ws - 1) * (2 * ws - 1);
+  uint16_t tab[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int i = tid + k * kThreads, h = i >> 8, e = i & 255;
+    tab[k] = i < NH * 256 && e < n_table ? reinterpret_cast<const uint16_t*>(g.table)[e * NH + h] : (uint16_t)0;
+  }
+  __nv_bfloat16 par[3] = {};
+  if (tid < C) {
+    par[0] = g.ln_g[tid];
+    par[1] = g.ln_b[tid];
+    par[2] = g.b_proj[tid];
   }
   for (int i = tid; i < na * A_BYTES / 16; i += kThreads) reinterpret_cast<uint4*>(sA)[i] = make_uint4(0, 0, 0, 0);
   for (int i = tid; i < na * AX_BYTES / 16; i += kThreads) reinterpret_cast<uint4*>(sAx)[i] = make_uint4(0, 0, 0, 0);
   for (int i = tid; i < ID_BYTES / 16; i += kThreads) reinterpret_cast<uint4*>(sId)[i] = make_uint4(0, 0, 0, 0);
   for (int i = tid; i < na * BM; i += kThreads) rstd_s[i] = 0.f;
   for (int i = tid; i < NRING * BM; i += kThreads) rowoff_s[i] = ROW_INVALID;
+  if (tid >= 128 && tid < 128 + TP) {
+    const int t = tid - 128;
+    tyx_s[t] = ((t / ws) << 8) | (t % ws);
+    int4 tk = make_int4(0, 0, 0, 0);
+    if (g.split >= 0 && t < T) {
+      const DevMapPart pt = devmap_part_rolled(g.rowmap, g.split, g.rowmap.n_atoms, (uint32_t)t);
+      tk = make_int4((int)pt.off, pt.u0, pt.u1, 0);
+    }
+    tok_s[t] = tk;
+  }
+  if (warp == 8 + 4 * NH && lane < 2 && U > 0 && g.split >= 0) {      // the first unit's windows under the map
+    const int n = 2 * ubase + lane;
+    int4 wp = make_int4(0, 0, 0, 0);
+    if (n < g.n_windows) {
+      const DevMapPart pw = devmap_part_rolled(g.rowmap, 0, g.split, (uint32_t)n);
+      wp = make_int4((int)(uint32_t)(pw.off & 0xFFFFFFFFll), (int)(pw.off >> 32), pw.u0, pw.u1);
+    }
+    win_s[lane] = wp;
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+    if (tid + k * kThreads < NH * 256) raw_s[tid + k * kThreads] = tab[k];
+  if (tid < C) {
+    lng_s[tid] = par[0];
+    ln_s[tid] = __bfloat162float(par[1]);
+    bp_s[tid] = __bfloat162float(par[2]);
+  }
   __syncthreads();
-  if (tid < 32)                                       // identity: row n has a one in column n
-    *reinterpret_cast<uint16_t*>(sId + sw64_off(tid, tid >> 3) + (tid & 7) * 2) = 0x3F80u;
+  if (warp == 7 + 4 * NH)                             // identity: row n has a one in column n
+    *reinterpret_cast<uint16_t*>(sId + sw64_off(lane, lane >> 3) + (lane & 7) * 2) = 0x3F80u;
   // keys below / right of the wrap line of a seam window (bit c = key c)
-  if (warp == 2) {
+  if (warp == 8 + 4 * NH) {
     const int c0 = lane, c1 = lane + 32;
     const bool y0 = c0 < T && (tyx_s[c0] >> 8) >= ws - g.shift, y1 = c1 < T && (tyx_s[c1] >> 8) >= ws - g.shift;
     const bool x0 = c0 < T && (tyx_s[c0] & 255) >= ws - g.shift, x1 = c1 < T && (tyx_s[c1] & 255) >= ws - g.shift;
@@ -237,36 +269,24 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
     const uint32_t m2 = __ballot_sync(0xFFFFFFFFu, x0), m3 = __ballot_sync(0xFFFFFFFFu, x1);
     if (lane == 0) { kmask_s[0] = m0; kmask_s[1] = m1; kmask_s[2] = m2; kmask_s[3] = m3; }
   }
-  // fold gamma into the resident QKV weights; the column terms c_n and b'_n go into the extra k-step (thread = one weight row)
-  const bool w_ok = ptx::mbar_wait(w_full, 0, abort_flag, g.status);
-  if (w_ok && tid < 2 * NH * WROWS) {                  // (whole warps: 2 * NH * 96 is a multiple of 32)
-    const int row = tid >> 1, half = tid & 1;          // two threads per weight row: the first and second half of its chunks
-    const int h = row / WROWS, rr = row - h * WROWS;
-    const int which = rr >> 5, j = rr & 31;
-    float csum = 0.f, bsum = half ? 0.f : __bfloat162float(g.b_qkv[which * C + h * D + j]);
-    float bsum2 = 0.f;
-#pragma unroll 2
-    for (int ci = half * (NCH / 2); ci < (half + 1) * (NCH / 2); ++ci) {     // chunk ci of the row: k-block ci / 4, chunk ci % 4
-      uint4* p = reinterpret_cast<uint4*>(sWq + (h * NH + (ci >> 2)) * WQ_TILE + sw64_off(rr, ci & 3));
-      const uint4 wv = *p;
-      const uint32_t w4[4] = {wv.x, wv.y, wv.z, wv.w};
-      const float4 ga0 = *reinterpret_cast<const float4*>(ln_s + ci * 8), ga1 = *reinterpret_cast<const float4*>(ln_s + ci * 8 + 4);
-      const float4 be0 = *reinterpret_cast<const float4*>(ln_s + C + ci * 8), be1 = *reinterpret_cast<const float4*>(ln_s + C + ci * 8 + 4);
-      const float ga[8] = {ga0.x, ga0.y, ga0.z, ga0.w, ga1.x, ga1.y, ga1.z, ga1.w};
-      const float be[8] = {be0.x, be0.y, be0.z, be0.w, be1.x, be1.y, be1.z, be1.w};
-      uint32_t o4[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 f = bf16x2_to_float2(w4[e]);
-        bsum = fmaf(be[2 * e], f.x, bsum);
-        bsum2 = fmaf(be[2 * e + 1], f.y, bsum2);
-        o4[e] = float2_to_bf16x2(ga[2 * e] * f.x, ga[2 * e + 1] * f.y);
-        const float2 r2 = bf16x2_to_float2(o4[e]);
-        csum += r2.x + r2.y;
-      }
-      *p = make_uint4(o4[0], o4[1], o4[2], o4[3]);
-    }
-    bsum += bsum2;
+  // fold gamma into the resident QKV weights, a head's as soon as they are in; the column terms c_n and b'_n go into the extra k-step
+  const int frow = tid >> 1, fhead = frow / WROWS, half = tid & 1;       // two threads per weight row: the first and second half of its chunks
+  const bool folds = tid < 2 * NH * WROWS;             // (six whole warps per head)
+  float b0 = 0.f;
+  if (folds && half == 0) {
+    const int rr = frow - fhead * WROWS;
+    b0 = __bfloat162float(g.b_qkv[(rr >> 5) * C + fhead * D + (rr & 31)]);
+  }
+  bool w_ok = true;
+  if (folds) w_ok = ptx::mbar_wait(&w_full[fhead], 0, abort_flag, g.status);
+  if (warp == 8 + 4 * NH) w_ok = ptx::mbar_wait(&w_full[NH], 0, abort_flag, g.status);      // (the projection's weights are not folded)
+  if (w_ok && folds) {
+    const int h = fhead, rr = frow - h * WROWS;
+    FoldSums f;
+#pragma unroll 1
+    for (int ci = half * (NCH / 2); ci < (half + 1) * (NCH / 2); ++ci)      // chunk ci of the row: k-block ci / 4, chunk ci % 4
+      fold_chunk(sWq + (h * NH + (ci >> 2)) * WQ_TILE + sw64_off(rr, ci & 3), lng_s + ci * 8, ln_s + ci * 8, f);
+    float csum = f.c(), bsum = b0 + f.b();
     csum += __shfl_xor_sync(0xFFFFFFFFu, csum, 1);
     bsum += __shfl_xor_sync(0xFFFFFFFFu, bsum, 1);
     if (half == 0) {
@@ -275,15 +295,6 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
       *reinterpret_cast<uint4*>(sWx + h * WX_TILE + plain_off(rr, 0)) = k0;
       *reinterpret_cast<uint4*>(sWx + h * WX_TILE + plain_off(rr, 1)) = k1;
     }
-  }
-  if (tid < 2 && U > 0 && g.split >= 0) {              // the first unit's windows under the map (parameters only)
-    const int n = 2 * ubase + tid;
-    int4 wp = make_int4(0, 0, 0, 0);
-    if (n < g.n_windows) {
-      const DevMapPart pw = devmap_part_rolled(g.rowmap, 0, g.split, (uint32_t)n);
-      wp = make_int4((int)(uint32_t)(pw.off & 0xFFFFFFFFll), (int)(pw.off >> 32), pw.u0, pw.u1);
-    }
-    win_s[tid] = wp;
   }
   ptx::fence_proxy_async();                           // the rewritten weights -> visible to the MMAs
   ptx::tc_fence_before();
@@ -827,7 +838,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
   }
   ptx::tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
+  if (warp == 2) {
     ptx::tc_fence_after();
     ptx::tmem_dealloc(tmem_base, TMEM_COLS);
   }
@@ -860,10 +871,12 @@ int launch_swin_attn_fused(const smartmem_swin_params_t& p, const DevMap& rowmap
   if (!p.rel_bias_table) return SMARTMEM_ERR_INVALID_ARG;
   CUtensorMap twq, twp, tx;
   int rc;
-  const long long wq_dims[3] = {C, C, 3}, wq_strides[2] = {C, (long long)C * C};
-  const int wq_box[3] = {D, D, 3};
-  if ((rc = tc_encode_nd_sw64(p.w_qkv, 3, wq_dims, wq_strides, wq_box, &twq)) != SMARTMEM_OK) return rc;
-  if ((rc = tc_encode_2d_sw64(p.w_proj, C, C, C, D, C, &twp)) != SMARTMEM_OK) return rc;
+  const long long wq_dims[4] = {D, C, 3, NH}, wq_strides[3] = {C, (long long)C * C, D};      // (column, row, q / k / v, k-block)
+  const int wq_box[4] = {D, D, 3, NH};
+  if ((rc = tc_encode_nd_sw64(p.w_qkv, 4, wq_dims, wq_strides, wq_box, &twq)) != SMARTMEM_OK) return rc;
+  const long long wp_dims[3] = {D, C, NH}, wp_strides[2] = {C, D};                           // (column, row, k-block)
+  const int wp_box[3] = {D, C, NH};
+  if ((rc = tc_encode_nd_sw64(p.w_proj, 3, wp_dims, wp_strides, wp_box, &twp)) != SMARTMEM_OK) return rc;
   memset(&tx, 0, sizeof(tx));
   const long long dims[4] = {C, p.W, p.H, p.B}, strides[3] = {C, (long long)p.W * C, (long long)p.H * p.W * C};
   const int box[4] = {D, p.window, p.window, 1};

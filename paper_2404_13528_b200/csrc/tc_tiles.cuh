@@ -9,6 +9,7 @@
 // bf16 pieces (24 significant bits), so that the accumulator only needs one multiply by rstd.
 #pragma once
 #include "common.cuh"
+#include "ptx.cuh"
 
 namespace smartmem {
 
@@ -66,6 +67,35 @@ __device__ __forceinline__ void extra_col(float c, float b, uint4& k0, uint4& k1
   split3(b, bh, bm, bl);
   k0 = make_uint4(ch | (cm << 16), ch | (cl << 16), ch | (cm << 16), bh | (bm << 16));
   k1 = make_uint4(bh | (bl << 16), bh | (bm << 16), 0u, 0u);
+}
+
+// gamma folded into eight weights of a row in place, their part of c and b' added up (even and odd columns apart).  In packed pairs
+// (a product of two bf16 values is exact in fp32, so the packed bf16 product rounds as fp32 multiply and convert do): a CTA folds all
+// its weights before it can start, up to 37 thousand, and is bound by issue slots meanwhile.
+struct FoldSums {
+  ptx::f32x2 c2 = 0ull, b2 = 0ull;
+  __device__ static float sum(ptx::f32x2 v) {
+    float lo, hi;
+    ptx::unpack2(v, lo, hi);
+    return lo + hi;
+  }
+  __device__ float c() const { return sum(c2); }
+  __device__ float b() const { return sum(b2); }
+};
+__device__ __forceinline__ void fold_chunk(void* weights, const __nv_bfloat16* gamma, const float* beta, FoldSums& f) {
+  const uint4 wv = *reinterpret_cast<const uint4*>(weights), gv = *reinterpret_cast<const uint4*>(gamma);
+  const float4 be[2] = {*reinterpret_cast<const float4*>(beta), *reinterpret_cast<const float4*>(beta + 4)};
+  const uint32_t w4[4] = {wv.x, wv.y, wv.z, wv.w}, g4[4] = {gv.x, gv.y, gv.z, gv.w};
+  const ptx::f32x2 e4[4] = {ptx::pack2(be[0].x, be[0].y), ptx::pack2(be[0].z, be[0].w), ptx::pack2(be[1].x, be[1].y), ptx::pack2(be[1].z, be[1].w)};
+  uint32_t o4[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const uint32_t o = ptx::mul_bf16x2(g4[e], w4[e]);
+    f.b2 = ptx::fma2(e4[e], ptx::pack2(__uint_as_float(w4[e] << 16), __uint_as_float(w4[e] & 0xFFFF0000u)), f.b2);
+    f.c2 = ptx::add2(f.c2, ptx::pack2(__uint_as_float(o << 16), __uint_as_float(o & 0xFFFF0000u)));
+    o4[e] = o;
+  }
+  *reinterpret_cast<uint4*>(weights) = make_uint4(o4[0], o4[1], o4[2], o4[3]);
 }
 
 }  // namespace smartmem
