@@ -37,7 +37,7 @@
 // exact to 2^-24), so the epilogue of the QKV product is one multiply per element.  Every CTA folds gamma into its resident
 // copy of the weights once (prologue); the row statistics are two passes over the row, fp32.
 //
-// Warp roles (9 + 4 heads warps):
+// Warp roles (10 + 4 heads warps):
 //   0-3   bring in the rows of the units ahead -- a window that does not straddle the seam of the shifted image is an affine
 //         box [32 channels, ws, ws] of x per k-block, one TMA copy each; a seam window is gathered row by row with 16-byte
 //         asynchronous copies through the index map -- and take their statistics, a thread per row;
@@ -45,9 +45,8 @@
 //         group issues its own S and P V products from an elected thread right after the group's barrier: those hand-offs
 //         are on the item's critical path, and a barrier is cheaper than a trip through another warp;
 //   then  four warps for the Y epilogue (one row per thread);
-//   last  one thread that issues, in item order, the products that have slack: QKV of the items ahead (into the buffer the
-//         item four before has left), the residual product that opens a unit's Y, and the heads' projections.  Issue order is
-//         accumulation order, and orders a buffer's next accumulator behind the projection that reads the buffer last.
+//   last  one warp that issues the QKV products of the items ahead (into the buffer the item four before has left) and one
+//         that issues, in item order, the residual product that opens a unit's Y and the heads' projections.
 // What bounds it (clock stamps at every hand-off, and builds with the arithmetic of one role removed): not arithmetic -- with
 // the whole softmax compiled out the kernel is 5 % faster -- but the chain of hand-offs of an item (tensor-memory round trips,
 // three barriers, two waits for small products behind other groups' products in the tensor pipe), about 9000 cycles per item
@@ -81,7 +80,7 @@ constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t TM_Y = NBUF * BUF_COLS;          // the projection's accumulator (C columns) after the item buffers
 constexpr uint32_t ROW_INVALID = 0xFFFFFFFFu;       // no such row (a padding row of the tile, or a window past the end)
 constexpr int WIN_MISSING = 0, WIN_GATHER = 1, WIN_BOX = 2;
-constexpr int N_BARS = 29;
+constexpr int N_BARS = 33;
 
 struct FusedArgs {
   int n_windows, n_pairs, T, ws, shift, H, W;
@@ -105,11 +104,11 @@ __device__ __forceinline__ float ex2f(float x) {
 }
 
 template <int NH, int KC>
-__global__ void __launch_bounds__(32 * (9 + 4 * NH), 1)
+__global__ void __launch_bounds__(32 * (10 + 4 * NH), 1)
 swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_constant__ CUtensorMap tmWp,
                        const __grid_constant__ CUtensorMap tmX, const __grid_constant__ FusedArgs g) {
   constexpr int C = NH * D, NCH = C / 8;             // channels, 16-byte chunks per row
-  constexpr int kThreads = 32 * (9 + 4 * NH);
+  constexpr int kThreads = 32 * (10 + 4 * NH);
   constexpr int A_BYTES = NH * KBT;                  // a unit's raw rows: NH k-blocks of 32 columns
   constexpr int WP_TILE = C * 64;                    // Wp[:, 32 h : 32 h + 32]: C rows x 64 bytes
   constexpr int BR = KC == 56 ? 28 : 36;             // 32-bit words per bias row (16-byte reads of 8 consecutive rows hit distinct banks)
@@ -140,7 +139,8 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
   uint64_t *a_full = bars + 4, *a_free = a_full + 3, *landed = a_free + 3;     // [3] each: per slot of the row ring
   uint64_t *s_full = landed + 3, *o_full = s_full + 3;             // [3] each: per group (the group issues these products itself)
   uint64_t *acc_full = o_full + 3, *ob_full = acc_full + NBUF;     // [NBUF] each: per item buffer (items 4 apart share one)
-  uint64_t *y_full = ob_full + NBUF, *y_empty = y_full + 1;
+  uint64_t *buf_free = ob_full + NBUF;                             // [NBUF]: the item's projection has read the buffer
+  uint64_t *y_full = buf_free + NBUF, *y_empty = y_full + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(y_empty + 1);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
   uint16_t* raw_s = reinterpret_cast<uint16_t*>(sKV);              // prologue scratch: the raw table columns, [NH][256]
@@ -198,6 +198,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
       for (int i = 0; i < NBUF; ++i) {
         ptx::mbar_init(&acc_full[i], 1);
         ptx::mbar_init(&ob_full[i], 4);
+        ptx::mbar_init(&buf_free[i], 1);
       }
       ptx::mbar_init(y_full, 1);
       ptx::mbar_init(y_empty, 4);
@@ -691,97 +692,82 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
       if (lane == 0) ptx::mbar_arrive(&ob_full[it & (NBUF - 1)]);       // the projection of this item may be issued
     }
   } else if (warp == 8 + 4 * NH) {
-    // ---- the products that have slack -- QKV of the items ahead, the projections -- are issued by a thread of their own, in item
-    // order, so that no group thread ever waits on their inputs.  Issue order is accumulation order (the heads of a unit add
-    // up in Y) and also orders a buffer's next accumulator behind the projection that reads the buffer last. -----------------
-    if (__all_sync(0xFFFFFFFFu, w_ok ? 1 : 0)) {          // the whole warp walks the queues; an elected lane issues
-      const uint32_t idesc_qkv = ptx::make_idesc_bf16(BM, WROWS, false, false);
+    // ---- the residual product that opens a unit's Y and the heads' projections, in item order (issue order is accumulation order).
+    // They and the QKV products have a warp each: together in one polling loop (about a thousand cycles a turn, beside the warps it
+    // shares a scheduler with) they were what the items waited for.  Whole warps walk the queues; an elected lane issues. ---------
+    if (__all_sync(0xFFFFFFFFu, w_ok ? 1 : 0)) {
       const uint32_t idesc_pj = ptx::make_idesc_bf16(BM, C, false, false);
       const uint32_t idesc_id = ptx::make_idesc_bf16(BM, D, false, false);
-      const uint32_t a_base = ptx::smem_u32(sA), ax_base = ptx::smem_u32(sAx), wq_base = ptx::smem_u32(sWq);
-      const uint32_t wx_base = ptx::smem_u32(sWx), wp_base = ptx::smem_u32(sWp);
-      int qi = 0, qh = 0, qu = 0, qab = 0, qaph = 0;   // QKV queue: item, head, unit, row-ring slot and its phase
-      int ji = 0, jh = 0, ju = 0;                      // projection queue
-      int xu = 0, xab = 0, xaph = 0;                   // residual queue: unit, its row-ring slot and phase
-      const uint32_t id_base = ptx::smem_u32(sId);
-      uint32_t idle = 0;
-      unsigned long long t_idle = 0;
-      while (ji < total) {
-        bool progress = false;
-        if (xu < U && xu <= ju && __all_sync(0xFFFFFFFFu, ptx::mbar_test(y_empty, (xu & 1) ^ 1) && ptx::mbar_test(&a_full[xab], xaph))) {
-          // Y = X I: the unit's raw rows open the accumulation (the epilogue of the unit before has read Y); exact, since every
-          // product is a bf16 value times one.  The product is the last reader of the unit's rows: its completion frees the slot.
-          ptx::tc_fence_after();
-          const uint64_t bd = desc_sw64(id_base);
-          const uint64_t ad0 = desc_sw64(a_base + xab * A_BYTES);
-          if (ptx::elect_one()) {
+      const uint64_t id_d = desc_sw64(ptx::smem_u32(sId)), a_d = desc_sw64(ptx::smem_u32(sA)), wp_d = desc_sw64(ptx::smem_u32(sWp));
+      bool ok = true;
+      int ab = 0, aph = 0, it = 0;
+#pragma unroll 1
+      for (int ul = 0; ul < U && ok; ++ul) {
+        // Y = X I: the unit's raw rows open the accumulation (the epilogue of the unit before has read Y); exact, since every
+        // product is a bf16 value times one.  The product is the last reader of the unit's rows: its completion frees the slot.
+        ok = __all_sync(0xFFFFFFFFu, GWAIT(&a_full[ab], aph) && GWAIT(y_empty, (ul & 1) ^ 1) ? 1 : 0) != 0;
+        if (!ok) break;
+        ptx::tc_fence_after();
+        const uint64_t ad0 = a_d + ab * (A_BYTES >> 4);
+        if (ptx::elect_one()) {
 #pragma unroll
-            for (int kb = 0; kb < NH; ++kb) {          // 32 channels at a time: Y[:, 32 kb : 32 kb + 32] = X[:, 32 kb : 32 kb + 32] I_32
-              const uint64_t ad = ad0 + kb * (KBT >> 4);
-              ptx::tc_mma_bf16(tmem_base + TM_Y + kb * D, ad, bd, idesc_id, 0u);
-              ptx::tc_mma_bf16(tmem_base + TM_Y + kb * D, ad + 2, bd + 2, idesc_id, 1u);
-            }
-            ptx::tc_commit(&a_free[xab]);
+          for (int kb = 0; kb < NH; ++kb) {            // 32 channels at a time: Y[:, 32 kb : 32 kb + 32] = X[:, 32 kb : 32 kb + 32] I_32
+            ptx::tc_mma_bf16(tmem_base + TM_Y + kb * D, ad0 + kb * (KBT >> 4), id_d, idesc_id, 0u);
+            ptx::tc_mma_bf16(tmem_base + TM_Y + kb * D, ad0 + kb * (KBT >> 4) + 2, id_d + 2, idesc_id, 1u);
           }
-          __syncwarp();
-          ++xu;
-          if (++xab == na) { xab = 0; xaph ^= 1; }
-          progress = true;
+          ptx::tc_commit(&a_free[ab]);
         }
-        if (xu > ju && __all_sync(0xFFFFFFFFu, ptx::mbar_test(&ob_full[ji & (NBUF - 1)], (ji >> 2) & 1))) {
+        __syncwarp();
+        if (++ab == na) { ab = 0; aph ^= 1; }
+#pragma unroll 1
+        for (int h = 0; h < NH && ok; ++h, ++it) {
           // Y += Ob_h Wp[:, 32 h : 32 h + 32]^T; the last head hands Y to the epilogue
+          ok = __all_sync(0xFFFFFFFFu, GWAIT(&ob_full[it & (NBUF - 1)], (it >> 2) & 1) ? 1 : 0) != 0;
+          if (!ok) break;
           ptx::tc_fence_after();
-          const uint32_t a = tmem_base + (ji & (NBUF - 1)) * BUF_COLS + 64;
-          const uint64_t bd = desc_sw64(wp_base + jh * WP_TILE);
+          const uint32_t a = tmem_base + (it & (NBUF - 1)) * BUF_COLS + 64;
+          const uint64_t bd = wp_d + h * (WP_TILE >> 4);
           if (ptx::elect_one()) {
             ptx::tc_mma_bf16_ta(tmem_base + TM_Y, a, bd, idesc_pj, 1u);
             ptx::tc_mma_bf16_ta(tmem_base + TM_Y, a + 8, bd + 2, idesc_pj, 1u);
-            if (jh == NH - 1) ptx::tc_commit(y_full);
+            ptx::tc_commit(&buf_free[it & (NBUF - 1)]);
+            if (h == NH - 1) ptx::tc_commit(y_full);
           }
           __syncwarp();
-          ++ji;
-          if (++jh == NH) { jh = 0; ++ju; }
-          progress = true;
-        }
-        if (qi < total && qi < ji + NBUF && __all_sync(0xFFFFFFFFu, ptx::mbar_test(&a_full[qab], qaph))) {
-          // acc = [X | e] [Wq_h; Wk_h; Wv_h | f]^T into the buffer item qi - NBUF has left (its projection was issued above)
-          ptx::tc_fence_after();
-          const uint32_t d = tmem_base + (qi & (NBUF - 1)) * BUF_COLS;
-          const uint64_t ad0 = desc_sw64(a_base + qab * A_BYTES), bd0 = desc_sw64(wq_base + qh * NH * WQ_TILE);
-          const uint64_t axd = desc_plain(ax_base + qab * AX_BYTES), wxd = desc_plain(wx_base + qh * WX_TILE);
-          if (ptx::elect_one()) {
-#pragma unroll
-            for (int kb = 0; kb < NH; ++kb) {
-              const uint64_t ad = ad0 + kb * (KBT >> 4), bd = bd0 + kb * (WQ_TILE >> 4);
-              ptx::tc_mma_bf16(d, ad, bd, idesc_qkv, kb ? 1u : 0u);
-              ptx::tc_mma_bf16(d, ad + 2, bd + 2, idesc_qkv, 1u);    // next 16 channels: +32 bytes
-            }
-            ptx::tc_mma_bf16(d, axd, wxd, idesc_qkv, 1u);
-            ptx::tc_commit(&acc_full[qi & (NBUF - 1)]);
-          }
-          __syncwarp();
-          ++qi;
-          if (++qh == NH) {
-            qh = 0; ++qu;
-            if (++qab == na) { qab = 0; qaph ^= 1; }
-          }
-          progress = true;
-        }
-        if (progress) {
-          idle = 0;
-        } else if ((++idle & 255u) == 0) {
-          if (__any_sync(0xFFFFFFFFu, *(volatile int*)abort_flag)) break;
-          const unsigned long long now = __shfl_sync(0xFFFFFFFFu, ptx::globaltimer(), 0);
-          if (idle == 256u) t_idle = now;
-          else if (now - t_idle > ptx::wait_limit_ns(g.status)) {
-            if (lane == 0) {
-              *abort_flag = 1;
-              atomicExch(g.status, (int)SMARTMEM_ERR_TIMEOUT);
-            }
-            break;
-          }
         }
       }
+    }
+  } else if (warp == 9 + 4 * NH) {
+    // ---- QKV of the items ahead: acc = [X | e] [Wq_h; Wk_h; Wv_h | f]^T into the buffer item it - NBUF has left (its projection, the
+    // buffer's last reader, is done) -------------------------------------------------------------------------------------------
+    const uint32_t idesc_qkv = ptx::make_idesc_bf16(BM, WROWS, false, false);
+    const uint64_t a_d = desc_sw64(ptx::smem_u32(sA)), w_d = desc_sw64(ptx::smem_u32(sWq));
+    const uint64_t ax_d = desc_plain(ptx::smem_u32(sAx)), wx_d = desc_plain(ptx::smem_u32(sWx));
+    bool ok = true;
+    int ab = 0, aph = 0, it = 0;
+#pragma unroll 1
+    for (int ul = 0; ul < U && ok; ++ul) {
+      ok = __all_sync(0xFFFFFFFFu, GWAIT(&a_full[ab], aph) ? 1 : 0) != 0;
+      const uint64_t ad0 = a_d + ab * (A_BYTES >> 4), axd = ax_d + ab * (AX_BYTES >> 4);
+#pragma unroll 1
+      for (int h = 0; h < NH && ok; ++h, ++it) {
+        ok = __all_sync(0xFFFFFFFFu, GWAIT(&buf_free[it & (NBUF - 1)], ((it >> 2) & 1) ^ 1) ? 1 : 0) != 0;
+        if (!ok) break;
+        ptx::tc_fence_after();
+        const uint32_t d = tmem_base + (it & (NBUF - 1)) * BUF_COLS;
+        const uint64_t bd0 = w_d + h * (NH * WQ_TILE >> 4);
+        if (ptx::elect_one()) {
+#pragma unroll
+          for (int kb = 0; kb < NH; ++kb) {
+            ptx::tc_mma_bf16(d, ad0 + kb * (KBT >> 4), bd0 + kb * (WQ_TILE >> 4), idesc_qkv, kb ? 1u : 0u);
+            ptx::tc_mma_bf16(d, ad0 + kb * (KBT >> 4) + 2, bd0 + kb * (WQ_TILE >> 4) + 2, idesc_qkv, 1u);    // next 16 channels: +32 bytes
+          }
+          ptx::tc_mma_bf16(d, axd, wx_d + h * (WX_TILE >> 4), idesc_qkv, 1u);
+          ptx::tc_commit(&acc_full[it & (NBUF - 1)]);
+        }
+        __syncwarp();
+      }
+      if (++ab == na) { ab = 0; aph ^= 1; }
     }
   } else {
     // ---- Y epilogue: Y already holds x_row + sum_h Ob_h Wp_h^T (the residual rode on the tensor core as a product with the
@@ -911,7 +897,7 @@ int launch_swin_attn_fused(const smartmem_swin_params_t& p, const DevMap& rowmap
   if ((rc = ensure_max_dynamic_smem(fn, (int)kMaxSmem)) != SMARTMEM_OK) return rc;
   const int sms = tc_sm_count();
   const unsigned grid = (unsigned)(g.n_pairs < sms ? g.n_pairs : sms);
-  const unsigned threads = 32u * (9 + 4 * NH);
+  const unsigned threads = 32u * (10 + 4 * NH);
   profile_tick("attn_half_fused", st);
   cudaError_t e;
   if (NH == 3) e = kc56 ? launch_pdl(swin_attn_fused_kernel<3, 56>, dim3(grid), dim3(threads), smem, st, twq, twp, tx, g)
