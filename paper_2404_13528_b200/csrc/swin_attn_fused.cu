@@ -25,9 +25,9 @@
 //   Ob   = bf16(O / rowsum)                    back into tensor memory as packed pairs
 //   Y   += Ob Wp[:, 32 h : 32 h + 32]^T        128 x C x 32: the head merge is the accumulation over heads
 //
-// and per unit  Y starts as X I (the unit's raw rows times the identity: the residual rides on the tensor core, exactly, since
-// every product is a bf16 value times one), the heads' projections accumulate on top, and the epilogue stores
-// y_row = Y + b_proj with 16-byte vectors at the row's offset under the map.
+// and per unit  the heads' projections accumulate in Y, and the epilogue stores  y_row = x_row + Y + b_proj  with 32-byte vectors at
+// the row's offset under the map.  x_row is read again (from L2) while the unit is under way: as a product of the raw rows with the
+// identity, which opened Y, the residual kept the unit's slot of the row ring until the epilogue of the unit before had left Y.
 //
 // LayerNorm without a normalised tile:  LN(x) W^T + b = rstd (x W'^T - mean c + sigma b'),  W' = bf16(gamma . W) (column
 // scaling), c_n = sum_k W'_nk, b'_n = b_n + sum_k beta_k W_nk, sigma = 1 / rstd.  c is summed from the ROUNDED W', so the
@@ -40,18 +40,21 @@
 // Warp roles (10 + 4 heads warps):
 //   0-3   bring in the rows of the units ahead -- a window that does not straddle the seam of the shifted image is an affine
 //         box [32 channels, ws, ws] of x per k-block, one TMA copy each; a seam window is gathered row by row with 16-byte
-//         asynchronous copies through the index map -- and take their statistics, a thread per row;
+//         asynchronous copies through the index map;
 //   then  one group of four warps per head (q/k/v epilogue, softmax, O epilogue: one row of the pair tile per thread).  A
 //         group issues its own S and P V products from an elected thread right after the group's barrier: those hand-offs
 //         are on the item's critical path, and a barrier is cheaper than a trip through another warp;
-//   then  four warps for the Y epilogue (one row per thread);
+//   then  four warps for the row statistics and the Y epilogue (one row per thread);
 //   last  one warp that issues the QKV products of the items ahead (into the buffer the item four before has left) and one
-//         that issues, in item order, the residual product that opens a unit's Y and the heads' projections.
-// What bounds it (clock stamps at every hand-off, and builds with the arithmetic of one role removed): not arithmetic -- with
-// the whole softmax compiled out the kernel is 5 % faster -- but the chain of hand-offs of an item (tensor-memory round trips,
-// three barriers, two waits for small products behind other groups' products in the tensor pipe), about 9000 cycles per item
-// with three items in flight; and instruction fetch: code that runs once per unit (statistics, epilogue, the prologue) is
-// kept in rolled loops because its straight-line form ran at the speed of the instruction cache misses.  Every wait is bounded.
+//         that issues, in item order, the heads' projections.
+// What bounds it (clock stamps at every hand-off): not arithmetic -- with the whole softmax compiled out the kernel is 5 % faster --
+// but the chain of hand-offs of an item (tensor-memory round trips, three barriers, two waits for small products behind other
+// groups' products in the tensor pipe; 4500 cycles) and the wait for its QKV product.  That wait was the loading warps' chain,
+// 6500 cycles a unit (copies issued, rows awaited, statistics taken, then the next unit's copies): with the statistics in the
+// epilogue warps, which take them whenever rows are in, and slots freed by the QKV products, the next rows are on their way
+// meanwhile (32 x 56 x 56 x 64, three slots: 27.3 -> 23.9 us; 96 channels have room for two slots: 32.9 -> 32.7).  A single warp
+// for the copies is too slow for the gathered windows (59.7).  Code that runs once per unit (statistics, the prologue) is kept in
+// rolled loops because its straight-line form ran at the speed of the instruction cache misses.  Every wait is bounded.
 #include "attn.cuh"
 #include "gemm_tc.cuh"
 #include "ptx.cuh"
@@ -73,8 +76,10 @@ constexpr int WQ_TILE = WROWS * 64;
 constexpr int WX_TILE = WROWS * 32;                 // the extra k-step of a head's weights
 constexpr int KV_SLOT = 2 * KBT;                    // k, v tiles of one item
 constexpr int NBUF = 4, BUF_COLS = 96;              // item buffers of tensor memory
-constexpr int ID_BYTES = 32 * 64;                   // the identity tile
-constexpr int NRING = 4;                            // units whose row offsets are kept (a unit's epilogue runs long after its gather)
+// Units whose row offsets are kept.  The rows of unit u come in once the QKV products of unit u - 3 are done at the latest, which waited
+// for a projection of unit u - 5 (two heads; three: u - 4), which waited until the epilogue of unit u - 6 had read Y and, before
+// that, its offsets: six would do.
+constexpr int NRING = 8;
 constexpr int kLoaderThreads = 128;
 constexpr uint32_t TMEM_COLS = 512;
 constexpr uint32_t TM_Y = NBUF * BUF_COLS;          // the projection's accumulator (C columns) after the item buffers
@@ -122,8 +127,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
   uint8_t* sWp = sWq + NH * NH * WQ_TILE;                          // [NH heads][C rows x 64 B]
   uint8_t* sAx = sWp + NH * WP_TILE;                               // [na][128 rows x 32 B]
   uint8_t* sWx = sAx + na * AX_BYTES;                              // [NH heads][96 rows x 32 B]
-  uint8_t* sId = sWx + NH * WX_TILE;                               // [32 rows x 64 B]: the 32 x 32 identity (the residual rides on the tensor core)
-  uint32_t* bias_s = reinterpret_cast<uint32_t*>(sId + ID_BYTES);  // [NH][T][BR]: bf16 pairs
+  uint32_t* bias_s = reinterpret_cast<uint32_t*>(sWx + NH * WX_TILE);   // [NH][T][BR]: bf16 pairs
   float* bp_s = reinterpret_cast<float*>(bias_s + NH * T * BR);    // [C]
   float* rstd_s = bp_s + C;                                        // [na][128]
   uint32_t* rowoff_s = reinterpret_cast<uint32_t*>(rstd_s + na * BM);   // [NRING][128]: row offset in 16-byte units
@@ -189,8 +193,8 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
 #pragma unroll 1
       for (int i = 0; i < 3; ++i) {
         ptx::mbar_init(&a_full[i], 4);
-        ptx::mbar_init(&a_free[i], NH + 1);
-        ptx::mbar_init(&landed[i], 4);
+        ptx::mbar_init(&a_free[i], 4 * NH);
+        ptx::mbar_init(&landed[i], 128 + 4);
         ptx::mbar_init(&s_full[i], 1);
         ptx::mbar_init(&o_full[i], 1);
       }
@@ -228,7 +232,6 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
   }
   for (int i = tid; i < na * A_BYTES / 16; i += kThreads) reinterpret_cast<uint4*>(sA)[i] = make_uint4(0, 0, 0, 0);
   for (int i = tid; i < na * AX_BYTES / 16; i += kThreads) reinterpret_cast<uint4*>(sAx)[i] = make_uint4(0, 0, 0, 0);
-  for (int i = tid; i < ID_BYTES / 16; i += kThreads) reinterpret_cast<uint4*>(sId)[i] = make_uint4(0, 0, 0, 0);
   for (int i = tid; i < na * BM; i += kThreads) rstd_s[i] = 0.f;
   for (int i = tid; i < NRING * BM; i += kThreads) rowoff_s[i] = ROW_INVALID;
   if (tid >= 128 && tid < 128 + TP) {
@@ -259,8 +262,6 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
     bp_s[tid] = __bfloat162float(par[2]);
   }
   __syncthreads();
-  if (warp == 7 + 4 * NH)                             // identity: row n has a one in column n
-    *reinterpret_cast<uint16_t*>(sId + sw64_off(lane, lane >> 3) + (lane & 7) * 2) = 0x3F80u;
   // keys below / right of the wrap line of a seam window (bit c = key c)
   if (warp == 8 + 4 * NH) {
     const int c0 = lane, c1 = lane + 32;
@@ -311,14 +312,10 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
     constexpr int RPI = kLoaderThreads / NCH;          // rows per round of the gather loop: a row by NCH consecutive threads
     const int my_ch = lt % NCH, my_slot = lt / NCH;
     bool ok = true;
-    auto vote = [&](bool pred, bool all) {             // OR (all = false) or AND (all = true) over the loader threads; also a barrier
+    auto vote = [&](bool pred) {                       // OR over the loader threads; also a barrier
       uint32_t res;
-      if (all)
-        asm volatile("{\n\t.reg .pred pin, pout;\n\tsetp.ne.u32 pin, %1, 0;\n\tbar.red.and.pred pout, 1, 128, pin;\n\tselp.u32 %0, 1, 0, pout;\n\t}"
-                     : "=r"(res) : "r"(pred ? 1u : 0u) : "memory");
-      else
-        asm volatile("{\n\t.reg .pred pin, pout;\n\tsetp.ne.u32 pin, %1, 0;\n\tbar.red.or.pred pout, 1, 128, pin;\n\tselp.u32 %0, 1, 0, pout;\n\t}"
-                     : "=r"(res) : "r"(pred ? 1u : 0u) : "memory");
+      asm volatile("{\n\t.reg .pred pin, pout;\n\tsetp.ne.u32 pin, %1, 0;\n\tbar.red.or.pred pout, 1, 128, pin;\n\tselp.u32 %0, 1, 0, pout;\n\t}"
+                   : "=r"(res) : "r"(pred ? 1u : 0u) : "memory");
       return res != 0;
     };
     auto window_part = [&](int ul) {                   // threads 0, 1: the leading atoms' contribution of the unit's two windows
@@ -335,8 +332,9 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
     auto issue_loads = [&](int ul) {
       const int ab = ul % na;
       const int p = ubase + ul;
-      {                                                 // a thread per row of the pair tile: the window's kind, the row's offset
-        const int w = lt >> 6, i = lt & 63, n = 2 * p + w;
+      {
+        // two warps per window; the copies first (their latency is what a unit waits for), issued by an elected lane
+        const int w = warp >> 1, i = lt & 63, n = 2 * p + w;
         int kind = WIN_MISSING, wy = 0, wx = 0, b = 0;
         if (n < g.n_windows) {
           b = (int)fd_div((uint32_t)n, g.fd_wpi);
@@ -346,8 +344,22 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
           const bool seam = g.shift > 0 && (wy == g.nWh - 1 || wx == g.nWw - 1);
           kind = (seam || !g.use_box) ? WIN_GATHER : WIN_BOX;
         }
+        if ((warp & 1) == 0) {
+          if (kind == WIN_BOX) {                        // (no arrival: the loader warps arrive below)
+            if (ptx::elect_one()) ptx::mbar_add_tx(&landed[ab], (uint32_t)(T * C * 2));
+            __syncwarp();
+#pragma unroll
+            for (int kb = 0; kb < NH; ++kb) {
+              if (ptx::elect_one())
+                ptx::tma_load_4d(sA + ab * A_BYTES + kb * KBT + w * (64 * 64), &tmX, &landed[ab], kb * D, wx * ws + g.shift, wy * ws + g.shift, b);
+              __syncwarp();
+            }
+          }
+          if (lane == 0) wkind_s[ab * 2 + w] = kind;
+        }
+        // a thread per row of the pair tile: its offset under the map (the gather of a seam window and the scatter use it)
         uint32_t off16 = ROW_INVALID;
-        if (i < T && kind != WIN_MISSING) {            // the offset under the map: the gather of a seam window, the residual and the scatter use it
+        if (i < T && kind != WIN_MISSING) {
           long long off;
           if (g.split >= 0) {
             const int4 wp = win_s[(ul & 1) * 2 + w], tk = tok_s[i];
@@ -359,16 +371,6 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
           off16 = (uint32_t)(off >> 3);
         }
         rowoff_s[(ul % NRING) * BM + lt] = off16;
-        if (i == 0) {
-          wkind_s[ab * 2 + w] = kind;
-          if (kind == WIN_BOX) {                        // this thread moves the window (no arrival: the loader warps arrive below)
-            ptx::mbar_add_tx(&landed[ab], (uint32_t)(T * C * 2));
-#pragma unroll
-            for (int kb = 0; kb < NH; ++kb)
-              ptx::tma_load_4d(sA + ab * A_BYTES + kb * KBT + w * (64 * 64), &tmX, &landed[ab], kb * D, wx * ws + g.shift,
-                               wy * ws + g.shift, b);
-          }
-        }
       }
       asm volatile("bar.sync 2, 128;" ::: "memory");
       const int kind0 = wkind_s[ab * 2], kind1 = wkind_s[ab * 2 + 1];
@@ -383,90 +385,16 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
             ptx::cp_async16(dst, g.x + ((size_t)rowoff_s[(ul % NRING) * BM + row] << 3) + my_ch * 8);
         }
       }
-      ptx::cp_async_commit();
+      ptx::cp_async_arrive(&landed[ab]);               // every thread, once its copies are in
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&landed[ab]);
       window_part(ul + 1);                             // read after the next barrier of the loader threads
     };
-    auto statistics = [&](int ul) {
-      const int ab = ul % na;
-      const int r = lt, i = lt & 63;
-      if (i < T) {
-        float rstd = 0.f;
-        uint4 k0 = make_uint4(0, 0, 0, 0), k1 = k0;
-        if (rowoff_s[(ul % NRING) * BM + r] != ROW_INVALID) {
-          // two passes over the row in shared memory (mean, then squared deviations); the loops are only partly unrolled: this code
-          // runs once per unit, and fetching its instructions costs as much as executing them
-          f32x2 s2[2] = {0ull, 0ull};
-#pragma unroll 4
-          for (int ch = 0; ch < NCH; ++ch) {
-            const uint4 xv = *reinterpret_cast<const uint4*>(sA + ab * A_BYTES + (ch >> 2) * KBT + sw64_off(r, ch & 3));
-            const uint32_t x4[4] = {xv.x, xv.y, xv.z, xv.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-              s2[e & 1] = ptx::add2(s2[e & 1], ptx::pack2(__uint_as_float(x4[e] << 16), __uint_as_float(x4[e] & 0xFFFF0000u)));
-          }
-          float a0, a1, a2, a3;
-          ptx::unpack2(s2[0], a0, a1);
-          ptx::unpack2(s2[1], a2, a3);
-          const float mean = ((a0 + a1) + (a2 + a3)) * (1.0f / (float)C);
-          const f32x2 nm2 = ptx::pack2(-mean, -mean);
-          f32x2 q2[2] = {0ull, 0ull};
-#pragma unroll 4
-          for (int ch = 0; ch < NCH; ++ch) {
-            const uint4 xv = *reinterpret_cast<const uint4*>(sA + ab * A_BYTES + (ch >> 2) * KBT + sw64_off(r, ch & 3));
-            const uint32_t x4[4] = {xv.x, xv.y, xv.z, xv.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const f32x2 d2 = ptx::add2(ptx::pack2(__uint_as_float(x4[e] << 16), __uint_as_float(x4[e] & 0xFFFF0000u)), nm2);
-              q2[e & 1] = ptx::fma2(d2, d2, q2[e & 1]);
-            }
-          }
-          ptx::unpack2(q2[0], a0, a1);
-          ptx::unpack2(q2[1], a2, a3);
-          const float var = ((a0 + a1) + (a2 + a3)) * (1.0f / (float)C) + g.eps;
-          rstd = rsqrtf(var);
-          extra_row(-mean, var * rstd, k0, k1);          // sigma = var / sqrt(var)
-        }
-        rstd_s[ab * BM + r] = rstd;
-        *reinterpret_cast<uint4*>(sAx + ab * AX_BYTES + plain_off(r, 0)) = k0;
-        *reinterpret_cast<uint4*>(sAx + ab * AX_BYTES + plain_off(r, 1)) = k1;
-      }
-      ptx::fence_proxy_async();                        // the extra k-step -> visible to the MMAs
-      __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(&a_full[ab]);
-    };
-    // A unit's rows are requested as soon as its ring slot is free (the QKV products of the unit that held it are done); when
-    // no slot is free the oldest request in flight is waited for and handed to the statistics warps.
-    int issued = 0, done = 0;
-    while (done < U) {
-      if (issued < U && issued - done < na) {
-        uint64_t* bar = &a_free[issued % na];
-        const uint32_t par = (uint32_t)(((issued / na) & 1) ^ 1);
-        bool ready;
-        if (issued == done) {
-          ok = ptx::mbar_wait_relaxed(bar, par, abort_flag, g.status, 64);
-          if (vote(!ok, false)) break;
-          ready = true;
-        } else {
-          ready = vote(ptx::mbar_test(bar, par), true);
-        }
-        if (ready) {
-          issue_loads(issued);
-          ++issued;
-          continue;
-        }
-      }
-      const int pending = issued - done;               // cp.async groups in flight; the oldest belongs to unit `done`
-      if (pending >= 3) ptx::cp_async_wait<2>();
-      else if (pending == 2) ptx::cp_async_wait<1>();
-      else ptx::cp_async_wait<0>();
-      ptx::fence_proxy_async();                        // the gathered rows -> visible to the MMAs
-      __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(&landed[done % na]);
-      // every row of the unit is in (the loader warps' copies and the TMA boxes): its statistics, a thread per row
-      ok = ptx::mbar_wait_relaxed(&landed[done % na], (done / na) & 1, abort_flag, g.status, 32);
-      if (vote(!ok, false)) break;
-      statistics(done);
-      ++done;
+#pragma unroll 1
+    for (int ul = 0; ul < U; ++ul) {
+      ok = ptx::mbar_wait_relaxed(&a_free[ul % na], ((ul / na) & 1) ^ 1, abort_flag, g.status, 64);
+      if (vote(!ok)) break;                     // (also the barrier between window_part and its readers)
+      issue_loads(ul);
     }
   } else if (warp < 4 + 4 * NH) {
     // ---- row groups: group h takes head h of every unit; one row of the pair tile per thread.  The group's elected thread issues
@@ -476,7 +404,6 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
     const int q = warp & 3;                            // TMEM lane quadrant
     const int r = q * 32 + lane;
     const int w = r >> 6, i = r & 63;                  // window of the pair, token
-    const bool elected = q == 0 && lane == 0;          // (arrivals on behalf of the group)
     const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
     const int my_ty = tyx_s[i] >> 8, my_tx = tyx_s[i] & 255;
     const uint32_t ky_lo = kmask_s[0], ky_hi = kmask_s[1], kx_lo = kmask_s[2], kx_hi = kmask_s[3];
@@ -526,11 +453,13 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
       // -- q, k, v of this row: rstd times the accumulator (the mean and bias terms rode on the extra k-step) --
       ok = ok && GWAIT(&a_full[ab], (ul / na) & 1) &&     // (long complete: orders the read of rstd)
            GWAIT(&acc_full[it & (NBUF - 1)], (it >> 2) & 1);
+      ok = __all_sync(0xFFFFFFFFu, ok ? 1 : 0) != 0;
       if (ok) {
-        if (elected) ptx::mbar_arrive(&a_free[ab]);      // this head's product has read the unit's rows
         ptx::tc_fence_after();
         const float rstd = rstd_s[ab * BM + r];
         const f32x2 r2 = ptx::pack2(rstd, rstd);
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&a_free[ab]);    // this head's product has read the unit's rows, this warp their statistics
         uint32_t rv[32], q16[16];
         auto scaled_pairs = [&](uint32_t* out) {         // 32 accumulator columns in rv -> 16 bf16 pairs of rstd * acc
 #pragma unroll
@@ -692,33 +621,17 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
       if (lane == 0) ptx::mbar_arrive(&ob_full[it & (NBUF - 1)]);       // the projection of this item may be issued
     }
   } else if (warp == 8 + 4 * NH) {
-    // ---- the residual product that opens a unit's Y and the heads' projections, in item order (issue order is accumulation order).
-    // They and the QKV products have a warp each: together in one polling loop (about a thousand cycles a turn, beside the warps it
-    // shares a scheduler with) they were what the items waited for.  Whole warps walk the queues; an elected lane issues. ---------
+    // ---- the heads' projections, in item order (issue order is accumulation order).  They and the QKV products have a warp each:
+    // together in one polling loop (about a thousand cycles a turn, beside the warps it shares a scheduler with) they were what the
+    // items waited for.  Whole warps walk the queues; an elected lane issues. --------------------------------------------------
     if (__all_sync(0xFFFFFFFFu, w_ok ? 1 : 0)) {
       const uint32_t idesc_pj = ptx::make_idesc_bf16(BM, C, false, false);
-      const uint32_t idesc_id = ptx::make_idesc_bf16(BM, D, false, false);
-      const uint64_t id_d = desc_sw64(ptx::smem_u32(sId)), a_d = desc_sw64(ptx::smem_u32(sA)), wp_d = desc_sw64(ptx::smem_u32(sWp));
+      const uint64_t wp_d = desc_sw64(ptx::smem_u32(sWp));
       bool ok = true;
-      int ab = 0, aph = 0, it = 0;
+      int it = 0;
 #pragma unroll 1
       for (int ul = 0; ul < U && ok; ++ul) {
-        // Y = X I: the unit's raw rows open the accumulation (the epilogue of the unit before has read Y); exact, since every
-        // product is a bf16 value times one.  The product is the last reader of the unit's rows: its completion frees the slot.
-        ok = __all_sync(0xFFFFFFFFu, GWAIT(&a_full[ab], aph) && GWAIT(y_empty, (ul & 1) ^ 1) ? 1 : 0) != 0;
-        if (!ok) break;
-        ptx::tc_fence_after();
-        const uint64_t ad0 = a_d + ab * (A_BYTES >> 4);
-        if (ptx::elect_one()) {
-#pragma unroll
-          for (int kb = 0; kb < NH; ++kb) {            // 32 channels at a time: Y[:, 32 kb : 32 kb + 32] = X[:, 32 kb : 32 kb + 32] I_32
-            ptx::tc_mma_bf16(tmem_base + TM_Y + kb * D, ad0 + kb * (KBT >> 4), id_d, idesc_id, 0u);
-            ptx::tc_mma_bf16(tmem_base + TM_Y + kb * D, ad0 + kb * (KBT >> 4) + 2, id_d + 2, idesc_id, 1u);
-          }
-          ptx::tc_commit(&a_free[ab]);
-        }
-        __syncwarp();
-        if (++ab == na) { ab = 0; aph ^= 1; }
+        ok = __all_sync(0xFFFFFFFFu, GWAIT(y_empty, (ul & 1) ^ 1) ? 1 : 0) != 0;      // the epilogue of the unit before has read Y
 #pragma unroll 1
         for (int h = 0; h < NH && ok; ++h, ++it) {
           // Y += Ob_h Wp[:, 32 h : 32 h + 32]^T; the last head hands Y to the epilogue
@@ -728,7 +641,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
           const uint32_t a = tmem_base + (it & (NBUF - 1)) * BUF_COLS + 64;
           const uint64_t bd = wp_d + h * (WP_TILE >> 4);
           if (ptx::elect_one()) {
-            ptx::tc_mma_bf16_ta(tmem_base + TM_Y, a, bd, idesc_pj, 1u);
+            ptx::tc_mma_bf16_ta(tmem_base + TM_Y, a, bd, idesc_pj, h ? 1u : 0u);
             ptx::tc_mma_bf16_ta(tmem_base + TM_Y, a + 8, bd + 2, idesc_pj, 1u);
             ptx::tc_commit(&buf_free[it & (NBUF - 1)]);
             if (h == NH - 1) ptx::tc_commit(y_full);
@@ -770,53 +683,133 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
       if (++ab == na) { ab = 0; aph ^= 1; }
     }
   } else {
-    // ---- Y epilogue: Y already holds x_row + sum_h Ob_h Wp_h^T (the residual rode on the tensor core as a product with the
-    // identity); add the bias, round once, store the row at its offset under the map.  One row per thread. ------------------
+    // ---- statistics of the units ahead as their rows come in, and the Y epilogue: the residual and the bias, rounded once, stored at
+    // the row's offset under the map.  One row per thread; each warp on its own. ---------------------------------------------
     const int q = warp & 3;
     const int r = q * 32 + lane;
     const int i = r & 63;
     const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
     const bool wide_store = (reinterpret_cast<uintptr_t>(g.y) & 31) == 0;
+    auto statistics = [&](int ul) {
+      const int ab = ul % na;
+      if (i < T) {
+        float rstd = 0.f;
+        uint4 k0 = make_uint4(0, 0, 0, 0), k1 = k0;
+        if (rowoff_s[(ul % NRING) * BM + r] != ROW_INVALID) {
+          // two passes over the row in shared memory (mean, then squared deviations); the loops are only partly unrolled: this code
+          // runs once per unit, and fetching its instructions costs as much as executing them
+          f32x2 s2[2] = {0ull, 0ull};
+#pragma unroll 4
+          for (int ch = 0; ch < NCH; ++ch) {
+            const uint4 xv = *reinterpret_cast<const uint4*>(sA + ab * A_BYTES + (ch >> 2) * KBT + sw64_off(r, ch & 3));
+            const uint32_t x4[4] = {xv.x, xv.y, xv.z, xv.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              s2[e & 1] = ptx::add2(s2[e & 1], ptx::pack2(__uint_as_float(x4[e] << 16), __uint_as_float(x4[e] & 0xFFFF0000u)));
+          }
+          float a0, a1, a2, a3;
+          ptx::unpack2(s2[0], a0, a1);
+          ptx::unpack2(s2[1], a2, a3);
+          const float mean = ((a0 + a1) + (a2 + a3)) * (1.0f / (float)C);
+          const f32x2 nm2 = ptx::pack2(-mean, -mean);
+          f32x2 q2[2] = {0ull, 0ull};
+#pragma unroll 4
+          for (int ch = 0; ch < NCH; ++ch) {
+            const uint4 xv = *reinterpret_cast<const uint4*>(sA + ab * A_BYTES + (ch >> 2) * KBT + sw64_off(r, ch & 3));
+            const uint32_t x4[4] = {xv.x, xv.y, xv.z, xv.w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const f32x2 d2 = ptx::add2(ptx::pack2(__uint_as_float(x4[e] << 16), __uint_as_float(x4[e] & 0xFFFF0000u)), nm2);
+              q2[e & 1] = ptx::fma2(d2, d2, q2[e & 1]);
+            }
+          }
+          ptx::unpack2(q2[0], a0, a1);
+          ptx::unpack2(q2[1], a2, a3);
+          const float var = ((a0 + a1) + (a2 + a3)) * (1.0f / (float)C) + g.eps;
+          rstd = rsqrtf(var);
+          extra_row(-mean, var * rstd, k0, k1);          // sigma = var / sqrt(var)
+        }
+        rstd_s[ab * BM + r] = rstd;
+        *reinterpret_cast<uint4*>(sAx + ab * AX_BYTES + plain_off(r, 0)) = k0;
+        *reinterpret_cast<uint4*>(sAx + ab * AX_BYTES + plain_off(r, 1)) = k1;
+      }
+      ptx::fence_proxy_async();                        // the gathered rows and the extra k-step -> visible to the MMAs
+      __syncwarp();
+      if (lane == 0) ptx::mbar_arrive(&a_full[ab]);
+    };
     bool ok = true;
-    for (int ul = 0; ul < U && ok; ++ul) {
-      ok = ptx::mbar_wait_relaxed(y_full, ul & 1, abort_flag, g.status, 32);
-      if (!ok) break;
-      ptx::tc_fence_after();
+    int su = 0;                                        // statistics taken of the units below it
+    // Waits for `bar`, taking the statistics of units whose rows come in meanwhile: they are what the next products wait for.
+    auto wait_working = [&](uint64_t* bar, uint32_t par, bool until_statistics, int ul) {
+      uint32_t idle = 0;
+      unsigned long long t_idle = 0;
+      while (true) {
+        if (su < U && __all_sync(0xFFFFFFFFu, ptx::mbar_test(&landed[su % na], (su / na) & 1) ? 1 : 0)) {
+          statistics(su);
+          ++su;
+          idle = 0;
+        } else if (until_statistics ? su > ul : __all_sync(0xFFFFFFFFu, ptx::mbar_test(bar, par) ? 1 : 0) != 0) {
+          return true;
+        } else if ((++idle & 63u) == 0) {
+          if (__any_sync(0xFFFFFFFFu, *(volatile int*)abort_flag)) return false;
+          const unsigned long long now = __shfl_sync(0xFFFFFFFFu, ptx::globaltimer(), 0);
+          if (idle == 64u) t_idle = now;
+          else if (now - t_idle > ptx::wait_limit_ns(g.status)) {
+            if (lane == 0) {
+              *abort_flag = 1;
+              atomicExch(g.status, (int)SMARTMEM_ERR_TIMEOUT);
+            }
+            return false;
+          }
+        }
+      }
+    };
+#pragma unroll 1
+    for (int ul = 0; ul < U; ++ul) {
+      // (the row's offset is written before the rows come in)
+      if (!wait_working(nullptr, 0, true, ul)) break;
       const uint32_t my_off = rowoff_s[(ul % NRING) * BM + r];
       const bool valid = i < T && my_off != ROW_INVALID;
       uint4* yg = reinterpret_cast<uint4*>(g.y + ((size_t)(valid ? my_off : 0u) << 3));
-#pragma unroll 1
-      for (int k = 0; k < NH; ++k) {                   // 32 columns = 4 chunks of the row at a time
-        uint32_t rv[32];
-        ptx::tmem_ld32(tmem_base + TM_Y + lane_addr + k * 32, rv);
+      const uint4* xg = reinterpret_cast<const uint4*>(g.x + ((size_t)(valid ? my_off : 0u) << 3));
+      uint4 xr[NCH];
+#pragma unroll
+      for (int c = 0; c < NCH; ++c) xr[c] = valid ? xg[c] : make_uint4(0, 0, 0, 0);
+      ok = wait_working(y_full, ul & 1, false, ul);
+      if (!ok) break;
+      ptx::tc_fence_after();
+#pragma unroll
+      for (int k = 0; k < NCH / 2; ++k) {              // 16 columns at a time (two chunks: a sector)
+        uint32_t rv[16], o[8];
+        ptx::tmem_ld16(tmem_base + TM_Y + lane_addr + k * 16, rv);
         ptx::tmem_ld_wait();
-        if (k == NH - 1) {                             // Y is in registers: the next unit's products may overwrite it
+        if (k == NCH / 2 - 1) {                        // Y is in registers: the next unit's products may overwrite it
           ptx::tc_fence_before();
           __syncwarp();
           if (lane == 0) ptx::mbar_arrive(y_empty);
         }
+        const uint32_t xw[8] = {xr[2 * k].x, xr[2 * k].y, xr[2 * k].z, xr[2 * k].w, xr[2 * k + 1].x, xr[2 * k + 1].y, xr[2 * k + 1].z, xr[2 * k + 1].w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float4 b4 = *reinterpret_cast<const float4*>(bp_s + k * 16 + 4 * e);
+          const f32x2 bb[2] = {ptx::pack2(b4.x, b4.y), ptx::pack2(b4.z, b4.w)};
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const uint32_t xp = xw[2 * e + j];
+            const f32x2 acc = ptx::pack2(__uint_as_float(rv[4 * e + 2 * j]), __uint_as_float(rv[4 * e + 2 * j + 1]));
+            const f32x2 res = ptx::pack2(__uint_as_float(xp << 16), __uint_as_float(xp & 0xFFFF0000u));
+            float v0, v1;
+            ptx::unpack2(ptx::add2(ptx::add2(acc, res), bb[j]), v0, v1);
+            o[2 * e + j] = float2_to_bf16x2(v0, v1);
+          }
+        }
         if (valid) {
-          uint4 o_prev = make_uint4(0, 0, 0, 0);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const float4 b0 = *reinterpret_cast<const float4*>(bp_s + k * 32 + c * 8);
-            const float4 b1 = *reinterpret_cast<const float4*>(bp_s + k * 32 + c * 8 + 4);
-            const f32x2 bb[4] = {ptx::pack2(b0.x, b0.y), ptx::pack2(b0.z, b0.w), ptx::pack2(b1.x, b1.y), ptx::pack2(b1.z, b1.w)};
-            uint32_t o4[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-              const int col = c * 8 + 2 * e;
-              float v0, v1;
-              ptx::unpack2(ptx::add2(ptx::pack2(__uint_as_float(rv[col]), __uint_as_float(rv[col + 1])), bb[e]), v0, v1);
-              o4[e] = float2_to_bf16x2(v0, v1);
-            }
-            // whole 32-byte sectors per store when y is aligned for it (rows are 128 or 192 bytes apart)
-            if (wide_store) {
-              if (c & 1) ptx::st_global_v8(yg + k * 4 + c - 1, o_prev, make_uint4(o4[0], o4[1], o4[2], o4[3]));
-              else o_prev = make_uint4(o4[0], o4[1], o4[2], o4[3]);
-            } else {
-              yg[k * 4 + c] = make_uint4(o4[0], o4[1], o4[2], o4[3]);
-            }
+          // whole 32-byte sectors per store when y is aligned for it (rows are 128 or 192 bytes apart)
+          if (wide_store) {
+            ptx::st_global_v8(yg + 2 * k, make_uint4(o[0], o[1], o[2], o[3]), make_uint4(o[4], o[5], o[6], o[7]));
+          } else {
+            yg[2 * k] = make_uint4(o[0], o[1], o[2], o[3]);
+            yg[2 * k + 1] = make_uint4(o[4], o[5], o[6], o[7]);
           }
         }
       }
@@ -836,7 +829,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
 static size_t fused_smem_need(int NH, int T, int na) {
   const int C = NH * D, br = T <= 56 ? 28 : 36;
   return (size_t)na * NH * KBT + (size_t)NH * KV_SLOT + (size_t)NH * NH * WQ_TILE + (size_t)NH * C * 64 +
-         (size_t)na * AX_BYTES + (size_t)NH * WX_TILE + (size_t)ID_BYTES + (size_t)NH * T * br * 4 + (size_t)C * 4 +
+         (size_t)na * AX_BYTES + (size_t)NH * WX_TILE + (size_t)NH * T * br * 4 + (size_t)C * 4 +
          (size_t)na * BM * 4 + (size_t)NRING * BM * 4 + (size_t)2 * C * 4 + TP * 4 + 16 + TP * 16 + 4 * 16 + 32 + N_BARS * 8 + 16;
 }
 static constexpr size_t kMaxSmem = 232448;
