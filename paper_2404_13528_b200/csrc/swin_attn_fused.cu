@@ -739,17 +739,17 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
     };
     bool ok = true;
     int su = 0;                                        // statistics taken of the units below it
-    // Waits for `bar`, taking the statistics of units whose rows come in meanwhile: they are what the next products wait for.
+    // Waits for `bar`, or for the statistics of unit `ul`, taking the statistics of units whose rows come in meanwhile.
     auto wait_working = [&](uint64_t* bar, uint32_t par, bool until_statistics, int ul) {
       uint32_t idle = 0;
       unsigned long long t_idle = 0;
       while (true) {
-        if (su < U && __all_sync(0xFFFFFFFFu, ptx::mbar_test(&landed[su % na], (su / na) & 1) ? 1 : 0)) {
+        if (until_statistics ? su > ul : __all_sync(0xFFFFFFFFu, ptx::mbar_test(bar, par) ? 1 : 0) != 0) {
+          return true;
+        } else if (su < U && __all_sync(0xFFFFFFFFu, ptx::mbar_test(&landed[su % na], (su / na) & 1) ? 1 : 0)) {
           statistics(su);
           ++su;
           idle = 0;
-        } else if (until_statistics ? su > ul : __all_sync(0xFFFFFFFFu, ptx::mbar_test(bar, par) ? 1 : 0) != 0) {
-          return true;
         } else if ((++idle & 63u) == 0) {
           if (__any_sync(0xFFFFFFFFu, *(volatile int*)abort_flag)) return false;
           const unsigned long long now = __shfl_sync(0xFFFFFFFFu, ptx::globaltimer(), 0);
