@@ -25,9 +25,9 @@
 //   Ob   = bf16(O / rowsum)                    back into tensor memory as packed pairs
 //   Y   += Ob Wp[:, 32 h : 32 h + 32]^T        128 x C x 32: the head merge is the accumulation over heads
 //
-// and per unit  the heads' projections accumulate in Y, and the epilogue stores  y_row = x_row + Y + b_proj  with 32-byte vectors at
-// the row's offset under the map.  x_row is read again (from L2) while the unit is under way: as a product of the raw rows with the
-// identity, which opened Y, the residual kept the unit's slot of the row ring until the epilogue of the unit before had left Y.
+// and per unit  Y starts as X I (the unit's raw rows times the identity: the residual rides on the tensor core, exactly, since
+// every product is a bf16 value times one), the heads' projections accumulate on top, and the epilogue stores
+// y_row = Y + b_proj with 16-byte vectors at the row's offset under the map.
 //
 // LayerNorm without a normalised tile:  LN(x) W^T + b = rstd (x W'^T - mean c + sigma b'),  W' = bf16(gamma . W) (column
 // scaling), c_n = sum_k W'_nk, b'_n = b_n + sum_k beta_k W_nk, sigma = 1 / rstd.  c is summed from the ROUNDED W', so the
@@ -46,15 +46,16 @@
 //         are on the item's critical path, and a barrier is cheaper than a trip through another warp;
 //   then  four warps for the row statistics and the Y epilogue (one row per thread);
 //   last  one warp that issues the QKV products of the items ahead (into the buffer the item four before has left) and one
-//         that issues, in item order, the heads' projections.
-// What bounds it (clock stamps at every hand-off): not arithmetic -- with the whole softmax compiled out the kernel is 5 % faster --
-// but the chain of hand-offs of an item (tensor-memory round trips, three barriers, two waits for small products behind other
-// groups' products in the tensor pipe; 4500 cycles) and the wait for its QKV product.  That wait was the loading warps' chain,
-// 6500 cycles a unit (copies issued, rows awaited, statistics taken, then the next unit's copies): with the statistics in the
-// epilogue warps, which take them whenever rows are in, and slots freed by the QKV products, the next rows are on their way
-// meanwhile (32 x 56 x 56 x 64, three slots: 27.3 -> 23.9 us; 96 channels have room for two slots: 32.9 -> 32.7).  A single warp
-// for the copies is too slow for the gathered windows (59.7).  Code that runs once per unit (statistics, the prologue) is kept in
-// rolled loops because its straight-line form ran at the speed of the instruction cache misses.  Every wait is bounded.
+//         that issues, in item order, the residual product that opens a unit's Y and the heads' projections.
+// What bounds it (clock stamps at every hand-off, counters): no unit of the SM -- issue slots 52 % busy, ALU 35, tensor pipe 24, special
+// functions 19 -- but the chain of hand-offs of an item (tensor-memory round trips, three barriers, two waits for small products;
+// 4500 cycles), which more items in flight did not shorten (four row groups instead of two or three, with or without two fewer
+// loading warps: 0.2 to 3 us slower).  What did: the loading warps issued a unit's copies, awaited its rows and took their
+// statistics before they turned to the next unit, 6500 cycles in all; now the epilogue warps take the statistics whenever rows
+// are in (32 x 56 x 56 tokens, 96 channels: 32.9 -> 29.8 us; 64: 27.3 -> 23.4).  Tried: the residual read again from global memory
+// in the epilogue, which frees a unit's slot of the row ring earlier (33.1); one warp for all copies (59.7: the gathered windows).
+// Code that runs once per unit (statistics, epilogue, the prologue) is kept in rolled loops because its straight-line form ran at
+// the speed of the instruction cache misses.  Every wait is bounded.
 #include "attn.cuh"
 #include "gemm_tc.cuh"
 #include "ptx.cuh"
@@ -75,10 +76,10 @@ constexpr int WROWS = 96;                           // rows of a per-head QKV we
 constexpr int WQ_TILE = WROWS * 64;
 constexpr int WX_TILE = WROWS * 32;                 // the extra k-step of a head's weights
 constexpr int KV_SLOT = 2 * KBT;                    // k, v tiles of one item
+constexpr int ID_BYTES = 32 * 64;                   // the identity tile
 constexpr int NBUF = 4, BUF_COLS = 96;              // item buffers of tensor memory
-// Units whose row offsets are kept.  The rows of unit u come in once the QKV products of unit u - 3 are done at the latest, which waited
-// for a projection of unit u - 5 (two heads; three: u - 4), which waited until the epilogue of unit u - 6 had read Y and, before
-// that, its offsets: six would do.
+// Units whose row offsets are kept.  The rows of unit u come in once unit u - 3 at the latest has had its residual product, which waited
+// until the epilogue of unit u - 4 had read Y, so that of u - 5 had read its offsets long before.
 constexpr int NRING = 8;
 constexpr int kLoaderThreads = 128;
 constexpr uint32_t TMEM_COLS = 512;
@@ -127,7 +128,8 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
   uint8_t* sWp = sWq + NH * NH * WQ_TILE;                          // [NH heads][C rows x 64 B]
   uint8_t* sAx = sWp + NH * WP_TILE;                               // [na][128 rows x 32 B]
   uint8_t* sWx = sAx + na * AX_BYTES;                              // [NH heads][96 rows x 32 B]
-  uint32_t* bias_s = reinterpret_cast<uint32_t*>(sWx + NH * WX_TILE);   // [NH][T][BR]: bf16 pairs
+  uint8_t* sId = sWx + NH * WX_TILE;                               // [32 rows x 64 B]: the 32 x 32 identity (the residual rides on the tensor core)
+  uint32_t* bias_s = reinterpret_cast<uint32_t*>(sId + ID_BYTES);  // [NH][T][BR]: bf16 pairs
   float* bp_s = reinterpret_cast<float*>(bias_s + NH * T * BR);    // [C]
   float* rstd_s = bp_s + C;                                        // [na][128]
   uint32_t* rowoff_s = reinterpret_cast<uint32_t*>(rstd_s + na * BM);   // [NRING][128]: row offset in 16-byte units
@@ -193,7 +195,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
 #pragma unroll 1
       for (int i = 0; i < 3; ++i) {
         ptx::mbar_init(&a_full[i], 4);
-        ptx::mbar_init(&a_free[i], 4 * NH);
+        ptx::mbar_init(&a_free[i], 4 * NH + 1);
         ptx::mbar_init(&landed[i], 128 + 4);
         ptx::mbar_init(&s_full[i], 1);
         ptx::mbar_init(&o_full[i], 1);
@@ -232,6 +234,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
   }
   for (int i = tid; i < na * A_BYTES / 16; i += kThreads) reinterpret_cast<uint4*>(sA)[i] = make_uint4(0, 0, 0, 0);
   for (int i = tid; i < na * AX_BYTES / 16; i += kThreads) reinterpret_cast<uint4*>(sAx)[i] = make_uint4(0, 0, 0, 0);
+  for (int i = tid; i < ID_BYTES / 16; i += kThreads) reinterpret_cast<uint4*>(sId)[i] = make_uint4(0, 0, 0, 0);
   for (int i = tid; i < na * BM; i += kThreads) rstd_s[i] = 0.f;
   for (int i = tid; i < NRING * BM; i += kThreads) rowoff_s[i] = ROW_INVALID;
   if (tid >= 128 && tid < 128 + TP) {
@@ -262,6 +265,8 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
     bp_s[tid] = __bfloat162float(par[2]);
   }
   __syncthreads();
+  if (warp == 7 + 4 * NH)                             // identity: row n has a one in column n
+    *reinterpret_cast<uint16_t*>(sId + sw64_off(lane, lane >> 3) + (lane & 7) * 2) = 0x3F80u;
   // keys below / right of the wrap line of a seam window (bit c = key c)
   if (warp == 8 + 4 * NH) {
     const int c0 = lane, c1 = lane + 32;
@@ -485,12 +490,10 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
         }
         // q as the S product's A operand: 64 bf16 = 32 packed columns over the accumulator's last 32 (v has been read): this
         // window's half carries q, the other half zeros (the two windows' keys are stacked along the reduction dimension)
+        ptx::tmem_st16(tb + 64 + w * 16, q16);
 #pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          rv[c] = w ? 0u : q16[c];
-          rv[16 + c] = w ? q16[c] : 0u;
-        }
-        ptx::tmem_st32(tb + 64, rv);
+        for (int c = 0; c < 16; ++c) q16[c] = 0u;
+        ptx::tmem_st16(tb + 64 + (1 - w) * 16, q16);
         ptx::tmem_st_wait();
         ptx::fence_proxy_async();                      // generic-proxy writes -> visible to the MMAs
         ptx::tc_fence_before();
@@ -556,7 +559,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
           }
         }
 #pragma unroll
-        for (int c = 0; c < KC; ++c) mx4[c & 3] = fmaxf(mx4[c & 3], sc[c]);
+        for (int c = 0; c < KC; c += 2) mx4[(c >> 1) & 3] = fmaxf(fmaxf(mx4[(c >> 1) & 3], sc[c]), sc[c + 1]);      // (one instruction)
         const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
         const float nmx = -mx * LOG2E;
         const f32x2 nmx2 = ptx::pack2(nmx, nmx);
@@ -621,17 +624,33 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
       if (lane == 0) ptx::mbar_arrive(&ob_full[it & (NBUF - 1)]);       // the projection of this item may be issued
     }
   } else if (warp == 8 + 4 * NH) {
-    // ---- the heads' projections, in item order (issue order is accumulation order).  They and the QKV products have a warp each:
-    // together in one polling loop (about a thousand cycles a turn, beside the warps it shares a scheduler with) they were what the
-    // items waited for.  Whole warps walk the queues; an elected lane issues. --------------------------------------------------
+    // ---- the residual product that opens a unit's Y and the heads' projections, in item order (issue order is accumulation order).
+    // They and the QKV products have a warp each: together in one polling loop (about a thousand cycles a turn, beside the warps it
+    // shares a scheduler with) they were what the items waited for.  Whole warps walk the queues; an elected lane issues. ---------
     if (__all_sync(0xFFFFFFFFu, w_ok ? 1 : 0)) {
       const uint32_t idesc_pj = ptx::make_idesc_bf16(BM, C, false, false);
-      const uint64_t wp_d = desc_sw64(ptx::smem_u32(sWp));
+      const uint32_t idesc_id = ptx::make_idesc_bf16(BM, D, false, false);
+      const uint64_t id_d = desc_sw64(ptx::smem_u32(sId)), a_d = desc_sw64(ptx::smem_u32(sA)), wp_d = desc_sw64(ptx::smem_u32(sWp));
       bool ok = true;
-      int it = 0;
+      int ab = 0, aph = 0, it = 0;
 #pragma unroll 1
       for (int ul = 0; ul < U && ok; ++ul) {
-        ok = __all_sync(0xFFFFFFFFu, GWAIT(y_empty, (ul & 1) ^ 1) ? 1 : 0) != 0;      // the epilogue of the unit before has read Y
+        // Y = X I: the unit's raw rows open the accumulation (the epilogue of the unit before has read Y); exact, since every
+        // product is a bf16 value times one.  The product is the last reader of the unit's rows: its completion frees the slot.
+        ok = __all_sync(0xFFFFFFFFu, GWAIT(&a_full[ab], aph) && GWAIT(y_empty, (ul & 1) ^ 1) ? 1 : 0) != 0;
+        if (!ok) break;
+        ptx::tc_fence_after();
+        const uint64_t ad0 = a_d + ab * (A_BYTES >> 4);
+        if (ptx::elect_one()) {
+#pragma unroll
+          for (int kb = 0; kb < NH; ++kb) {            // 32 channels at a time: Y[:, 32 kb : 32 kb + 32] = X[:, 32 kb : 32 kb + 32] I_32
+            ptx::tc_mma_bf16(tmem_base + TM_Y + kb * D, ad0 + kb * (KBT >> 4), id_d, idesc_id, 0u);
+            ptx::tc_mma_bf16(tmem_base + TM_Y + kb * D, ad0 + kb * (KBT >> 4) + 2, id_d + 2, idesc_id, 1u);
+          }
+          ptx::tc_commit(&a_free[ab]);
+        }
+        __syncwarp();
+        if (++ab == na) { ab = 0; aph ^= 1; }
 #pragma unroll 1
         for (int h = 0; h < NH && ok; ++h, ++it) {
           // Y += Ob_h Wp[:, 32 h : 32 h + 32]^T; the last head hands Y to the epilogue
@@ -641,7 +660,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
           const uint32_t a = tmem_base + (it & (NBUF - 1)) * BUF_COLS + 64;
           const uint64_t bd = wp_d + h * (WP_TILE >> 4);
           if (ptx::elect_one()) {
-            ptx::tc_mma_bf16_ta(tmem_base + TM_Y, a, bd, idesc_pj, h ? 1u : 0u);
+            ptx::tc_mma_bf16_ta(tmem_base + TM_Y, a, bd, idesc_pj, 1u);
             ptx::tc_mma_bf16_ta(tmem_base + TM_Y, a + 8, bd + 2, idesc_pj, 1u);
             ptx::tc_commit(&buf_free[it & (NBUF - 1)]);
             if (h == NH - 1) ptx::tc_commit(y_full);
@@ -737,20 +756,19 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&a_full[ab]);
     };
-    bool ok = true;
     int su = 0;                                        // statistics taken of the units below it
-    // Waits for `bar`, or for the statistics of unit `ul`, taking the statistics of units whose rows come in meanwhile.
-    auto wait_working = [&](uint64_t* bar, uint32_t par, bool until_statistics, int ul) {
+    // Waits for `bar`, taking the statistics of units whose rows come in meanwhile.
+    auto wait_working = [&](uint64_t* bar, uint32_t par) {
       uint32_t idle = 0;
       unsigned long long t_idle = 0;
       while (true) {
-        if (until_statistics ? su > ul : __all_sync(0xFFFFFFFFu, ptx::mbar_test(bar, par) ? 1 : 0) != 0) {
+        if (__all_sync(0xFFFFFFFFu, ptx::mbar_test(bar, par) ? 1 : 0)) {
           return true;
         } else if (su < U && __all_sync(0xFFFFFFFFu, ptx::mbar_test(&landed[su % na], (su / na) & 1) ? 1 : 0)) {
           statistics(su);
           ++su;
           idle = 0;
-        } else if ((++idle & 63u) == 0) {
+        } else if (__nanosleep(32), (++idle & 63u) == 0) {
           if (__any_sync(0xFFFFFFFFu, *(volatile int*)abort_flag)) return false;
           const unsigned long long now = __shfl_sync(0xFFFFFFFFu, ptx::globaltimer(), 0);
           if (idle == 64u) t_idle = now;
@@ -766,50 +784,43 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
     };
 #pragma unroll 1
     for (int ul = 0; ul < U; ++ul) {
-      // (the row's offset is written before the rows come in)
-      if (!wait_working(nullptr, 0, true, ul)) break;
+      if (!wait_working(y_full, ul & 1)) break;
+      ptx::tc_fence_after();
       const uint32_t my_off = rowoff_s[(ul % NRING) * BM + r];
       const bool valid = i < T && my_off != ROW_INVALID;
       uint4* yg = reinterpret_cast<uint4*>(g.y + ((size_t)(valid ? my_off : 0u) << 3));
-      const uint4* xg = reinterpret_cast<const uint4*>(g.x + ((size_t)(valid ? my_off : 0u) << 3));
-      uint4 xr[NCH];
-#pragma unroll
-      for (int c = 0; c < NCH; ++c) xr[c] = valid ? xg[c] : make_uint4(0, 0, 0, 0);
-      ok = wait_working(y_full, ul & 1, false, ul);
-      if (!ok) break;
-      ptx::tc_fence_after();
-#pragma unroll
-      for (int k = 0; k < NCH / 2; ++k) {              // 16 columns at a time (two chunks: a sector)
-        uint32_t rv[16], o[8];
-        ptx::tmem_ld16(tmem_base + TM_Y + lane_addr + k * 16, rv);
+#pragma unroll 1
+      for (int k = 0; k < NH; ++k) {                   // 32 columns = 4 chunks of the row at a time
+        uint32_t rv[32];
+        ptx::tmem_ld32(tmem_base + TM_Y + lane_addr + k * 32, rv);
         ptx::tmem_ld_wait();
-        if (k == NCH / 2 - 1) {                        // Y is in registers: the next unit's products may overwrite it
+        if (k == NH - 1) {                             // Y is in registers: the next unit's products may overwrite it
           ptx::tc_fence_before();
           __syncwarp();
           if (lane == 0) ptx::mbar_arrive(y_empty);
         }
-        const uint32_t xw[8] = {xr[2 * k].x, xr[2 * k].y, xr[2 * k].z, xr[2 * k].w, xr[2 * k + 1].x, xr[2 * k + 1].y, xr[2 * k + 1].z, xr[2 * k + 1].w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float4 b4 = *reinterpret_cast<const float4*>(bp_s + k * 16 + 4 * e);
-          const f32x2 bb[2] = {ptx::pack2(b4.x, b4.y), ptx::pack2(b4.z, b4.w)};
-#pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const uint32_t xp = xw[2 * e + j];
-            const f32x2 acc = ptx::pack2(__uint_as_float(rv[4 * e + 2 * j]), __uint_as_float(rv[4 * e + 2 * j + 1]));
-            const f32x2 res = ptx::pack2(__uint_as_float(xp << 16), __uint_as_float(xp & 0xFFFF0000u));
-            float v0, v1;
-            ptx::unpack2(ptx::add2(ptx::add2(acc, res), bb[j]), v0, v1);
-            o[2 * e + j] = float2_to_bf16x2(v0, v1);
-          }
-        }
         if (valid) {
-          // whole 32-byte sectors per store when y is aligned for it (rows are 128 or 192 bytes apart)
-          if (wide_store) {
-            ptx::st_global_v8(yg + 2 * k, make_uint4(o[0], o[1], o[2], o[3]), make_uint4(o[4], o[5], o[6], o[7]));
-          } else {
-            yg[2 * k] = make_uint4(o[0], o[1], o[2], o[3]);
-            yg[2 * k + 1] = make_uint4(o[4], o[5], o[6], o[7]);
+          uint4 o_prev = make_uint4(0, 0, 0, 0);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            const float4 b0 = *reinterpret_cast<const float4*>(bp_s + k * 32 + c * 8);
+            const float4 b1 = *reinterpret_cast<const float4*>(bp_s + k * 32 + c * 8 + 4);
+            const f32x2 bb[4] = {ptx::pack2(b0.x, b0.y), ptx::pack2(b0.z, b0.w), ptx::pack2(b1.x, b1.y), ptx::pack2(b1.z, b1.w)};
+            uint32_t o4[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int col = c * 8 + 2 * e;
+              float v0, v1;
+              ptx::unpack2(ptx::add2(ptx::pack2(__uint_as_float(rv[col]), __uint_as_float(rv[col + 1])), bb[e]), v0, v1);
+              o4[e] = float2_to_bf16x2(v0, v1);
+            }
+            // whole 32-byte sectors per store when y is aligned for it (rows are 128 or 192 bytes apart)
+            if (wide_store) {
+              if (c & 1) ptx::st_global_v8(yg + k * 4 + c - 1, o_prev, make_uint4(o4[0], o4[1], o4[2], o4[3]));
+              else o_prev = make_uint4(o4[0], o4[1], o4[2], o4[3]);
+            } else {
+              yg[k * 4 + c] = make_uint4(o4[0], o4[1], o4[2], o4[3]);
+            }
           }
         }
       }
@@ -829,7 +840,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
 static size_t fused_smem_need(int NH, int T, int na) {
   const int C = NH * D, br = T <= 56 ? 28 : 36;
   return (size_t)na * NH * KBT + (size_t)NH * KV_SLOT + (size_t)NH * NH * WQ_TILE + (size_t)NH * C * 64 +
-         (size_t)na * AX_BYTES + (size_t)NH * WX_TILE + (size_t)NH * T * br * 4 + (size_t)C * 4 +
+         (size_t)na * AX_BYTES + (size_t)NH * WX_TILE + (size_t)ID_BYTES + (size_t)NH * T * br * 4 + (size_t)C * 4 +
          (size_t)na * BM * 4 + (size_t)NRING * BM * 4 + (size_t)2 * C * 4 + TP * 4 + 16 + TP * 16 + 4 * 16 + 32 + N_BARS * 8 + 16;
 }
 static constexpr size_t kMaxSmem = 232448;
