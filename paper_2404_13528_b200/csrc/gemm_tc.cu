@@ -990,11 +990,13 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
     // the first tile, and for every further wave its k-blocks or, where the reduction is short, its epilogue.  A narrow tile
     // costs more per column but splits the columns over more SMs: M = 666, N = K = 2048 (48 tiles of 128 x 256, 96 of half
     // that) 16.1 us on 256-wide single tiles, 9.6 on 128-wide pairs; M = 196, N = 512, K = 2048 14.1 -> 8.8 us on 64-wide ones.
+    // With many waves, narrow pair tiles pay for the operand they read twice: M = 16384, N = 512, K = 1024 17.1 us on four waves of
+    // 128-wide pairs, 16.2 on two of 256; M = 12544, K = 2048 23.3 on three, 24.8 on two.
     struct Option { int bn; bool pair, lean; double fixed, per_kb, wave, wave_min; };
     static const Option options[] = {{64, false, false, 2.4, 0.185, 0.55, 0.95}, {96, false, false, 2.9, 0.22, 0.8, 1.2},
                                      {128, false, true, 2.6, 0.26, 0.7, 1.15},   {256, false, true, 3.9, 0.5, -0.2, 1.65},
                                      {128, false, false, 2.6, 0.27, 0.4, 2.8},   {256, false, false, 4.4, 0.36, 0.5, 4.0},
-                                     {128, true, false, 3.0, 0.185, 0.2, 2.2},   {256, true, false, 4.6, 0.33, 0.4, 3.0}};
+                                     {128, true, false, 3.0, 0.185, 0.6, 2.2},   {256, true, false, 5.4, 0.33, 0.4, 3.0}};
     double best = 0.0;
     for (const Option& o : options) {
       if (o.pair && !pair_ok) continue;
