@@ -22,16 +22,18 @@ int ensure_max_dynamic_smem(const void* kernel, int bytes, int carveout = -1);
 // set up its barriers and tensor memory, prefetch its descriptors and constants) while the kernel
 // before it in the stream is still draining; it must call `pdl_wait()` before it reads or writes
 // anything that kernel could touch.  The wait returns once the whole preceding grid has finished
-// and its writes are visible.  `pdl_launch_dependents()` lets the NEXT kernel in the stream begin
+// and its writes are visible.  What no kernel in flight can be writing may be read earlier: parameters of a layer call, in a kernel
+// that follows another one of the same call (that one has waited for whatever preceded the call); its launcher says so with
+// `settled`, and without it gives up the early start.  `pdl_launch_dependents()` lets the NEXT kernel in the stream begin
 // that early start as soon as every CTA of this one has called it.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// `cluster_x` > 1 launches thread-block clusters of that many CTAs (neighbours in blockIdx.x).
+// `cluster_x` > 1 launches thread-block clusters of that many CTAs (neighbours in blockIdx.x).  `early` false: ordinary stream order.
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, unsigned cluster_x,
-                                      Args&&... args) {
+inline cudaError_t launch_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, unsigned cluster_x, bool early,
+                                  Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -41,7 +43,7 @@ inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   // SMARTMEM_NO_PDL=1 launches every kernel with ordinary stream ordering (for measuring what the overlap buys)
   static const int allow = [] { const char* e = getenv("SMARTMEM_NO_PDL"); return (e && e[0] == '1') ? 0 : 1; }();
-  attr[0].val.programmaticStreamSerializationAllowed = allow;
+  attr[0].val.programmaticStreamSerializationAllowed = early ? allow : 0;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   if (cluster_x > 1) {
@@ -52,6 +54,11 @@ inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 
     cfg.numAttrs = 2;
   }
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, unsigned cluster_x,
+                                      Args&&... args) {
+  return launch_cluster(kernel, grid, block, smem, st, cluster_x, true, static_cast<Args&&>(args)...);
 }
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {

@@ -475,6 +475,7 @@ EXPORT int smartmem_attn_decode(const smartmem_attn_params_t* pp, int32_t pos, c
       ep.seg_out[1] = kc + (long long)pos * hid;   ep.seg_ld[1] = Smax * hid;
       ep.seg_out[2] = vc + (long long)pos * hid;   ep.seg_ld[2] = Smax * hid;
     }
+    ep.b_settled = norm_in_gemm ? 0 : 1;             // (with RMSNorm inside it is the call's first kernel)
     if (norm_in_gemm) { ep.rms_gamma = p.rms_g; ep.rms_eps = p.rms_eps; }
     SM_TRY(launch_gemm_tc(tc_operand_plain(norm_in_gemm ? x : at(L.xn), B, hid, hid), tc_operand_plain(p.w_qkv, 3 * hid, hid, hid), ep, 1,
                           B, 3 * hid, hid, st));
@@ -502,6 +503,7 @@ EXPORT int smartmem_attn_decode(const smartmem_attn_params_t* pp, int32_t pos, c
     ep.out = y;
     ep.ldc = hid;
     ep.residual = p.add_residual ? x : nullptr;
+    ep.b_settled = 1;
     SM_TRY(launch_gemm_tc(tc_operand_plain(at(L.ao), B, hid, hid), tc_operand_plain(p.w_o, hid, hid, hid), ep, 1, B, hid,
                           hid, st));
   }

@@ -71,12 +71,10 @@ ln_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       *abort_flag = 0;
       ptx::fence_barrier_init();
       ptx::fence_proxy_async();
-      ptx::prefetch_tensormap(&tmW);
-      ptx::mbar_expect_tx(w_full, (uint32_t)(HW * K * 2));
+      // A chain's weights are inputs like any other, perhaps still being written by the kernel before this one: before the dependency
+      // wait they only come as far as L2
+      ptx::tma_prefetch_3d(&tmW, 0, n0 + rank * HW, 0);
     }
-    __syncwarp();
-    // a parameter: fetched before the dependency wait, all k-blocks in one copy
-    if (ptx::elect_one()) ptx::tma_load_3d(sW, &tmW, w_full, 0, n0 + rank * HW, 0);
     __syncwarp();
     ptx::tmem_alloc_pair(tmem_slot, TMEM_COLS);
   }
@@ -85,14 +83,10 @@ ln_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   if (tid >= 256 && tid - 256 < K / 8) {
     const int v = tid - 256;
     col_s[v] = (int)devmap_part_rolled(g.map, g.split, g.map.n_atoms, (uint32_t)v).off;
-    const uint4 ga = *reinterpret_cast<const uint4*>(g.ln_g + v * 8), be = *reinterpret_cast<const uint4*>(g.ln_b + v * 8);
-    const float2 g0 = bf16x2_to_float2(ga.x), g1 = bf16x2_to_float2(ga.y), g2 = bf16x2_to_float2(ga.z), g3 = bf16x2_to_float2(ga.w);
-    const float2 b0 = bf16x2_to_float2(be.x), b1 = bf16x2_to_float2(be.y), b2 = bf16x2_to_float2(be.z), b3 = bf16x2_to_float2(be.w);
-    float4* p = reinterpret_cast<float4*>(par);
-    p[v] = make_float4(g0.x, g0.y, g1.x, g1.y);
-    p[K / 8 + v] = make_float4(g2.x, g2.y, g3.x, g3.y);
-    p[2 * (K / 8) + v] = make_float4(b0.x, b0.y, b1.x, b1.y);
-    p[3 * (K / 8) + v] = make_float4(b2.x, b2.y, b3.x, b3.y);
+    if (v < K / 64) {
+      ptx::prefetch_l2(g.ln_g + v * 64);
+      ptx::prefetch_l2(g.ln_b + v * 64);
+    }
   }
   // the warp's eight row offsets in tile t, one evaluation of the map per lane
   auto offset_of = [&](int t) {
@@ -160,6 +154,16 @@ ln_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         be[2 * h + 1] = ptx::pack2(__uint_as_float(b.z), __uint_as_float(b.w));
       }
     };
+    auto widen_affine = [&](int v) {
+      const uint4 ga = *reinterpret_cast<const uint4*>(g.ln_g + v * 8), be = *reinterpret_cast<const uint4*>(g.ln_b + v * 8);
+      const float2 g0 = bf16x2_to_float2(ga.x), g1 = bf16x2_to_float2(ga.y), g2 = bf16x2_to_float2(ga.z), g3 = bf16x2_to_float2(ga.w);
+      const float2 b0 = bf16x2_to_float2(be.x), b1 = bf16x2_to_float2(be.y), b2 = bf16x2_to_float2(be.z), b3 = bf16x2_to_float2(be.w);
+      float4* p = reinterpret_cast<float4*>(par);
+      p[v] = make_float4(g0.x, g0.y, g1.x, g1.y);
+      p[K / 8 + v] = make_float4(g2.x, g2.y, g3.x, g3.y);
+      p[2 * (K / 8) + v] = make_float4(b0.x, b0.y, b1.x, b1.y);
+      p[3 * (K / 8) + v] = make_float4(b2.x, b2.y, b3.x, b3.y);
+    };
     pdl_wait();
     pdl_launch_dependents();
     auto normalise = [&](auto& x, int row0, auto&& free) {
@@ -172,6 +176,15 @@ ln_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     };
     uint4 x0[J0][V], x1[J1][V];                    // rows being normalised, rows on their way
     if (first < g.tiles) request(x0, first, 0, row_off);
+    if (warp == 0) {                               // all k-blocks of the slice in one copy
+      if (ptx::elect_one()) {
+        ptx::mbar_expect_tx(w_full, (uint32_t)(HW * K * 2));
+        ptx::tma_load_3d(sW, &tmW, w_full, 0, n0 + rank * HW, 0);
+      }
+      __syncwarp();
+    }
+    if (tid >= 256 && tid - 256 < K / 8) widen_affine(tid - 256);
+    __syncthreads();
     int it = 0;
     for (int t = first; t < g.tiles; t += g.pairs, ++it) {
       request(x1, t, 4, row_off);

@@ -3,7 +3,7 @@
 // The kernel for K = 64 and 96 keeps all of W in shared memory and streams the rows past it; here W does not fit, and with a few
 // thousand rows there is nothing to stream: a launch, a dependency and a drain cost the normalisation and the product each more
 // than their work.  A CTA takes 128 rows and a slice of the output columns, normalises the rows (again in every slice: they come
-// from L2) straight into the operand, and multiplies them with its slice of W, fetched before the dependency wait.  Bound by that
+// from L2) straight into the operand, and multiplies them with its slice of W, which is in L2 by then.  Bound by that
 // chain (1.5 us rows, 0.9 product, 0.6 output and the dependency).  Measured, a block's attention half with norm + QKV linear
 // before -> with this: 3920 x 192 17.4 -> 15.4 us (93 CTAs), 7840 x 128 19.1 -> 16.3 (124), 1568 x 256 16.6 -> 14.8 (78), 4704 x 256
 // 20.5 -> 18.4 (148); an MLP half with norm + fc1 + GELU: 1568 x 256 13.1 -> 11.3.
@@ -22,7 +22,7 @@ constexpr int BM = 128, BK = 64;
 constexpr int kWorkers = 16, kThreads = 32 * (kWorkers + 1);
 
 struct LnWaveArgs {
-  int M, N, slices, has_map, gelu, wide;
+  int M, N, slices, has_map, gelu, wide, w_settled;
   float eps;
   const __nv_bfloat16 *x, *ln_g, *ln_b, *bias;
   __nv_bfloat16* out;
@@ -59,17 +59,21 @@ ln_wave_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       *abort_flag = 0;
       ptx::fence_barrier_init();
       ptx::fence_proxy_async();
-      ptx::prefetch_tensormap(&tmW);
       ptx::mbar_expect_tx(w_full, (uint32_t)(NS * K * 2));
+      // W, all k-blocks in one copy: before the dependency wait where nothing in flight can be writing it, else only as far as L2
+      if (g.w_settled) ptx::tma_load_3d(sW, &tmW, w_full, 0, n0, 0);
+      else ptx::tma_prefetch_3d(&tmW, 0, n0, 0);
     }
     __syncwarp();
-    // a parameter: fetched before the dependency wait, all k-blocks in one copy
-    if (ptx::elect_one()) ptx::tma_load_3d(sW, &tmW, w_full, 0, n0, 0);
-    __syncwarp();
     ptx::tmem_alloc(tmem_slot, TMEM_COLS);
+  } else if (warp == 0) {
+    if (lane < K / 64) {
+      ptx::prefetch_l2(g.ln_g + lane * 64);
+      ptx::prefetch_l2(g.ln_b + lane * 64);
+    } else if (g.bias && lane - K / 64 < NB) {
+      ptx::prefetch_l2(g.bias + n0 + (lane - K / 64) * 64);
+    }
   }
-  if (tid < NS / 8)
-    *reinterpret_cast<uint4*>(bias_s + tid * 8) = g.bias ? *reinterpret_cast<const uint4*>(g.bias + n0 + tid * 8) : make_uint4(0, 0, 0, 0);
   ptx::tc_fence_before();
   __syncthreads();
   ptx::tc_fence_after();
@@ -77,6 +81,11 @@ ln_wave_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 
   if (warp == kWorkers) {
     const uint32_t a0 = ptx::smem_u32(sA), w0 = ptx::smem_u32(sW);
+    if (!g.w_settled) {
+      pdl_wait();
+      if (ptx::elect_one()) ptx::tma_load_3d(sW, &tmW, w_full, 0, n0, 0);
+      __syncwarp();
+    }
     const bool ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(w_full, 0, abort_flag, g.status) && ptx::mbar_wait(a_ready, 0, abort_flag, g.status) ? 1 : 0) != 0;
     if (ok) {
       ptx::tc_fence_after();
@@ -95,12 +104,6 @@ ln_wave_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   } else {
     constexpr int L = ln_lanes(NV), J = L / 4, V = 8 * NV / L;
     const int sub = lane % L, rsub = lane / L;
-    uint4 ga[V], be[V];
-#pragma unroll
-    for (int k = 0; k < V; ++k) {
-      ga[k] = *reinterpret_cast<const uint4*>(g.ln_g + (sub + L * k) * 8);
-      be[k] = *reinterpret_cast<const uint4*>(g.ln_b + (sub + L * k) * 8);
-    }
     // the warp's eight row offsets, one evaluation of the map per lane
     const int mrow = m0 + warp * 8 + (lane & 7);
     long long row_off = 0;
@@ -118,10 +121,19 @@ ln_wave_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         if (m0 + warp * 8 + r < g.M) x[j][k] = *reinterpret_cast<const uint4*>(g.x + off + (sub + L * k) * 8);
       }
     }
+    uint4 ga[V], be[V];                              // (behind the wait as well, their latency under the rows')
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      ga[k] = *reinterpret_cast<const uint4*>(g.ln_g + (sub + L * k) * 8);
+      be[k] = *reinterpret_cast<const uint4*>(g.ln_b + (sub + L * k) * 8);
+    }
     ln_rows_to_operand<NV>(x, ga, be, g.eps, sA, warp * 8, lane);
     ptx::fence_proxy_async();
     __syncwarp();
     if (lane == 0) ptx::mbar_arrive(a_ready);
+    if (tid < NS / 8)
+      *reinterpret_cast<uint4*>(bias_s + tid * 8) = g.bias ? *reinterpret_cast<const uint4*>(g.bias + n0 + tid * 8) : make_uint4(0, 0, 0, 0);
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * kWorkers) : "memory");
 
     // ---- output: a thread per row and quarter of the columns, rows leave the registers as whole sectors ---------------------
     const int q = warp & 3, grp = warp >> 2, m = m0 + q * 32 + lane;
@@ -192,7 +204,7 @@ int blocks_of(long long M, long long N, long long K) {
 bool gemm_ln_wave_wins(long long M, long long N, long long K) { return blocks_of(M, N, K) != 0; }
 
 int launch_gemm_ln_wave(const void* X, const DevMap* rowmap, const void* gamma, const void* beta, float eps, const void* W, const void* bias,
-                        int gelu, void* out, long long M, long long N, long long K, cudaStream_t st) {
+                        int gelu, void* out, long long M, long long N, long long K, bool w_settled, cudaStream_t st) {
   const int nb = M < 1 ? 0 : blocks_of(M, N, K), ns = 64 * nb;
   if (nb == 0) return SMARTMEM_ERR_UNSUPPORTED;
   const void* ptrs[] = {X, gamma, beta, W, out};
@@ -201,7 +213,7 @@ int launch_gemm_ln_wave(const void* X, const DevMap* rowmap, const void* gamma, 
   if ((uintptr_t)bias & 15) return SMARTMEM_ERR_ALIGNMENT;
   LnWaveArgs g;
   memset(&g, 0, sizeof(g));
-  g.M = (int)M; g.N = (int)N; g.slices = (int)(N / ns); g.has_map = rowmap ? 1 : 0; g.gelu = gelu;
+  g.M = (int)M; g.N = (int)N; g.slices = (int)(N / ns); g.has_map = rowmap ? 1 : 0; g.gelu = gelu; g.w_settled = w_settled ? 1 : 0;
   if (rowmap) g.rowmap = *rowmap;
   g.eps = eps;
   g.x = (const __nv_bfloat16*)X; g.ln_g = (const __nv_bfloat16*)gamma; g.ln_b = (const __nv_bfloat16*)beta; g.bias = (const __nv_bfloat16*)bias; g.out = (__nv_bfloat16*)out;

@@ -6,7 +6,7 @@
 // splits the hidden features: every CTA normalises the rows (redundantly), multiplies them with its slice of W1, keeps the GELU of
 // its slice on chip as fc2's operand and multiplies that with its slice of W2; the fp32 partial results are exchanged as bulk
 // copies between the CTAs' shared memories, each CTA adding up its share of the rows.  The weight slices are fetched before the
-// dependency wait.  Measured against the three kernels: C = 192 (four slices), 3920 rows 14.8 -> 12.3 us, 196 rows 9.9 -> 10.1
+// dependency wait where nothing in flight can be writing them.  Measured against the three kernels: C = 192 (four slices), 3920 rows 14.8 -> 12.3 us, 196 rows 9.9 -> 10.1
 // (24 -> 18 us of host time); C = 128 (two slices), 7840 rows 13.5 -> 10.2.
 //
 // Bound by the chain of its phases (at C = 192 about 1.5 us rows, 0.9 first product, 1.3 GELU, 0.9 second product, 0.6 drain, 2.2
@@ -300,7 +300,7 @@ bool mlp_cluster_wins(long long M, long long C, long long hidden) {
 }
 
 int launch_mlp_cluster(const void* x, const void* ln_g, const void* ln_b, float eps, const void* W1, const void* b1, const void* W2,
-                       const void* b2, void* out, long long M, long long C, long long hidden, cudaStream_t st) {
+                       const void* b2, void* out, long long M, long long C, long long hidden, bool settled, cudaStream_t st) {
   MlpClusterArgs g;
   memset(&g, 0, sizeof(g));
   g.splits = splits_of(C, hidden);
@@ -328,7 +328,7 @@ int launch_mlp_cluster(const void* x, const void* ln_g, const void* ln_b, float 
   if (ensure_max_dynamic_smem((const void*)fn, 227 * 1024) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   profile_tick("mlp_cluster", st);
   const unsigned grid = (unsigned)((M + BM - 1) / BM * g.splits);
-  if (launch_pdl_cluster(fn, dim3(grid), dim3(kThreads), z.smem, st, (unsigned)g.splits, t1, t2, g) != cudaSuccess) return SMARTMEM_ERR_CUDA;
+  if (launch_cluster(fn, dim3(grid), dim3(kThreads), z.smem, st, (unsigned)g.splits, settled, t1, t2, g) != cudaSuccess) return SMARTMEM_ERR_CUDA;
   count_launch();
   return SMARTMEM_OK;
 }

@@ -13,7 +13,9 @@
 //     the normalised row itself is stored;
 //   * W and X have rings of their own: X comes from L2 and is scaled well ahead of the products, so that a stage of W is
 //     only held for its copy and its product (with one ring the scaling's latency came off the depth of W's);
-//   * W does not depend on the kernel before this one in the stream: the ring is filled with it before the dependency wait.
+//   * where nothing in flight writes W (TcEpilogue::b_settled) the ring is filled with it before the dependency wait, otherwise the
+//     same boxes are only prefetched into L2 there: W may be the second operand of a product, or a weight that the kernel before this
+//     one is still writing.
 //
 // Warp roles (8 warps): 0 TMA producer of W, 1 TMEM owner and MMA issuer, 2-6 scale X (RMSNorm), 7 TMA producer of X, 2-5
 // drain the accumulator; all eight finish the rows.
@@ -44,7 +46,7 @@ struct SplitArgs {
   __nv_bfloat16* out;
   long long ldc;
   const __nv_bfloat16 *bias, *residual;
-  int gelu, has_rowmap;
+  int gelu, has_rowmap, w_settled;
   int rope_cols, rope_S, rope_pos0, rope_half;
   float rope_c;
   int seg_cols;
@@ -100,19 +102,22 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   }
   __syncwarp();
   if (warp == 0) {
-    // the ring's first round of W: parameters only
+    // the ring's first round of W
     for (int s = 0; s < g.stages && s < nk; ++s) {
       if (ptx::elect_one()) {
-        ptx::mbar_expect_tx(&full[s], W_STAGE);
-        ptx::tma_load_2d(smem + s * W_STAGE, &tmW, &full[s], (kb0 + s) * BK, n0);
+        if (g.w_settled) {
+          ptx::mbar_expect_tx(&full[s], W_STAGE);
+          ptx::tma_load_2d(smem + s * W_STAGE, &tmW, &full[s], (kb0 + s) * BK, n0);
+        } else {
+          ptx::tma_prefetch_2d(&tmW, (kb0 + s) * BK, n0);
+        }
       }
       __syncwarp();
     }
   }
   if (warp == 1) ptx::tmem_alloc(tmem_slot, g.tmem_cols);
-  if (norm)
-    for (int i = tid; i < nk * (BK / 8); i += kThreads)
-      reinterpret_cast<uint4*>(gamma_s)[i] = *reinterpret_cast<const uint4*>(g.gamma + kb0 * BK + i * 8);
+  if (norm)                                         // (a line per k-block)
+    for (int i = tid; i < nk; i += kThreads) ptx::prefetch_l2(g.gamma + (kb0 + i) * BK);
   {
     const int sg = g.seg_cols > 0 ? n0 / g.seg_cols : 0;
     const long long ld = g.seg_cols > 0 ? g.seg_ld[sg] : g.ldc;
@@ -135,7 +140,7 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     const uint32_t bytes = w_side ? (uint32_t)W_STAGE : g.x_bytes;
     uint8_t* ring = w_side ? smem : sx;
     const CUtensorMap* tm = w_side ? &tmW : &tmX;
-    const int row0 = w_side ? n0 : m0, first = w_side ? min(ns, nk) : 0;      // (W: the first round is on its way already)
+    const int row0 = w_side ? n0 : m0, first = w_side && g.w_settled ? min(ns, nk) : 0;      // (settled W: the first round is on its way already)
     bool ok = true;
     int issued = first;
     uint32_t s = first == ns ? 0 : (uint32_t)first, ph = first == ns ? 0 : 1;
@@ -185,6 +190,9 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   } else {                                          // warps 2-6
     bool ok = true;
     if (norm) {
+      for (int i = tid - 64; i < nk * (BK / 8); i += 32 * kScaleWarps)
+        reinterpret_cast<uint4*>(gamma_s)[i] = *reinterpret_cast<const uint4*>(g.gamma + kb0 * BK + i * 8);
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * kScaleWarps) : "memory");
       // a warp scales whole stages, always the same ones of the ring, so that it sees every phase of their barriers; lane l
       // owns 16-byte chunk l % 8 of rows l / 8 + 4 i, so its eight gammas are the same for all of them.  Four chunks are
       // loaded before the first is worked on.
@@ -418,6 +426,7 @@ int launch_gemm_splitk(const TcOperand& X, const TcOperand& W, const TcEpilogue&
   g.gamma = (const __nv_bfloat16*)ep.rms_gamma; g.eps = ep.rms_eps; g.invK = 1.0f / (float)K;
   g.out = (__nv_bfloat16*)ep.out; g.ldc = ep.ldc;
   g.bias = (const __nv_bfloat16*)ep.bias; g.residual = (const __nv_bfloat16*)ep.residual; g.gelu = ep.gelu;
+  g.w_settled = ep.b_settled;
   g.has_rowmap = ep.rowmap ? 1 : 0;
   if (ep.rowmap) g.rowmap = *ep.rowmap;
   const int rope_dim = ep.rope_dim ? ep.rope_dim : 128;

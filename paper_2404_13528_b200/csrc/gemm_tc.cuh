@@ -45,6 +45,9 @@ struct TcEpilogue {
   // RMSNorm of A's rows inside the GEMM (null: none): gamma [K].  Few rows only (gemm_splitk.cu).
   const void* rms_gamma;
   float rms_eps;
+  // Non-zero: nothing in flight writes B -- parameters of a layer call, in a kernel that follows another one of the same call, which has
+  // waited for whatever preceded the call.  The few-row kernel then fetches B before its dependency wait.
+  int b_settled;
 };
 
 int tc_operand_from_map(const smartmem_index_map_t& m, int n_batch_atoms, int n_row_atoms, const void* ptr,
@@ -90,25 +93,25 @@ int tc_cluster_ctas(int size);
 bool mlp_fused_supported(long long C, long long hidden);
 int launch_mlp_fused(const void* A, const void* ln_gamma, const void* ln_beta, float ln_eps, const void* W1, const void* b1,
                      const void* W2, const void* b2, void* out, long long M, long long C, long long hidden,
-                     cudaStream_t st);
+                     bool settled, cudaStream_t st);
 
 // The same for few rows where the weights do not fit one SM: the hidden features split over a cluster (gemm_mlp_cluster.cu).
 // mlp_cluster_wins: it covers the shape and beats the separate kernels.
 bool mlp_cluster_wins(long long M, long long C, long long hidden);
 int launch_mlp_cluster(const void* x, const void* ln_g, const void* ln_b, float eps, const void* W1, const void* b1, const void* W2,
-                       const void* b2, void* out, long long M, long long C, long long hidden, cudaStream_t st);
+                       const void* b2, void* out, long long M, long long C, long long hidden, bool settled, cudaStream_t st);
 
 // LayerNorm o row-gather o linear for narrow rows: out[m, :] = LN(X[src(m), :]) W^T + bias, with X rows of
 // K in {64, 96} elements, W [N, K], N a multiple of 96 (at most 288).  `rowmap` (null: identity) gives
 // the element offset of consumer row m in X; gamma/beta null: no normalisation (plain gather).
 bool gemm_ln_supported(long long N, long long K);
 int launch_gemm_ln(const void* X, const DevMap* rowmap, const void* gamma, const void* beta, float eps, const void* W,
-                   const void* bias, void* out, long long M, long long N, long long K, cudaStream_t st);
+                   const void* bias, void* out, long long M, long long N, long long K, bool settled, cudaStream_t st);
 // The same, with an optional GELU, for few rows of 128, 192 or 256 elements (gemm_ln_wave.cu).  gemm_ln_wave_wins: it covers the shape and
-// beats the separate kernels.
+// beats the separate kernels.  w_settled: as TcEpilogue::b_settled, for W.
 bool gemm_ln_wave_wins(long long M, long long N, long long K);
 int launch_gemm_ln_wave(const void* X, const DevMap* rowmap, const void* gamma, const void* beta, float eps, const void* W, const void* bias,
-                        int gelu, void* out, long long M, long long N, long long K, cudaStream_t st);
+                        int gelu, void* out, long long M, long long N, long long K, bool w_settled, cudaStream_t st);
 // LayerNorm o gather o linear without bias for rows of 256, 384 or 512 elements, gathered in 16-byte vectors through a map over
 // [M, K] without rolls (gemm_ln_pair.cu; SMARTMEM_ERR_UNSUPPORTED where the map does not split into rows).  out may not overlap X.
 bool gemm_ln_pair_wins(const smartmem_index_map_t& map, long long M, long long N, long long K);

@@ -122,6 +122,7 @@ EXPORT int smartmem_attn_layer(const smartmem_attn_params_t* pp, const void* x, 
     memset(&ep, 0, sizeof(ep));
     ep.out = at(L.qkv);
     ep.ldc = 3 * hid;
+    ep.b_settled = 1;
     if (elim) { ep.rope_cols = (int)(2 * hid); ep.rope_S = (int)S; ep.rope_log2_theta = log2f(p.rope_theta); ep.rope_dim = rot; }
     SM_TRY(launch_gemm_tc(tc_operand_plain(at(L.xn), M, hid, hid), tc_operand_plain(p.w_qkv, 3 * hid, hid, hid), ep, 1, M,
                           3 * hid, hid, st));
@@ -158,6 +159,7 @@ EXPORT int smartmem_attn_layer(const smartmem_attn_params_t* pp, const void* x, 
     ep.out = y;
     ep.ldc = hid;
     ep.residual = p.add_residual ? x : nullptr;
+    ep.b_settled = 1;
     SM_TRY(launch_gemm_tc(tc_operand_plain(proj_in, M, hid, hid), tc_operand_plain(p.w_o, hid, hid, hid), ep, 1, M, hid,
                           hid, st));
   }

@@ -69,12 +69,12 @@ __device__ __forceinline__ void gemm_any(const float* A, int pa, const float* W,
   else tile_gemm<2, 2>(A, pa, W, pw, M, N, K, epi);
 }
 
-// rows [0, n) of `cols` floats from global memory (row r at src(r)) into shared memory with pitch `pitch`
+// rows [0, n) of `vpr.d` 16-byte vectors from global memory (row r at src(r)) into shared memory with pitch `pitch`
 template <typename Src>
-__device__ __forceinline__ void load_rows(float* dst, int pitch, int n, int cols, Src src) {
-  const int vpr = cols / 4;
-  for (int i = threadIdx.x; i < n * vpr; i += kThreads) {
-    const int r = i / vpr, v = i - r * vpr;
+__device__ __forceinline__ void load_rows(float* dst, int pitch, int n, const FastDiv& vpr, Src src) {
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n * (int)vpr.d; i += kThreads) {
+    const int r = (int)fd_div((uint32_t)i, vpr), v = i - r * (int)vpr.d;
     ptx::cp_async16(dst + r * pitch + v * 4, src(r) + v * 4);
   }
 }
@@ -103,6 +103,7 @@ struct AttnF32Args {
   float* y;
   int C, heads, d, T, ws, shift, H, W, nWw, win_per_img;
   float eps, scale;
+  FastDiv fd_vpr, fd_d;                                // vectors of a row, head dimension
   int tp;                                              // pitch of P and of v transposed: T rounded up to an odd number of vectors
   DevMap rowmap;
 };
@@ -123,21 +124,27 @@ __global__ void __launch_bounds__(kThreads) swin_attn_f32_kernel(const __grid_co
   const int n = (int)blockIdx.x / g.heads;             // window
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-  // parameters only: weights of this head, its bias column, the rows' offsets
-  for (int which = 0; which < 3; ++which)
-    load_rows(wq + which * d * pc, pc, d, C, [&](int r) { return g.w_qkv + (size_t)(which * C + h * d + r) * C; });
-  load_rows(wp, pc, d, C, [&](int r) { return g.w_proj + (size_t)(h * d + r) * C; });
-  ptx::cp_async_commit();
-  const int nt = (2 * g.ws - 1) * (2 * g.ws - 1);
-  for (int i = tid; i < nt; i += kThreads) tab[i] = g.table[i * g.heads + h];
+  // The head's weights as far as L2: they may still be written by the kernel before this one.  (A line per 32 floats of a head's rows,
+  // which lie one behind the other.)
+  for (int i = tid * 32; i < d * C; i += kThreads * 32) {
+    for (int which = 0; which < 3; ++which) ptx::prefetch_l2(g.w_qkv + (size_t)(which * C + h * d) * C + i);
+    ptx::prefetch_l2(g.w_proj + (size_t)h * d * C + i);
+  }
   for (int i = tid; i < T; i += kThreads) offs[i] = devmap_eval(g.rowmap, (uint32_t)(n * T + i));
   for (int i = tid; i < d * tp; i += kThreads) vt[i] = 0.f;
   for (int i = tid; i < T * tp; i += kThreads) P[i] = 0.f;
   __syncthreads();
   pdl_wait();
   pdl_launch_dependents();
-  load_rows(xs, pc, T, C, [&](int r) { return g.x + offs[r]; });
+  load_rows(xs, pc, T, g.fd_vpr, [&](int r) { return g.x + offs[r]; });
+  // (rows of q, k, v and of the projection lie one behind the other in shared memory)
+  load_rows(wq, pc, 4 * d, g.fd_vpr, [&](int r) {
+    const int which = (int)fd_div((uint32_t)r, g.fd_d), e = h * d + r - which * d;
+    return which < 3 ? g.w_qkv + (size_t)(which * C + e) * C : g.w_proj + (size_t)e * C;
+  });
   ptx::cp_async_commit();
+  const int nt = (2 * g.ws - 1) * (2 * g.ws - 1);
+  for (int i = tid; i < nt; i += kThreads) tab[i] = g.table[i * g.heads + h];
   ptx::cp_async_wait<0>();
   __syncthreads();
   norm_rows(xs, pc, T, C, g.ln_g, g.ln_b, g.eps);
@@ -193,6 +200,7 @@ struct MlpF32Args {
   float* y;
   int M, C, hidden, slice, splits;
   float eps;
+  FastDiv fd_vpr, fd_vps;                              // vectors of a row, of a slice
 };
 constexpr int kMlpRows = 16;
 
@@ -206,12 +214,12 @@ __global__ void __launch_bounds__(kThreads) swin_mlp_f32_kernel(const MlpF32Args
   float* part = hid + kMlpRows * ph;                   // [16][C]: this slice's share of fc2
   const int rank = g.splits > 1 ? (int)ptx::cluster_ctarank() : 0;
   const int m0 = (int)blockIdx.x / g.splits * kMlpRows, rows = min(kMlpRows, g.M - m0);
-  load_rows(w1, pc, hs, C, [&](int r) { return g.w1 + (size_t)(rank * hs + r) * C; });
-  load_rows(w2, ph, C, hs, [&](int r) { return g.w2 + (size_t)r * g.hidden + rank * hs; });
+  load_rows(w1, pc, hs, g.fd_vpr, [&](int r) { return g.w1 + (size_t)(rank * hs + r) * C; });
+  load_rows(w2, ph, C, g.fd_vps, [&](int r) { return g.w2 + (size_t)r * g.hidden + rank * hs; });
   ptx::cp_async_commit();
   pdl_wait();
   pdl_launch_dependents();
-  load_rows(xs, pc, rows, C, [&](int r) { return g.x + (size_t)(m0 + r) * C; });
+  load_rows(xs, pc, rows, g.fd_vpr, [&](int r) { return g.x + (size_t)(m0 + r) * C; });
   ptx::cp_async_commit();
   ptx::cp_async_wait<0>();
   __syncthreads();
@@ -274,6 +282,8 @@ int launch_swin_attn_f32(const smartmem_swin_params_t& p, const DevMap& rowmap, 
   g.nWw = p.W / p.window; g.win_per_img = g.nWw * (p.H / p.window);
   g.eps = p.ln_eps; g.scale = 1.0f / sqrtf((float)g.d);
   g.tp = pitch_of(g.T);
+  g.fd_vpr = make_fastdiv((uint32_t)g.C / 4);
+  g.fd_d = make_fastdiv((uint32_t)g.d);
   g.rowmap = rowmap;
   const long long ctas = (long long)p.B * g.win_per_img * p.heads;
   if (ctas >= (1ll << 31) || (long long)p.B * p.H * p.W >= (1ll << 31)) return SMARTMEM_ERR_UNSUPPORTED;
@@ -285,7 +295,7 @@ int launch_swin_attn_f32(const smartmem_swin_params_t& p, const DevMap& rowmap, 
   return SMARTMEM_OK;
 }
 
-int launch_swin_mlp_f32(const smartmem_swin_params_t& p, const void* x, void* y, long long M, cudaStream_t st) {
+int launch_swin_mlp_f32(const smartmem_swin_params_t& p, const void* x, void* y, long long M, bool settled, cudaStream_t st) {
   MlpF32Args g;
   memset(&g, 0, sizeof(g));
   g.x = (const float*)x; g.y = (float*)y;
@@ -295,12 +305,14 @@ int launch_swin_mlp_f32(const smartmem_swin_params_t& p, const void* x, void* y,
   g.splits = mlp_f32_splits(g.C, g.hidden);
   if (g.splits == 0) return SMARTMEM_ERR_UNSUPPORTED;
   g.slice = g.hidden / g.splits;
+  g.fd_vpr = make_fastdiv((uint32_t)g.C / 4);
+  g.fd_vps = make_fastdiv((uint32_t)g.slice / 4);
   const long long ctas = (M + kMlpRows - 1) / kMlpRows * g.splits;
   if (ctas >= (1ll << 31)) return SMARTMEM_ERR_UNSUPPORTED;
   const size_t smem = mlp_f32_smem(g.C, g.slice);
   if (ensure_max_dynamic_smem((const void*)swin_mlp_f32_kernel, (int)kMaxSmem) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   profile_tick("swin_mlp_f32", st);
-  if (launch_pdl_cluster(swin_mlp_f32_kernel, dim3((unsigned)ctas), dim3(kThreads), smem, st, (unsigned)g.splits, g) != cudaSuccess) return SMARTMEM_ERR_CUDA;
+  if (launch_cluster(swin_mlp_f32_kernel, dim3((unsigned)ctas), dim3(kThreads), smem, st, (unsigned)g.splits, settled, g) != cudaSuccess) return SMARTMEM_ERR_CUDA;
   count_launch();
   return SMARTMEM_OK;
 }
