@@ -149,7 +149,8 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
   uint64_t *y_full = buf_free + NBUF, *y_empty = y_full + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(y_empty + 1);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
-  uint16_t* raw_s = reinterpret_cast<uint16_t*>(sKV);              // prologue scratch: the raw table columns, [NH][256]
+  // prologue scratch: a head's raw table column (256 entries), over its own group's k tile
+  auto raw_of = [&](int h) { return reinterpret_cast<uint16_t*>(sKV + h * KV_SLOT); };
 
   if (pad + (uint32_t)(reinterpret_cast<uint8_t*>(tmem_slot + 4) - smem) > g.smem_bytes) {
     if (threadIdx.x == 0) atomicExch(g.status, (int)SMARTMEM_ERR_UNSUPPORTED);
@@ -258,7 +259,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
   }
 #pragma unroll
   for (int k = 0; k < 2; ++k)
-    if (tid + k * kThreads < NH * 256) raw_s[tid + k * kThreads] = tab[k];
+    if (tid + k * kThreads < NH * 256) raw_of((tid + k * kThreads) >> 8)[(tid + k * kThreads) & 255] = tab[k];
   if (tid < C) {
     lng_s[tid] = par[0];
     ln_s[tid] = __bfloat162float(par[1]);
@@ -423,11 +424,11 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
     const uint32_t* brow = bias_s + (gi * T + (i < T ? i : 0)) * BR;
     const f32x2 scale2 = ptx::pack2(g.scale, g.scale), log2e2 = ptx::pack2(LOG2E, LOG2E);
     // This head's bias as a [T, T] table of bf16 pairs, -inf for the padded keys, built by the group itself while the first unit's
-    // rows are on their way (a task = a quarter of a row).  The first group barrier below orders it before the first softmax.
+    // rows are on their way (a task = a quarter of a row).  The barrier behind it: the raw column lies where the group's first k rows go.
     for (int task = (warp - 4 - 4 * gi) * 32 + lane; task < T * 4; task += 128) {
       const int r = task >> 2, qtr = task & 3;                        // row, quarter of the row's key pairs
       const int ry = tyx_s[r] >> 8, rx = tyx_s[r] & 255;
-      const uint16_t* tab = raw_s + gi * 256 + (ry + ws - 1) * (2 * ws - 1) + (rx + ws - 1);
+      const uint16_t* tab = raw_of(gi) + (ry + ws - 1) * (2 * ws - 1) + (rx + ws - 1);
 #pragma unroll 1
       for (int c2 = qtr * (KC / 8); c2 < (qtr + 1) * (KC / 8); ++c2) {
         uint32_t word = 0;
@@ -457,6 +458,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
           : "memory");
       return gave_up != 0;
     };
+    group_sync();
     for (int ul = 0; ul < U; ++ul) {
       const int it = ul * NH + gi;
       const int ab = ul % na;

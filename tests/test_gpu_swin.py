@@ -174,3 +174,24 @@ def test_block_halves_compose_to_the_block(cfg):
     with pytest.raises(sm.SmartmemError) as e:
         sm.smartmem_swin_block_half(p, dev["x"].data_ptr(), out.data_ptr(), ws.data_ptr(), n, sm.ELIMINATE, 2, stream())
     assert e.value.code == sm.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("C,heads", [(64, 2), (96, 3)])
+def test_fused_attention_half_bias_of_every_cta(C, heads):
+    """The same image 148 times, a bias that decides the softmax: whichever CTA builds a head's bias table (from scratch memory that its
+    first keys take over), every image comes out bit for bit the same, and as the oracle has it."""
+    B, H, W = 148, 14, 14
+    inp = synth.swin_inputs(24, 1, H, W, C, heads, 7, 0, "bf16")
+    dev = {k: to_dev(v) for k, v in inp.items()}
+    table = (100 * dev["rel_bias_table"].float()).bfloat16()          # std 2
+    dev["rel_bias_table"] = table
+    pf = {k: synth.to_f64(v) for k, v in inp.items() if k not in ("x", "rel_bias_table")}
+    pf["rel_bias_table"] = to_host_f64(table)
+    ref = oswin.swin_block(synth.to_f64(inp["x"]), pf, heads=heads, window=7, shift=3, mlp_ratio=0)
+    x = dev["x"].repeat(B, 1, 1, 1)
+    first = None
+    for _ in range(10):
+        y = run_block(inp, dev, B=B, H=H, W=W, C=C, heads=heads, window=7, shift=3, mlp_ratio=0, dtype="bf16", mode=sm.ELIMINATE, x_dev=x)
+        first = y[:1].clone() if first is None else first
+        assert torch.equal(y, first.expand_as(y))
+    assert_close_bf16(to_host_f64(first), ref, "one image")
