@@ -446,8 +446,8 @@ EXPORT int smartmem_attn_decode(const smartmem_attn_params_t* pp, int32_t pos, c
   __nv_bfloat16* vc = (__nv_bfloat16*)v_cache;
 
 #define SM_TRY(expr) do { rc = (expr); if (rc != SMARTMEM_OK) return rc; } while (0)
-  // few rows: RMSNorm rides along in the QKV GEMM
-  const bool norm_in_gemm = B <= 128;
+  // few rows: RMSNorm rides along in the QKV GEMM, where its share of gamma fits (hidden up to 27392 at B = 49..64, more at others)
+  const bool norm_in_gemm = B <= 128 && gemm_splitk_norm_fits(B, 3 * hid, hid);
   if (!norm_in_gemm) SM_TRY(launch_norm(SMARTMEM_BF16, true, x, at(L.xn), p.rms_g, nullptr, p.rms_eps, B, (int)hid, nullptr, st));
   DecodeAttnArgs a;
   memset(&a, 0, sizeof(a));

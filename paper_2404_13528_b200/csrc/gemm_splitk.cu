@@ -360,6 +360,55 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   }
 }
 
+// Sizes of a launch; returns the bytes of shared memory, 0 if a CTA's part does not fit (with RMSNorm: gamma of its K range lies beside
+// the rings).
+size_t plan_launch(long long M, long long N, long long K, bool norm, SplitArgs& g) {
+  // row tiles of at most 256 rows and at most 15 rows of padding each
+  g.tiles_m = (int)((M + 255) / 256);
+  g.NB = (int)(((M + g.tiles_m - 1) / g.tiles_m + 15) / 16 * 16);
+  if (norm && g.NB > kMaxNormRows) return 0;
+  g.nkb = (int)(K / BK);
+  const long long tiles = (N + BN_W - 1) / BN_W * g.tiles_m;
+  g.x_bytes = (uint32_t)(g.NB * BK * 2);
+  // Two CTAs per SM where X is narrow enough to leave each a ring of four or more stages of W.  As many splits as there are
+  // CTA slots for: a second wave of clusters costs more than the shorter K ranges gain (N = 12288, K = 4096, 96 tiles:
+  // 18.8 us in clusters of 2, 24 us in clusters of 3, 135 of which do not fit).
+  const int per_sm = g.NB <= 64 ? 2 : 1;
+  int splits = 1;
+  for (int s = 2; s <= kMaxSplits && s <= g.nkb; ++s)
+    if (tiles * s <= (long long)per_sm * tc_cluster_ctas(s)) splits = s;
+  g.splits = splits;
+  const int nk_max = (g.nkb + splits - 1) / splits;
+  const uint32_t gamma_bytes = norm ? (uint32_t)(nk_max * BK * 2) : 0u;
+  const uint32_t rows_bytes = (uint32_t)g.NB * 12u + (norm ? (uint32_t)(kScaleWarps * g.NB * 4) : 0u);
+  const uint32_t bar_bytes = (2 * kMaxStages + 3 * kMaxXStages + 1) * 8 + 16;
+  const uint32_t space = (per_sm == 2 ? 113u : 226u) * 1024u, fixed = 1024u + gamma_bytes + rows_bytes + bar_bytes + 32;
+  if (space < fixed) return 0;
+  const uint32_t budget = space - fixed;
+  // X comes from L2 and needs less depth than W: a quarter of the space, but three stages at least, and one for each scaling
+  // warp
+  const int min_x = norm ? kScaleWarps : 3;
+  int xstages = (int)(budget / 4 / g.x_bytes);
+  xstages = xstages > kMaxXStages ? kMaxXStages : xstages < min_x ? min_x : xstages;
+  if (xstages > nk_max) xstages = nk_max;
+  if (budget < xstages * g.x_bytes + W_STAGE) return 0;
+  int stages = (int)((budget - xstages * g.x_bytes) / W_STAGE);
+  if (stages > kMaxStages) stages = kMaxStages;
+  if (stages > nk_max) stages = nk_max;
+  const uint32_t acc_bytes = (uint32_t)g.NB * BN_W * 4;              // the fp32 tile lies over the drained rings
+  uint32_t ring = stages * W_STAGE + xstages * g.x_bytes;
+  if (ring < acc_bytes) ring = (acc_bytes + 1023) / 1024 * 1024;
+  if (ring > budget) return 0;
+  g.stages = stages;
+  g.xstages = xstages;
+  g.x_off = stages * W_STAGE;
+  g.gamma_off = (int)ring;
+  g.table_off = (g.gamma_off + (int)gamma_bytes + 15) & ~15;
+  g.bar_off = (g.table_off + (int)rows_bytes + 15) & ~15;
+  g.tmem_cols = g.NB <= 32 ? 32 : g.NB <= 64 ? 64 : g.NB <= 128 ? 128 : 256;
+  return 1024 + g.bar_off + bar_bytes;
+}
+
 }  // namespace
 
 bool gemm_splitk_supported(const TcOperand& X, const TcOperand& W, const TcEpilogue& ep, long long batch, long long M, long long N,
@@ -377,51 +426,16 @@ double gemm_splitk_us(long long M, long long N, long long K) {
   return M > 128 ? 1e30 : M < 32 ? 0.0 : 3.0 + 0.018 * nb + (double)N * (double)K * 2.0 / 6.2e6 * (1.0 + nb / 260.0);
 }
 
+bool gemm_splitk_norm_fits(long long M, long long N, long long K) {
+  SplitArgs g;
+  return M >= 1 && K % BK == 0 && plan_launch(M, N, K, true, g) != 0;
+}
+
 int launch_gemm_splitk(const TcOperand& X, const TcOperand& W, const TcEpilogue& ep, long long M, long long N, long long K, cudaStream_t st) {
   SplitArgs g;
   memset(&g, 0, sizeof(g));
-  // row tiles of at most 256 rows and at most 15 rows of padding each
-  g.tiles_m = (int)((M + 255) / 256);
-  g.NB = (int)(((M + g.tiles_m - 1) / g.tiles_m + 15) / 16 * 16);
-  if (ep.rms_gamma && g.NB > kMaxNormRows) return SMARTMEM_ERR_UNSUPPORTED;
-  g.nkb = (int)(K / BK);
-  const long long tiles = (N + BN_W - 1) / BN_W * g.tiles_m;
-  g.x_bytes = (uint32_t)(g.NB * BK * 2);
-  // Two CTAs per SM where X is narrow enough to leave each a ring of four or more stages of W.  As many splits as there are
-  // CTA slots for: a second wave of clusters costs more than the shorter K ranges gain (N = 12288, K = 4096, 96 tiles:
-  // 18.8 us in clusters of 2, 24 us in clusters of 3, 135 of which do not fit).
-  const int per_sm = g.NB <= 64 ? 2 : 1;
-  int splits = 1;
-  for (int s = 2; s <= kMaxSplits && s <= g.nkb; ++s)
-    if (tiles * s <= (long long)per_sm * tc_cluster_ctas(s)) splits = s;
-  g.splits = splits;
-  const int nk_max = (g.nkb + splits - 1) / splits;
-  const uint32_t gamma_bytes = ep.rms_gamma ? (uint32_t)(nk_max * BK * 2) : 0u;
-  const uint32_t rows_bytes = (uint32_t)g.NB * 12u + (ep.rms_gamma ? (uint32_t)(kScaleWarps * g.NB * 4) : 0u);
-  const uint32_t bar_bytes = (2 * kMaxStages + 3 * kMaxXStages + 1) * 8 + 16;
-  const uint32_t budget = (per_sm == 2 ? 113u : 226u) * 1024u - 1024u - gamma_bytes - rows_bytes - bar_bytes - 32;
-  // X comes from L2 and needs less depth than W: a quarter of the space, but three stages at least, and one for each scaling
-  // warp
-  const int min_x = ep.rms_gamma ? kScaleWarps : 3;
-  int xstages = (int)(budget / 4 / g.x_bytes);
-  xstages = xstages > kMaxXStages ? kMaxXStages : xstages < min_x ? min_x : xstages;
-  if (xstages > nk_max) xstages = nk_max;
-  if (budget < xstages * g.x_bytes + W_STAGE) return SMARTMEM_ERR_UNSUPPORTED;
-  int stages = (int)((budget - xstages * g.x_bytes) / W_STAGE);
-  if (stages > kMaxStages) stages = kMaxStages;
-  if (stages > nk_max) stages = nk_max;
-  const uint32_t acc_bytes = (uint32_t)g.NB * BN_W * 4;              // the fp32 tile lies over the drained rings
-  uint32_t ring = stages * W_STAGE + xstages * g.x_bytes;
-  if (ring < acc_bytes) ring = (acc_bytes + 1023) / 1024 * 1024;
-  if (ring > budget) return SMARTMEM_ERR_UNSUPPORTED;
-  g.stages = stages;
-  g.xstages = xstages;
-  g.x_off = stages * W_STAGE;
-  g.gamma_off = (int)ring;
-  g.table_off = (g.gamma_off + (int)gamma_bytes + 15) & ~15;
-  g.bar_off = (g.table_off + (int)rows_bytes + 15) & ~15;
-  const size_t smem = 1024 + g.bar_off + bar_bytes;
-  g.tmem_cols = g.NB <= 32 ? 32 : g.NB <= 64 ? 64 : g.NB <= 128 ? 128 : 256;
+  const size_t smem = plan_launch(M, N, K, ep.rms_gamma != nullptr, g);
+  if (smem == 0) return SMARTMEM_ERR_UNSUPPORTED;
   g.M = (int)M; g.N = (int)N;
   g.gamma = (const __nv_bfloat16*)ep.rms_gamma; g.eps = ep.rms_eps; g.invK = 1.0f / (float)K;
   g.out = (__nv_bfloat16*)ep.out; g.ldc = ep.ldc;
@@ -442,7 +456,8 @@ int launch_gemm_splitk(const TcOperand& X, const TcOperand& W, const TcEpilogue&
   if (rc != SMARTMEM_OK) return rc;
   if (ensure_max_dynamic_smem((const void*)gemm_splitk_kernel, 227 * 1024) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   profile_tick("gemm_splitk", st);
-  if (launch_pdl_cluster(gemm_splitk_kernel, dim3((unsigned)(tiles * splits)), dim3(kThreads), smem, st, (unsigned)splits, tw, tx, g) != cudaSuccess)
+  const unsigned grid = (unsigned)((N + BN_W - 1) / BN_W * g.tiles_m * g.splits);
+  if (launch_pdl_cluster(gemm_splitk_kernel, dim3(grid), dim3(kThreads), smem, st, (unsigned)g.splits, tw, tx, g) != cudaSuccess)
     return SMARTMEM_ERR_CUDA;
   count_launch();
   return SMARTMEM_OK;

@@ -61,6 +61,8 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
 bool gemm_splitk_supported(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep, long long batch, long long M, long long N,
                            long long K);
 double gemm_splitk_us(long long M, long long N, long long K);
+// Whether the kernel takes these sizes with RMSNorm inside (TcEpilogue::rms_gamma): few rows, and room for a CTA's share of gamma.
+bool gemm_splitk_norm_fits(long long M, long long N, long long K);
 int launch_gemm_splitk(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep, long long M, long long N, long long K, cudaStream_t st);
 
 // bf16 row-major [outer, inner] matrix as a 2-D tensor map with 128-byte swizzle (box_inner = 64).

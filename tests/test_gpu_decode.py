@@ -132,3 +132,32 @@ def test_decode_rejects_bad_arguments():
     with pytest.raises(sm.SmartmemError) as e:        # no such mode for this entry point
         run_decode(dev, kc, vc, B=2, pos=3, s_max=8, hidden=256, heads=2, add_residual=0, mode=sm.ELIMINATE_NAIVE)
     assert e.value.code == sm.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("B,hidden", [
+    (49, 27392), (49, 27648),        # the widest layer whose RMSNorm fits the QKV GEMM of four 16-row steps, and the next
+    (1, 43776),                      # the same for one row
+])
+def test_widest_layers(B, hidden):
+    """At position 0 the attention's output is the new value row, so fp32 products on the device are the reference."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(46)
+
+    def normal(*shape, std, mean=0.0):
+        return torch.empty(shape, dtype=torch.bfloat16, device="cuda").normal_(mean, std, generator=gen)
+
+    dev = dict(x=normal(B, hidden, std=1.0), rms_g=normal(hidden, std=0.02, mean=1.0), w_qkv=normal(3 * hidden, hidden, std=hidden ** -0.5),
+               w_o=normal(hidden, hidden, std=hidden ** -0.5))
+    kc, vc = (torch.full((B, 2, hidden // 128, 128), float("nan"), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+    y = run_decode(dev, kc, vc, B=B, pos=0, s_max=2, hidden=hidden, heads=hidden // 128, add_residual=0, mode=sm.ELIMINATE)
+    x = dev["x"].float()
+    xn = x * torch.rsqrt((x * x).mean(-1, keepdim=True) + 1e-5) * dev["rms_g"].float()
+
+    def product(a, w):
+        return torch.cat([a @ part.float().T for part in w.split(4096)], dim=1)
+
+    for name, cache, rows in (("k", kc, slice(hidden, 2 * hidden)), ("v", vc, slice(2 * hidden, 3 * hidden))):
+        ref = product(xn, dev["w_qkv"][rows])                  # (rotated by position 0: as it is)
+        assert_close_bf16(to_host_f64(cache[:, 0]).reshape(B, hidden), ref.double().cpu().numpy(), name)
+    ref = product(vc[:, 0].reshape(B, hidden).float(), dev["w_o"])
+    assert_close_bf16(to_host_f64(y), ref.double().cpu().numpy(), "y")
