@@ -317,8 +317,8 @@ int smartmem_attn_layer(const smartmem_attn_params_t* p, const void* x, void* y,
  *   SMARTMEM_EXPLICIT   [B, heads, S_max, head_dim]  -- the per-head layout of the materialised
  *       chain: plain QKV GEMM, head-split copy, stand-alone rotary pass, append copy into the cache,
  *       attention on contiguous per-head tensors.
- * head_dim must be 128, hidden a multiple of 256, pos + 1 <= 16384; otherwise
- * SMARTMEM_ERR_UNSUPPORTED.  Errors as for smartmem_attn_layer. */
+ * head_dim must be 128, hidden a multiple of 256, pos + 1 <= 16384, and a cache must have fewer than 2^31 rows
+ * (ELIMINATE: B * S_max, EXPLICIT: B * heads * S_max); otherwise SMARTMEM_ERR_UNSUPPORTED.  Errors as for smartmem_attn_layer. */
 int smartmem_attn_decode_workspace_bytes(const smartmem_attn_params_t* p, int32_t mode, size_t* bytes);
 int smartmem_attn_decode(const smartmem_attn_params_t* p, int32_t pos, const void* x, void* k_cache, void* v_cache,
                          void* y, void* workspace, size_t workspace_bytes, int32_t mode, void* cuda_stream);

@@ -426,7 +426,8 @@ EXPORT int smartmem_attn_decode(const smartmem_attn_params_t* pp, int32_t pos, c
   if (rc != SMARTMEM_OK) return rc;
   const smartmem_attn_params_t& p = *pp;
   if (pos < 0 || pos >= p.S) return SMARTMEM_ERR_SHAPE;
-  if (pos + 1 > DEC_MAX_S || (long long)p.B * p.heads * p.S >= (1ll << 31)) return SMARTMEM_ERR_UNSUPPORTED;
+  // rows of the caches as the attention kernel's tensor maps count them: [B S_max] or [B heads S_max]
+  if (pos + 1 > DEC_MAX_S || (long long)p.B * p.S * (mode == SMARTMEM_ELIMINATE ? 1 : p.heads) >= (1ll << 31)) return SMARTMEM_ERR_UNSUPPORTED;
   if (!x || !y || !k_cache || !v_cache || !workspace || x == y || !p.rms_g || !p.w_qkv || !p.w_o)
     return SMARTMEM_ERR_INVALID_ARG;
   const void* al16[] = {x, y, k_cache, v_cache, workspace, p.rms_g, p.w_qkv, p.w_o};

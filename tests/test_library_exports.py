@@ -3,6 +3,8 @@ import ctypes
 import os
 import re
 
+import pytest
+
 from paper_2404_13528_b200 import binding as sm
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -22,6 +24,20 @@ def test_every_declared_symbol_is_exported_and_bound():
         assert hasattr(L, n), f"{n} declared in smartmem.h but not exported"
         assert n in sm.EXPORTED, f"{n} has no entry in the Python binding"
         assert hasattr(sm, n), f"binding lacks a function named {n}"
+
+
+@pytest.mark.parametrize("mode,B,S,code", [
+    (sm.ELIMINATE, 1, 1 << 30, sm.ERR_WORKSPACE),           # heads do not count: the cache's rows hold all of them
+    (sm.ELIMINATE, 2, 1 << 30, sm.ERR_UNSUPPORTED),
+    (sm.EXPLICIT, 1, 1 << 30, sm.ERR_UNSUPPORTED), (sm.EXPLICIT, 1, (1 << 30) - 1, sm.ERR_WORKSPACE),
+])
+def test_decode_cache_rows_limit(mode, B, S, code):
+    p = sm.AttnParams()
+    p.dtype, p.B, p.S, p.hidden, p.heads, p.head_dim, p.rms_eps, p.rope_theta = sm.BF16, B, S, 256, 2, 128, 1e-5, 1e4
+    p.rms_g = p.w_qkv = p.w_o = 16
+    with pytest.raises(sm.SmartmemError) as e:              # refused on the host, nothing is launched: no workspace is given
+        sm.smartmem_attn_decode(p, 3, 16, 32, 48, 64, 80, 0, mode, 0)
+    assert e.value.code == code
 
 
 def test_host_only_calls_work_without_a_gpu():
