@@ -2,7 +2,8 @@
 
 Argument marshalling only: every step of the hot path runs inside the CUDA library.  The
 functions keep the C names.  The calls a program makes per step go through a small CPython extension
-(csrc/fastcall.c) that converts their arguments without ctypes.  Device buffers are passed as integers (``tensor.data_ptr()``),
+(csrc/fastcall.c) that converts their plain forms without ctypes; everything else, and all calls where the extension could not be
+built, goes through ctypes.  Device buffers are passed as integers (``tensor.data_ptr()``),
 streams as ``torch.cuda.current_stream().cuda_stream``.  If the shared library is missing
 the import of any entry point raises -- there is no fallback.
 """
@@ -131,13 +132,23 @@ def lib() -> C.CDLL:
     return L
 
 
+class _NoFast:
+    """Stands in for the extension where it has not been built: every call goes through ctypes."""
+    swin_block = attn_layer = attn_decode = run_chain = staticmethod(lambda *args: None)
+
+
 def _bind_fast():
-    """Loads _fastcall.so (built next to the library) and hands it the addresses of the per-step calls."""
+    """Loads the extension (built next to the library) and hands it the addresses of the per-step calls and the types of their
+    parameter blocks."""
     global _fast
     L = lib()
-    from . import _fastcall
+    try:
+        from . import _fastcall
+    except ImportError:
+        _fast = _NoFast
+        return _fast
     _fastcall.bind(*(C.cast(getattr(L, n), C.c_void_p).value for n in
-                     ("smartmem_swin_block", "smartmem_attn_layer", "smartmem_attn_decode", "smartmem_run_chain")))
+                     ("smartmem_swin_block", "smartmem_attn_layer", "smartmem_attn_decode", "smartmem_run_chain")), SwinParams, AttnParams)
     _fast = _fastcall
     return _fast
 
@@ -262,6 +273,10 @@ def smartmem_plan_eval_sequential(plan: int, step: int, operand: int, i: int) ->
 def smartmem_run_chain(plan: int, inputs, outputs, workspace: int, workspace_bytes: int, stream: int):
     """inputs / outputs: lists of device pointers (ints)."""
     rc = (_fast or _bind_fast()).run_chain(plan, inputs, outputs, workspace, workspace_bytes, stream)
+    if rc is None:
+        ai = (C.c_void_p * len(inputs))(*inputs)
+        ao = (C.c_void_p * len(outputs))(*outputs)
+        rc = lib().smartmem_run_chain(plan, ai, ao, workspace, workspace_bytes, stream)
     if rc:
         raise SmartmemError(rc, "smartmem_run_chain")
 
@@ -274,6 +289,8 @@ def smartmem_swin_block_workspace_bytes(p: SwinParams, mode: int) -> int:
 
 def smartmem_swin_block(p: SwinParams, x: int, y: int, workspace: int, workspace_bytes: int, mode: int, stream: int):
     rc = (_fast or _bind_fast()).swin_block(p, x, y, workspace, workspace_bytes, mode, stream)
+    if rc is None:
+        rc = lib().smartmem_swin_block(C.byref(p), x, y, workspace, workspace_bytes, mode, stream)
     if rc:
         raise SmartmemError(rc, "smartmem_swin_block")
 
@@ -315,6 +332,8 @@ def smartmem_attn_layer_workspace_bytes(p: AttnParams, mode: int) -> int:
 
 def smartmem_attn_layer(p: AttnParams, x: int, y: int, workspace: int, workspace_bytes: int, mode: int, stream: int):
     rc = (_fast or _bind_fast()).attn_layer(p, x, y, workspace, workspace_bytes, mode, stream)
+    if rc is None:
+        rc = lib().smartmem_attn_layer(C.byref(p), x, y, workspace, workspace_bytes, mode, stream)
     if rc:
         raise SmartmemError(rc, "smartmem_attn_layer")
 
@@ -328,6 +347,8 @@ def smartmem_attn_decode_workspace_bytes(p: AttnParams, mode: int) -> int:
 def smartmem_attn_decode(p: AttnParams, pos: int, x: int, k_cache: int, v_cache: int, y: int, workspace: int,
                          workspace_bytes: int, mode: int, stream: int):
     rc = (_fast or _bind_fast()).attn_decode(p, pos, x, k_cache, v_cache, y, workspace, workspace_bytes, mode, stream)
+    if rc is None:
+        rc = lib().smartmem_attn_decode(C.byref(p), pos, x, k_cache, v_cache, y, workspace, workspace_bytes, mode, stream)
     if rc:
         raise SmartmemError(rc, "smartmem_attn_decode")
 
