@@ -36,8 +36,8 @@ struct LnPairArgs {
 
 template <int NV, int NB>
 constexpr int pair_smem_bytes() {
-  // rows, slice of W, gamma and beta widened, offsets of a row's vectors, barriers
-  return 1024 + NV * kLnBlockBytes + NV * NB * 32 * 128 + NV * 64 * 8 + NV * 8 * 4 + 4 * 8 + 8;
+  // rows, slice of W, gamma and beta widened and as they come, offsets of a row's vectors, barriers
+  return 1024 + NV * kLnBlockBytes + NV * NB * 32 * 128 + NV * 64 * 8 + NV * 64 * 4 + NV * 8 * 4 + 5 * 8 + 8;
 }
 
 template <int NV, int NB, int RW>                  // K / 64, columns of a slice / 64, rows of a tile per warp
@@ -52,10 +52,11 @@ ln_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   uint8_t* sW = sA + NV * kLnBlockBytes;           // [NV][HW x 128 B]
   // gamma and beta, widened once: floats 0-3 of every vector of eight, then floats 4-7 (16 bytes apart for neighbouring lanes)
   float* par = reinterpret_cast<float*>(sW + NV * HW * 128);
-  int* col_s = reinterpret_cast<int*>(par + 2 * K);                  // element offset of each vector inside a row
+  uint4* raw = reinterpret_cast<uint4*>(par + 2 * K);                // vectors of gamma, then of beta
+  int* col_s = reinterpret_cast<int*>(raw + 2 * (K / 8));            // element offset of each vector inside a row
   uint64_t* w_full = reinterpret_cast<uint64_t*>(col_s + NV * 8);
-  uint64_t *a_ready = w_full + 1, *d_full = w_full + 2;              // (a_ready: the even CTA's)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(w_full + 4);
+  uint64_t *a_ready = w_full + 1, *d_full = w_full + 2, *par_full = w_full + 4;      // (a_ready: the even CTA's)
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(w_full + 5);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
 
   const int tid = threadIdx.x, warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0), lane = tid & 31;
@@ -68,6 +69,7 @@ ln_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       ptx::mbar_init(a_ready, 2 * kWorkers);
       ptx::mbar_init(&d_full[0], 1);
       ptx::mbar_init(&d_full[1], 1);
+      ptx::mbar_init(par_full, K / 8);
       *abort_flag = 0;
       ptx::fence_barrier_init();
       ptx::fence_proxy_async();
@@ -155,7 +157,7 @@ ln_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       }
     };
     auto widen_affine = [&](int v) {
-      const uint4 ga = *reinterpret_cast<const uint4*>(g.ln_g + v * 8), be = *reinterpret_cast<const uint4*>(g.ln_b + v * 8);
+      const uint4 ga = raw[v], be = raw[K / 8 + v];
       const float2 g0 = bf16x2_to_float2(ga.x), g1 = bf16x2_to_float2(ga.y), g2 = bf16x2_to_float2(ga.z), g3 = bf16x2_to_float2(ga.w);
       const float2 b0 = bf16x2_to_float2(be.x), b1 = bf16x2_to_float2(be.y), b2 = bf16x2_to_float2(be.z), b3 = bf16x2_to_float2(be.w);
       float4* p = reinterpret_cast<float4*>(par);
@@ -175,7 +177,6 @@ ln_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
                                              [&] { return j > 0 || free(); });
     };
     uint4 x0[J0][V], x1[J1][V];                    // rows being normalised, rows on their way
-    if (first < g.tiles) request(x0, first, 0, row_off);
     if (warp == 0) {                               // all k-blocks of the slice in one copy
       if (ptx::elect_one()) {
         ptx::mbar_expect_tx(w_full, (uint32_t)(HW * K * 2));
@@ -183,12 +184,26 @@ ln_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       }
       __syncwarp();
     }
-    if (tid >= 256 && tid - 256 < K / 8) widen_affine(tid - 256);
-    __syncthreads();
+    // Gamma and beta, requested ahead of the rows; widened under the statistics of the first ones.
+    const bool widens = tid >= 256 && tid - 256 < K / 8;
+    if (widens) {
+      ptx::cp_async16(raw + tid - 256, g.ln_g + (tid - 256) * 8);
+      ptx::cp_async16(raw + K / 8 + tid - 256, g.ln_b + (tid - 256) * 8);
+      ptx::cp_async_commit();
+    }
+    if (first < g.tiles) request(x0, first, 0, row_off);
+    if (widens) {
+      ptx::cp_async_wait<0>();
+      widen_affine(tid - 256);
+      ptx::mbar_arrive(par_full);
+    }
     int it = 0;
     for (int t = first; t < g.tiles; t += g.pairs, ++it) {
       request(x1, t, 4, row_off);
-      normalise(x0, 0, [&] { return it == 0 ? ok : product_done(it - 1); });
+      normalise(x0, 0, [&] {
+        if (it > 0) return product_done(it - 1);
+        return ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(par_full, 0, abort_flag, g.status) ? 1 : 0) != 0;
+      });
       if (t + g.pairs < g.tiles) {
         row_off = offset_of(t + g.pairs);
         request(x0, t + g.pairs, 0, row_off);
