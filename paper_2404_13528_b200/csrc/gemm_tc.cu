@@ -920,7 +920,7 @@ int tc_operand_from_map(const smartmem_index_map_t& m, int n_batch_atoms, int n_
                         TcOperand* op) {
   if (m.klass == 3 || m.n_rolls > 0) return SMARTMEM_ERR_UNSUPPORTED;
   const int nk = m.n_atoms - n_batch_atoms - n_row_atoms;
-  if (nk != 1 || n_row_atoms < 1 || n_row_atoms > 3 || n_batch_atoms > 3) return SMARTMEM_ERR_UNSUPPORTED;
+  if (nk != 1 || n_row_atoms < 0 || n_row_atoms > 3 || n_batch_atoms > 3) return SMARTMEM_ERR_UNSUPPORTED;
   memset(op, 0, sizeof(*op));
   op->ptr = (const char*)ptr + m.base * 2;
   op->n_batch_atoms = n_batch_atoms;
@@ -935,6 +935,11 @@ int tc_operand_from_map(const smartmem_index_map_t& m, int n_batch_atoms, int n_
   }
   op->K = m.extent[m.n_atoms - 1];
   op->k_stride = m.src_stride[m.n_atoms - 1];
+  if (n_row_atoms == 0) {                              // one row: the map has no atom for it
+    op->n_row_atoms = 1;
+    op->row_extent[0] = 1;
+    op->row_stride[0] = (op->K + 7) / 8 * 8;
+  }
   return SMARTMEM_OK;
 }
 

@@ -93,3 +93,23 @@ def test_norm_linear_in_one_wave(cfg):
 ])
 def test_merge_in_one_kernel(B, H, W, C):
     patch_merging_case(B, H, W, C)
+
+
+@pytest.mark.parametrize("M,K,N", [
+    (300, 256, 384),                          # three slices of the columns over two tiles
+    (1568, 256, 1280), (1568, 256, 1408),     # ten slices: 70 pairs of 74; eleven are 77: two kernels
+    (9472, 384, 384), (9473, 384, 384),       # two slices, 37 tiles: every pair; a row more
+    (3200, 384, 960),                         # five slices, 13 tiles
+    (6272, 512, 256), (6144, 512, 256),       # rows of 512: 25 tiles, and one tile fewer than a third of the pairs
+    (6272, 512, 384),                         # three slices: two kernels
+    (1, 256, 128), (1, 384, 192), (1, 128, 64),   # one row
+])
+def test_norm_linear_chains(M, K, N):
+    """LayerNorm -> linear, rows as they lie, at the edges of the rule that makes one kernel of them."""
+    x, g, b = synth.normal(506, 0, (M, K), dtype="bf16"), synth.normal(506, 1, (K,), 0.02, 1.0, "bf16"), synth.normal(506, 2, (K,), 0.02, 0.0, "bf16")
+    w = synth.normal(506, 3, (N, K), std=K ** -0.5, dtype="bf16")
+    ops = [sm.make_op(sm.OP_LAYERNORM, side_input=(1, 2), eps=1e-5), sm.make_op(sm.OP_LINEAR, side_input=(3, 0))]
+    out = run_plan(ops, [sm.make_desc(t.shape) for t in (x, g, b, w)], sm.ELIMINATE, [to_dev(t) for t in (x, g, b, w)], (M, N))
+    xf = synth.to_f64(x)
+    xn = (xf - xf.mean(-1, keepdims=True)) / np.sqrt(xf.var(-1, keepdims=True) + 1e-5) * synth.to_f64(g) + synth.to_f64(b)
+    assert_close_bf16(to_host_f64(out), xn @ synth.to_f64(w).T, f"{M} x {K} -> {N}")
