@@ -910,10 +910,41 @@ int tc_encode_2d_blocks(const void* ptr, long long inner, long long outer, long 
 
 int tc_sm_count() { return sm_count(); }
 
+namespace {
+constexpr int kProbeSmem = 120 * 1024;                   // (two of them do not fit an SM)
+__global__ void cluster_probe_kernel() {}                // never launched: asked for its occupancy
+constexpr int kMaxDevices = 64, kMaxCluster = 8;
+std::mutex g_cluster_mu;
+int g_cluster_ctas[kMaxDevices][kMaxCluster + 1];        // 0: not asked yet
+}  // namespace
+
+// How the SMs are dealt out to GPCs differs from board to board, so the device is asked, once per size.  (One with 148 SMs said 148, 148,
+// 135, 132, 130, 132, 105 and 120 for sizes 1 to 8; what stands in where there is no device to ask, for the host-only calls.)
 int tc_cluster_ctas(int size) {
-  // of 148 SMs: cudaOccupancyMaxActiveClusters, one CTA per SM
-  static const int ctas[9] = {0, 148, 148, 135, 132, 130, 132, 105, 120};
-  return ctas[size] * sm_count() / 148;
+  static const int typical[kMaxCluster + 1] = {0, 148, 148, 135, 132, 130, 132, 105, 120};
+  const int guess = typical[size] * sm_count() / 148;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return guess;
+  std::lock_guard<std::mutex> lk(g_cluster_mu);
+  int& known = g_cluster_ctas[dev][size];
+  if (known) return known;
+  if (ensure_max_dynamic_smem((const void*)cluster_probe_kernel, kProbeSmem) != SMARTMEM_OK) return guess;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)size);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = kProbeSmem;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = (unsigned)size;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  int clusters = 0;
+  if (cudaOccupancyMaxActiveClusters(&clusters, cluster_probe_kernel, &cfg) != cudaSuccess || clusters < 1) {
+    cudaGetLastError();                                  // (nothing was launched: the guess serves)
+    return guess;
+  }
+  return known = clusters * size;
 }
 
 int tc_operand_from_map(const smartmem_index_map_t& m, int n_batch_atoms, int n_row_atoms, const void* ptr,

@@ -85,7 +85,7 @@ int tc_encode_2d_blocks(const void* ptr, long long inner, long long outer, long 
 int tc_encode_2d_plain(const void* ptr, long long inner, long long outer, long long pitch_elems, int box_inner, int box_outer,
                        CUtensorMap* out);
 int tc_sm_count();
-// SMs that clusters of `size` (1..8) CTAs, one per SM, fill: a cluster must find its CTAs inside one GPC.
+// SMs of the current device that clusters of `size` (1..8) CTAs, one per SM, fill: a cluster must find its CTAs inside one GPC.
 int tc_cluster_ctas(int size);
 
 // Fused MLP half of a block: out = A + GELU(LN(A) W1^T + b1) W2^T + b2 with the hidden activation and the
