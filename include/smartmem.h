@@ -269,8 +269,9 @@ int smartmem_profile_end(void* cuda_stream, float* kernel_ms, char* kernel_names
  *
  *  - Same arguments, requirements and results as smartmem_swin_block, minus the workspace.
  *  - A block whose intermediates need more than the fixed array (see
- *    smartmem_swin_block_workspace_bytes) is rejected with SMARTMEM_ERR_WORKSPACE
- *    ("workspace too small"); nothing is launched.
+ *    smartmem_swin_block_workspace_bytes) is run by kernels that keep more of them on chip, where
+ *    such kernels exist (an fp32 MLP half whose weights fit a cluster: fp32 sums in another order),
+ *    and otherwise rejected with SMARTMEM_ERR_WORKSPACE ("workspace too small"); nothing is launched.
  *  - The call itself performs no device allocation and frees nothing: no cudaMalloc / cudaFree and
  *    no allocating library routine.  The first call on each device looks up the array's device
  *    address (the device must be current); make that first call before starting any stream

@@ -37,6 +37,7 @@ __device__ __forceinline__ int region_label2(int ty, int tx, int ws, int wy, int
 // `rowmap` (windowed row -> element offset of the token in x and y).
 bool swin_attn_f32_supported(int C, int heads, int window);
 bool swin_mlp_f32_supported(int C, long long hidden);
+bool swin_mlp_f32_wins(long long M, int C, long long hidden);      // supported, and faster than the separate kernels
 int launch_swin_attn_f32(const smartmem_swin_params_t& p, const DevMap& rowmap, const void* x, void* y, cudaStream_t st);
 int launch_swin_mlp_f32(const smartmem_swin_params_t& p, const void* x, void* y, long long M, bool settled, cudaStream_t st);
 

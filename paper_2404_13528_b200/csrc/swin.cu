@@ -93,7 +93,8 @@ struct Path {
   bool mlp_cluster;                // (fuse_mlp) the hidden features split over a cluster
   bool ln2_wave;                   // LN2 + fc1 + GELU in one kernel
 };
-Path choose_path(const smartmem_swin_params_t& p, int mode) {
+// `compact`: a kernel that keeps intermediates on chip also where the kernels that write them are faster.
+Path choose_path(const smartmem_swin_params_t& p, int mode, bool compact) {
   const bool bf16 = p.dtype == SMARTMEM_BF16;
   Path t;
   t.fuse_attn = mode == SMARTMEM_ELIMINATE && (bf16 ? swin_attn_fused_supported(p.dtype, p.C, p.heads, p.window)
@@ -101,7 +102,8 @@ Path choose_path(const smartmem_swin_params_t& p, int mode) {
   t.ln1_wave = bf16 && gemm_ln_wave_wins((long long)p.B * p.H * p.W, 3 * (long long)p.C, p.C);
   t.fuse_ln1 = t.ln1_wave || (bf16 && gemm_ln_supported(3 * (long long)p.C, p.C));
   t.fuse_mlp = p.mlp_ratio > 0 && (bf16 ? mlp_fused_supported(p.C, (long long)p.C * p.mlp_ratio)
-                                        : swin_mlp_f32_supported(p.C, (long long)p.C * p.mlp_ratio));
+                                        : compact ? swin_mlp_f32_supported(p.C, (long long)p.C * p.mlp_ratio)
+                                                  : swin_mlp_f32_wins((long long)p.B * p.H * p.W, p.C, (long long)p.C * p.mlp_ratio));
   t.mlp_cluster = bf16 && p.mlp_ratio > 0 && !t.fuse_mlp && mlp_cluster_wins((long long)p.B * p.H * p.W, p.C, (long long)p.C * p.mlp_ratio);
   t.fuse_mlp = t.fuse_mlp || t.mlp_cluster;
   t.ln2_wave = bf16 && p.mlp_ratio > 0 && !t.fuse_mlp && gemm_ln_wave_wins((long long)p.B * p.H * p.W, (long long)p.C * p.mlp_ratio, p.C);
@@ -109,10 +111,10 @@ Path choose_path(const smartmem_swin_params_t& p, int mode) {
 }
 
 // Only the intermediates the chosen path writes are reserved.
-Layout ws_layout(const smartmem_swin_params_t& p, int mode) {
+Layout ws_layout(const smartmem_swin_params_t& p, int mode, bool compact) {
   const size_t esz = p.dtype == SMARTMEM_F32 ? 4 : 2;
   const size_t MC = al((size_t)p.B * p.H * p.W * p.C * esz);
-  const Path t = choose_path(p, mode);
+  const Path t = choose_path(p, mode, compact);
   Layout L;
   memset(&L, 0, sizeof(L));
   size_t off = 0;
@@ -163,7 +165,7 @@ EXPORT int smartmem_swin_block_workspace_bytes(const smartmem_swin_params_t* p, 
   int rc = validate(p, mode);
   if (rc != SMARTMEM_OK) return rc;
   if (!bytes) return SMARTMEM_ERR_INVALID_ARG;
-  *bytes = ws_layout(*p, mode).total;
+  *bytes = ws_layout(*p, mode, false).total;
   return SMARTMEM_OK;
 }
 
@@ -184,7 +186,7 @@ struct KernelTimer {
 
 // half: -1 the whole block, 0 the attention half only, 1 the MLP half only (x is then the attention half's result)
 int run_block(const smartmem_swin_params_t* pp, const void* x, void* y, void* workspace, size_t workspace_bytes,
-              int32_t mode, void* cuda_stream, KernelTimer* tm, int half = -1) {
+              int32_t mode, void* cuda_stream, KernelTimer* tm, int half = -1, bool compact = false) {
   int rc = validate(pp, mode);
   if (rc != SMARTMEM_OK) return rc;
   if (half < -1 || half > 1 || (half == 1 && pp->mlp_ratio == 0)) return SMARTMEM_ERR_INVALID_ARG;
@@ -201,7 +203,7 @@ int run_block(const smartmem_swin_params_t* pp, const void* x, void* y, void* wo
                         p.ln2_g, p.ln2_b, p.w_fc1, p.b_fc1, p.w_fc2, p.b_fc2};
   for (const void* q : al16)
     if ((uintptr_t)q & 15) return SMARTMEM_ERR_ALIGNMENT;
-  const Layout L = ws_layout(p, mode);
+  const Layout L = ws_layout(p, mode, compact);
   if (workspace_bytes < L.total) return SMARTMEM_ERR_WORKSPACE;
   int ndev = 0;
   if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev < 1) return SMARTMEM_ERR_CUDA;
@@ -213,7 +215,7 @@ int run_block(const smartmem_swin_params_t* pp, const void* x, void* y, void* wo
   const bool f32 = p.dtype == SMARTMEM_F32;
   const int esz = f32 ? 4 : 2;
   const bool elim = mode != SMARTMEM_EXPLICIT;
-  const Path path = choose_path(p, mode);
+  const Path path = choose_path(p, mode, compact);
   const long long C = p.C, nH = p.heads, d = C / nH, ws = p.window, T = ws * ws;
   const long long M = (long long)p.B * p.H * p.W, nW = M / T, hid = C * p.mlp_ratio;
   char* w = (char*)workspace;
@@ -413,8 +415,9 @@ EXPORT int smartmem_swin_block_noalloc(const smartmem_swin_params_t* p, const vo
                                        void* cuda_stream) {
   int rc = validate(p, mode);
   if (rc != SMARTMEM_OK) return rc;
-  if (ws_layout(*p, mode).total > SMARTMEM_STATIC_SCRATCH_BYTES) return SMARTMEM_ERR_WORKSPACE;
+  const bool compact = ws_layout(*p, mode, false).total > SMARTMEM_STATIC_SCRATCH_BYTES;
+  if (compact && ws_layout(*p, mode, true).total > SMARTMEM_STATIC_SCRATCH_BYTES) return SMARTMEM_ERR_WORKSPACE;
   void* scratch = nullptr;
   if ((rc = static_scratch(&scratch)) != SMARTMEM_OK) return rc;
-  return run_block(p, x, y, scratch, SMARTMEM_STATIC_SCRATCH_BYTES, mode, cuda_stream, nullptr);
+  return run_block(p, x, y, scratch, SMARTMEM_STATIC_SCRATCH_BYTES, mode, cuda_stream, nullptr, -1, compact);
 }

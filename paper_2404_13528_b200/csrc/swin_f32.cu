@@ -3,8 +3,9 @@
 //   attention half: y = x + unshift(unpartition(proj(window_attention(qkv(LN1(partition(shift(x))))))))
 //   MLP half:       y = x + fc2(GELU(fc1(LN2(x))))
 //
-// fp32 blocks are small models at small batches: what bounds them is the chain of launches and of latencies inside each, so
-// the seven kernels of the block became two.  A cluster of CTAs shares one unit of work:
+// fp32 blocks are mostly small models at small batches: what bounds them is the chain of launches and of latencies inside each, so
+// the seven kernels of the block became two (the MLP half's where it wins at that size; the attention half's at every size measured, 1
+// to 64 images of 28 x 28 or 56 x 56 x 16 to 256 channels).  A cluster of CTAs shares one unit of work:
 //   * attention: a window per cluster, a head per CTA.  Every CTA gathers and normalises the window's rows (redundantly: they
 //     are few), computes q, k, v of its head, the scores, softmax and P v; the heads' outputs are exchanged through
 //     distributed shared memory and every CTA projects onto its share of the output columns, adds the residual and scatters.
@@ -271,6 +272,17 @@ bool swin_attn_f32_supported(int C, int heads, int window) {
   return heads <= kMaxCluster && C % 4 == 0 && d % 4 == 0 && T <= 64 && attn_f32_smem(C, d, T, window) <= kMaxSmem;
 }
 bool swin_mlp_f32_supported(int C, long long hidden) { return C % 4 == 0 && hidden < (1 << 20) && mlp_f32_splits(C, (int)hidden) > 0; }
+
+// Every cluster of sixteen rows loads the weights and walks through its phases on its own, about 0.055 us of a full chip beside its
+// products; the tiled kernels spend next to nothing per row but run their products at less than half the rate, and their launches cost
+// more.  Both estimates in us, fitted to (cluster / LayerNorm and two linears, hidden = 4 C): 784 x 32 8.0 / 9.8, 3136 x 32 17.6 / 16.2,
+// 25088 x 32 111 / 72, 784 x 48 12.0 / 15.6, 25088 x 48 141 / 147, 25088 x 64 161 / 257, 50176 x 96 554 / 1170, 12544 x 192 802 / 1088,
+// 12544 x 256 1935 / 1929; hidden = C: 784 x 16 6.7 / 6.9, 25088 x 16 88 / 11, 25088 x 64 118 / 72.
+bool swin_mlp_f32_wins(long long M, int C, long long hidden) {
+  if (!swin_mlp_f32_supported(C, hidden)) return false;
+  const double groups = (double)((M + kMlpRows - 1) / kMlpRows), mflop = 4e-6 * kMlpRows * C * (double)hidden;
+  return 4.5 + groups * (0.055 + mflop / 15.0) < 8.0 + groups * (mflop / 6.4);
+}
 
 int launch_swin_attn_f32(const smartmem_swin_params_t& p, const DevMap& rowmap, const void* x, void* y, cudaStream_t st) {
   AttnF32Args g;

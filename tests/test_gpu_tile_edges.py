@@ -59,6 +59,22 @@ def test_fp32_blocks(cfg):
     case(503, dtype="f32", **cfg)
 
 
+@pytest.mark.parametrize("cfg,fused", [
+    (dict(B=1, H=28, W=56, C=32, heads=2, window=7, shift=3, mlp_ratio=4), True),      # 98 groups of sixteen rows: one kernel
+    (dict(B=2, H=28, W=56, C=32, heads=2, window=7, shift=3, mlp_ratio=4), False),     # 196: three
+    (dict(B=1, H=28, W=56, C=16, heads=1, window=7, shift=0, mlp_ratio=1), False),
+    (dict(B=2, H=28, W=56, C=64, heads=2, window=7, shift=3, mlp_ratio=4), True),
+])
+def test_fp32_mlp_half_by_size(cfg, fused):
+    p = sm.SwinParams()
+    p.dtype = sm.F32
+    for k, v in cfg.items():
+        setattr(p, k, v)
+    rows = cfg["B"] * cfg["H"] * cfg["W"] * cfg["C"] * 4
+    assert (sm.smartmem_swin_block_workspace_bytes(p, sm.ELIMINATE) < 2 * rows) == fused      # only the tensor between the halves
+    case(507, dtype="f32", images=[cfg["B"] - 1], **cfg)
+
+
 @pytest.mark.parametrize("cfg", [
     dict(B=1, H=7, W=7, C=192, heads=6, window=7, shift=0, mlp_ratio=4),      # one tile of 49 rows, hidden features over four CTAs
     dict(B=3, H=14, W=14, C=192, heads=6, window=7, shift=3, mlp_ratio=2),    # over two CTAs, ragged last 76 rows

@@ -70,3 +70,19 @@ def test_noalloc_rejects_blocks_beyond_the_fixed_array():
         sm.smartmem_swin_block_noalloc(p, x.data_ptr(), x.data_ptr(), sm.ELIMINATE, stream())
     assert e.value.code == sm.ERR_WORKSPACE
     assert "workspace too small" in str(e.value)
+
+
+def test_noalloc_fp32_block_beyond_the_fixed_array():
+    """32 x 28 x 56 tokens of 32 channels: kernel by kernel the MLP half wants more than the array, in one kernel it does not."""
+    cfg = dict(B=32, H=28, W=56, C=32, heads=2, window=7, shift=3, mlp_ratio=4)
+    inp = synth.swin_inputs(42, cfg["B"], cfg["H"], cfg["W"], cfg["C"], cfg["heads"], cfg["window"], cfg["mlp_ratio"], "f32")
+    dev = {k: to_dev(v) for k, v in inp.items()}
+    p = _params(cfg, dev, "f32")
+    n = sm.smartmem_swin_block_workspace_bytes(p, sm.ELIMINATE)
+    assert n > sm.smartmem_swin_block_static_scratch_bytes()
+    ws, ref, got = torch.empty(n, dtype=torch.uint8, device="cuda"), torch.empty_like(dev["x"]), torch.empty_like(dev["x"])
+    sm.smartmem_swin_block(p, dev["x"].data_ptr(), ref.data_ptr(), ws.data_ptr(), n, sm.ELIMINATE, stream())
+    sm.smartmem_swin_block_noalloc(p, dev["x"].data_ptr(), got.data_ptr(), sm.ELIMINATE, stream())
+    check_status()
+    # fp32 sums of at most 128 products of O(1) values in another order, through two linears
+    assert (got - ref).abs().max() <= 1e-5
