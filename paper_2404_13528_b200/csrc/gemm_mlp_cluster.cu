@@ -1,17 +1,15 @@
-// Fused MLP half of a Swin block whose weights do not fit one SM: out = x + fc2(GELU(fc1(LN(x)))), C a multiple of 64 up to 192,
-// for few rows.
+// Fused MLP half of a Swin block whose weights do not fit one SM: out = x + fc2(GELU(fc1(LN(x)))), C = 64 or 128, for few rows.
 //
-// With a few thousand rows the three kernels it replaces (LayerNorm, fc1 + GELU, fc2 + residual) are each a launch, a
+// With a few thousand rows the kernels it replaces (LayerNorm + fc1 + GELU, together or apart, and fc2 + residual) are each a launch, a
 // dependency, a first load and a drain around a fraction of a microsecond of products.  Here a cluster of CTAs takes 128 rows and
 // splits the hidden features: every CTA normalises the rows (redundantly), multiplies them with its slice of W1, keeps the GELU of
 // its slice on chip as fc2's operand and multiplies that with its slice of W2; the fp32 partial results are exchanged as bulk
 // copies between the CTAs' shared memories, each CTA adding up its share of the rows.  The weight slices are fetched before the
-// dependency wait where nothing in flight can be writing them.  Measured against the three kernels: C = 192 (four slices), 3920 rows 14.8 -> 12.3 us, 196 rows 9.9 -> 10.1
-// (24 -> 18 us of host time); C = 128 (two slices), 7840 rows 13.5 -> 10.2.
+// dependency wait where nothing in flight can be writing them.  What it gave is beside the rule at the end.
 //
-// Bound by the chain of its phases (at C = 192 about 1.5 us rows, 0.9 first product, 1.3 GELU, 0.9 second product, 0.6 drain, 2.2
-// exchange of 72 KB at the 18 bytes a cycle that shared memory takes from its peers, 1.2 sum), one tile per cluster: beyond one wave
-// the second tile cannot overlap the first and the three kernels win.  Tried and slower: the shares sent into W1's memory
+// Bound by the chain of its phases (with four slices of 192 about 1.5 us rows, 0.9 first product, 1.3 GELU, 0.9 second product, 0.6
+// drain, 2.2 exchange of 72 KB at the 18 bytes a cycle that shared memory takes from its peers, 1.2 sum), one tile per cluster: beyond
+// one wave the second tile cannot overlap the first and the separate kernels win.  Tried and slower: the shares sent into W1's memory
 // while the second product runs (12.8 us).
 //
 // Shared memory: the normalised rows (later the hidden slice) and both weight slices as K-major 128-byte-swizzled operands; once
@@ -284,7 +282,7 @@ Sizes sizes_of(int C, int hs, int S) {
 }
 // the fewest slices whose operands fit an SM (0: none)
 int splits_of(long long C, long long hidden) {
-  if (C % 64 || C > 192) return 0;
+  if (C != 64 && C != 128) return 0;
   for (int s = 1; s <= kMaxSplits; s *= 2)
     if (hidden % (64 * s) == 0 && hidden / s <= 256 && sizes_of((int)C, (int)(hidden / s), s).smem <= 227 * 1024) return s;
   return 0;
@@ -293,10 +291,14 @@ int splits_of(long long C, long long hidden) {
 }  // namespace
 
 bool mlp_cluster_wins(long long M, long long C, long long hidden) {
+  // Whole blocks, us, separate kernels -> this one.  C = 64 (hidden 64 and 768, which the kernel with resident weights does not take): 196
+  // rows 15.5 -> 10.9 and 16.8 -> 13.1, 3136 20.1 -> 13.3.  C = 128, hidden 512: 7840 rows 28.8 -> 27.5, 2352 23.4 -> 22.8, but 1568 21.0 ->
+  // 21.2, 196 20.1 -> 20.6, 49 18.0 -> 19.0, hidden 256 alike; hidden 128 and 768 win at every size (196 rows 18.8 -> 18.1, 21.0 -> 20.2).
+  // C = 192 lost or tied at every size once LayerNorm and fc1 were one kernel (784 rows 22.4 -> 23.3, 3920 29.2 -> 29.3) and is not covered.
+  // One wave of clusters: a second one took C = 128 at 15680 rows from 18.7 to 20.8 us, the MLP half alone.
   const int s = splits_of(C, hidden);
-  if (s == 0) return false;
-  // one wave of clusters: a second one took C = 192 at 6272 rows from 15.3 (three kernels) to 23 us, C = 128 at 15680 from 18.7 to 20.8
-  return (M + BM - 1) / BM <= tc_cluster_ctas(s) / s;
+  if (s == 0 || (M + BM - 1) / BM > tc_cluster_ctas(s) / s) return false;
+  return C == 64 || M >= 2304 || hidden < 256 || hidden > 512;
 }
 
 int launch_mlp_cluster(const void* x, const void* ln_g, const void* ln_b, float eps, const void* W1, const void* b1, const void* W2,
@@ -320,10 +322,9 @@ int launch_mlp_cluster(const void* x, const void* ln_g, const void* ln_b, float 
   int rc = tc_encode_2d_blocks(W1, C, hidden, C / BK, g.hs, &t1);
   if (rc == SMARTMEM_OK) rc = tc_encode_2d_blocks(W2, hidden, C, g.hs / BK, C, &t2);
   if (rc != SMARTMEM_OK) return rc;
-  static constexpr decltype(&mlp_cluster_kernel<1, 1>) kernels[3][4] = {
+  static constexpr decltype(&mlp_cluster_kernel<1, 1>) kernels[2][4] = {
       {mlp_cluster_kernel<1, 1>, mlp_cluster_kernel<1, 2>, mlp_cluster_kernel<1, 3>, mlp_cluster_kernel<1, 4>},
-      {mlp_cluster_kernel<2, 1>, mlp_cluster_kernel<2, 2>, mlp_cluster_kernel<2, 3>, mlp_cluster_kernel<2, 4>},
-      {mlp_cluster_kernel<3, 1>, mlp_cluster_kernel<3, 2>, mlp_cluster_kernel<3, 3>, mlp_cluster_kernel<3, 4>}};
+      {mlp_cluster_kernel<2, 1>, mlp_cluster_kernel<2, 2>, mlp_cluster_kernel<2, 3>, mlp_cluster_kernel<2, 4>}};
   auto* fn = kernels[C / 64 - 1][g.hs / 64 - 1];
   if (ensure_max_dynamic_smem((const void*)fn, 227 * 1024) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   profile_tick("mlp_cluster", st);

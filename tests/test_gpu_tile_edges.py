@@ -81,6 +81,10 @@ def test_fp32_mlp_half_by_size(cfg, fused):
     dict(B=1, H=16, W=8, C=128, heads=4, window=4, shift=2, mlp_ratio=4),     # exactly one tile, the widest slice (256)
     dict(B=2, H=14, W=14, C=128, heads=4, window=7, shift=3, mlp_ratio=1),    # one CTA per tile
     dict(B=1, H=14, W=14, C=192, heads=6, window=7, shift=3, mlp_ratio=3),    # 576 does not split into whole blocks: kernel by kernel
+    dict(B=1, H=48, W=48, C=128, heads=4, window=8, shift=4, mlp_ratio=4),    # 2304 rows, the fewest that two CTAs per tile take
+    dict(B=1, H=40, W=56, C=128, heads=4, window=8, shift=0, mlp_ratio=4),    # 2240: kernel by kernel
+    dict(B=3, H=14, W=14, C=128, heads=4, window=7, shift=3, mlp_ratio=6),    # four CTAs per tile, ragged last 76 rows
+    dict(B=1, H=14, W=14, C=64, heads=2, window=7, shift=3, mlp_ratio=12),    # the narrowest, four CTAs per tile
 ])
 def test_mlp_over_a_cluster(cfg):
     case(504, dtype="bf16", **cfg)
