@@ -419,11 +419,16 @@ bool gemm_splitk_supported(const TcOperand& X, const TcOperand& W, const TcEpilo
 }
 
 // Microseconds, fitted to measurements: a fixed part, the exchange of the partial sums (distributed shared memory moves about
-// 14 bytes per clock and SM, which is what ends the range at 128 rows), and the stream of W.  Below 32 rows always: the tiled
-// kernel's copies of a mostly empty A tile are slower than full ones (two rows, N = 12288, K = 4096: 31 us against 19).
+// 14 bytes per clock and SM, which is what ends the range at 128 rows), and the stream of W.  Below 32 rows the tiled kernel's estimate
+// does not hold (its copies of a mostly empty A tile are slower than full ones), so the line is drawn by measurement, tiled -> this one:
+// a long reduction, 2 rows, N = 4096: K = 512 5.1 -> 4.9, 1024 7.7 -> 5.5, 4096 23.6 -> 10.0; 31 rows, N = 512: K = 512 4.4 -> 4.6, 1024
+// 5.9 -> 4.8.  A shorter one only where there are tiles enough for every SM and W is not yet all of the cost: 2 rows, K = 256, N = 1024
+// 3.7 -> 4.0, 12288 5.1 -> 4.7, 32768 7.8 -> 5.6, 65536 10.3 -> 10.0, 131072 15.9 -> 18.3; 31 rows, 12288 4.8 -> 5.9, 32768 7.4 -> 6.2,
+// 65536 10.0 -> 11.2; K = 128, N = 65536 7.3 -> 8.2.
 double gemm_splitk_us(long long M, long long N, long long K) {
   const double nb = (double)((M + 15) / 16 * 16);
-  return M > 128 ? 1e30 : M < 32 ? 0.0 : 3.0 + 0.018 * nb + (double)N * (double)K * 2.0 / 6.2e6 * (1.0 + nb / 260.0);
+  if (M < 32) return K >= (M > 16 ? 768 : 512) || (K >= 256 && N * K >= (1ll << 23) && N < 65536) ? 0.0 : 1e30;
+  return M > 128 ? 1e30 : 3.0 + 0.018 * nb + (double)N * (double)K * 2.0 / 6.2e6 * (1.0 + nb / 260.0);
 }
 
 bool gemm_splitk_norm_fits(long long M, long long N, long long K) {

@@ -1,7 +1,5 @@
 """GPU parity of the GEMM for few rows (reduction split over a cluster) and of the decode attention at the edges of its tiles."""
-import numpy as np
 import pytest
-import torch
 
 from paper_2404_13528_b200 import binding as sm
 from paper_2404_13528_b200 import synth
@@ -19,6 +17,10 @@ pytestmark = pytest.mark.gpu
     (64, 1024, 4096),        # the widest X with two CTAs per SM
     (65, 256, 512),          # the narrowest with one
     (128, 40, 2048),         # most rows, fewer columns than a tile
+    (1, 136, 512), (16, 136, 576),   # the shortest reductions, a ragged column tile; nine k-blocks over eight CTAs
+    (16, 136, 448), (17, 136, 704),  # a k-block fewer: the tiled kernel
+    (17, 128, 768), (31, 264, 1088),
+    (3, 32776, 256), (31, 65528, 256),   # four k-blocks, a large W: no split
 ])
 def test_few_row_linear(M, N, K):
     x = synth.normal(401, 0, (M, K), dtype="bf16")
