@@ -101,25 +101,25 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constan
     uint32_t s = 0, ph = 1;
     int issued = 0;
     for (int unit = unit0; unit < a.units && ok; unit += unit_step) {
-    const int b = unit / a.heads, h = unit - b * a.heads;
-    const int row = b * a.rows_b + h * a.rows_h, col = h * a.cols_h;
-    for (int i = 0; i < n_st; ++i) {
-      const int p0 = s_lo + i * DEC_STEP, np = min(DEC_STEP, s_hi - p0), nbox = (np + DEC_BOX - 1) / DEC_BOX;
-      ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(&empty[s], ph, &abort_flag, a.status) ? 1 : 0) != 0;
-      if (!ok) break;
-      if (!waited && p0 + nbox * DEC_BOX >= a.S) { pdl_wait(); waited = true; }
-      if (ptx::elect_one()) {
-        uint8_t* st = ring + s * DEC_STAGE_BYTES;
-        ptx::mbar_expect_tx(&full[s], (uint32_t)nbox * 2u * DEC_BOX_BYTES);
-        for (int x = 0; x < nbox; ++x) {
-          ptx::tma_load_2d(st + x * DEC_BOX_BYTES, &tmK, &full[s], col, row + p0 + x * DEC_BOX);
-          ptx::tma_load_2d(st + DEC_STAGE_BYTES / 2 + x * DEC_BOX_BYTES, &tmV, &full[s], col, row + p0 + x * DEC_BOX);
+      const int b = unit / a.heads, h = unit - b * a.heads;
+      const int row = b * a.rows_b + h * a.rows_h, col = h * a.cols_h;
+      for (int i = 0; i < n_st; ++i) {
+        const int p0 = s_lo + i * DEC_STEP, np = min(DEC_STEP, s_hi - p0), nbox = (np + DEC_BOX - 1) / DEC_BOX;
+        ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(&empty[s], ph, &abort_flag, a.status) ? 1 : 0) != 0;
+        if (!ok) break;
+        if (!waited && p0 + nbox * DEC_BOX >= a.S) { pdl_wait(); waited = true; }
+        if (ptx::elect_one()) {
+          uint8_t* st = ring + s * DEC_STAGE_BYTES;
+          ptx::mbar_expect_tx(&full[s], (uint32_t)nbox * 2u * DEC_BOX_BYTES);
+          for (int x = 0; x < nbox; ++x) {
+            ptx::tma_load_2d(st + x * DEC_BOX_BYTES, &tmK, &full[s], col, row + p0 + x * DEC_BOX);
+            ptx::tma_load_2d(st + DEC_STAGE_BYTES / 2 + x * DEC_BOX_BYTES, &tmV, &full[s], col, row + p0 + x * DEC_BOX);
+          }
         }
+        __syncwarp();
+        ++issued;
+        if (++s == DEC_STAGES) { s = 0; ph ^= 1; }
       }
-      __syncwarp();
-      ++issued;
-      if (++s == DEC_STAGES) { s = 0; ph ^= 1; }
-    }
     }
     if (abort_flag && lane == 0) {                    // unwinding: copies in flight get a bounded chance to land
       for (int k = issued > DEC_STAGES ? issued - DEC_STAGES : 0; k < issued; ++k) {
@@ -141,100 +141,100 @@ decode_attn_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constan
     uint32_t s = 0, ph = 0;
     int pb = 0;
     for (int unit = unit0; unit < a.units; unit += unit_step, pb ^= 1) {
-    float qf[8];
-    unpack8(q_next, qf);
-    q_next = q_of(unit + unit_step);
+      float qf[8];
+      unpack8(q_next, qf);
+      q_next = q_of(unit + unit_step);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) qf[j] *= a.scale_log2e;
-    float m = -INFINITY, l = 0.f, acc[8];
+      for (int j = 0; j < 8; ++j) qf[j] *= a.scale_log2e;
+      float m = -INFINITY, l = 0.f, acc[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) acc[j] = 0.f;
-    for (int i = 0; i < n_st; ++i) {
-      const int np = min(DEC_STEP, s_hi - (s_lo + i * DEC_STEP));
-      if (!ptx::mbar_wait(&full[s], ph, &abort_flag, a.status)) break;
-      const uint8_t* kt = ring + s * DEC_STAGE_BYTES + grp * (DH * 2) + l16 * 16;
-      uint4 kv[DEC_UNROLL], vv[DEC_UNROLL];
+      for (int j = 0; j < 8; ++j) acc[j] = 0.f;
+      for (int i = 0; i < n_st; ++i) {
+        const int np = min(DEC_STEP, s_hi - (s_lo + i * DEC_STEP));
+        if (!ptx::mbar_wait(&full[s], ph, &abort_flag, a.status)) break;
+        const uint8_t* kt = ring + s * DEC_STAGE_BYTES + grp * (DH * 2) + l16 * 16;
+        uint4 kv[DEC_UNROLL], vv[DEC_UNROLL];
 #pragma unroll
-      for (int u = 0; u < DEC_UNROLL; ++u) {
-        kv[u] = *reinterpret_cast<const uint4*>(kt + u * (DEC_GROUPS * DH * 2));
-        vv[u] = *reinterpret_cast<const uint4*>(kt + DEC_STAGE_BYTES / 2 + u * (DEC_GROUPS * DH * 2));
-      }
-      float d[DEC_UNROLL], vf[DEC_UNROLL][8];
-#pragma unroll
-      for (int u = 0; u < DEC_UNROLL; ++u) {
-        float kf[8];
-        unpack8(kv[u], kf);
-        float d0 = 0.f, d1 = 0.f;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          d0 = fmaf(qf[2 * j], kf[2 * j], d0);
-          d1 = fmaf(qf[2 * j + 1], kf[2 * j + 1], d1);
+        for (int u = 0; u < DEC_UNROLL; ++u) {
+          kv[u] = *reinterpret_cast<const uint4*>(kt + u * (DEC_GROUPS * DH * 2));
+          vv[u] = *reinterpret_cast<const uint4*>(kt + DEC_STAGE_BYTES / 2 + u * (DEC_GROUPS * DH * 2));
         }
-        d[u] = d0 + d1;
-        // rows past the share are whatever lay in the ring or behind the cache's last used row: never multiplied
-        const bool in = grp + u * DEC_GROUPS < np;
-        unpack8(in ? vv[u] : make_uint4(0, 0, 0, 0), vf[u]);
+        float d[DEC_UNROLL], vf[DEC_UNROLL][8];
+#pragma unroll
+        for (int u = 0; u < DEC_UNROLL; ++u) {
+          float kf[8];
+          unpack8(kv[u], kf);
+          float d0 = 0.f, d1 = 0.f;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            d0 = fmaf(qf[2 * j], kf[2 * j], d0);
+            d1 = fmaf(qf[2 * j + 1], kf[2 * j + 1], d1);
+          }
+          d[u] = d0 + d1;
+          // rows past the share are whatever lay in the ring or behind the cache's last used row: never multiplied
+          const bool in = grp + u * DEC_GROUPS < np;
+          unpack8(in ? vv[u] : make_uint4(0, 0, 0, 0), vf[u]);
+        }
+        __syncwarp();
+        if (lane == 0) ptx::mbar_arrive(&empty[s]);
+        if (++s == DEC_STAGES) { s = 0; ph ^= 1; }
+#pragma unroll
+        for (int x = 8; x >= 1; x >>= 1)
+#pragma unroll
+          for (int u = 0; u < DEC_UNROLL; ++u) d[u] += __shfl_xor_sync(0xFFFFFFFFu, d[u], x);
+        float mn = m;
+#pragma unroll
+        for (int u = 0; u < DEC_UNROLL; ++u) {
+          if (grp + u * DEC_GROUPS >= np) d[u] = -INFINITY;
+          mn = fmaxf(mn, d[u]);
+        }
+        const float ref = mn == -INFINITY ? 0.f : mn;   // (a half-warp that has seen no position yet)
+        const float c = exp2f(m - ref);
+        l *= c;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[j] *= c;
+#pragma unroll
+        for (int u = 0; u < DEC_UNROLL; ++u) {
+          const float p = exp2f(d[u] - ref);
+          l += p;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) acc[j] = fmaf(p, vf[u][j], acc[j]);
+        }
+        m = mn;
       }
-      __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(&empty[s]);
-      if (++s == DEC_STAGES) { s = 0; ph ^= 1; }
+      {                                                 // the warp's two halves
+        const float mo = __shfl_xor_sync(0xFFFFFFFFu, m, 16), lo = __shfl_xor_sync(0xFFFFFFFFu, l, 16);
+        const float mn = fmaxf(m, mo), ref = mn == -INFINITY ? 0.f : mn, w = exp2f(m - ref), wo = exp2f(mo - ref);
+        l = l * w + lo * wo;
 #pragma unroll
-      for (int x = 8; x >= 1; x >>= 1)
-#pragma unroll
-        for (int u = 0; u < DEC_UNROLL; ++u) d[u] += __shfl_xor_sync(0xFFFFFFFFu, d[u], x);
-      float mn = m;
-#pragma unroll
-      for (int u = 0; u < DEC_UNROLL; ++u) {
-        if (grp + u * DEC_GROUPS >= np) d[u] = -INFINITY;
-        mn = fmaxf(mn, d[u]);
+        for (int j = 0; j < 8; ++j) acc[j] = acc[j] * w + __shfl_xor_sync(0xFFFFFFFFu, acc[j], 16) * wo;
+        m = mn;
       }
-      const float ref = mn == -INFINITY ? 0.f : mn;   // (a half-warp that has seen no position yet)
-      const float c = exp2f(m - ref);
-      l *= c;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) acc[j] *= c;
-#pragma unroll
-      for (int u = 0; u < DEC_UNROLL; ++u) {
-        const float p = exp2f(d[u] - ref);
-        l += p;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) acc[j] = fmaf(p, vf[u][j], acc[j]);
+      if (lane < 16) {
+        *reinterpret_cast<float4*>(&part[pb][warp][l16 * 8]) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        *reinterpret_cast<float4*>(&part[pb][warp][l16 * 8 + 4]) = make_float4(acc[4], acc[5], acc[6], acc[7]);
       }
-      m = mn;
-    }
-    {                                                 // the warp's two halves
-      const float mo = __shfl_xor_sync(0xFFFFFFFFu, m, 16), lo = __shfl_xor_sync(0xFFFFFFFFu, l, 16);
-      const float mn = fmaxf(m, mo), ref = mn == -INFINITY ? 0.f : mn, w = exp2f(m - ref), wo = exp2f(mo - ref);
-      l = l * w + lo * wo;
+      if (lane == 0) { gm[pb][warp] = m; gl[pb][warp] = l; }
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * DEC_WARPS) : "memory");
+      if (tid < DH) {
+        float o = 0.f, lt = 0.f, mt = -INFINITY;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) acc[j] = acc[j] * w + __shfl_xor_sync(0xFFFFFFFFu, acc[j], 16) * wo;
-      m = mn;
-    }
-    if (lane < 16) {
-      *reinterpret_cast<float4*>(&part[pb][warp][l16 * 8]) = make_float4(acc[0], acc[1], acc[2], acc[3]);
-      *reinterpret_cast<float4*>(&part[pb][warp][l16 * 8 + 4]) = make_float4(acc[4], acc[5], acc[6], acc[7]);
-    }
-    if (lane == 0) { gm[pb][warp] = m; gl[pb][warp] = l; }
-    asm volatile("bar.sync 1, %0;" ::"n"(32 * DEC_WARPS) : "memory");
-    if (tid < DH) {
-      float o = 0.f, lt = 0.f, mt = -INFINITY;
+        for (int g = 0; g < DEC_WARPS; ++g) mt = fmaxf(mt, gm[pb][g]);
+        const float ref = mt == -INFINITY ? 0.f : mt;
 #pragma unroll
-      for (int g = 0; g < DEC_WARPS; ++g) mt = fmaxf(mt, gm[pb][g]);
-      const float ref = mt == -INFINITY ? 0.f : mt;
-#pragma unroll
-      for (int g = 0; g < DEC_WARPS; ++g) {
-        const float w = exp2f(gm[pb][g] - ref);
-        lt = fmaf(w, gl[pb][g], lt);
-        o = fmaf(w, part[pb][g][tid], o);
+        for (int g = 0; g < DEC_WARPS; ++g) {
+          const float w = exp2f(gm[pb][g] - ref);
+          lt = fmaf(w, gl[pb][g], lt);
+          o = fmaf(w, part[pb][g][tid], o);
+        }
+        if (a.split > 1) {                              // (one unit per CTA then)
+          cta_o[tid] = o;
+          if (tid == 0) { cta_ml[0] = mt; cta_ml[1] = lt; }
+        } else {
+          const int b = unit / a.heads, h = unit - b * a.heads;
+          a.o[b * a.o_sb + h * a.o_sh + tid] = __float2bfloat16_rn(o / lt);
+        }
       }
-      if (a.split > 1) {                              // (one unit per CTA then)
-        cta_o[tid] = o;
-        if (tid == 0) { cta_ml[0] = mt; cta_ml[1] = lt; }
-      } else {
-        const int b = unit / a.heads, h = unit - b * a.heads;
-        a.o[b * a.o_sb + h * a.o_sh + tid] = __float2bfloat16_rn(o / lt);
-      }
-    }
     }
   }
   if (a.split > 1) {

@@ -502,13 +502,13 @@ int launch_norm_t(const void* src, void* dst, const void* gamma, const void* bet
       launch_pdl(norm_wide_kernel<T, RMS>, dim3((unsigned)rows), dim3(256), 0, st, s, d, g, b, eps, C);
     else SM_LAUNCH(32, 1, true)
   } else {
-  if (nvec <= 16) SM_LAUNCH(4, 1, false)
-  else if (nvec <= 32) SM_LAUNCH(8, 2, false)
-  else if (nvec <= 64) SM_LAUNCH(16, 1, false)
-  else if (nvec <= 128) SM_LAUNCH(32, 1, false)
-  else if (!rowmap && nvec <= 1024)
-    launch_pdl(norm_wide_kernel<T, RMS>, dim3((unsigned)rows), dim3(256), 0, st, s, d, g, b, eps, C);
-  else SM_LAUNCH(32, 1, true)
+    if (nvec <= 16) SM_LAUNCH(4, 1, false)
+    else if (nvec <= 32) SM_LAUNCH(8, 2, false)
+    else if (nvec <= 64) SM_LAUNCH(16, 1, false)
+    else if (nvec <= 128) SM_LAUNCH(32, 1, false)
+    else if (!rowmap && nvec <= 1024)
+      launch_pdl(norm_wide_kernel<T, RMS>, dim3((unsigned)rows), dim3(256), 0, st, s, d, g, b, eps, C);
+    else SM_LAUNCH(32, 1, true)
   }
 #undef SM_LAUNCH
   count_launch();

@@ -10,7 +10,7 @@
 // moves 11 C through HBM.
 //
 // Unit of work: a pair of windows = one 128-row MMA tile (window w of the pair in rows 64 w .. 64 w + T - 1,
-// the rows between T and 64 stay zero), taken round-robin by persistent CTAs that keep every weight resident.
+// the rows between T and 64 stay zero); persistent CTAs that keep every weight resident take a contiguous run of units each.
 // An "item" is (unit, head); head h is the work of row group h.  Per item, all in one 96-column buffer of tensor
 // memory (four buffers in rotation):
 //
@@ -410,8 +410,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
     }
   } else if (warp < 4 + 4 * NH) {
     // ---- row groups: group h takes head h of every unit; one row of the pair tile per thread.  The group's elected thread issues
-    // the item's S, P V and projection products, and the QKV product of its NEXT item as soon as the tensor-memory buffer that
-    // item rotates into is free (the projection of the item before this one has completed). ------------------------------------
+    // the item's S and P V products; the QKV products and the projections come from the last two warps. ------------------------
     const int gi = (warp - 4) >> 2;                    // group = head
     const int q = warp & 3;                            // TMEM lane quadrant
     const int r = q * 32 + lane;

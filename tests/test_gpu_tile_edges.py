@@ -1,7 +1,6 @@
 """GPU parity of the row-norm, ragged-transpose, batched-score and fp32 block kernels at the edges of their tiles."""
 import numpy as np
 import pytest
-import torch
 
 from oracle import chains
 from paper_2404_13528_b200 import binding as sm
