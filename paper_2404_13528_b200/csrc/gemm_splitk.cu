@@ -102,21 +102,28 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   }
   __syncwarp();
   if (warp == 0) {
-    // the ring's first round of W
-    for (int s = 0; s < g.stages && s < nk; ++s) {
-      if (ptx::elect_one()) {
-        if (g.w_settled) {
+    // the ring's first round of W (two loops: with the choice inside the elected branch a copy took longer to issue, 0.4 us a launch)
+    const int first = min(g.stages, nk);
+    if (g.w_settled) {
+#pragma unroll 1
+      for (int s = 0; s < first; ++s) {
+        if (ptx::elect_one()) {
           ptx::mbar_expect_tx(&full[s], W_STAGE);
           ptx::tma_load_2d(smem + s * W_STAGE, &tmW, &full[s], (kb0 + s) * BK, n0);
-        } else {
-          ptx::tma_prefetch_2d(&tmW, (kb0 + s) * BK, n0);
         }
+        __syncwarp();
       }
-      __syncwarp();
+    } else {
+#pragma unroll 1
+      for (int s = 0; s < first; ++s) {
+        if (ptx::elect_one()) ptx::tma_prefetch_2d(&tmW, (kb0 + s) * BK, n0);
+        __syncwarp();
+      }
     }
   }
   if (warp == 1) ptx::tmem_alloc(tmem_slot, g.tmem_cols);
   if (norm)                                         // (a line per k-block)
+#pragma unroll 1
     for (int i = tid; i < nk; i += kThreads) ptx::prefetch_l2(g.gamma + (kb0 + i) * BK);
   {
     const int sg = g.seg_cols > 0 ? n0 / g.seg_cols : 0;
@@ -190,6 +197,7 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   } else {                                          // warps 2-6
     bool ok = true;
     if (norm) {
+#pragma unroll 1
       for (int i = tid - 64; i < nk * (BK / 8); i += 32 * kScaleWarps)
         reinterpret_cast<uint4*>(gamma_s)[i] = *reinterpret_cast<const uint4*>(g.gamma + kb0 * BK + i * 8);
       asm volatile("bar.sync 1, %0;" ::"n"(32 * kScaleWarps) : "memory");
