@@ -1052,8 +1052,14 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
     // fewer idle SMs in the last wave (time of a wave ~ tile width plus a fixed part), for short reductions only: a 128-wide tile
     // reads as many operand bytes per product as shared memory delivers, so over a long K the wider tile wins even with a
     // ragged last wave (measured at K = 2048)
+    // Short reductions are bound by their stores, which the wide tile makes in whole rows, so it takes them whatever N is (128 heads,
+    // 1000 x 1000 scores of 64: 89 us in 128-wide tiles, 58 in 256; 704 x 704 55 in 64-wide ones, 34), but for an N that 96-wide tiles fill
+    // and 256-wide ones do not: one of those takes as long as 2.05 narrow ones (288 x 288: 10.2 us in three, 14.3 in two; 576 x 576 with
+    // 24 heads 7.8 in six, 9.3 in three; 960 x 960 71 in ten, 55 in four).
+    const long long wide = (N + 255) / 256;
+    const bool fill96 = N % 128 && N % 96 == 0 && 100 * (N / 96) < 205 * wide;
     if (ep.rope_cols > 0) bn = 256;
-    else if (nkb <= 2 && N >= 192 && !a_mn && tiles_m1 * batch * ((N + 255) / 256) >= tc_sm_count()) bn = 256;   // bound by its stores
+    else if (nkb <= 2 && N >= 192 && !a_mn && !fill96 && tiles_m1 * batch * wide >= tc_sm_count()) bn = 256;
     else if (N % 256 == 0) {
       const long long tm = tiles_m1 * batch, sms = tc_sm_count();
       const long long w256 = (tm * (N / 256) + sms - 1) / sms, w128 = (tm * (N / 128) + sms - 1) / sms;
