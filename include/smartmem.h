@@ -28,10 +28,9 @@
  *   - Calls validate on the host, enqueue work on the given stream and return without
  *     synchronising.  The return value is a smartmem_status_t.  Nothing aborts or prints.
  *   - Whatever a call reads may be the result of work enqueued before it on the same stream: activations, chain inputs,
- *     and the weights, scales, biases and tables of a parameter block.  One exception: a bf16 Swin block of 2 or 3 heads of
- *     32 (C = 64 or 96) in SMARTMEM_ELIMINATE fetches ln1_g, ln1_b, w_qkv, b_qkv, rel_bias_table, w_proj and b_proj while the
- *     kernel before it on the stream is finishing, so that kernel must not be the one that writes them: let another kernel,
- *     a copy or a synchronisation come between.
+ *     and the weights, scales, biases and tables of a parameter block.  One exception: the first kernel of a bf16 Swin block
+ *     of C = 64 or 96 (or of one of its halves) fetches its parameters while the kernel before it on the stream is finishing,
+ *     so that kernel must not be the one that writes them: let another kernel, a copy or a synchronisation come between.
  *   - Device-side waits are bounded; a wait that runs out sets a device status word that
  *     smartmem_last_device_status() reads back.
  *   - There is no CPU fallback: without a CUDA device the run entry points return

@@ -24,7 +24,8 @@ int ensure_max_dynamic_smem(const void* kernel, int bytes, int carveout = -1);
 // anything that kernel could touch.  The wait returns once the whole preceding grid has finished
 // and its writes are visible.  What no kernel in flight can be writing may be read earlier: parameters of a layer call, in a kernel
 // that follows another one of the same call (that one has waited for whatever preceded the call); its launcher says so with
-// `settled`, and without it gives up the early start.  `pdl_launch_dependents()` lets the NEXT kernel in the stream begin
+// `settled`, and without it gives up the early start.  (The kernels of narrow bf16 Swin blocks read parameters early in any place;
+// the header tells callers.)  `pdl_launch_dependents()` lets the NEXT kernel in the stream begin
 // that early start as soon as every CTA of this one has called it.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -302,10 +302,10 @@ gemm_ln_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 }
 
 template <int KDIM>
-int launch_t(const CUtensorMap& tw, const CUtensorMap& toa, const CUtensorMap& tob, LnGemmArgs& g, size_t smem, bool settled, cudaStream_t st) {
+int launch_t(const CUtensorMap& tw, const CUtensorMap& toa, const CUtensorMap& tob, LnGemmArgs& g, size_t smem, cudaStream_t st) {
   if (ensure_max_dynamic_smem((const void*)gemm_ln_kernel<KDIM>, 232448) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   const unsigned grid = (unsigned)(g.tiles < tc_sm_count() ? g.tiles : tc_sm_count());
-  if (launch_cluster(gemm_ln_kernel<KDIM>, dim3(grid), dim3(kThreads), smem, st, 1u, settled, tw, toa, tob, g) != cudaSuccess) return SMARTMEM_ERR_CUDA;
+  if (launch_pdl(gemm_ln_kernel<KDIM>, dim3(grid), dim3(kThreads), smem, st, tw, toa, tob, g) != cudaSuccess) return SMARTMEM_ERR_CUDA;
   count_launch();
   return SMARTMEM_OK;
 }
@@ -317,7 +317,7 @@ bool gemm_ln_supported(long long N, long long K) {
 }
 
 int launch_gemm_ln(const void* X, const DevMap* rowmap, const void* gamma, const void* beta, float eps, const void* W,
-                   const void* bias, void* out, long long M, long long N, long long K, bool settled, cudaStream_t st) {
+                   const void* bias, void* out, long long M, long long N, long long K, cudaStream_t st) {
   if (!gemm_ln_supported(N, K) || M < 1 || M >= (1ll << 31) - BM) return SMARTMEM_ERR_UNSUPPORTED;
   const void* ptrs[] = {X, gamma, beta, W, bias, out};
   for (const void* p : ptrs)
@@ -347,7 +347,7 @@ int launch_gemm_ln(const void* X, const DevMap* rowmap, const void* gamma, const
   if (need > smem) return SMARTMEM_ERR_UNSUPPORTED;
   g.smem_bytes = (uint32_t)smem;
   profile_tick("gemm_ln", st);
-  return K == 96 ? launch_t<96>(tw, toa, tob, g, smem, settled, st) : launch_t<64>(tw, toa, tob, g, smem, settled, st);
+  return K == 96 ? launch_t<96>(tw, toa, tob, g, smem, st) : launch_t<64>(tw, toa, tob, g, smem, st);
 }
 
 }  // namespace smartmem

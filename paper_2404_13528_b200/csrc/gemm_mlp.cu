@@ -514,7 +514,7 @@ bool mlp_fused_supported(long long C, long long hidden) {
 
 int launch_mlp_fused(const void* A, const void* ln_gamma, const void* ln_beta, float ln_eps, const void* W1, const void* b1,
                      const void* W2, const void* b2, void* out, long long M, long long C, long long hidden,
-                     bool settled, cudaStream_t st) {
+                     cudaStream_t st) {
   if (!mlp_fused_supported(C, hidden) || M < 1 || M >= (1ll << 31) - BM) return SMARTMEM_ERR_UNSUPPORTED;
   const void* ptrs[] = {A, W1, b1, W2, b2, out, ln_gamma, ln_beta};
   for (const void* p : ptrs) {
@@ -555,7 +555,7 @@ int launch_mlp_fused(const void* A, const void* ln_gamma, const void* ln_beta, f
   if (ensure_max_dynamic_smem((const void*)kern, 232448) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   profile_tick("mlp_fused", st);
   const unsigned grid = (unsigned)(g.tiles < tc_sm_count() ? g.tiles : tc_sm_count());
-  launch_cluster(kern, dim3(grid), dim3(kThreads), smem, st, 1u, settled, ta, tw1, tw2, g);
+  launch_pdl(kern, dim3(grid), dim3(kThreads), smem, st, ta, tw1, tw2, g);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? SMARTMEM_OK : SMARTMEM_ERR_CUDA;
 }

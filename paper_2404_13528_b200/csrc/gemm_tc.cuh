@@ -95,7 +95,7 @@ int tc_cluster_ctas(int size);
 bool mlp_fused_supported(long long C, long long hidden);
 int launch_mlp_fused(const void* A, const void* ln_gamma, const void* ln_beta, float ln_eps, const void* W1, const void* b1,
                      const void* W2, const void* b2, void* out, long long M, long long C, long long hidden,
-                     bool settled, cudaStream_t st);
+                     cudaStream_t st);
 
 // The same for few rows where the weights do not fit one SM: the hidden features split over a cluster (gemm_mlp_cluster.cu).
 // mlp_cluster_wins: it covers the shape and beats the separate kernels.
@@ -108,7 +108,7 @@ int launch_mlp_cluster(const void* x, const void* ln_g, const void* ln_b, float 
 // the element offset of consumer row m in X; gamma/beta null: no normalisation (plain gather).
 bool gemm_ln_supported(long long N, long long K);
 int launch_gemm_ln(const void* X, const DevMap* rowmap, const void* gamma, const void* beta, float eps, const void* W,
-                   const void* bias, void* out, long long M, long long N, long long K, bool settled, cudaStream_t st);
+                   const void* bias, void* out, long long M, long long N, long long K, cudaStream_t st);
 // The same, with an optional GELU, for few rows of 128, 192 or 256 elements (gemm_ln_wave.cu).  gemm_ln_wave_wins: it covers the shape and
 // beats the separate kernels.  w_settled: as TcEpilogue::b_settled, for W.
 bool gemm_ln_wave_wins(long long M, long long N, long long K);

@@ -251,7 +251,7 @@ int run_block(const smartmem_swin_params_t* pp, const void* x, void* y, void* wo
   const bool fuse_ln1 = path.fuse_ln1;
   auto ln1_qkv = [&](const void* rows, const DevMap* map) {
     return path.ln1_wave ? launch_gemm_ln_wave(rows, map, p.ln1_g, p.ln1_b, p.ln_eps, p.w_qkv, p.b_qkv, 0, at(L.qkv), M, 3 * C, C, !elim, st)
-                         : launch_gemm_ln(rows, map, p.ln1_g, p.ln1_b, p.ln_eps, p.w_qkv, p.b_qkv, at(L.qkv), M, 3 * C, C, !elim, st);
+                         : launch_gemm_ln(rows, map, p.ln1_g, p.ln1_b, p.ln_eps, p.w_qkv, p.b_qkv, at(L.qkv), M, 3 * C, C, st);
   };
 #define SM_TRY(label, expr) do { if (tm) tm->tick(label); rc = (expr); if (rc != SMARTMEM_OK) return rc; } while (0)
   if (half == 1) {
@@ -317,7 +317,7 @@ int run_block(const smartmem_swin_params_t* pp, const void* x, void* y, void* wo
       SM_TRY("mlp_fused_ln2_fc1_gelu_fc2_residual",
              f32 ? launch_swin_mlp_f32(p, y1, y, M, half != 1, st)
              : path.mlp_cluster ? launch_mlp_cluster(y1, p.ln2_g, p.ln2_b, p.ln_eps, p.w_fc1, p.b_fc1, p.w_fc2, p.b_fc2, y, M, C, hid, half != 1, st)
-                                : launch_mlp_fused(y1, p.ln2_g, p.ln2_b, p.ln_eps, p.w_fc1, p.b_fc1, p.w_fc2, p.b_fc2, y, M, C, hid, half != 1, st));
+                                : launch_mlp_fused(y1, p.ln2_g, p.ln2_b, p.ln_eps, p.w_fc1, p.b_fc1, p.w_fc2, p.b_fc2, y, M, C, hid, st));
     } else {
       if (path.ln2_wave) {
         SM_TRY("ln2_fc1_gemm_gelu", launch_gemm_ln_wave(y1, nullptr, p.ln2_g, p.ln2_b, p.ln_eps, p.w_fc1, p.b_fc1, 1, at(L.hid), M, hid, C, half != 1, st));

@@ -122,7 +122,8 @@ def test_weights_then_decode_step(B):
     ("w_qkv", sm.BF16, 192, 32, 14, -1),     # norm + QKV in one kernel
     ("w_qkv", sm.BF16, 512, 32, 14, -1),     # kernel by kernel
     ("w_qkv", sm.F32, 32, 16, 8, -1),
-    ("w_fc1", sm.BF16, 96, 32, 14, 1), ("w_fc1", sm.BF16, 192, 32, 14, 1), ("w_fc1", sm.BF16, 256, 32, 14, 1), ("w_fc1", sm.F32, 32, 16, 8, 1),   # the MLP half on its own
+    ("w_fc1", sm.BF16, 192, 32, 14, 1), ("w_fc1", sm.BF16, 256, 32, 14, 1), ("w_fc1", sm.F32, 32, 16, 8, 1),   # the MLP half on its own
+    ("w_fc1", sm.BF16, 128, 32, 49, 1),      # the same over a cluster
 ])
 def test_weights_then_block(which, dtype, C, head_dim, H, half):
     td = torch.float32 if dtype == sm.F32 else torch.bfloat16
