@@ -73,7 +73,7 @@ __device__ __forceinline__ void gemm_any(const float* A, int pa, const float* W,
 // rows [0, n) of `vpr.d` 16-byte vectors from global memory (row r at src(r)) into shared memory with pitch `pitch`
 template <typename Src>
 __device__ __forceinline__ void load_rows(float* dst, int pitch, int n, const FastDiv& vpr, Src src) {
-#pragma unroll 4
+#pragma unroll 1                                       // (runs once: the unrolled form costs more in instruction fetches)
   for (int i = threadIdx.x; i < n * (int)vpr.d; i += kThreads) {
     const int r = (int)fd_div((uint32_t)i, vpr), v = i - r * (int)vpr.d;
     ptx::cp_async16(dst + r * pitch + v * 4, src(r) + v * 4);
