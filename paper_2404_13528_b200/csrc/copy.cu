@@ -181,8 +181,8 @@ __global__ void __launch_bounds__(256) copy_transpose16_kernel(const __grid_cons
 }
 
 // The same for any extents: tiles at the edges are ragged, loads are LV and stores SV elements wide (the widest vectors that
-// divide the extents and every stride and offset of their side).  [4,256,57,57] -> channels last: 2-byte gathers through the
-// map took 34 us, the tiles (2-byte loads, 16-byte stores) take 8.
+// divide the extents and every stride and offset of their side).  [4,256,57,57] -> channels last, us of a stream of calls: 2-byte
+// gathers through the map 19.1, the tiles (2-byte loads, 16-byte stores) 9.6.
 template <int LV, int SV>
 __global__ void __launch_bounds__(256) copy_transpose_any_kernel(const __grid_constant__ TransposeArgs a, const uint16_t* __restrict__ src,
                                                                  uint16_t* __restrict__ dst) {

@@ -5,8 +5,8 @@
 // operand, and multiplies them with a slice of W that stays in shared memory: only a pair has room for both (each CTA its 128
 // rows and half of the slice's rows of W).  Bound by the work of one tile after the other: of about 7000 cycles for a tile of 256 x 384,
 // the normalisation is 4500 (issue slots: 16 warps), the product 2000 and the output 2000, the latter two overlapped with the
-// next tile's rows.  Measured against norm and linear as two kernels (us of a stream of calls): 25088 x 384 18.5 -> 13.0, 18816 x 384
-// 15.2 -> 9.0, 37632 x 256 15.6 -> 11.1, 9408 x 512 11.8 -> 10.5; small ones, bound by the launches, 9.8 -> 7.1.
+// next tile's rows.  Measured against norm and linear as two kernels (us of a stream of calls, gathered rows): 25088 x 384 16.8 ->
+// 14.1, 18816 x 384 14.2 -> 10.1, 37632 x 256 14.4 -> 12.1, 9408 x 512 12.3 -> 11.9; where it is taken stands at the end.
 //
 // Sixteen warps of rows and output (a seventeenth would leave 96 registers a thread for the 48 of rows in flight); warp 0 also
 // fetches W and, in the even CTA, issues the products.  The statistics of the next tile overlap the product of this one, its

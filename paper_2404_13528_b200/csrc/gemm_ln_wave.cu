@@ -4,9 +4,9 @@
 // thousand rows there is nothing to stream: a launch, a dependency and a drain cost the normalisation and the product each more
 // than their work.  A CTA takes 128 rows and a slice of the output columns, normalises the rows (again in every slice: they come
 // from L2) straight into the operand, and multiplies them with its slice of W, which is in L2 by then.  Bound by that
-// chain (1.5 us rows, 0.9 product, 0.6 output and the dependency).  Measured, a block's attention half with norm + QKV linear
-// before -> with this: 3920 x 192 17.4 -> 15.4 us (93 CTAs), 7840 x 128 19.1 -> 16.3 (124), 1568 x 256 16.6 -> 14.8 (78), 4704 x 256
-// 20.5 -> 18.4 (148); an MLP half with norm + fc1 + GELU: 1568 x 256 13.1 -> 11.3.
+// chain (1.5 us rows, 0.9 product, 0.6 output and the dependency).  Measured, a block's attention half with norm and QKV linear as two
+// kernels -> with this: 3920 x 192 19.2 -> 17.1 us (93 CTAs), 7840 x 128 20.6 -> 17.2 (124), 1568 x 256 18.2 -> 15.7 (78), 4704 x 256
+// 21.9 -> 19.5 (148); whole blocks, norm + fc1 + GELU as well: 1568 x 256 32.8 -> 27.9, 3920 x 192 35.3 -> 29.2.
 //
 // Warp roles: 0-15 rows, then bias and output; 16 fetches W, owns the tensor memory and issues the product.
 #include <cstring>

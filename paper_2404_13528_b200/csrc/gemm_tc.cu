@@ -617,7 +617,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if constexpr (QTMA) {
         // Very short reductions (batched q k^T): the tile's store is all there is, and with one staging tile the store path
         // idled while the next tile was converted.  Two tiles, and a warp sends one 32 x 64 box of its quadrant (rows and
-        // columns past the edge are clipped): 8 x 16 heads, 1024 x 1024 scores of 64: 70.5 -> 52 us.
+        // columns past the edge are clipped): 8 x 16 heads, 1024 x 1024 scores of 64: 72.2 -> 55.7 us in a short stream of calls, 73.4 ->
+        // 62.8 in a long one.
         ptx::fence_proxy_async();
         asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory");
         if (lane == 0) {

@@ -47,8 +47,8 @@
 //   then  four warps for the row statistics and the Y epilogue (one row per thread);
 //   last  one warp that issues the QKV products of the items ahead (into the buffer the item four before has left) and one
 //         that issues, in item order, the residual product that opens a unit's Y and the heads' projections.
-// What bounds it (clock stamps at every hand-off, counters): no unit of the SM -- issue slots 52 % busy, ALU 35, tensor pipe 24, special
-// functions 19 -- but the chain of hand-offs of an item (tensor-memory round trips, three barriers, two waits for small products;
+// What bounds it (clock stamps at every hand-off, counters): no unit of the SM -- issue slots 54 % busy, ALU 34, tensor pipe 27, special
+// functions 21 -- but the chain of hand-offs of an item (tensor-memory round trips, three barriers, two waits for small products;
 // 4500 cycles), which more items in flight did not shorten (four row groups instead of two or three, with or without two fewer
 // loading warps: 0.2 to 3 us slower).  What did: the loading warps issued a unit's copies, awaited its rows and took their
 // statistics before they turned to the next unit, 6500 cycles in all; now the epilogue warps take the statistics whenever rows
