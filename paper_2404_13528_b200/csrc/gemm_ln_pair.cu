@@ -269,17 +269,16 @@ int launch_pair(const CUtensorMap& tw, const LnPairArgs& g, cudaStream_t st) {
 // linear as two kernels -> this one, us of a stream of calls, gathered rows: 3136 x 256 in 3 slices 7.1 -> 6.5, 9408 x 256 in 2 8.7 -> 7.6,
 // 9408 x 384 in 2 12.3 -> 10.0, 9408 x 512 in 2 12.3 -> 11.9; beyond a round 12544 x 256 in 2 10.0 -> 10.4, 12544 x 384 in 2 12.6 -> 13.8,
 // 12544 x 512 in 2 13.8 -> 16.0, 25088 x 384 in 6 (LayerNorm into a QKV projection) 33 -> 60.  One slice wins with any number of rounds
-// for rows of 256 and 384 (25088: 11.5 -> 10.7, 16.8 -> 14.1).  Longer rows with less than a third of the pairs at work take longer than
-// the two kernels, whose launches overlap in a stream: 1568 x 384 in one slice 6.3 against 7.4; rows of 512 in more than two slices, or
-// with fewer tiles than that, as well: 1568 x 512 in 4 7.4 against 8.7.
+// for rows of 256 and 384 (25088: 11.5 -> 10.7, 16.8 -> 14.1).
+// Small calls are bound by the host, and what decides there is the second launch it saves: through the Python binding 10.3 -> 7.5 us.
+// (On the device alone two kernels whose launches overlap are the shorter ones: 1568 x 384 in one slice 6.3 against 7.4, 784 x 512 in
+// eight 7.1 against 8.4.)
 bool gemm_ln_pair_wins(const smartmem_index_map_t& map, long long M, long long N, long long K) {
   const int nb = blocks_of(K);
   if (!nb || N % (64 * nb) || M < 1) return false;
   const long long tiles = (M + 2 * BM - 1) / (2 * BM);
   const long long slices = N / (64 * nb), work = tiles * slices, pairs = tc_cluster_ctas(2) / 2;
   if (work > pairs && (slices > 1 || K == 512)) return false;
-  if (K > 256 && 3 * work < pairs) return false;
-  if (K == 512 && (slices > 2 || 3 * tiles < pairs)) return false;
   return M < (1ll << 31) / 4 && map.klass < 2 && map.vec_elems == 8 &&
          map.n_elements == M * K;
 }

@@ -120,8 +120,8 @@ def test_merge_in_one_kernel(B, H, W, C):
     (1568, 256, 1280), (1568, 256, 1408),     # ten slices: 70 pairs of 74; eleven are 77: two kernels
     (9472, 384, 384), (9473, 384, 384),       # two slices, 37 tiles: every pair; a row more
     (3200, 384, 960),                         # five slices, 13 tiles
-    (6272, 512, 256), (6144, 512, 256),       # rows of 512: 25 tiles, and one tile fewer than a third of the pairs
-    (6272, 512, 384),                         # three slices: two kernels
+    (6144, 512, 384), (6145, 512, 384),       # rows of 512 in three slices: 24 tiles, and one more than fits a round
+    (18944, 512, 128), (18945, 512, 128),     # in one: 74 tiles, and a second round
     (1, 256, 128), (1, 384, 192), (1, 128, 64),   # one row
 ])
 def test_norm_linear_chains(M, K, N):
