@@ -140,7 +140,9 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
   int4* tok_s = reinterpret_cast<int4*>(kmask_s + 4);              // [64]: the map's contribution of token t: (offset, u0, u1, -)
   int4* win_s = tok_s + TP;                                        // [2 units][2 windows]: the contribution of window n: (offset lo, hi, u0, u1)
   int* wkind_s = reinterpret_cast<int*>(win_s + 4);                // [na][2 windows] (+ pad): how the window's rows come in
-  uint64_t* bars = reinterpret_cast<uint64_t*>(wkind_s + 8);
+  uint16_t* raw_s = reinterpret_cast<uint16_t*>(wkind_s + 8);      // [NH][256]: the raw table columns (memory of their own: a fast group's
+                                                                   // first keys may be in place while another still builds its table)
+  uint64_t* bars = reinterpret_cast<uint64_t*>(raw_s + NH * 256);
   uint64_t* w_full = bars;                                         // [NH] QKV weights of a head, then the projection's
   uint64_t *a_full = bars + 4, *a_free = a_full + 3, *landed = a_free + 3;     // [3] each: per slot of the row ring
   uint64_t *s_full = landed + 3, *o_full = s_full + 3;             // [3] each: per group (the group issues these products itself)
@@ -149,8 +151,6 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
   uint64_t *y_full = buf_free + NBUF, *y_empty = y_full + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(y_empty + 1);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
-  // prologue scratch: a head's raw table column (256 entries), over its own group's k tile
-  auto raw_of = [&](int h) { return reinterpret_cast<uint16_t*>(sKV + h * KV_SLOT); };
 
   if (pad + (uint32_t)(reinterpret_cast<uint8_t*>(tmem_slot + 4) - smem) > g.smem_bytes) {
     if (threadIdx.x == 0) atomicExch(g.status, (int)SMARTMEM_ERR_UNSUPPORTED);
@@ -259,7 +259,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
   }
 #pragma unroll
   for (int k = 0; k < 2; ++k)
-    if (tid + k * kThreads < NH * 256) raw_of((tid + k * kThreads) >> 8)[(tid + k * kThreads) & 255] = tab[k];
+    if (tid + k * kThreads < NH * 256) raw_s[tid + k * kThreads] = tab[k];
   if (tid < C) {
     lng_s[tid] = par[0];
     ln_s[tid] = __bfloat162float(par[1]);
@@ -423,11 +423,11 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
     const uint32_t* brow = bias_s + (gi * T + (i < T ? i : 0)) * BR;
     const f32x2 scale2 = ptx::pack2(g.scale, g.scale), log2e2 = ptx::pack2(LOG2E, LOG2E);
     // This head's bias as a [T, T] table of bf16 pairs, -inf for the padded keys, built by the group itself while the first unit's
-    // rows are on their way (a task = a quarter of a row).  The barrier behind it: the raw column lies where the group's first k rows go.
+    // rows are on their way (a task = a quarter of a row).  The first group barrier below orders it before the first softmax.
     for (int task = (warp - 4 - 4 * gi) * 32 + lane; task < T * 4; task += 128) {
       const int r = task >> 2, qtr = task & 3;                        // row, quarter of the row's key pairs
       const int ry = tyx_s[r] >> 8, rx = tyx_s[r] & 255;
-      const uint16_t* tab = raw_of(gi) + (ry + ws - 1) * (2 * ws - 1) + (rx + ws - 1);
+      const uint16_t* tab = raw_s + gi * 256 + (ry + ws - 1) * (2 * ws - 1) + (rx + ws - 1);
 #pragma unroll 1
       for (int c2 = qtr * (KC / 8); c2 < (qtr + 1) * (KC / 8); ++c2) {
         uint32_t word = 0;
@@ -457,7 +457,6 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
           : "memory");
       return gave_up != 0;
     };
-    group_sync();
     for (int ul = 0; ul < U; ++ul) {
       const int it = ul * NH + gi;
       const int ab = ul % na;
@@ -848,7 +847,7 @@ static size_t fused_smem_need(int NH, int T, int na) {
   const int C = NH * D, br = T <= 56 ? 28 : 36;
   return (size_t)na * NH * KBT + (size_t)NH * KV_SLOT + (size_t)NH * NH * WQ_TILE + (size_t)NH * C * 64 +
          (size_t)na * AX_BYTES + (size_t)NH * WX_TILE + (size_t)ID_BYTES + (size_t)NH * T * br * 4 + (size_t)C * 4 +
-         (size_t)na * BM * 4 + (size_t)NRING * BM * 4 + (size_t)2 * C * 4 + TP * 4 + 16 + TP * 16 + 4 * 16 + 32 + N_BARS * 8 + 16;
+         (size_t)na * BM * 4 + (size_t)NRING * BM * 4 + (size_t)2 * C * 4 + TP * 4 + 16 + TP * 16 + 4 * 16 + 32 + NH * 512 + N_BARS * 8 + 16;
 }
 static constexpr size_t kMaxSmem = 232448;
 
@@ -899,7 +898,7 @@ int launch_swin_attn_fused(const smartmem_swin_params_t& p, const DevMap& rowmap
   if (!g.status) return SMARTMEM_ERR_CUDA;
   const bool kc56 = T <= 56;
   auto need = [&](int na) { return fused_smem_need(NH, T, na); };
-  g.na = need(3) <= kMaxSmem ? 3 : 2;
+  g.na = need(3) + 1024 <= kMaxSmem ? 3 : 2;
   if (need(g.na) > kMaxSmem) return SMARTMEM_ERR_UNSUPPORTED;
   const size_t smem = need(g.na) + 1024 <= kMaxSmem ? need(g.na) + 1024 : kMaxSmem;   // alignment slack only while it fits
   g.smem_bytes = (uint32_t)smem;
