@@ -41,6 +41,7 @@ struct OpCoord {
 struct GemmArgs {
   int M, N, K;
   int tiles_n, tiles_m, batch;
+  uint32_t wide_tiles;                   // 256-wide pair tiles from this one on come as two halves each (tile_item)
   FastDiv fd_tiles_n, fd_tiles_m;        // tile index -> (tile_n, tile_m, batch) without hardware division
   OpCoord ca, cb;
   __nv_bfloat16* out;
@@ -103,6 +104,28 @@ __device__ __forceinline__ TileIdx split_tile(uint32_t t, const FastDiv& fn, con
   return {t - r * fn.d, r - b * fm.d, b};
 }
 
+// The work items of a kernel: its tiles, and where 256-wide pair tiles leave a last round of which fewer than half the pairs have a
+// tile, that round's tiles as two 128-wide halves each.  A half takes 0.56 of a tile's time, so the round ends that much earlier.
+struct TileItem {
+  TileIdx ti;
+  int n_off;                             // first column of the item inside its tile
+  bool half;
+};
+template <bool HALVES>
+struct HalfMap {                         // tensor map of a half's B rows: only the kernels that take halves pay for the parameter
+  CUtensorMap map;
+};
+template <>
+struct HalfMap<false> {};
+template <bool HALVES>
+__device__ __forceinline__ TileItem tile_item(uint32_t t, const GemmArgs& g) {
+  if (HALVES && t >= g.wide_tiles) {
+    const uint32_t u = t - g.wide_tiles;
+    return {split_tile(g.wide_tiles + (u >> 1), g.fd_tiles_n, g.fd_tiles_m), (int)(u & 1) * 128, true};
+  }
+  return {split_tile(t, g.fd_tiles_n, g.fd_tiles_m), 0, false};
+}
+
 constexpr int kEpiWarps = 16;
 constexpr int kThreads = 64 + 32 * kEpiWarps + 32;      // + a second TMA producer warp (B operand)
 
@@ -123,7 +146,8 @@ constexpr int kThreads = 64 + 32 * kEpiWarps + 32;      // + a second TMA produc
 template <int BN, int STAGES, bool A_MN, bool PAIR, bool LEAN>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-               const __grid_constant__ CUtensorMap tmC, const __grid_constant__ GemmArgs g) {
+               const __grid_constant__ CUtensorMap tmC, const __grid_constant__ HalfMap<PAIR && BN == 256> tmBh,
+               const __grid_constant__ GemmArgs g) {
   static_assert(!PAIR || ((BN == 256 || BN == 128) && !A_MN), "CTA pairs: 256- or 128-wide tiles, K-major A");
   static_assert(!LEAN || BN % 128 == 0, "the lean epilogue's boxes are 32 columns wide");
   constexpr bool RES = !LEAN || BN == 128;                 // the epilogue can add a residual
@@ -132,6 +156,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   constexpr uint32_t ACC_COLS = BN <= 32 ? 32 : BN <= 64 ? 64 : BN <= 128 ? 128 : 256;   // one accumulator buffer
   constexpr uint32_t TMEM_COLS = 2 * ACC_COLS;
   constexpr uint32_t IDESC = ptx::make_idesc_bf16(PAIR ? 2 * BM : BM, BN, A_MN, false);
+  constexpr bool HALVES = PAIR && BN == 256;               // the last round's tiles may come as halves
+  const CUtensorMap* map_half = &tmB;
+  if constexpr (HALVES) map_half = &tmBh.map;
+  constexpr uint32_t IDESC_HALF = ptx::make_idesc_bf16(2 * BM, BN / 2, false, false);
 
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -155,7 +183,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int nkb = (g.K + BK - 1) / BK;
   const int last_ksteps = (g.K - (nkb - 1) * BK + 15) / 16;
   const bool two_producers = nkb >= 8;
-  const uint32_t total_tiles = (uint32_t)g.tiles_n * g.tiles_m * g.batch;   // PAIR: tiles_m counts 256-row tiles
+  const uint32_t tiles = (uint32_t)g.tiles_n * g.tiles_m * g.batch;         // PAIR: tiles_m counts 256-row tiles
+  const uint32_t total_tiles = HALVES ? 2 * tiles - g.wide_tiles : tiles;   // (work items)
   const uint32_t rank = PAIR ? ptx::cluster_ctarank() : 0u;                  // which half of the pair's tile
   const bool leader = rank == 0;
   const uint32_t cta_first = PAIR ? blockIdx.x >> 1 : blockIdx.x, cta_step = PAIR ? gridDim.x >> 1 : gridDim.x;
@@ -176,6 +205,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   if (warp == 0 && lane == 0) {
     ptx::prefetch_tensormap(&tmA);
     ptx::prefetch_tensormap(&tmB);
+    if constexpr (HALVES) {
+      if (g.wide_tiles < tiles) ptx::prefetch_tensormap(&tmBh.map);
+    }
     if (QTMA || (LEAN && g.tma_out)) ptx::prefetch_tensormap(&tmC);
   }
   if (warp == 1) {
@@ -202,18 +234,22 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     bool ok = true;
     const uint32_t full0 = PAIR ? ptx::mapa(ptx::smem_u32(full), 0) : 0u;     // the even CTA's `full` barriers
     for (uint32_t t = cta_first; t < total_tiles && ok; t += cta_step) {
-      const TileIdx ti_ = split_tile(t, g.fd_tiles_n, g.fd_tiles_m);
+      const TileItem item = tile_item<HALVES>(t, g);
+      const TileIdx& ti_ = item.ti;
       const uint32_t tile_n = ti_.tile_n, tile_m = PAIR ? 2 * ti_.tile_m + rank : ti_.tile_m, batch = ti_.batch;
       const TileCoord ta = op_coords(g.ca, tile_m, batch, BM), tb = op_coords(g.cb, tile_n, batch, BN);
-      const int brow0 = tb.row0 + (int)rank * BN_CTA;
+      const bool half = HALVES && item.half;
+      const int brow0 = tb.row0 + (HALVES ? item.n_off : 0) + (int)rank * (half ? BN_CTA / 2 : BN_CTA);
+      const uint32_t b_bytes = half ? B_STAGE_BYTES / 2 : B_STAGE_BYTES;
+      const CUtensorMap* mapB = half ? map_half : &tmB;
       for (int kb = 0; kb < nkb; ++kb, ++kbg) {
         ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(&empty[s], ph ^ 1, abort_flag, g.status) ? 1 : 0) != 0;
         if (!ok) break;
         if (ptx::elect_one()) {
           if constexpr (PAIR) {
-            if (leader) ptx::mbar_expect_tx(&full[s], 2 * (two_producers ? A_STAGE_BYTES : A_STAGE_BYTES + B_STAGE_BYTES));
+            if (leader) ptx::mbar_expect_tx(&full[s], 2 * (two_producers ? A_STAGE_BYTES : A_STAGE_BYTES + b_bytes));
             tma_load_op_pair(g.ca, sA + s * A_STAGE_BYTES, &tmA, full0 + s * 8, kb * BK, ta.row0, ta);
-            if (!two_producers) tma_load_op_pair(g.cb, sB + s * B_STAGE_BYTES, &tmB, full0 + s * 8, kb * BK, brow0, tb);
+            if (!two_producers) tma_load_op_pair(g.cb, sB + s * B_STAGE_BYTES, mapB, full0 + s * 8, kb * BK, brow0, tb);
           } else {
             ptx::mbar_expect_tx(&full[s], two_producers ? A_STAGE_BYTES : A_STAGE_BYTES + B_STAGE_BYTES);
             tma_load_op(g.ca, sA + s * A_STAGE_BYTES, &tmA, &full[s], kb * BK, ta.row0, ta);
@@ -255,6 +291,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (!ok) break;
         ptx::tc_fence_after();
         const uint32_t d_tmem = tmem_base + buf * ACC_COLS;
+        const uint32_t idesc = HALVES && t >= g.wide_tiles ? IDESC_HALF : IDESC;
         for (int kb = 0; kb < nkb; ++kb) {
           ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(&full[s], ph, abort_flag, g.status) ? 1 : 0) != 0;
           if (!ok) break;
@@ -269,7 +306,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           constexpr uint64_t A_STEP = (A_MN ? 2048 : 32) >> 4, B_STEP = 32 >> 4;
           const bool last_kb = kb == nkb - 1;
           auto mma = [&](uint64_t ad, uint64_t bd, uint32_t acc) {
-            if constexpr (PAIR) ptx::tc_mma_bf16_pair(d_tmem, ad, bd, IDESC, acc);
+            if constexpr (PAIR) ptx::tc_mma_bf16_pair(d_tmem, ad, bd, idesc, acc);
             else ptx::tc_mma_bf16(d_tmem, ad, bd, IDESC, acc);
           };
           if (ptx::elect_one()) {
@@ -301,17 +338,20 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       bool ok = true;
       const uint32_t full0 = PAIR ? ptx::mapa(ptx::smem_u32(full), 0) : 0u;
       for (uint32_t t = cta_first; t < total_tiles && ok; t += cta_step) {
-        const TileIdx ti_ = split_tile(t, g.fd_tiles_n, g.fd_tiles_m);
-        const uint32_t tile_n = ti_.tile_n, batch = ti_.batch;
+        const TileItem item = tile_item<HALVES>(t, g);
+        const uint32_t tile_n = item.ti.tile_n, batch = item.ti.batch;
         const TileCoord tb = op_coords(g.cb, tile_n, batch, BN);
-        const int brow0 = tb.row0 + (int)rank * BN_CTA;
+        const bool half = HALVES && item.half;
+        const int brow0 = tb.row0 + (HALVES ? item.n_off : 0) + (int)rank * (half ? BN_CTA / 2 : BN_CTA);
+        const uint32_t b_bytes = half ? B_STAGE_BYTES / 2 : B_STAGE_BYTES;
+        const CUtensorMap* mapB = half ? map_half : &tmB;
         for (int kb = 0; kb < nkb; ++kb) {
           ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(&empty[s], ph, abort_flag, g.status) ? 1 : 0) != 0;
           if (!ok) break;
           if (ptx::elect_one()) {
             if constexpr (PAIR) {
-              if (leader) ptx::mbar_expect_tx(&full[s], 2 * B_STAGE_BYTES);
-              tma_load_op_pair(g.cb, sB + s * B_STAGE_BYTES, &tmB, full0 + s * 8, kb * BK, brow0, tb);
+              if (leader) ptx::mbar_expect_tx(&full[s], 2 * b_bytes);
+              tma_load_op_pair(g.cb, sB + s * B_STAGE_BYTES, mapB, full0 + s * 8, kb * BK, brow0, tb);
             } else {
               ptx::mbar_expect_tx(&full[s], B_STAGE_BYTES);
               tma_load_op(g.cb, sB + s * B_STAGE_BYTES, &tmB, &full[s], kb * BK, tb.row0, tb);
@@ -352,10 +392,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint4 res_next[VPR];
     const uint32_t tmem_empty0 = PAIR ? ptx::mapa(ptx::smem_u32(tmem_empty), 0) : 0u;   // the even CTA's barriers
     for (uint32_t t = cta_first; t < total_tiles && ok; t += cta_step, ++it) {
-      const TileIdx ti_ = split_tile(t, g.fd_tiles_n, g.fd_tiles_m);
+      const TileItem item = tile_item<HALVES>(t, g);
+      const TileIdx& ti_ = item.ti;
       const uint32_t tile_n = ti_.tile_n, tile_m = PAIR ? 2 * ti_.tile_m + rank : ti_.tile_m, batch = ti_.batch;
       const uint32_t buf = it & 1, use = it >> 1;
-      const int n0 = tile_n * BN;
+      if (HALVES && item.half && grp >= 2) {                 // a half's 128 columns are the first two groups'
+        ok = ptx::mbar_wait(&tmem_full[buf], use & 1, abort_flag, g.status);
+        if (!ok) break;
+        if (lane == 0) ptx::mbar_arrive_cluster(tmem_empty0 + buf * 8);
+        continue;
+      }
+      const int n0 = tile_n * BN + (HALVES ? item.n_off : 0);
       const int row = tile_m * BM + q * 32 + lane;
       const bool row_ok = row < g.M;
       long long o2_base = 0;                                 // second copy: row = b * S + s goes to out2[b][col][s]
@@ -829,22 +876,25 @@ int sm_count() {
 }
 
 template <int BN, int STAGES, bool A_MN, bool PAIR = false, bool LEAN = false>
-int launch_t(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, const GemmArgs& g, cudaStream_t st) {
+int launch_t(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, const CUtensorMap& tbh, const GemmArgs& g, cudaStream_t st) {
   constexpr bool QST = !PAIR && !(BN == 256 && STAGES == 4);
   constexpr int RCc = !QST ? 16 : ((BN / 4) > 32 ? 32 : (BN / 4));
   constexpr size_t smem = 1024 + STAGES * (A_STAGE_BYTES + (PAIR ? BN / 2 : BN) * BK * 2) + (2 * STAGES + 4) * 8 + 16 +
                           (LEAN ? kEpiWarps * 32 * 64 : PAIR ? 0 : STAGES == 2 ? 2 * 4 * 32 * 512 : !QST ? kEpiWarps * 32 * (RCc * 2 + 16) : 4 * 32 * (BN * 2 + 16));   // pairs store from registers
   if (ensure_max_dynamic_smem((const void*)gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN>, (int)smem) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   profile_tick("gemm_tc", st);
-  const long long tiles = (long long)g.tiles_n * g.tiles_m * g.batch;
+  HalfMap<PAIR && BN == 256> hm;
+  if constexpr (PAIR && BN == 256) hm.map = tbh;
+  long long tiles = (long long)g.tiles_n * g.tiles_m * g.batch;
+  if (PAIR && BN == 256) tiles = 2 * tiles - g.wide_tiles;
   if constexpr (PAIR) {
     // one cluster of two CTAs per tile of 256 rows; the two CTAs of a cluster are neighbours in blockIdx.x
     const long long pairs = sm_count() / 2;
     const unsigned grid = (unsigned)(2 * (tiles < pairs ? tiles : pairs));
-    launch_pdl_cluster(gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN>, dim3(grid), dim3(kThreads), smem, st, 2u, ta, tb, tc, g);
+    launch_pdl_cluster(gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN>, dim3(grid), dim3(kThreads), smem, st, 2u, ta, tb, tc, hm, g);
   } else {
     const unsigned grid = (unsigned)(tiles < sm_count() ? tiles : sm_count());
-    launch_pdl(gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN>, dim3(grid), dim3(kThreads), smem, st, ta, tb, tc, g);
+    launch_pdl(gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN>, dim3(grid), dim3(kThreads), smem, st, ta, tb, tc, hm, g);
   }
   count_launch();
   return cudaGetLastError() == cudaSuccess ? SMARTMEM_OK : SMARTMEM_ERR_CUDA;
@@ -987,6 +1037,11 @@ TcOperand tc_operand_plain(const void* ptr, long long rows, long long K, long lo
   return op;
 }
 
+// The last round of 256-wide pair tiles in halves: where it is not the first and the halves still make one round.  Measured (us, whole
+// tiles -> halves): M = 435, K = 4096, N = 12288 (96 tiles on 74 pairs) 46.3 -> 42.2, M = 1268 (240) 108.8 -> 99.3, M = 2048 (384) 159.4 ->
+// 153.7; M = 12544, K = 512, N = 2048 (392) 24.2 -> 23.1; M = 20000, K = 512, N = 1024 21.3 -> 20.0.
+static bool tail_halves(long long tiles, long long pairs) { return tiles > pairs && tiles % pairs != 0 && 2 * (tiles % pairs) <= pairs; }
+
 int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep, long long batch, long long M,
                    long long N, long long K, cudaStream_t st) {
   if (M < 1 || N < 1 || K < 1 || batch < 1 ||  M >= (1ll << 31) || N >= (1ll << 31))
@@ -1021,7 +1076,7 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
   const bool lean128_ok = lean_ok && (lean256_ok || (N % 16 == 0 && ep.ldc % 16 == 0 && ((uintptr_t)ep.out & 31) == 0 && ((uintptr_t)ep.residual & 31) == 0 &&
                                                       (!ep.rowmap || devmap_offsets_multiple_of(*ep.rowmap, 16))));
   int bn = 128;
-  bool pair = false, lean = false;
+  bool pair = false, lean = false, halves = false;
   if (batch == 1) {
     // Tile width, and single CTAs or pairs: the smallest of the times fitted to measurements (us): a fixed part, the k-blocks of
     // the first tile, and for every further wave its k-blocks or, where the reduction is short, its epilogue.  A narrow tile
@@ -1044,8 +1099,10 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
       if (B.n_row_atoms > 1 && B.row_extent[B.n_row_atoms - 1] % o.bn) continue;
       const long long tiles = (o.pair ? (tiles_m1 + 1) / 2 : tiles_m1) * ((N + o.bn - 1) / o.bn), slots = tc_sm_count() / (o.pair ? 2 : 1);
       const double kbs = nkb * o.per_kb, wave = kbs + o.wave > o.wave_min ? kbs + o.wave : o.wave_min;
-      const double t = o.fixed + kbs + (double)((tiles + slots - 1) / slots - 1) * wave;
-      if (best == 0.0 || t < best) { best = t; bn = o.bn; pair = o.pair; lean = o.lean; }
+      double t = o.fixed + kbs + (double)((tiles + slots - 1) / slots - 1) * wave;
+      const bool tail = o.pair && o.bn == 256 && tail_halves(tiles, slots);
+      if (tail) t -= 0.44 * wave;
+      if (best == 0.0 || t < best) { best = t; bn = o.bn; pair = o.pair; lean = o.lean; halves = tail; }
     }
     if (splitk_ok && gemm_splitk_us(M, N, K) < best) return launch_gemm_splitk(A, B, ep, M, N, K, st);
   } else {
@@ -1118,6 +1175,14 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
   g.fd_tiles_m = make_fastdiv((uint32_t)g.tiles_m);
   g.batch = (int)batch;
   if ((long long)g.tiles_n * g.tiles_m * g.batch >= (1ll << 31)) return SMARTMEM_ERR_UNSUPPORTED;
+  const long long all_tiles = (long long)g.tiles_n * g.tiles_m * g.batch;
+  g.wide_tiles = (uint32_t)(halves ? all_tiles - all_tiles % (tc_sm_count() / 2) : all_tiles);
+  CUtensorMap tbh = tb;
+  if (halves) {
+    OpCoord same;
+    rc = build_operand(B, bn, bn / 4, &tbh, &same);
+    if (rc != SMARTMEM_OK) return rc;
+  }
   CUtensorMap tc = ta;                                     // (a valid map for the kernels that store without TMA)
   const bool pair_lean = pair && bn == 256 && nkb <= 16 && ep.rope_cols == 0 && !ep.residual;
   if ((pair_lean || lean) && batch == 1 && !ep.rowmap) {     // output as 32 x 32 boxes of [M, N] with pitch ldc
@@ -1127,19 +1192,19 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
     else if (lean) return SMARTMEM_ERR_CUDA;
     else tc = ta;
   }
-  if (pair_lean) return launch_t<256, 6, false, true, true>(ta, tb, tc, g, st);
-  if (lean) return bn == 128 ? launch_t<128, 5, false, false, true>(ta, tb, tc, g, st) : launch_t<256, 4, false, false, true>(ta, tb, tc, g, st);
-  if (pair && bn == 256) return launch_t<256, 6, false, true>(ta, tb, tc, g, st);
-  if (pair) return launch_t<128, 8, false, true>(ta, tb, tc, g, st);
+  if (pair_lean) return launch_t<256, 6, false, true, true>(ta, tb, tc, tbh, g, st);
+  if (lean) return bn == 128 ? launch_t<128, 5, false, false, true>(ta, tb, tc, tbh, g, st) : launch_t<256, 4, false, false, true>(ta, tb, tc, tbh, g, st);
+  if (pair && bn == 256) return launch_t<256, 6, false, true>(ta, tb, tc, tbh, g, st);
+  if (pair) return launch_t<128, 8, false, true>(ta, tb, tc, tbh, g, st);
   if (stages == 2) {
     const uint64_t dims[3] = {(uint64_t)N, (uint64_t)M, (uint64_t)batch};
     const uint64_t strides[2] = {(uint64_t)ep.ldc * 2, (uint64_t)(batch > 1 ? ep.out_batch_stride : ep.ldc * M) * 2};
     const uint32_t box[3] = {64, 32, 1};
-    if (encode_cached(ep.out, 3, dims, strides, box, &tc) == SMARTMEM_OK) return launch_t<256, 2, false>(ta, tb, tc, g, st);
+    if (encode_cached(ep.out, 3, dims, strides, box, &tc) == SMARTMEM_OK) return launch_t<256, 2, false>(ta, tb, tc, tbh, g, st);
     stages = 3;
   }
 #define SM_CASE(BN_, ST_, MN_)                                                                  \
-  if (bn == BN_ && stages == ST_ && a_mn == MN_) return launch_t<BN_, ST_, MN_>(ta, tb, tc, g, st);
+  if (bn == BN_ && stages == ST_ && a_mn == MN_) return launch_t<BN_, ST_, MN_>(ta, tb, tc, tbh, g, st);
   SM_CASE(256, 3, false) SM_CASE(256, 4, false) SM_CASE(128, 5, false) SM_CASE(96, 7, false) SM_CASE(64, 8, false)
   SM_CASE(256, 3, true) SM_CASE(256, 4, true) SM_CASE(128, 5, true)
 #undef SM_CASE

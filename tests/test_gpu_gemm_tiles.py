@@ -17,6 +17,8 @@ pytestmark = pytest.mark.gpu
     (300, 1024, 2048),       # pairs of CTAs, 128 wide, three row tiles: the last pair's second CTA has no rows
     (257, 2048, 4096),       # pairs, one row in the third tile
     (650, 3072, 1024),       # pairs, 256 wide
+    (400, 19200, 384),       # pairs, 256 wide, two tiles of the last round in halves
+    (513, 15616, 384),       # the same with 32 tiles in halves, one row in the last pair
 ])
 def test_linear_tile_choices(M, N, K):
     x = synth.normal(402, 0, (M, K), dtype="bf16")
