@@ -13,8 +13,15 @@
 //     distributed shared memory in the order of the CTAs.
 // Operands lie in shared memory with rows of K + 4 floats (an odd number of 16-byte vectors: eight lanes on eight rows hit
 // distinct banks), a thread computes TM x TN outputs with 16-byte reads along K.
-// [1,8,8,32] attention half (4 windows, 2 heads), us of a stream of calls: four kernels 16.7, one 9.4 (8.9 with the weights fetched
-// before the dependency wait, which nothing in front of the call would order).
+// What bounds the attention half is the length of its phases, one behind the other with a barrier between them, not their arithmetic (clock
+// stamps: 20 to 130 thousand cycles a window when it had 256 threads, a warp per row in LayerNorm and softmax, parameters read from
+// global memory where they were used, and index arithmetic per score).  So every phase is one round of one small tile a thread (512 threads
+// beyond 32 tokens), eight lanes share a row, parameters come to shared memory with the rows, and a token's place in the bias table and its
+// region are worked out once, ahead of the dependency wait.  Us of a stream of calls, that version -> this: [1,8,8,32] in 4 x 4 windows,
+// two heads of 16 9.3 -> 6.3 (the host's call); [1,28,28,96], 7 x 7, three heads of 32 34.2 -> 16.9; [16,28,28,96] 128 -> 84 (both resident
+// twice per SM: 64 registers; with 106 it was 100); [16,28,28,48], 4 x 4, three heads of 16 103 -> 56 (139 with 512 threads a window).
+// The MLP half had the same faults: [4,14,14,64] 12.3 -> 10.3, [128,14,14,96] 296 -> 265; one output row by two columns a thread instead of two by four
+// there: 307.
 #include <cstring>
 
 #include "attn.cuh"
@@ -24,39 +31,44 @@
 namespace smartmem {
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 256;                          // of the MLP half
 constexpr int kMaxCluster = 8;
 
-// out(r, c) = sum_k A[r][k] W[c][k] for r < M, c < N; K a multiple of 4; epi(r, c, value)
+// acc(i, j) = sum_k A[r0 + i][k] W[c0 + j * cs][k], rows and columns clamped to M and N (what lies beyond is not used); K a multiple of 4.
+template <int TM, int TN>
+__device__ __forceinline__ void tile_dot(const float* A, int pa, const float* W, int pw, int M, int N, int K, int r0, int c0, int cs, float (&acc)[TM][TN]) {
+  const float* a[TM];
+  const float* w[TN];
+#pragma unroll
+  for (int i = 0; i < TM; ++i) a[i] = A + min(r0 + i, M - 1) * pa;
+#pragma unroll
+  for (int j = 0; j < TN; ++j) w[j] = W + min(c0 + j * cs, N - 1) * pw;        // (neighbouring lanes on neighbouring rows)
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+#pragma unroll (TM * TN > 8 ? 1 : 2)
+  for (int k = 0; k < K; k += 4) {
+    float4 av[TM], wv[TN];
+#pragma unroll
+    for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const float4*>(a[i] + k);
+#pragma unroll
+    for (int j = 0; j < TN; ++j) wv[j] = *reinterpret_cast<const float4*>(w[j] + k);
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j)
+        acc[i][j] = fmaf(av[i].w, wv[j].w, fmaf(av[i].z, wv[j].z, fmaf(av[i].y, wv[j].y, fmaf(av[i].x, wv[j].x, acc[i][j]))));
+  }
+}
+// out(r, c) = sum_k A[r][k] W[c][k] for r < M, c < N; epi(r, c, value)
 template <int TM, int TN, typename Epi>
 __device__ __forceinline__ void tile_gemm(const float* A, int pa, const float* W, int pw, int M, int N, int K, Epi epi) {
   const int mt = (M + TM - 1) / TM, nt = (N + TN - 1) / TN;
   for (int idx = threadIdx.x; idx < mt * nt; idx += kThreads) {
     const int tm = idx / nt, tn = idx - tm * nt;
-    const float* a[TM];
-    const float* w[TN];
     float acc[TM][TN];
-#pragma unroll
-    for (int i = 0; i < TM; ++i) a[i] = A + min(tm * TM + i, M - 1) * pa;
-#pragma unroll
-    for (int j = 0; j < TN; ++j) w[j] = W + min(tn + j * nt, N - 1) * pw;      // (neighbouring lanes on neighbouring rows)
-#pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-      for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
-#pragma unroll 2
-    for (int k = 0; k < K; k += 4) {
-      float4 av[TM], wv[TN];
-#pragma unroll
-      for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const float4*>(a[i] + k);
-#pragma unroll
-      for (int j = 0; j < TN; ++j) wv[j] = *reinterpret_cast<const float4*>(w[j] + k);
-#pragma unroll
-      for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j)
-          acc[i][j] = fmaf(av[i].w, wv[j].w, fmaf(av[i].z, wv[j].z, fmaf(av[i].y, wv[j].y, fmaf(av[i].x, wv[j].x, acc[i][j]))));
-    }
+    tile_dot<TM, TN>(A, pa, W, pw, M, N, K, tm * TM, tn, nt, acc);
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
@@ -64,39 +76,51 @@ __device__ __forceinline__ void tile_gemm(const float* A, int pa, const float* W
         if (tm * TM + i < M && tn + j * nt < N) epi(tm * TM + i, tn + j * nt, acc[i][j]);
   }
 }
-// four rows x four columns per thread where that still gives most threads a tile, else two x two
-template <typename Epi>
-__device__ __forceinline__ void gemm_any(const float* A, int pa, const float* W, int pw, int M, int N, int K, Epi epi) {
-  if (M * N >= 16 * 160) tile_gemm<4, 4>(A, pa, W, pw, M, N, K, epi);
-  else tile_gemm<2, 2>(A, pa, W, pw, M, N, K, epi);
-}
 
 // rows [0, n) of `vpr.d` 16-byte vectors from global memory (row r at src(r)) into shared memory with pitch `pitch`
-template <typename Src>
+template <int THREADS, typename Src>
 __device__ __forceinline__ void load_rows(float* dst, int pitch, int n, const FastDiv& vpr, Src src) {
 #pragma unroll 1                                       // (runs once: the unrolled form costs more in instruction fetches)
-  for (int i = threadIdx.x; i < n * (int)vpr.d; i += kThreads) {
+  for (int i = threadIdx.x; i < n * (int)vpr.d; i += THREADS) {
     const int r = (int)fd_div((uint32_t)i, vpr), v = i - r * (int)vpr.d;
     ptx::cp_async16(dst + r * pitch + v * 4, src(r) + v * 4);
   }
 }
-__device__ __forceinline__ float warp_sum(float v) {
+template <int LANES>
+__device__ __forceinline__ float lanes_sum(float v) {
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+  for (int o = LANES / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
   return v;
 }
-// LayerNorm of `n` rows in place (a warp per row; mean, then centred squares)
-__device__ __forceinline__ void norm_rows(float* x, int pitch, int n, int C, const float* __restrict__ g, const float* __restrict__ b, float eps) {
-  const int lane = threadIdx.x & 31;
-  for (int r = threadIdx.x >> 5; r < n; r += kThreads / 32) {
-    float* p = x + r * pitch;
+// LayerNorm of `n` rows in place, LANES lanes per row (mean, then centred squares); gamma and beta in shared memory
+template <int THREADS, int LANES>
+__device__ __forceinline__ void norm_rows(float* x, int pitch, int n, int C, const float* g, const float* b, float eps) {
+  const int l = threadIdx.x & (LANES - 1);
+  const float inv = 1.0f / (float)C;
+  for (int r0 = 0; r0 < n; r0 += THREADS / LANES) {    // (all lanes of a warp run all rounds: shuffles)
+    const int r = r0 + (int)threadIdx.x / LANES;
+    const bool in = r < n;
+    float4* p = reinterpret_cast<float4*>(x + min(r, n - 1) * pitch);
+    const int nv = C / 4;
     float s = 0.f;
-    for (int c = lane; c < C; c += 32) s += p[c];
-    const float mean = warp_sum(s) / (float)C;
+#pragma unroll 2
+    for (int c = l; c < nv; c += LANES) { const float4 v = p[c]; s += (v.x + v.y) + (v.z + v.w); }
+    const float mean = lanes_sum<LANES>(s) * inv;
     float q = 0.f;
-    for (int c = lane; c < C; c += 32) q = fmaf(p[c] - mean, p[c] - mean, q);
-    const float rstd = rsqrtf(warp_sum(q) / (float)C + eps);
-    for (int c = lane; c < C; c += 32) p[c] = fmaf((p[c] - mean) * rstd, g[c], b[c]);
+#pragma unroll 2
+    for (int c = l; c < nv; c += LANES) {
+      const float4 v = p[c];
+      const float a0 = v.x - mean, a1 = v.y - mean, a2 = v.z - mean, a3 = v.w - mean;
+      q += fmaf(a0, a0, a1 * a1) + fmaf(a2, a2, a3 * a3);
+    }
+    const float rstd = rsqrtf(lanes_sum<LANES>(q) * inv + eps);
+    if (in)
+#pragma unroll 2
+      for (int c = l; c < nv; c += LANES) {
+        const float4 v = p[c], gv = reinterpret_cast<const float4*>(g)[c], bv = reinterpret_cast<const float4*>(b)[c];
+        p[c] = make_float4(fmaf((v.x - mean) * rstd, gv.x, bv.x), fmaf((v.y - mean) * rstd, gv.y, bv.y), fmaf((v.z - mean) * rstd, gv.z, bv.z),
+                           fmaf((v.w - mean) * rstd, gv.w, bv.w));
+      }
   }
 }
 
@@ -105,12 +129,34 @@ struct AttnF32Args {
   float* y;
   int C, heads, d, T, ws, shift, H, W, nWw, win_per_img;
   float eps, scale;
-  FastDiv fd_vpr, fd_d;                                // vectors of a row, head dimension
+  FastDiv fd_vpr, fd_d, fd_ws;                         // vectors of a row, head dimension, window
   int tp;                                              // pitch of P and of v transposed: T rounded up to an odd number of vectors
   DevMap rowmap;
 };
 
-__global__ void __launch_bounds__(kThreads) swin_attn_f32_kernel(const __grid_constant__ AttnF32Args g) {
+// q, k and v of one head: a TM x TN tile a thread
+template <int TM, int TN>
+__device__ __forceinline__ void qkv_phase(const AttnF32Args& g, const float* xs, int pc, const float* wq, const float* bq, float* q, float* k, float* vt, int pd) {
+  const int d = g.d, T = g.T, nt = 3 * d / TN;
+  const int tm = (int)threadIdx.x / nt, tn = (int)threadIdx.x - tm * nt;
+  if (tm * TM >= T) return;
+  float acc[TM][TN];
+  tile_dot<TM, TN>(xs, pc, wq, pc, T, 3 * d, g.C, tm * TM, tn, nt, acc);
+#pragma unroll
+  for (int j = 0; j < TN; ++j) {
+    const int c = tn + j * nt, which = c < d ? 0 : c < 2 * d ? 1 : 2, e = c - which * d;
+    const float b = bq[c], sc = which == 0 ? g.scale : 1.0f;
+    float* dst = which == 0 ? q + tm * TM * pd + e : which == 1 ? k + tm * TM * pd + e : vt + e * g.tp + tm * TM;
+    const int step = which == 2 ? 1 : pd;
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+      if (tm * TM + i < T) dst[i * step] = (acc[i][j] + b) * sc;
+  }
+}
+
+// THREADS: 256 up to 32 tokens, else 512: one output tile a thread in every phase.
+template <int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 3 : 2) swin_attn_f32_kernel(const __grid_constant__ AttnF32Args g) {
   extern __shared__ __align__(16) float sm[];
   const int C = g.C, d = g.d, T = g.T, pc = C + 4, pd = d + 4, tp = g.tp;
   float* xs = sm;                                      // [T][C]: the normalised rows, later every head's output
@@ -120,81 +166,140 @@ __global__ void __launch_bounds__(kThreads) swin_attn_f32_kernel(const __grid_co
   float* k = q + T * pd;                               // [T][d]
   float* vt = k + T * pd;                              // [d][T], zero beyond T
   float* P = vt + d * tp;                              // [T][T], zero beyond T
-  float* tab = P + T * tp;                             // the head's column of the bias table
-  long long* offs = reinterpret_cast<long long*>(tab + (((2 * g.ws - 1) * (2 * g.ws - 1) + 3) & ~3));
+  float* lng = P + T * tp;                             // gamma and beta [C], biases of q, k, v [3 d] and of the projection [d]
+  float* lnb = lng + C;
+  float* bq = lnb + C;
+  float* bp = bq + 3 * d;
+  const int nt = (2 * g.ws - 1) * (2 * g.ws - 1);
+  float* tab = bp + d;                                 // the head's column of the bias table
+  long long* offs = reinterpret_cast<long long*>(tab + ((nt + 3) & ~3));
+  int* code = reinterpret_cast<int*>(offs + T);        // a token's place in the bias table (differences index it) and its region
+  int* label = code + T;
   const int h = g.heads > 1 ? (int)ptx::cluster_ctarank() : 0;
   const int n = (int)blockIdx.x / g.heads;             // window
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
 
   // The head's weights as far as L2: they may still be written by the kernel before this one.  (A line per 32 floats of a head's rows,
   // which lie one behind the other.)
-  for (int i = tid * 32; i < d * C; i += kThreads * 32) {
+  for (int i = tid * 32; i < d * C; i += THREADS * 32) {
     for (int which = 0; which < 3; ++which) ptx::prefetch_l2(g.w_qkv + (size_t)(which * C + h * d) * C + i);
     ptx::prefetch_l2(g.w_proj + (size_t)h * d * C + i);
   }
-  for (int i = tid; i < T; i += kThreads) offs[i] = devmap_eval(g.rowmap, (uint32_t)(n * T + i));
-  for (int i = tid; i < d * tp; i += kThreads) vt[i] = 0.f;
-  for (int i = tid; i < T * tp; i += kThreads) P[i] = 0.f;
+  if (tid < T) {
+    offs[tid] = devmap_eval(g.rowmap, (uint32_t)(n * T + tid));
+    const int wl = n % g.win_per_img, wy = wl / g.nWw, wx = wl - wy * g.nWw;
+    const int ty = (int)fd_div((uint32_t)tid, g.fd_ws), tx = tid - ty * g.ws;
+    code[tid] = ty * (2 * g.ws - 1) + tx;
+    label[tid] = g.shift > 0 ? region_label2(ty, tx, g.ws, wy, wx, g.H, g.W, g.shift) : 0;
+  }
+  for (int i = tid; i < d * tp; i += THREADS) vt[i] = 0.f;
+  for (int i = tid; i < T * tp; i += THREADS) P[i] = 0.f;
   __syncthreads();
   pdl_wait();
   pdl_launch_dependents();
-  load_rows(xs, pc, T, g.fd_vpr, [&](int r) { return g.x + offs[r]; });
-  // (rows of q, k, v and of the projection lie one behind the other in shared memory)
-  load_rows(wq, pc, 4 * d, g.fd_vpr, [&](int r) {
+  load_rows<THREADS>(xs, pc, T, g.fd_vpr, [&](int r) { return g.x + offs[r]; });
+  for (int i = tid; i < C / 2; i += THREADS)
+    ptx::cp_async16(lng + i * 4, (i < C / 4 ? g.ln_g : g.ln_b - C) + i * 4);
+  ptx::cp_async_commit();
+  // (rows of q, k, v and of the projection lie one behind the other in shared memory, and so do their biases)
+  load_rows<THREADS>(wq, pc, 4 * d, g.fd_vpr, [&](int r) {
     const int which = (int)fd_div((uint32_t)r, g.fd_d), e = h * d + r - which * d;
     return which < 3 ? g.w_qkv + (size_t)(which * C + e) * C : g.w_proj + (size_t)e * C;
   });
   ptx::cp_async_commit();
-  const int nt = (2 * g.ws - 1) * (2 * g.ws - 1);
-  for (int i = tid; i < nt; i += kThreads) tab[i] = g.table[i * g.heads + h];
+  for (int i = tid; i < 4 * d + nt; i += THREADS) {
+    const int which = (int)fd_div((uint32_t)i, g.fd_d), e = h * d + i - which * d;
+    bq[i] = i >= 4 * d ? g.table[(i - 4 * d) * g.heads + h] : which < 3 ? g.b_qkv[which * C + e] : g.b_proj[e];
+  }
+  ptx::cp_async_wait<1>();
+  __syncthreads();
+  norm_rows<THREADS, 8>(xs, pc, T, C, lng, lnb, g.eps);
   ptx::cp_async_wait<0>();
   __syncthreads();
-  norm_rows(xs, pc, T, C, g.ln_g, g.ln_b, g.eps);
+  // the smallest tile that gives no thread two (T at most 64 and d 16 or 32: at most 192 and 384 of the largest)
+  const int t2 = (T + 1) / 2;
+  if (t2 * (3 * d / 2) <= THREADS) qkv_phase<2, 2>(g, xs, pc, wq, bq, q, k, vt, pd);
+  else if (t2 * (3 * d / 4) <= THREADS) qkv_phase<2, 4>(g, xs, pc, wq, bq, q, k, vt, pd);
+  else qkv_phase<4, 4>(g, xs, pc, wq, bq, q, k, vt, pd);
   __syncthreads();
-  gemm_any(xs, pc, wq, pc, T, 3 * d, C, [&](int r, int c, float v) {
-    const int which = c / d, e = c - which * d;
-    v += g.b_qkv[which * C + h * d + e];
-    if (which == 0) q[r * pd + e] = v * g.scale;
-    else if (which == 1) k[r * pd + e] = v;
-    else vt[e * tp + r] = v;
-  });
-  __syncthreads();
-  const int wl = n % g.win_per_img, wy = wl / g.nWw, wx = wl - wy * g.nWw;
-  gemm_any(q, pd, k, pd, T, T, d, [&](int i, int j, float s) {
-    const int ty = i / g.ws, tx = i - ty * g.ws, sy = j / g.ws, sx = j - sy * g.ws;
-    s += tab[(ty - sy + g.ws - 1) * (2 * g.ws - 1) + tx - sx + g.ws - 1];
-    if (g.shift > 0 && region_label2(ty, tx, g.ws, wy, wx, g.H, g.W, g.shift) != region_label2(sy, sx, g.ws, wy, wx, g.H, g.W, g.shift)) s -= 100.f;
-    P[i * tp + j] = s;
-  });
-  __syncthreads();
-  for (int i = warp; i < T; i += kThreads / 32) {      // softmax: a warp per row, at most two keys per lane
-    float* p = P + i * tp;
-    const float a = lane < T ? p[lane] : -INFINITY, b = lane + 32 < T ? p[lane + 32] : -INFINITY;
-    float m = fmaxf(a, b);
+  {
+    const int nk = (T + 3) / 4;
+    const int tm = tid / nk, tn = tid - tm * nk;
+    if (tm * 2 < T) {
+      float acc[2][4];
+      tile_dot<2, 4>(q, pd, k, pd, T, T, d, tm * 2, tn, nk, acc);
+      const int i0 = tm * 2, i1 = min(i0 + 1, T - 1), mid = (g.ws - 1) * 2 * g.ws;
+      const int c0 = code[i0] + mid, c1 = code[i1] + mid, l0 = label[i0], l1 = label[i1];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
-    const float ea = lane < T ? expf(a - m) : 0.f, eb = lane + 32 < T ? expf(b - m) : 0.f;
-    const float inv = 1.0f / warp_sum(ea + eb);
-    if (lane < T) p[lane] = ea * inv;
-    if (lane + 32 < T) p[lane + 32] = eb * inv;
+      for (int j = 0; j < 4; ++j) {
+        const int col = tn + j * nk;
+        if (col < T) {
+          const int cc = code[col], lc = label[col];
+          P[i0 * tp + col] = acc[0][j] + tab[c0 - cc] - (l0 != lc ? 100.f : 0.f);
+          if (i0 + 1 < T) P[i1 * tp + col] = acc[1][j] + tab[c1 - cc] - (l1 != lc ? 100.f : 0.f);
+        }
+      }
+    }
   }
   __syncthreads();
-  // o of this head goes straight into every CTA's row buffer: column h d + c of all of them
-  uint32_t peer[kMaxCluster];
+  {                                                    // softmax: eight lanes per row, eight keys per lane
+    const int r = min(tid >> 3, T - 1), l = tid & 7;
+    float* p = P + r * tp;
+    float v[8], m = -INFINITY;
 #pragma unroll
-  for (int r = 0; r < kMaxCluster; ++r) peer[r] = r < g.heads ? (g.heads > 1 ? ptx::mapa(ptx::smem_u32(xs), (uint32_t)r) : ptx::smem_u32(xs)) : 0u;
-  if (g.heads > 1) ptx::cluster_sync();                // everyone has read its normalised rows
-  gemm_any(P, tp, vt, tp, T, d, (T + 3) & ~3, [&](int i, int c, float v) {
-    const uint32_t o = (uint32_t)(i * pc + h * d + c) * 4u;
+    for (int j = 0; j < 8; ++j) {
+      v[j] = l + 8 * j < T ? p[l + 8 * j] : -INFINITY;
+      m = fmaxf(m, v[j]);
+    }
 #pragma unroll
-    for (int r = 0; r < kMaxCluster; ++r)
-      if (r < g.heads) ptx::st_cluster_f32(peer[r] + o, v);
-  });
-  if (g.heads > 1) ptx::cluster_sync(); else __syncthreads();
-  gemm_any(xs, pc, wp, pc, T, d, C, [&](int i, int c, float v) {
-    const long long o = offs[i] + h * d + c;
-    g.y[o] = v + g.b_proj[h * d + c] + g.x[o];
-  });
+    for (int o = 4; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xFFFFFFFFu, m, o));
+    float s = 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      v[j] = l + 8 * j < T ? expf(v[j] - m) : 0.f;
+      s += v[j];
+    }
+    const float inv = 1.0f / lanes_sum<8>(s);
+    if ((tid >> 3) < T)
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (l + 8 * j < T) p[l + 8 * j] = v[j] * inv;
+  }
+  __syncthreads();
+  // o of this head goes straight into every CTA's row buffer: column h d + c of all of them.  A thread has the same two rows and two
+  // columns of it and of the projection.
+  const int tm = tid / (d / 2), c0 = tid - tm * (d / 2), c1 = c0 + d / 2, r0 = tm * 2;
+  const bool in0 = r0 < T, in1 = r0 + 1 < T;
+  float acc[2][2], res[2][2] = {};
+  const long long o0 = in0 ? offs[r0] + h * d : 0, o1 = in1 ? offs[r0 + 1] + h * d : 0;
+  if (in0) { res[0][0] = g.x[o0 + c0]; res[0][1] = g.x[o0 + c1]; }
+  if (in1) { res[1][0] = g.x[o1 + c0]; res[1][1] = g.x[o1 + c1]; }
+  if (g.heads > 1) ptx::cluster_arrive();              // (everyone has read its normalised rows)
+  if (in0) tile_dot<2, 2>(P, tp, vt, tp, T, d, (T + 3) & ~3, r0, c0, d / 2, acc);
+  if (g.heads > 1) ptx::cluster_wait();
+  if (in0) {
+    const uint32_t xa = ptx::smem_u32(xs), o = (uint32_t)(r0 * pc + h * d + c0) * 4u;
+#pragma unroll 1
+    for (int r = 0; r < g.heads; ++r) {
+      const uint32_t peer = (g.heads > 1 ? ptx::mapa(xa, (uint32_t)r) : xa) + o;
+      ptx::st_cluster_f32(peer, acc[0][0]);
+      ptx::st_cluster_f32(peer + d * 2, acc[0][1]);
+      if (in1) {
+        ptx::st_cluster_f32(peer + pc * 4, acc[1][0]);
+        ptx::st_cluster_f32(peer + pc * 4 + d * 2, acc[1][1]);
+      }
+    }
+  }
+  if (g.heads > 1) { __syncwarp(); ptx::cluster_sync(); } else __syncthreads();
+  if (in0) {
+    tile_dot<2, 2>(xs, pc, wp, pc, T, d, C, r0, c0, d / 2, acc);
+    g.y[o0 + c0] = acc[0][0] + bp[c0] + res[0][0];
+    g.y[o0 + c1] = acc[0][1] + bp[c1] + res[0][1];
+    if (in1) {
+      g.y[o1 + c0] = acc[1][0] + bp[c0] + res[1][0];
+      g.y[o1 + c1] = acc[1][1] + bp[c1] + res[1][1];
+    }
+  }
 }
 
 struct MlpF32Args {
@@ -202,7 +307,7 @@ struct MlpF32Args {
   float* y;
   int M, C, hidden, slice, splits;
   float eps;
-  FastDiv fd_vpr, fd_vps;                              // vectors of a row, of a slice
+  FastDiv fd_vpr, fd_vps, fd_C;                        // vectors of a row, of a slice; floats of a row
 };
 constexpr int kMlpRows = 16;
 
@@ -214,22 +319,34 @@ __global__ void __launch_bounds__(kThreads) swin_mlp_f32_kernel(const MlpF32Args
   float* w2 = w1 + hs * pc;                            // [C][slice]
   float* hid = w2 + C * ph;                            // [16][slice]
   float* part = hid + kMlpRows * ph;                   // [16][C]: this slice's share of fc2
+  float* lng = part + kMlpRows * C;                    // gamma, beta, the second bias [C], the first [slice]
+  float* lnb = lng + C;
+  float* b2 = lnb + C;
+  float* b1 = b2 + C;
   const int rank = g.splits > 1 ? (int)ptx::cluster_ctarank() : 0;
   const int m0 = (int)blockIdx.x / g.splits * kMlpRows, rows = min(kMlpRows, g.M - m0);
-  load_rows(w1, pc, hs, g.fd_vpr, [&](int r) { return g.w1 + (size_t)(rank * hs + r) * C; });
-  load_rows(w2, ph, C, g.fd_vps, [&](int r) { return g.w2 + (size_t)r * g.hidden + rank * hs; });
+  load_rows<kThreads>(w1, pc, hs, g.fd_vpr, [&](int r) { return g.w1 + (size_t)(rank * hs + r) * C; });
+  load_rows<kThreads>(w2, ph, C, g.fd_vps, [&](int r) { return g.w2 + (size_t)r * g.hidden + rank * hs; });
+  const int C4 = C / 4, h4 = hs / 4;
+  for (int i = threadIdx.x; i < 3 * C4 + h4; i += kThreads)
+    ptx::cp_async16(lng + i * 4, (i < C4 ? g.ln_g : i < 2 * C4 ? g.ln_b - C : i < 3 * C4 ? g.b2 - 2 * C : g.b1 + rank * hs - 3 * C) + i * 4);
   ptx::cp_async_commit();
   pdl_wait();
   pdl_launch_dependents();
-  load_rows(xs, pc, rows, g.fd_vpr, [&](int r) { return g.x + (size_t)(m0 + r) * C; });
+  load_rows<kThreads>(xs, pc, rows, g.fd_vpr, [&](int r) { return g.x + (size_t)(m0 + r) * C; });
   ptx::cp_async_commit();
   ptx::cp_async_wait<0>();
   __syncthreads();
-  norm_rows(xs, pc, rows, C, g.ln_g, g.ln_b, g.eps);
+  norm_rows<kThreads, 16>(xs, pc, rows, C, lng, lnb, g.eps);
   __syncthreads();
-  tile_gemm<2, 4>(xs, pc, w1, pc, rows, hs, C, [&](int r, int c, float v) { hid[r * ph + c] = gelu_erf(v + g.b1[rank * hs + c]); });
+  // (eight outputs a thread, but for the narrowest: latency is all they cost)
+  auto gelu_out = [&](int r, int c, float v) { hid[r * ph + c] = gelu_erf(v + b1[c]); };
+  if (hs >= 48) tile_gemm<2, 4>(xs, pc, w1, pc, rows, hs, C, gelu_out);
+  else tile_gemm<1, 2>(xs, pc, w1, pc, rows, hs, C, gelu_out);
   __syncthreads();
-  tile_gemm<2, 4>(hid, ph, w2, ph, rows, C, hs, [&](int r, int c, float v) { part[r * C + c] = v; });
+  auto part_out = [&](int r, int c, float v) { part[r * C + c] = v; };
+  if (C >= 48) tile_gemm<2, 4>(hid, ph, w2, ph, rows, C, hs, part_out);
+  else tile_gemm<1, 2>(hid, ph, w2, ph, rows, C, hs, part_out);
   if (g.splits > 1) ptx::cluster_sync(); else __syncthreads();
   const int ra = rows * rank / g.splits, rb = rows * (rank + 1) / g.splits;            // this CTA finishes a share of the rows
   for (int i = ra * C + (int)threadIdx.x; i < rb * C; i += kThreads) {
@@ -244,7 +361,7 @@ __global__ void __launch_bounds__(kThreads) swin_mlp_f32_kernel(const MlpF32Args
       v = part[i];
     }
     const size_t o = (size_t)m0 * C + i;
-    g.y[o] = v + g.b2[i % C] + g.x[o];
+    g.y[o] = v + b2[i - (int)fd_div((uint32_t)i, g.fd_C) * C] + g.x[o];
   }
   if (g.splits > 1) ptx::cluster_sync();               // no CTA leaves while its share is still being read
 }
@@ -253,10 +370,10 @@ __global__ void __launch_bounds__(kThreads) swin_mlp_f32_kernel(const MlpF32Args
 int pitch_of(int n) { return (((n + 3) >> 2) | 1) << 2; }
 size_t attn_f32_smem(int C, int d, int T, int ws) {
   const size_t pc = C + 4, pd = d + 4, tp = pitch_of(T), nt = ((2 * ws - 1) * (2 * ws - 1) + 3) & ~3;
-  return (T * pc + 4 * d * pc + 2 * T * pd + d * tp + T * tp + nt) * 4 + (size_t)T * 8;
+  return (T * pc + 4 * d * pc + 2 * T * pd + d * tp + T * tp + 2 * C + 4 * d + nt) * 4 + (size_t)T * 16;
 }
 size_t mlp_f32_smem(int C, int slice) {
-  return ((size_t)kMlpRows * (C + 4) + (size_t)slice * (C + 4) + (size_t)C * (slice + 4) + (size_t)kMlpRows * (slice + 4) + (size_t)kMlpRows * C) * 4;
+  return ((size_t)kMlpRows * (C + 4) + (size_t)slice * (C + 4) + (size_t)C * (slice + 4) + (size_t)kMlpRows * (slice + 4) + (size_t)kMlpRows * C + 3 * C + slice) * 4;
 }
 constexpr size_t kMaxSmem = 227 * 1024;
 // the fewest slices of the hidden features (4 or 8) that fit
@@ -270,19 +387,20 @@ int mlp_f32_splits(int C, int hidden) {
 
 bool swin_attn_f32_supported(int C, int heads, int window) {
   const int d = C / heads, T = window * window;
-  return heads <= kMaxCluster && C % 4 == 0 && d % 4 == 0 && T <= 64 && attn_f32_smem(C, d, T, window) <= kMaxSmem;
+  return heads <= kMaxCluster && C % 4 == 0 && (d == 16 || d == 32) && T <= 64 && attn_f32_smem(C, d, T, window) <= kMaxSmem;
 }
 bool swin_mlp_f32_supported(int C, long long hidden) { return C % 4 == 0 && hidden < (1 << 20) && mlp_f32_splits(C, (int)hidden) > 0; }
 
-// Every cluster of sixteen rows loads the weights and walks through its phases on its own, about 0.055 us of a full chip beside its
+// Every cluster of sixteen rows loads the weights and walks through its phases on its own, about 0.04 us of a full chip beside its
 // products; the tiled kernels spend next to nothing per row but run their products at less than half the rate, and their launches cost
-// more.  Both estimates in us, fitted to (cluster / LayerNorm and two linears, hidden = 4 C): 784 x 32 8.0 / 9.8, 3136 x 32 17.6 / 16.2,
-// 25088 x 32 111 / 72, 784 x 48 12.0 / 15.6, 25088 x 48 141 / 147, 25088 x 64 161 / 257, 50176 x 96 554 / 1170, 12544 x 192 802 / 1088,
-// 12544 x 256 1935 / 1929; hidden = C: 784 x 16 6.7 / 6.9, 25088 x 16 88 / 11, 25088 x 64 118 / 72.
+// more.  Both estimates in us, fitted to (cluster / LayerNorm and two linears, hidden = 4 C): 784 x 32 8.2 / 10.5, 3136 x 32 14.4 / 16.2,
+// 6272 x 32 25.6 / 24.5, 25088 x 32 86 / 70, 784 x 48 9.4 / 14.3, 25088 x 48 114 / 143, 25088 x 64 133 / 252, 25088 x 96 265 / 553,
+// 25088 x 192 1486 / 2165; hidden = C: 1568 x 16 6.2 / 8.6, 3136 x 16 11.3 / 8.1, 25088 x 16 63 / 10, 3136 x 64 14.4 / 16.3, 25088 x 64 84 / 70.
+// (Within an eighth of one another the separate kernels keep the block.)
 bool swin_mlp_f32_wins(long long M, int C, long long hidden) {
   if (!swin_mlp_f32_supported(C, hidden)) return false;
   const double groups = (double)((M + kMlpRows - 1) / kMlpRows), mflop = 4e-6 * kMlpRows * C * (double)hidden;
-  return 4.5 + groups * (0.055 + mflop / 15.0) < 8.0 + groups * (mflop / 6.4);
+  return 4.5 + groups * (0.044 + mflop / 17.0) < 8.0 + groups * (mflop / 6.4);
 }
 
 int launch_swin_attn_f32(const smartmem_swin_params_t& p, const DevMap& rowmap, const void* x, void* y, cudaStream_t st) {
@@ -297,13 +415,15 @@ int launch_swin_attn_f32(const smartmem_swin_params_t& p, const DevMap& rowmap, 
   g.tp = pitch_of(g.T);
   g.fd_vpr = make_fastdiv((uint32_t)g.C / 4);
   g.fd_d = make_fastdiv((uint32_t)g.d);
+  g.fd_ws = make_fastdiv((uint32_t)g.ws);
   g.rowmap = rowmap;
   const long long ctas = (long long)p.B * g.win_per_img * p.heads;
   if (ctas >= (1ll << 31) || (long long)p.B * p.H * p.W >= (1ll << 31)) return SMARTMEM_ERR_UNSUPPORTED;
   const size_t smem = attn_f32_smem(g.C, g.d, g.T, g.ws);
-  if (ensure_max_dynamic_smem((const void*)swin_attn_f32_kernel, (int)kMaxSmem) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
+  auto kernel = g.T <= 32 ? swin_attn_f32_kernel<256> : swin_attn_f32_kernel<512>;
+  if (ensure_max_dynamic_smem((const void*)kernel, (int)kMaxSmem) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   profile_tick("swin_attn_f32", st);
-  if (launch_pdl_cluster(swin_attn_f32_kernel, dim3((unsigned)ctas), dim3(kThreads), smem, st, (unsigned)p.heads, g) != cudaSuccess) return SMARTMEM_ERR_CUDA;
+  if (launch_pdl_cluster(kernel, dim3((unsigned)ctas), dim3(g.T <= 32 ? 256 : 512), smem, st, (unsigned)p.heads, g) != cudaSuccess) return SMARTMEM_ERR_CUDA;
   count_launch();
   return SMARTMEM_OK;
 }
@@ -320,6 +440,7 @@ int launch_swin_mlp_f32(const smartmem_swin_params_t& p, const void* x, void* y,
   g.slice = g.hidden / g.splits;
   g.fd_vpr = make_fastdiv((uint32_t)g.C / 4);
   g.fd_vps = make_fastdiv((uint32_t)g.slice / 4);
+  g.fd_C = make_fastdiv((uint32_t)g.C);
   const long long ctas = (M + kMlpRows - 1) / kMlpRows * g.splits;
   if (ctas >= (1ll << 31)) return SMARTMEM_ERR_UNSUPPORTED;
   const size_t smem = mlp_f32_smem(g.C, g.slice);
