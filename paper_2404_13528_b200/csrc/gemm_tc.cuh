@@ -125,5 +125,9 @@ int launch_gemm_ln_pair(const void* X, const smartmem_index_map_t& map, const vo
 // row gather / row scatter through `rowmap` (windowed row -> element offset of the token in x and y).  x and y must not alias.
 bool swin_attn_fused_supported(int dtype, int C, int heads, int window);
 int launch_swin_attn_fused(const smartmem_swin_params_t& p, const DevMap& rowmap, const void* x, void* y, cudaStream_t st);
+// The same for wider blocks of few windows (C = 128, 192, 256, 384, 512, head dimension 32): a cluster of C / 64 CTAs per two windows
+// (swin_attn_cluster.cu).  swin_attn_cluster_wins: it covers the shape and beats the separate kernels.
+bool swin_attn_cluster_wins(const smartmem_swin_params_t& p);
+int launch_swin_attn_cluster(const smartmem_swin_params_t& p, const DevMap& rowmap, const void* x, void* y, cudaStream_t st);
 
 }  // namespace smartmem

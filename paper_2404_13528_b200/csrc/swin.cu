@@ -89,6 +89,7 @@ size_t al(size_t b) { return (b + 255) & ~(size_t)255; }
 // Which fused kernels a block takes (they decide which intermediates exist at all).
 struct Path {
   bool fuse_attn, fuse_ln1, fuse_mlp;
+  bool attn_cluster;               // (fuse_attn) two heads per CTA of a cluster
   bool ln1_wave;                   // (fuse_ln1) a slice of the columns per CTA
   bool mlp_cluster;                // (fuse_mlp) the hidden features split over a cluster
   bool ln2_wave;                   // LN2 + fc1 + GELU in one kernel
@@ -99,6 +100,8 @@ Path choose_path(const smartmem_swin_params_t& p, int mode, bool compact) {
   Path t;
   t.fuse_attn = mode == SMARTMEM_ELIMINATE && (bf16 ? swin_attn_fused_supported(p.dtype, p.C, p.heads, p.window)
                                                     : swin_attn_f32_supported(p.C, p.heads, p.window));
+  t.attn_cluster = mode == SMARTMEM_ELIMINATE && !t.fuse_attn && swin_attn_cluster_wins(p);
+  t.fuse_attn = t.fuse_attn || t.attn_cluster;
   t.ln1_wave = bf16 && gemm_ln_wave_wins((long long)p.B * p.H * p.W, 3 * (long long)p.C, p.C);
   t.fuse_ln1 = t.ln1_wave || (bf16 && gemm_ln_supported(3 * (long long)p.C, p.C));
   t.fuse_mlp = p.mlp_ratio > 0 && (bf16 ? mlp_fused_supported(p.C, (long long)p.C * p.mlp_ratio)
@@ -257,8 +260,11 @@ int run_block(const smartmem_swin_params_t* pp, const void* x, void* y, void* wo
   if (half == 1) {
     // MLP half only
   } else if (path.fuse_attn) {
-    // narrow blocks: the whole attention half in one kernel (rows gathered and scattered through the composed map)
-    SM_TRY("attn_half_fused", f32 ? launch_swin_attn_f32(p, m.e1_rows, x, y1, st) : launch_swin_attn_fused(p, m.e1_rows, x, y1, st));
+    // narrow blocks, and wide ones of few windows: the whole attention half in one kernel (rows gathered and scattered through the
+    // composed map)
+    SM_TRY("attn_half_fused", f32 ? launch_swin_attn_f32(p, m.e1_rows, x, y1, st)
+                              : path.attn_cluster ? launch_swin_attn_cluster(p, m.e1_rows, x, y1, st)
+                                                  : launch_swin_attn_fused(p, m.e1_rows, x, y1, st));
   } else if (elim) {
     if (fuse_ln1) {
       // narrow blocks: LN1, the shift o partition gather and the QKV projection in one kernel
