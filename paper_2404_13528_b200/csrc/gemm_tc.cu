@@ -41,7 +41,6 @@ struct OpCoord {
 struct GemmArgs {
   int M, N, K;
   int tiles_n, tiles_m, batch;
-  uint32_t wide_tiles;                   // 256-wide pair tiles from this one on come as two halves each (tile_item)
   FastDiv fd_tiles_n, fd_tiles_m;        // tile index -> (tile_n, tile_m, batch) without hardware division
   OpCoord ca, cb;
   __nv_bfloat16* out;
@@ -112,16 +111,19 @@ struct TileItem {
   bool half;
 };
 template <bool HALVES>
-struct HalfMap {                         // tensor map of a half's B rows: only the kernels that take halves pay for the parameter
-  CUtensorMap map;
+struct Halves {                          // (only the kernels that take halves pay for the parameter)
+  CUtensorMap map;                       // a half's B rows
+  uint32_t wide_tiles;                   // tiles from this one on come as halves
 };
 template <>
-struct HalfMap<false> {};
+struct Halves<false> {};
 template <bool HALVES>
-__device__ __forceinline__ TileItem tile_item(uint32_t t, const GemmArgs& g) {
-  if (HALVES && t >= g.wide_tiles) {
-    const uint32_t u = t - g.wide_tiles;
-    return {split_tile(g.wide_tiles + (u >> 1), g.fd_tiles_n, g.fd_tiles_m), (int)(u & 1) * 128, true};
+__device__ __forceinline__ TileItem tile_item(uint32_t t, const GemmArgs& g, const Halves<HALVES>& hv) {
+  if constexpr (HALVES) {
+    if (t >= hv.wide_tiles) {
+      const uint32_t u = t - hv.wide_tiles;
+      return {split_tile(hv.wide_tiles + (u >> 1), g.fd_tiles_n, g.fd_tiles_m), (int)(u & 1) * 128, true};
+    }
   }
   return {split_tile(t, g.fd_tiles_n, g.fd_tiles_m), 0, false};
 }
@@ -146,8 +148,8 @@ constexpr int kThreads = 64 + 32 * kEpiWarps + 32;      // + a second TMA produc
 template <int BN, int STAGES, bool A_MN, bool PAIR, bool LEAN>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-               const __grid_constant__ CUtensorMap tmC, const __grid_constant__ HalfMap<PAIR && BN == 256> tmBh,
-               const __grid_constant__ GemmArgs g) {
+               const __grid_constant__ CUtensorMap tmC, const __grid_constant__ GemmArgs g,
+               const __grid_constant__ Halves<PAIR && BN == 256> hv) {
   static_assert(!PAIR || ((BN == 256 || BN == 128) && !A_MN), "CTA pairs: 256- or 128-wide tiles, K-major A");
   static_assert(!LEAN || BN % 128 == 0, "the lean epilogue's boxes are 32 columns wide");
   constexpr bool RES = !LEAN || BN == 128;                 // the epilogue can add a residual
@@ -158,7 +160,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   constexpr uint32_t IDESC = ptx::make_idesc_bf16(PAIR ? 2 * BM : BM, BN, A_MN, false);
   constexpr bool HALVES = PAIR && BN == 256;               // the last round's tiles may come as halves
   const CUtensorMap* map_half = &tmB;
-  if constexpr (HALVES) map_half = &tmBh.map;
+  if constexpr (HALVES) map_half = &hv.map;
   constexpr uint32_t IDESC_HALF = ptx::make_idesc_bf16(2 * BM, BN / 2, false, false);
 
   extern __shared__ uint8_t smem_raw[];
@@ -184,7 +186,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   const int last_ksteps = (g.K - (nkb - 1) * BK + 15) / 16;
   const bool two_producers = nkb >= 8;
   const uint32_t tiles = (uint32_t)g.tiles_n * g.tiles_m * g.batch;         // PAIR: tiles_m counts 256-row tiles
-  const uint32_t total_tiles = HALVES ? 2 * tiles - g.wide_tiles : tiles;   // (work items)
+  uint32_t total_tiles = tiles;                                             // (work items)
+  if constexpr (HALVES) total_tiles = 2 * tiles - hv.wide_tiles;
   const uint32_t rank = PAIR ? ptx::cluster_ctarank() : 0u;                  // which half of the pair's tile
   const bool leader = rank == 0;
   const uint32_t cta_first = PAIR ? blockIdx.x >> 1 : blockIdx.x, cta_step = PAIR ? gridDim.x >> 1 : gridDim.x;
@@ -206,7 +209,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     ptx::prefetch_tensormap(&tmA);
     ptx::prefetch_tensormap(&tmB);
     if constexpr (HALVES) {
-      if (g.wide_tiles < tiles) ptx::prefetch_tensormap(&tmBh.map);
+      if (hv.wide_tiles < tiles) ptx::prefetch_tensormap(&hv.map);
     }
     if (QTMA || (LEAN && g.tma_out)) ptx::prefetch_tensormap(&tmC);
   }
@@ -234,8 +237,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     bool ok = true;
     const uint32_t full0 = PAIR ? ptx::mapa(ptx::smem_u32(full), 0) : 0u;     // the even CTA's `full` barriers
     for (uint32_t t = cta_first; t < total_tiles && ok; t += cta_step) {
-      const TileItem item = tile_item<HALVES>(t, g);
-      const TileIdx& ti_ = item.ti;
+      const TileItem item = tile_item<HALVES>(t, g, hv);
+      const TileIdx ti_ = item.ti;
       const uint32_t tile_n = ti_.tile_n, tile_m = PAIR ? 2 * ti_.tile_m + rank : ti_.tile_m, batch = ti_.batch;
       const TileCoord ta = op_coords(g.ca, tile_m, batch, BM), tb = op_coords(g.cb, tile_n, batch, BN);
       const bool half = HALVES && item.half;
@@ -291,7 +294,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         if (!ok) break;
         ptx::tc_fence_after();
         const uint32_t d_tmem = tmem_base + buf * ACC_COLS;
-        const uint32_t idesc = HALVES && t >= g.wide_tiles ? IDESC_HALF : IDESC;
+        uint32_t idesc = IDESC;
+        if constexpr (HALVES) idesc = t >= hv.wide_tiles ? IDESC_HALF : IDESC;
         for (int kb = 0; kb < nkb; ++kb) {
           ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(&full[s], ph, abort_flag, g.status) ? 1 : 0) != 0;
           if (!ok) break;
@@ -338,7 +342,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       bool ok = true;
       const uint32_t full0 = PAIR ? ptx::mapa(ptx::smem_u32(full), 0) : 0u;
       for (uint32_t t = cta_first; t < total_tiles && ok; t += cta_step) {
-        const TileItem item = tile_item<HALVES>(t, g);
+        const TileItem item = tile_item<HALVES>(t, g, hv);
         const uint32_t tile_n = item.ti.tile_n, batch = item.ti.batch;
         const TileCoord tb = op_coords(g.cb, tile_n, batch, BN);
         const bool half = HALVES && item.half;
@@ -392,8 +396,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint4 res_next[VPR];
     const uint32_t tmem_empty0 = PAIR ? ptx::mapa(ptx::smem_u32(tmem_empty), 0) : 0u;   // the even CTA's barriers
     for (uint32_t t = cta_first; t < total_tiles && ok; t += cta_step, ++it) {
-      const TileItem item = tile_item<HALVES>(t, g);
-      const TileIdx& ti_ = item.ti;
+      const TileItem item = tile_item<HALVES>(t, g, hv);
+      const TileIdx ti_ = item.ti;
       const uint32_t tile_n = ti_.tile_n, tile_m = PAIR ? 2 * ti_.tile_m + rank : ti_.tile_m, batch = ti_.batch;
       const uint32_t buf = it & 1, use = it >> 1;
       if (HALVES && item.half && grp >= 2) {                 // a half's 128 columns are the first two groups'
@@ -876,25 +880,27 @@ int sm_count() {
 }
 
 template <int BN, int STAGES, bool A_MN, bool PAIR = false, bool LEAN = false>
-int launch_t(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, const CUtensorMap& tbh, const GemmArgs& g, cudaStream_t st) {
+int launch_t(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, const Halves<true>& halves, const GemmArgs& g, cudaStream_t st) {
   constexpr bool QST = !PAIR && !(BN == 256 && STAGES == 4);
   constexpr int RCc = !QST ? 16 : ((BN / 4) > 32 ? 32 : (BN / 4));
   constexpr size_t smem = 1024 + STAGES * (A_STAGE_BYTES + (PAIR ? BN / 2 : BN) * BK * 2) + (2 * STAGES + 4) * 8 + 16 +
                           (LEAN ? kEpiWarps * 32 * 64 : PAIR ? 0 : STAGES == 2 ? 2 * 4 * 32 * 512 : !QST ? kEpiWarps * 32 * (RCc * 2 + 16) : 4 * 32 * (BN * 2 + 16));   // pairs store from registers
   if (ensure_max_dynamic_smem((const void*)gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN>, (int)smem) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   profile_tick("gemm_tc", st);
-  HalfMap<PAIR && BN == 256> hm;
-  if constexpr (PAIR && BN == 256) hm.map = tbh;
   long long tiles = (long long)g.tiles_n * g.tiles_m * g.batch;
-  if (PAIR && BN == 256) tiles = 2 * tiles - g.wide_tiles;
+  Halves<PAIR && BN == 256> hv;
+  if constexpr (PAIR && BN == 256) {
+    hv = halves;
+    tiles = 2 * tiles - halves.wide_tiles;
+  }
   if constexpr (PAIR) {
     // one cluster of two CTAs per tile of 256 rows; the two CTAs of a cluster are neighbours in blockIdx.x
     const long long pairs = sm_count() / 2;
     const unsigned grid = (unsigned)(2 * (tiles < pairs ? tiles : pairs));
-    launch_pdl_cluster(gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN>, dim3(grid), dim3(kThreads), smem, st, 2u, ta, tb, tc, hm, g);
+    launch_pdl_cluster(gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN>, dim3(grid), dim3(kThreads), smem, st, 2u, ta, tb, tc, g, hv);
   } else {
     const unsigned grid = (unsigned)(tiles < sm_count() ? tiles : sm_count());
-    launch_pdl(gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN>, dim3(grid), dim3(kThreads), smem, st, ta, tb, tc, hm, g);
+    launch_pdl(gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN>, dim3(grid), dim3(kThreads), smem, st, ta, tb, tc, g, hv);
   }
   count_launch();
   return cudaGetLastError() == cudaSuccess ? SMARTMEM_OK : SMARTMEM_ERR_CUDA;
@@ -1176,11 +1182,12 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
   g.batch = (int)batch;
   if ((long long)g.tiles_n * g.tiles_m * g.batch >= (1ll << 31)) return SMARTMEM_ERR_UNSUPPORTED;
   const long long all_tiles = (long long)g.tiles_n * g.tiles_m * g.batch;
-  g.wide_tiles = (uint32_t)(halves ? all_tiles - all_tiles % (tc_sm_count() / 2) : all_tiles);
-  CUtensorMap tbh = tb;
+  Halves<true> hv;
+  hv.map = tb;
+  hv.wide_tiles = (uint32_t)(halves ? all_tiles - all_tiles % (tc_sm_count() / 2) : all_tiles);
   if (halves) {
     OpCoord same;
-    rc = build_operand(B, bn, bn / 4, &tbh, &same);
+    rc = build_operand(B, bn, bn / 4, &hv.map, &same);
     if (rc != SMARTMEM_OK) return rc;
   }
   CUtensorMap tc = ta;                                     // (a valid map for the kernels that store without TMA)
@@ -1192,19 +1199,19 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
     else if (lean) return SMARTMEM_ERR_CUDA;
     else tc = ta;
   }
-  if (pair_lean) return launch_t<256, 6, false, true, true>(ta, tb, tc, tbh, g, st);
-  if (lean) return bn == 128 ? launch_t<128, 5, false, false, true>(ta, tb, tc, tbh, g, st) : launch_t<256, 4, false, false, true>(ta, tb, tc, tbh, g, st);
-  if (pair && bn == 256) return launch_t<256, 6, false, true>(ta, tb, tc, tbh, g, st);
-  if (pair) return launch_t<128, 8, false, true>(ta, tb, tc, tbh, g, st);
+  if (pair_lean) return launch_t<256, 6, false, true, true>(ta, tb, tc, hv, g, st);
+  if (lean) return bn == 128 ? launch_t<128, 5, false, false, true>(ta, tb, tc, hv, g, st) : launch_t<256, 4, false, false, true>(ta, tb, tc, hv, g, st);
+  if (pair && bn == 256) return launch_t<256, 6, false, true>(ta, tb, tc, hv, g, st);
+  if (pair) return launch_t<128, 8, false, true>(ta, tb, tc, hv, g, st);
   if (stages == 2) {
     const uint64_t dims[3] = {(uint64_t)N, (uint64_t)M, (uint64_t)batch};
     const uint64_t strides[2] = {(uint64_t)ep.ldc * 2, (uint64_t)(batch > 1 ? ep.out_batch_stride : ep.ldc * M) * 2};
     const uint32_t box[3] = {64, 32, 1};
-    if (encode_cached(ep.out, 3, dims, strides, box, &tc) == SMARTMEM_OK) return launch_t<256, 2, false>(ta, tb, tc, tbh, g, st);
+    if (encode_cached(ep.out, 3, dims, strides, box, &tc) == SMARTMEM_OK) return launch_t<256, 2, false>(ta, tb, tc, hv, g, st);
     stages = 3;
   }
 #define SM_CASE(BN_, ST_, MN_)                                                                  \
-  if (bn == BN_ && stages == ST_ && a_mn == MN_) return launch_t<BN_, ST_, MN_>(ta, tb, tc, tbh, g, st);
+  if (bn == BN_ && stages == ST_ && a_mn == MN_) return launch_t<BN_, ST_, MN_>(ta, tb, tc, hv, g, st);
   SM_CASE(256, 3, false) SM_CASE(256, 4, false) SM_CASE(128, 5, false) SM_CASE(96, 7, false) SM_CASE(64, 8, false)
   SM_CASE(256, 3, true) SM_CASE(256, 4, true) SM_CASE(128, 5, true)
 #undef SM_CASE
