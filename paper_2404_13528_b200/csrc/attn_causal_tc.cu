@@ -29,7 +29,7 @@ constexpr int BQ = 128, BKV = 64, D = 128;
 constexpr int KB = 128 * 64 * 2;                      // one 128 x 64 bf16 block (Q, P)
 constexpr int KBK = BKV * 64 * 2;                     // one 64 x 64 bf16 block (K, V)
 constexpr uint32_t TM_S = 0, TM_O = 128, TMEM_COLS = 256;   // two S buffers of 64 columns, O of 128: two CTAs share an SM's 512
-constexpr int KSTAGES = 3, N_BARS = 1 + 2 * KSTAGES + 4 + 4 + 3;
+constexpr int KSTAGES = 3, N_BARS = 1 + 2 * KSTAGES + 4 + 4 + 4;
 constexpr uint32_t SMEM_BYTES = 2 * KB + (2 * KSTAGES + 4) * KBK + N_BARS * 8 + 16;
 constexpr int kThreads = 192;
 constexpr float kRescaleThreshold = 8.0f;             // log2 units
@@ -68,7 +68,7 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   uint8_t* sV = sK + 2 * KSTAGES * KBK;                // [2 stages][2 d-chunks][8 KB]
   uint64_t* bars = reinterpret_cast<uint64_t*>(sV + 4 * KBK);
   uint64_t *q_full = bars, *k_full = bars + 1, *k_empty = k_full + KSTAGES, *v_full = k_empty + KSTAGES, *v_empty = v_full + 2;
-  uint64_t *s_full = v_empty + 2, *s_empty = s_full + 2, *p_full = s_empty + 2, *p_empty = p_full + 1, *o_done = p_empty + 1;
+  uint64_t *s_full = v_empty + 2, *s_empty = s_full + 2, *p_full = s_empty + 2, *p_empty = p_full + 2, *o_done = p_empty + 1;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + N_BARS);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
 
@@ -97,7 +97,9 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       ptx::mbar_init(&s_full[i], 1);
       ptx::mbar_init(&s_empty[i], 1);                 // P(j) lives in S buffer j & 1: freed by the commit of P V (j)
     }
-    ptx::mbar_init(p_full, 4);
+    // (a barrier per S buffer: the softmax may be two tiles ahead of P V, and with one for both the issuing warp, held up for that long by a
+    // slow read in its wait, found the phase that it waited for already followed by another and waited for good)
+    for (int i = 0; i < 2; ++i) ptx::mbar_init(&p_full[i], 4);
     ptx::mbar_init(p_empty, 1);
     ptx::mbar_init(o_done, 1);
     *abort_flag = 0;
@@ -184,7 +186,7 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       };
       auto issue_pv = [&](int j) {
         const int s = j & 1;
-        ok = ok && ptx::mbar_wait(p_full, j & 1, abort_flag, g.status);
+        ok = ok && ptx::mbar_wait(&p_full[s], (j >> 1) & 1, abort_flag, g.status);
         ok = ok && ptx::mbar_wait(&v_full[s], (j >> 1) & 1, abort_flag, g.status);
         ok = __all_sync(0xFFFFFFFFu, ok ? 1 : 0) != 0;
         if (!ok) return;
@@ -288,7 +290,7 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       ptx::tmem_st_wait();
       ptx::tc_fence_before();
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(p_full);
+      if (lane == 0) ptx::mbar_arrive(&p_full[sb]);
     }
     if (ok) ok = ptx::mbar_wait(o_done, 0, abort_flag, g.status);
     if (ok) {
