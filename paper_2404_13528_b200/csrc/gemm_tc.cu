@@ -47,7 +47,7 @@ struct GemmArgs {
   long long ldc, out_batch_stride;
   const __nv_bfloat16* bias;
   const __nv_bfloat16* residual;
-  int gelu, has_rowmap;
+  int gelu, has_rowmap, b_settled;
   int rope_cols, rope_S, rope_pos0;      // columns [0, rope_cols) are rotated; position = rope_pos0 + row % rope_S
   int rope_half;                         // R / 2: the first R columns of each 128-wide head rotate, pairs (i, i + R/2)
   float rope_c;                          // log2(theta) / (R / 2)
@@ -226,8 +226,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   }
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  pdl_wait();                       // everything above overlapped the previous kernel's tail
-  pdl_launch_dependents();
+  // Everything above overlapped the previous kernel's tail, and so does the B operand's first round of the ring where nothing in flight
+  // writes it (TcEpilogue::b_settled): its producer waits behind that.  (Not in its ring: a thousand lanes that poll for the length of a kernel
+  // slow down those that they wait for.)
+  if (warp < 2 + kEpiWarps || !two_producers || !g.b_settled) {
+    pdl_wait();
+    pdl_launch_dependents();
+  }
 
   if (warp == 0) {
     // The whole warp walks the loop and one elected lane issues (as for the products below): under a branch on one lane every
@@ -339,7 +344,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // cheaper to feed from one thread)
     if (two_producers) {
       uint32_t s = 0, ph = 1;
-      bool ok = true;
+      bool ok = true, waited = !g.b_settled;
       const uint32_t full0 = PAIR ? ptx::mapa(ptx::smem_u32(full), 0) : 0u;
       for (uint32_t t = cta_first; t < total_tiles && ok; t += cta_step) {
         const TileItem item = tile_item<HALVES>(t, g, hv);
@@ -350,6 +355,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const uint32_t b_bytes = half ? B_STAGE_BYTES / 2 : B_STAGE_BYTES;
         const CUtensorMap* mapB = half ? map_half : &tmB;
         for (int kb = 0; kb < nkb; ++kb) {
+          if (!waited && kb == STAGES) {
+            pdl_wait();
+            waited = true;
+          }
           ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(&empty[s], ph, abort_flag, g.status) ? 1 : 0) != 0;
           if (!ok) break;
           if (ptx::elect_one()) {
@@ -364,6 +373,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           __syncwarp();
           if (++s == STAGES) { s = 0; ph ^= 1; }
         }
+        if (!waited) pdl_wait();                             // (a reduction no longer than the ring)
+        waited = true;
       }
     }
   } else {
@@ -1158,6 +1169,7 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
   g.bias = (const __nv_bfloat16*)ep.bias;
   g.residual = (const __nv_bfloat16*)ep.residual;
   g.gelu = ep.gelu;
+  g.b_settled = ep.b_settled;
   g.has_rowmap = ep.rowmap ? 1 : 0;
   if (ep.rowmap) g.rowmap = *ep.rowmap;
   g.rope_cols = ep.rope_cols;
