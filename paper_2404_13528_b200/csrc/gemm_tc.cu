@@ -396,6 +396,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int grp = e >> 2;
     constexpr bool QSTAGE = !DIRECT && !(BN == 256 && STAGES == 4);  // per-quadrant staging of whole rows
     constexpr bool QBULK = BN == 256 && !A_MN && !QTMA;      // staged rows leave as bulk copies (512-byte rows; not the MN-major-A kernel: 13.1 vs 12.1 us)
+    constexpr bool BARE = QTMA;                              // nothing but conversion and store: no bias, GELU, residual, rotation, map or second copy
     constexpr int QROW = BN * 2 + 16;                        // bytes; the pad keeps phase 1 conflict-free
     uint8_t* stage = stage_base + e * (32 * STG_ROW);
     uint8_t* qstage = stage_base + q * (32 * QROW);
@@ -421,7 +422,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const int row = tile_m * BM + q * 32 + lane;
       const bool row_ok = row < g.M;
       long long o2_base = 0;                                 // second copy: row = b * S + s goes to out2[b][col][s]
-      if (!LEAN && g.out2) {
+      if (!LEAN && !BARE && g.out2) {
         const uint32_t b2 = fd_div((uint32_t)row, g.fd_out2_S);
         o2_base = (long long)b2 * g.N * g.fd_out2_S.d + ((uint32_t)row - b2 * g.fd_out2_S.d);
       }
@@ -433,7 +434,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       // the whole tile has one base and one pitch; the base is biased by the segment's first column
       __nv_bfloat16* out_t = g.out;
       long long ld_t = g.ldc;
-      if (g.seg_cols > 0) {
+      if (!BARE && g.seg_cols > 0) {
         const int sg = n0 / g.seg_cols;
         out_t = g.seg_out[sg] - (long long)sg * g.seg_cols;
         ld_t = g.seg_ld[sg];
@@ -441,13 +442,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       long long off;
       if (PREFETCH_NEXT && it > 0) {
         off = off_next;
+      } else if (BARE) {
+        off = 0;                                             // (the boxes go by coordinates)
       } else {
         off = 0;
         if (row_ok) off = g.has_rowmap ? devmap_eval_unrolled(g.rowmap, (uint32_t)row) : (long long)row * ld_t;
         off += (long long)batch * g.out_batch_stride;
       }
-      const __nv_bfloat16* __restrict__ rrow = (RES && g.residual) ? g.residual + off : nullptr;
-      const bool rope_tile = !LEAN && (BN == 256 || BN == 128) && g.rope_cols > 0 && n0 < g.rope_cols;
+      const __nv_bfloat16* __restrict__ rrow = (RES && !BARE && g.residual) ? g.residual + off : nullptr;
+      const bool rope_tile = !LEAN && !BARE && (BN == 256 || BN == 128) && g.rope_cols > 0 && n0 < g.rope_cols;
       auto col_of = [&](int rd) {
         return BN == 256 ? 128 * (grp >> 1) + 32 * (grp & 1) + RC * (rd % RH) + 64 * (rd / RH) : grp * CG;
       };
@@ -473,7 +476,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if (PREFETCH_NEXT && it > 0) {
 #pragma unroll
         for (int v = 0; v < VPR; ++v) res[v] = res_next[v];
-      } else {
+      } else if (!BARE) {
         fetch_res(col_of(0));                                // in flight while this tile's MMAs still run
       }
       if (PREFETCH_NEXT) {                                   // request the next tile's row offset and residual now
@@ -529,7 +532,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const int c0 = col_of(rd);
         float acc[RC];
         uint4 bv[VPR];                                       // this round's bias columns: requested before the wait on tensor memory
-        if (g.bias) {
+        if (!BARE && g.bias) {
 #pragma unroll
           for (int v = 0; v < VPR; ++v) {
             bv[v] = make_uint4(0, 0, 0, 0);
@@ -578,7 +581,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             for (int j = 0; j < RC; ++j) acc[j] = __uint_as_float(rv[j]);
           }
         }
-        if (g.bias) {
+        if (!BARE && g.bias) {
 #pragma unroll
           for (int v = 0; v < VPR; ++v) {
             const uint32_t w[4] = {bv[v].x, bv[v].y, bv[v].z, bv[v].w};
@@ -590,11 +593,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
           }
         }
-        if (g.gelu) {
+        if (!BARE && g.gelu) {
 #pragma unroll
           for (int j = 0; j < RC; ++j) acc[j] = gelu_tanh(acc[j]);
         }
-        if (rrow) {
+        if (!BARE && rrow) {
 #pragma unroll
           for (int v = 0; v < VPR; ++v) {
             const uint32_t w[4] = {res[v].x, res[v].y, res[v].z, res[v].w};
@@ -607,7 +610,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           }
           if (rd + 1 < ROUNDS) fetch_res(col_of(rd + 1));
         }
-        if (!LEAN && g.out2 && row_ok) {
+        if (!LEAN && !BARE && g.out2 && row_ok) {
           // The redundant copy of a producer with consumers of different reduction dimensions: the same values with the
           // row's position inside its group as the contiguous dimension.  A warp's 32 rows write 64 contiguous bytes per column.
 #pragma unroll
@@ -683,7 +686,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // 62.8 in a long one.
         ptx::fence_proxy_async();
         asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory");
-        if (lane == 0) {
+        if (lane == 0) {                                     // (the lane that waits for its boxes: groups are a thread's own)
           if ((int)tile_m * BM + q * 32 < g.M && n0 + grp * 64 < g.N)
             ptx::tma_store_3d(&tmC, qtile + grp * 4096, n0 + grp * 64, (int)tile_m * BM + q * 32, (int)batch);
           ptx::bulk_commit_group();
@@ -1153,7 +1156,7 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
   }
   // single CTAs: 256 wide, short K: wider store rounds instead of a 4th stage.  Narrow tiles: their stages are
   // small, and a tile is consumed faster than a load's latency, so the ring runs several tiles ahead.
-  const bool plain_out = !pair && !a_mn && !ep.rowmap && ep.seg_cols == 0 && !ep.out2;
+  const bool plain_out = !pair && !a_mn && !ep.rowmap && ep.seg_cols == 0 && !ep.out2 && !ep.bias && !ep.gelu && !ep.residual && ep.rope_cols == 0;
   int stages = bn == 256 ? (nkb <= 2 && plain_out ? 2 : nkb <= 4 ? 3 : 4) : bn == 64 ? 8 : bn == 96 ? 7 : 5;
   GemmArgs g;
   memset(&g, 0, sizeof(g));
