@@ -116,15 +116,20 @@ EXPORT int smartmem_attn_layer(const smartmem_attn_params_t* pp, const void* x, 
 #define SM_TRY(expr) do { rc = (expr); if (rc != SMARTMEM_OK) return rc; } while (0)
   const int rot = p.rotary_dim ? p.rotary_dim : (int)D;
   if (!elim) SM_TRY(launch_rope_table(tab, (int)S, rot, p.rope_theta, st));   // only the stand-alone RoPE pass reads it
-  SM_TRY(launch_norm(SMARTMEM_BF16, true, x, at(L.xn), p.rms_g, nullptr, p.rms_eps, M, (int)hid, nullptr, st));
+  // Few rows: RMSNorm rides along in the QKV product (gemm_splitk.cu), which saves a launch but not the products' slack once there are many
+  // rows to scale (us of a layer, apart -> together: hidden 1024 8 rows 16.0 -> 14.6, 40 18.2 -> 17.9, 64 20.4 -> 20.9; 2048 8 18.5 -> 17.9, 40 22.2 ->
+  // 21.4, 64 24.4 -> 24.6; 3072 64 32.5 -> 30.6; 4096 16 35.7 -> 34.2, 64 44.7 -> 40.9, 80 45.7 -> 49.4).
+  const bool norm_in_gemm = M <= (hid >= 3072 ? 64 : 40) && gemm_splitk_norm_fits(M, 3 * hid, hid);
+  if (!norm_in_gemm) SM_TRY(launch_norm(SMARTMEM_BF16, true, x, at(L.xn), p.rms_g, nullptr, p.rms_eps, M, (int)hid, nullptr, st));
   {
     TcEpilogue ep;
     memset(&ep, 0, sizeof(ep));
     ep.out = at(L.qkv);
     ep.ldc = 3 * hid;
-    ep.b_settled = 1;
+    ep.b_settled = norm_in_gemm ? 0 : 1;             // (with RMSNorm inside it is the call's first kernel, or follows the table's)
+    if (norm_in_gemm) { ep.rms_gamma = p.rms_g; ep.rms_eps = p.rms_eps; }
     if (elim) { ep.rope_cols = (int)(2 * hid); ep.rope_S = (int)S; ep.rope_log2_theta = log2f(p.rope_theta); ep.rope_dim = rot; }
-    SM_TRY(launch_gemm_tc(tc_operand_plain(at(L.xn), M, hid, hid), tc_operand_plain(p.w_qkv, 3 * hid, hid, hid), ep, 1, M,
+    SM_TRY(launch_gemm_tc(tc_operand_plain(norm_in_gemm ? x : at(L.xn), M, hid, hid), tc_operand_plain(p.w_qkv, 3 * hid, hid, hid), ep, 1, M,
                           3 * hid, hid, st));
   }
   CausalAttnArgs a;
