@@ -37,12 +37,14 @@ namespace {
 constexpr int D = 32, TP = 64;
 constexpr int OP_BYTES = 128 * 64;                    // one operand of a pair: 128 rows x 64 bytes
 constexpr int STAGE_BYTES = 3 * OP_BYTES;             // q, k, v
-constexpr int NSTAGE = 6;
-constexpr uint32_t TM_S = 0, TM_O = 256, TM_P = 320, TMEM_COLS = 512;   // S 2 x 128 columns, O 2 x 32, P 2 x 64 (128 keys as bf16 pairs)
+constexpr int NSTAGE = 8;
+constexpr uint32_t TM_S = 0, TM_O = 256, TM_P = 384, TMEM_COLS = 512;   // per group: S 64 columns, O 32, P 32 (64 keys as bf16 pairs)
 constexpr int BIAS_ROW = 36;                          // 32-bit words per bias row: 64 bf16 + pad, so that 16-byte row reads of
                                                       // eight consecutive threads fall into distinct banks
-constexpr int kSoftmaxWarps = 4, kGroups = 2, kLoaderWarps = 4;   // two softmax groups alternate over the units
-constexpr int kThreads = 32 * (3 + kGroups * kSoftmaxWarps + kLoaderWarps);   // + producer, P V issuer, S issuer
+constexpr int kSoftmaxWarps = 4, kMaxGroups = 4, kLoaderWarps = 4;
+// softmax groups taking turns over the units: four, or two beside the warps that load operands TMA cannot address
+constexpr int groups_of(bool manual) { return manual ? 2 : kMaxGroups; }
+constexpr int threads_of(bool manual) { return 32 * (3 + groups_of(manual) * kSoftmaxWarps + (manual ? kLoaderWarps : 0)); }   // + producer, P V issuer, S issuer
 
 struct WinTcArgs {
   WinAttnArgs a;
@@ -71,10 +73,12 @@ __device__ __forceinline__ float ex2f(float x) {
 
 // KC: key columns a softmax thread works on (56 when the window has at most 56 tokens -- a 7 x 7 window
 // has 49 -- else 64).  Columns [T, 64) of a score row are padding whose probability is zero.
-template <int KC>
-__global__ void __launch_bounds__(kThreads, 1)
+// MANUAL: some operand is not TMA's to load.
+template <int KC, bool MANUAL>
+__global__ void __launch_bounds__(threads_of(MANUAL), 1)
 win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
                    const __grid_constant__ CUtensorMap tm2, const __grid_constant__ WinTcArgs g) {
+  constexpr int kGroups = groups_of(MANUAL), kThreads = threads_of(MANUAL);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u);
   uint8_t* sIn = smem;                                 // [NSTAGE][q, k, v][128 rows x 64 B]
@@ -82,11 +86,11 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
   int* lab_s = reinterpret_cast<int*>(bias_s + TP * BIAS_ROW);   // scratch: the head's raw table column (<= 256 bf16), then 4 key-mask words
   uint16_t* raw_s = reinterpret_cast<uint16_t*>(lab_s);
   uint32_t* kmask_s = reinterpret_cast<uint32_t*>(lab_s) + 128;
-  int* tyx_s = lab_s + kGroups * 2 * TP;                         // [64]: ty << 8 | tx
+  int* tyx_s = lab_s + 4 * TP;                                   // [64]: ty << 8 | tx
   uint64_t* bars = reinterpret_cast<uint64_t*>(tyx_s + TP);
-  uint64_t *in_full = bars, *in_empty = bars + NSTAGE, *s_full = bars + 2 * NSTAGE, *s_empty = s_full + 2;
-  uint64_t *p_full = s_empty + 2, *p_empty = p_full + 2, *o_full = p_empty + 2, *o_empty = o_full + 2;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_empty + 2);
+  uint64_t *in_full = bars, *in_empty = bars + NSTAGE, *s_full = bars + 2 * NSTAGE, *s_empty = s_full + kMaxGroups;
+  uint64_t *p_full = s_empty + kMaxGroups, *p_empty = p_full + kMaxGroups, *o_full = p_empty + kMaxGroups, *o_empty = o_full + kMaxGroups;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(o_empty + kMaxGroups);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
 
   const WinAttnArgs& a = g.a;
@@ -95,21 +99,18 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
   const int T = a.T, ws = a.ws;
   const int h = blockIdx.x % a.heads;
   const int cidx = blockIdx.x / a.heads, cstride = gridDim.x / a.heads;
-  const bool any_manual = g.tma_mask != 7;
   const float LOG2E = 1.4426950408889634f;
 
   if (tid == 0) {
     for (int i = 0; i < NSTAGE; ++i) {
-      ptx::mbar_init(&in_full[i], 1 + (any_manual ? 32 * kLoaderWarps : 0));
+      ptx::mbar_init(&in_full[i], 1 + (MANUAL ? 32 * kLoaderWarps : 0));
       ptx::mbar_init(&in_empty[i], 1);
     }
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kGroups; ++i) {
       ptx::mbar_init(&s_full[i], 1);
       ptx::mbar_init(&s_empty[i], kSoftmaxWarps);
       ptx::mbar_init(&o_full[i], 1);
       ptx::mbar_init(&o_empty[i], kSoftmaxWarps);
-    }
-    for (int i = 0; i < 2; ++i) {
       ptx::mbar_init(&p_full[i], kSoftmaxWarps);
       ptx::mbar_init(&p_empty[i], 1);
     }
@@ -119,16 +120,13 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
   }
   if (warp == 1) ptx::tmem_alloc(tmem_slot, TMEM_COLS);   // first: its latency overlaps the table set-up below
   // one-time tables.  First the inputs of the table (one global load per thread, one latency): the
-  // head's column of the relative-position table and the token coordinates; P's off-diagonal blocks
-  // (and, for hand-loaded operands, the padded rows of the input stages) are zeroed meanwhile.
+  // head's column of the relative-position table and the token coordinates; for hand-loaded operands
+  // the padded rows of the input stages are zeroed meanwhile.
   const int n_table = (2 * ws - 1) * (2 * ws - 1);
   for (int i = tid; i < n_table && i < 256; i += kThreads) raw_s[i] = reinterpret_cast<const uint16_t*>(a.table)[i * a.heads + h];
   if (tid < TP) tyx_s[tid] = ((tid / ws) << 8) | (tid % ws);
-  {
-    uint8_t* z0 = smem;
-    const int zbytes = any_manual ? NSTAGE * STAGE_BYTES : 0;
-    for (int i = tid; i < zbytes / 16; i += kThreads) reinterpret_cast<uint4*>(z0)[i] = make_uint4(0, 0, 0, 0);
-  }
+  if constexpr (MANUAL)
+    for (int i = tid; i < NSTAGE * STAGE_BYTES / 16; i += kThreads) reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
   __syncthreads();
   // the head's bias as a [T, T] table of bf16 pairs, -inf for padded keys
   for (int i = tid; i < TP * (TP / 2); i += kThreads) {
@@ -169,7 +167,6 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
   const uint32_t tmem_base = *tmem_slot;
   pdl_wait();                       // the tables above depend on parameters only: they overlapped the previous kernel's tail
   pdl_launch_dependents();
-  const AttnOperand* ops[3] = {&a.q, &a.k, &a.v};
 
   if (warp == 0) {
     // ---- TMA producer ------------------------------------------------------------------------
@@ -204,20 +201,21 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
       bool ok = true;
       const int my_units = cidx < g.n_pairs ? (g.n_pairs - cidx + cstride - 1) / cstride : 0;
       for (int u = 0; u < my_units && ok; ++u) {
-        const int s = u % NSTAGE, ob = u & 1;
-        ok = ptx::mbar_wait(&p_full[ob], (u >> 1) & 1, abort_flag, g.status);
-        ok = ok && ptx::mbar_wait(&o_empty[ob], ((u >> 1) & 1) ^ 1, abort_flag, g.status);
+        const int s = u % NSTAGE, ob = u % kGroups, turn = (u / kGroups) & 1;
+        ok = ptx::mbar_wait(&p_full[ob], turn, abort_flag, g.status);
+        ok = ok && ptx::mbar_wait(&o_empty[ob], turn ^ 1, abort_flag, g.status);
         ok = __all_sync(0xFFFFFFFFu, ok ? 1 : 0) != 0;
         if (!ok) break;
         ptx::tc_fence_after();
         const uint32_t v0 = ptx::smem_u32(sIn + s * STAGE_BYTES + 2 * OP_BYTES);
         const uint64_t vd = make_desc_sw64(v0, 16, 512);
-        const uint32_t od = tmem_base + TM_O + ob * D, pa = tmem_base + TM_P + ob * 64;
+        const uint32_t od = tmem_base + TM_O + ob * D, pa = tmem_base + TM_P + ob * 32;
         if (ptx::elect_one()) {
-          ptx::tc_mma_bf16_ta(od, pa, vd, idesc_pv, 0u);
 #pragma unroll
-          for (int ks = 1; ks < 8; ++ks)               // 16 keys per step: P +8 packed columns, V +1024 bytes
-            ptx::tc_mma_bf16_ta(od, pa + 8 * ks, vd + ks * (1024 >> 4), idesc_pv, 1u);
+          for (int ks = 0; ks < 8; ++ks) {             // 16 keys per step: P +8 packed columns, V +1024 bytes; steps 4-7: the second window
+            const uint32_t first = ks < 4 ? 0u : ~0u;
+            ptx::tc_mma_bf16_ta_lanes(od, pa + 8 * (ks & 3), vd + ks * (1024 >> 4), idesc_pv, (ks & 3) ? 1u : 0u, first, ~first);
+          }
           ptx::tc_commit(&in_empty[s]);
           ptx::tc_commit(&p_empty[ob]);
           ptx::tc_commit(&o_full[ob]);
@@ -225,16 +223,16 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
         __syncwarp();
       }
     }
-  } else if (warp == 2 + kGroups * kSoftmaxWarps + kLoaderWarps) {
-    // ---- S issuer: runs ahead of P V as far as the two S buffers and the input ring allow, so a
+  } else if (warp == kThreads / 32 - 1) {
+    // ---- S issuer: runs ahead of P V as far as the S buffers and the input ring allow, so a
     // softmax group finds its next score tile waiting when it has written P ---------------------
     {
-      const uint32_t idesc_s = ptx::make_idesc_bf16(128, 128, false, false);
+      const uint32_t idesc_s = ptx::make_idesc_bf16(128, TP, false, false);
       bool ok = true;
       const int my_units = cidx < g.n_pairs ? (g.n_pairs - cidx + cstride - 1) / cstride : 0;
       for (int u = 0; u < my_units && ok; ++u) {
-        const int s = u % NSTAGE, sb = u & 1;
-        ok = ptx::mbar_wait(&s_empty[sb], ((u >> 1) & 1) ^ 1, abort_flag, g.status);
+        const int s = u % NSTAGE, sb = u % kGroups;
+        ok = ptx::mbar_wait(&s_empty[sb], ((u / kGroups) & 1) ^ 1, abort_flag, g.status);
         ok = ok && ptx::mbar_wait(&in_full[s], (u / NSTAGE) & 1, abort_flag, g.status);
         ok = __all_sync(0xFFFFFFFFu, ok ? 1 : 0) != 0;
         if (!ok) break;
@@ -242,15 +240,19 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
         const uint32_t q0 = ptx::smem_u32(sIn + s * STAGE_BYTES), k0 = q0 + OP_BYTES;
         const uint64_t qd = make_desc_sw64(q0, 16, 512), kd = make_desc_sw64(k0, 16, 512);
         if (ptx::elect_one()) {
-          ptx::tc_mma_bf16(tmem_base + TM_S + sb * 128, qd, kd, idesc_s, 0u);
-          ptx::tc_mma_bf16(tmem_base + TM_S + sb * 128, qd + 2, kd + 2, idesc_s, 1u);  // next 16 features: +32 bytes
+#pragma unroll
+          for (int ks = 0; ks < 4; ++ks) {             // 16 features per step: +32 bytes; steps 2-3: the second window's keys, +4096 bytes
+            const uint32_t first = ks < 2 ? 0u : ~0u;
+            ptx::tc_mma_bf16_lanes(tmem_base + TM_S + sb * TP, qd + 2 * (ks & 1), kd + 2 * (ks & 1) + (ks >> 1) * (4096 >> 4), idesc_s,
+                                   ks & 1, first, ~first);
+          }
           ptx::tc_commit(&s_full[sb]);
         }
         __syncwarp();
       }
     }
   } else if (warp < 2 + kGroups * kSoftmaxWarps) {
-    // ---- softmax + epilogue: one query row per thread; group gi takes the units u = gi (mod 2) ----
+    // ---- softmax + epilogue: one query row per thread; group gi takes the units u = gi (mod kGroups) ----
     const int gi = (warp - 2) / kSoftmaxWarps;
     const int q = warp & 3;                            // TMEM lane quadrant
     const int r = q * 32 + lane;                       // row of the pair tile
@@ -258,13 +260,6 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
     const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
     const int my_ty = tyx_s[i] >> 8, my_tx = tyx_s[i] & 255;
     const uint32_t* brow = bias_s + i * BIAS_ROW;
-    {                                                  // block-diagonal P: the other window's keys contribute nothing to this row
-      uint32_t zero[32];
-#pragma unroll
-      for (int c = 0; c < 32; ++c) zero[c] = 0u;
-      ptx::tmem_st32(tmem_base + TM_P + gi * 64 + lane_addr + (1 - w) * 32, zero);
-      ptx::tmem_st_wait();
-    }
     // keys below / right of the wrap line of a seam window (bit c = key c), and this row's own side
     const uint32_t ky_lo = kmask_s[0], ky_hi = kmask_s[1], kx_lo = kmask_s[2], kx_hi = kmask_s[3];
     const uint32_t my_fy = my_ty >= ws - a.shift ? 0xFFFFFFFFu : 0u, my_fx = my_tx >= ws - a.shift ? 0xFFFFFFFFu : 0u;
@@ -272,9 +267,9 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
     int n_prev = -1;
     bool ok = true;
     const bool wide_store = (reinterpret_cast<uintptr_t>(a.o.ptr) & 31) == 0 && a.o.sn % 16 == 0 && a.o.sh % 16 == 0 && a.o.st % 16 == 0;
-    auto epilogue = [&](int u, float inv, int n) {     // O(u) -> global
-      const int ob = u & 1;                            // == gi
-      ok = ok && ptx::mbar_wait(&o_full[ob], (u >> 1) & 1, abort_flag, g.status);
+    auto epilogue = [&](int turn, float inv, int n) {  // O of the group's unit number `turn` -> global
+      const int ob = gi;
+      ok = ok && ptx::mbar_wait(&o_full[ob], turn & 1, abort_flag, g.status);
       if (!ok) return;
       ptx::tc_fence_after();
       uint32_t rv[32];
@@ -305,10 +300,8 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
         }
       }
     };
-    int u = gi;
     int done = 0;
-    for (int p = cidx + gi * cstride; p < g.n_pairs && ok; p += 2 * cstride, u += 2, ++done) {
-      const int sb = u & 1;
+    for (int p = cidx + gi * cstride; p < g.n_pairs && ok; p += kGroups * cstride, ++done) {
       const int n = 2 * p + w;
       // Shifted blocks: only windows in the last window row or column straddle the seam.  There a key
       // lies in another region than this row iff the two sit on different sides of the wrap line at
@@ -324,11 +317,11 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
         if (last_row) { diff_lo |= ky_lo ^ my_fy; diff_hi |= ky_hi ^ my_fy; }
         if (last_col) { diff_lo |= kx_lo ^ my_fx; diff_hi |= kx_hi ^ my_fx; }
       }
-      ok = ptx::mbar_wait(&s_full[sb], (u >> 1) & 1, abort_flag, g.status);
+      ok = ptx::mbar_wait(&s_full[gi], done & 1, abort_flag, g.status);
       if (!ok) break;
       ptx::tc_fence_after();
       uint32_t rv[KC];
-      const uint32_t ts = tmem_base + TM_S + sb * 128 + lane_addr + w * 64;    // this window's 64 key columns
+      const uint32_t ts = tmem_base + TM_S + gi * TP + lane_addr;
       ptx::tmem_ld32(ts, rv);
       if constexpr (KC == 64) {
         ptx::tmem_ld32(ts + 32, rv + 32);
@@ -339,7 +332,7 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
       ptx::tmem_ld_wait();
       ptx::tc_fence_before();
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(&s_empty[sb]);
+      if (lane == 0) ptx::mbar_arrive(&s_empty[gi]);
       float sc[KC];
       float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};   // independent chains
       // scores in natural units: q.k * scale + bias (the row's 64 biases come as eight 16-byte reads
@@ -380,15 +373,13 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
       const float inv = 1.f / ((sum4[0] + sum4[1]) + (sum4[2] + sum4[3]));
       // drain this group's previous unit: its P V has finished by now, and the O buffer it frees is
       // the one this unit's P V accumulates into
-      if (done > 0) epilogue(u - 2, inv_prev, n_prev);
+      if (done > 0) epilogue(done - 1, inv_prev, n_prev);
       if (!ok) break;
       // previous P V must have completed before P is overwritten
-      ok = ptx::mbar_wait(&p_empty[gi], ((u >> 1) & 1) ^ 1, abort_flag, g.status);
+      ok = ptx::mbar_wait(&p_empty[gi], (done & 1) ^ 1, abort_flag, g.status);
       if (!ok) break;
-      // P row r (bf16 pairs): its window's 64 keys are packed columns w*32 .. w*32+31 of the group's P region;
-      // the other window's half of the row was zeroed once and is never written
       ptx::tc_fence_after();
-      ptx::tmem_st32(tmem_base + TM_P + gi * 64 + lane_addr + w * 32, pk);
+      ptx::tmem_st32(tmem_base + TM_P + gi * 32 + lane_addr, pk);
       ptx::tmem_st_wait();
       ptx::tc_fence_before();
       __syncwarp();
@@ -396,10 +387,11 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
       inv_prev = inv;
       n_prev = n;
     }
-    if (ok && done > 0) epilogue(u - 2, inv_prev, n_prev);
-  } else if (warp < 2 + kGroups * kSoftmaxWarps + kLoaderWarps) {
+    if (ok && done > 0) epilogue(done - 1, inv_prev, n_prev);
+  } else {
     // ---- helper loaders for operands TMA cannot address (e.g. a materialised K^T) ----------------
-    if (any_manual) {
+    if constexpr (MANUAL) {
+      const AttnOperand* ops[3] = {&a.q, &a.k, &a.v};
       const int lt = tid - 32 * (2 + kGroups * kSoftmaxWarps);
       bool ok = true;
       uint32_t it = 0;
@@ -510,19 +502,19 @@ int launch_window_attention_tc(const WinAttnArgs& a_in, long long n_windows, cud
       g.merged = 1;
     }
   }
-  const size_t smem = 1024 + NSTAGE * STAGE_BYTES + TP * BIAS_ROW * 4 + (2 * kGroups + 1) * TP * 4 +
-                      (2 * NSTAGE + 12) * 8 + 16;
-  if (ensure_max_dynamic_smem((const void*)win_attn_tc_kernel<56>, (int)smem) != SMARTMEM_OK ||
-      ensure_max_dynamic_smem((const void*)win_attn_tc_kernel<64>, (int)smem) != SMARTMEM_OK)
-    return SMARTMEM_ERR_CUDA;
+  const size_t smem = 1024 + NSTAGE * STAGE_BYTES + TP * BIAS_ROW * 4 + 5 * TP * 4 +
+                      (2 * NSTAGE + 6 * kMaxGroups) * 8 + 16;
+  const bool manual = g.tma_mask != 7;
+  auto* kern = a.T <= 56 ? (manual ? win_attn_tc_kernel<56, true> : win_attn_tc_kernel<56, false>)
+                         : (manual ? win_attn_tc_kernel<64, true> : win_attn_tc_kernel<64, false>);
+  if (ensure_max_dynamic_smem((const void*)kern, (int)smem) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   const int sms = tc_sm_count();
   long long per_head = (long long)sms / a.heads;
   if (per_head < 1) per_head = 1;
   if (per_head > g.n_pairs) per_head = g.n_pairs;
   const unsigned grid = (unsigned)(per_head * a.heads);
   profile_tick("window_attention_tc", st);
-  if (a.T <= 56) launch_pdl(win_attn_tc_kernel<56>, dim3(grid), dim3(kThreads), smem, st, tm[0], tm[1], tm[2], g);
-  else launch_pdl(win_attn_tc_kernel<64>, dim3(grid), dim3(kThreads), smem, st, tm[0], tm[1], tm[2], g);
+  launch_pdl(kern, dim3(grid), dim3(threads_of(manual)), smem, st, tm[0], tm[1], tm[2], g);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? SMARTMEM_OK : SMARTMEM_ERR_CUDA;
 }
