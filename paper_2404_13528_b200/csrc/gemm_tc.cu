@@ -388,7 +388,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     constexpr bool EARLY = DIRECT && LEAN;                   // accumulator slice to registers first, buffer released at once
     constexpr int RC = (BN == 256 && STAGES == 4 && !PAIR && !LEAN) ? 16 : (CG > 32 ? 32 : CG);   // 4 stages leave less staging room
     constexpr int ROUNDS = CG / RC;
-    constexpr int RH = ROUNDS > 1 ? ROUNDS / 2 : 1;          // BN == 256: rounds [0, RH) hold the first halves of rotary pairs
+    constexpr int RH = ROUNDS > 1 ? ROUNDS / 2 : 1;
     constexpr int VPR = RC / 8;                              // 16-byte vectors per row per round
     constexpr int STG_ROW = RC * 2 + 16;                     // bytes; the pad keeps phase 1 conflict-free
     const int e = warp - 2;
@@ -397,6 +397,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     constexpr bool QSTAGE = !DIRECT && !(BN == 256 && STAGES == 4);  // per-quadrant staging of whole rows
     constexpr bool QBULK = BN == 256 && !A_MN && !QTMA;      // staged rows leave as bulk copies (512-byte rows; not the MN-major-A kernel: 13.1 vs 12.1 us)
     constexpr bool BARE = QTMA;                              // nothing but conversion and store: no bias, GELU, residual, rotation, map or second copy
+    constexpr bool ROPE = !LEAN && !BARE && !A_MN && BN >= 128;   // kernels that rotate columns
     constexpr int QROW = BN * 2 + 16;                        // bytes; the pad keeps phase 1 conflict-free
     uint8_t* stage = stage_base + e * (32 * STG_ROW);
     uint8_t* qstage = stage_base + q * (32 * QROW);
@@ -412,13 +413,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const TileIdx ti_ = item.ti;
       const uint32_t tile_n = ti_.tile_n, tile_m = PAIR ? 2 * ti_.tile_m + rank : ti_.tile_m, batch = ti_.batch;
       const uint32_t buf = it & 1, use = it >> 1;
-      if (HALVES && item.half && grp >= 2) {                 // a half's 128 columns are the first two groups'
+      const int n0 = tile_n * BN + (HALVES ? item.n_off : 0);
+      const bool rope_tile = ROPE && g.rope_cols > 0 && n0 < g.rope_cols;
+      if (HALVES && item.half && grp >= 2 && !rope_tile) {   // a half's 128 columns are the first two groups' (of a rotated one, everybody's)
         ok = ptx::mbar_wait(&tmem_full[buf], use & 1, abort_flag, g.status);
         if (!ok) break;
         if (lane == 0) ptx::mbar_arrive_cluster(tmem_empty0 + buf * 8);
         continue;
       }
-      const int n0 = tile_n * BN + (HALVES ? item.n_off : 0);
       const int row = tile_m * BM + q * 32 + lane;
       const bool row_ok = row < g.M;
       long long o2_base = 0;                                 // second copy: row = b * S + s goes to out2[b][col][s]
@@ -450,7 +452,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         off += (long long)batch * g.out_batch_stride;
       }
       const __nv_bfloat16* __restrict__ rrow = (RES && !BARE && g.residual) ? g.residual + off : nullptr;
-      const bool rope_tile = !LEAN && !BARE && (BN == 256 || BN == 128) && g.rope_cols > 0 && n0 < g.rope_cols;
       auto col_of = [&](int rd) {
         return BN == 256 ? 128 * (grp >> 1) + 32 * (grp & 1) + RC * (rd % RH) + 64 * (rd / RH) : grp * CG;
       };
@@ -497,6 +498,32 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
       }
 
+      // Rotated columns: pairs (i, i + R/2) of the first R columns of each 128-wide head (R = 128: the whole head).  A warp takes the 16 pairs
+      // i = 16 grp + j of every head of the tile (both halves of a pair, as two blocks of 16 columns), or past R two blocks that stay as they
+      // are, so each angle's sine and cosine are worked out once per row and tile, while the products still run.  One element at a time, after
+      // them, they were three operations of the special-function unit each, 3 us of a 128 x 256 tile: a layer of 666 rows, hidden 1024, was
+      // 4.1 us slower with all columns rotated than with 32 of 128.
+      const int rope_blocks = g.rope_half >> 4;              // blocks of 16 columns in half of R: 1, 2 or 4
+      const bool rotated = grp < rope_blocks;
+      float sn[ROPE ? 16 : 1], cs[ROPE ? 16 : 1];
+      if constexpr (ROPE) {
+        if (rope_tile && rotated) {
+          // angle = position * theta^(-i/(R/2)), reduced mod 2 pi in two steps, then the hardware sine / cosine: no table traffic (a [S, 64]
+          // table read 16 bytes per lane per row slowed the whole kernel by a fifth)
+          const float pos = (float)(row_ok ? g.rope_pos0 + row % g.rope_S : 0);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            float f;
+            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(-(float)(grp * 16 + j) * g.rope_c));
+            const float ang = pos * f;
+            const float kk = rintf(ang * 0.15915494309189535f);
+            float red = fmaf(-kk, 6.2831854820251465f, ang);
+            red = fmaf(kk, 1.7484556e-7f, red);
+            sn[j] = __sinf(red);
+            cs[j] = __cosf(red);
+          }
+        }
+      }
       ok = ptx::mbar_wait(&tmem_full[buf], use & 1, abort_flag, g.status);
       if (!ok) break;
       ptx::tc_fence_after();
@@ -527,6 +554,57 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           else ptx::mbar_arrive(&tmem_empty[buf]);
         }
       }
+      if constexpr (ROPE) {
+        if (rope_tile) {
+          const int b0 = rotated ? grp : grp / rope_blocks * 2 * rope_blocks + grp % rope_blocks;
+          auto put = [&](int c0, const uint32_t (&w)[8]) {   // 16 columns of the thread's row
+            const uint4 lo = make_uint4(w[0], w[1], w[2], w[3]), hi = make_uint4(w[4], w[5], w[6], w[7]);
+            if constexpr (DIRECT) {
+              if (row_ok) ptx::st_global_v8(out_t + off + n0 + c0, lo, hi);
+            } else if constexpr (QSTAGE) {
+              *reinterpret_cast<uint4*>(qstage + lane * QROW + c0 * 2) = lo;
+              *reinterpret_cast<uint4*>(qstage + lane * QROW + c0 * 2 + 16) = hi;
+            } else {
+              *reinterpret_cast<uint4*>(stage + lane * STG_ROW) = lo;
+              *reinterpret_cast<uint4*>(stage + lane * STG_ROW + 16) = hi;
+              __syncwarp();
+#pragma unroll
+              for (int i = 0; i < 2; ++i) {
+                const int rr = (lane + 32 * i) >> 1, seg = lane & 1;
+                const long long roff = __shfl_sync(0xFFFFFFFFu, off, rr);
+                const int rok = __shfl_sync(0xFFFFFFFFu, (int)row_ok, rr);
+                const uint4 pk = *reinterpret_cast<const uint4*>(stage + rr * STG_ROW + seg * 16);
+                if (rok) *reinterpret_cast<uint4*>(out_t + roff + n0 + c0 + seg * 8) = pk;
+              }
+              __syncwarp();
+            }
+          };
+          const int heads = HALVES && item.half ? 1 : BN / 128;
+#pragma unroll 1
+          for (int h = 0; h < heads; ++h) {
+            const int c0 = h * 128 + b0 * 16, c1 = c0 + rope_blocks * 16;
+            uint32_t x[16], y[16], w[8];
+            ptx::tmem_ld16(taddr + c0, x);
+            ptx::tmem_ld16(taddr + c1, y);
+            ptx::tmem_ld_wait();
+            if (rotated) {
+#pragma unroll
+              for (int j = 0; j < 16; ++j) {
+                const float a = __uint_as_float(x[j]), b = __uint_as_float(y[j]);
+                x[j] = __float_as_uint(a * cs[j] - b * sn[j]);
+                y[j] = __float_as_uint(b * cs[j] + a * sn[j]);
+              }
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) w[j] = float2_to_bf16x2(__uint_as_float(x[2 * j]), __uint_as_float(x[2 * j + 1]));
+            put(c0, w);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) w[j] = float2_to_bf16x2(__uint_as_float(y[2 * j]), __uint_as_float(y[2 * j + 1]));
+            put(c1, w);
+          }
+        }
+      }
+      if (!rope_tile) {
 #pragma unroll
       for (int rd = 0; rd < ROUNDS; ++rd) {
         const int c0 = col_of(rd);
@@ -540,46 +618,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           }
         }
         {
-          uint32_t rv_local[EARLY ? 1 : RC], rw[EARLY ? 1 : RC];
+          uint32_t rv_local[EARLY ? 1 : RC];
           uint32_t* rv = EARLY ? rall[EARLY ? rd : 0] : rv_local;
-          if constexpr (!EARLY) ptx::tmem_ld_cols<RC>(taddr + c0, rv);
-          // rotary pairs are (i, i + R/2) inside the first R columns of a 128-column head (R = 128: the
-          // whole head).  This round's RC columns start at head-local column hc0; they rotate iff hc0 < R,
-          // and their partners are the RC columns R/2 further up or down (or, when R/2 < RC, the other
-          // half of this very round), read from TMEM a second time.
-          const int hc0 = c0 & 127, half = g.rope_half;
-          if (rope_tile && hc0 < 2 * half) {
-            const bool in_round = half < RC;                 // R = 32 with 32-column rounds: pairs (j, j + 16) of this round
-            const bool first_half = hc0 < half;
-            if constexpr (!EARLY) {
-              if (!in_round) ptx::tmem_ld_cols<RC>(taddr + (first_half ? c0 + half : c0 - half), rw);
-              ptx::tmem_ld_wait();
-            }
-            // angle = position * theta^(-i/(R/2)), reduced mod 2 pi in two steps, then the hardware
-            // sine / cosine: no table traffic (a [S, 64] table read 16 bytes per lane per row
-            // slowed the whole kernel by a fifth)
-            const float pos = (float)(row_ok ? g.rope_pos0 + row % g.rope_S : 0);
-            const int i0 = in_round ? 0 : hc0 - (first_half ? 0 : half);
-#pragma unroll
-            for (int j = 0; j < RC; ++j) {
-              const bool fh = in_round ? j < RC / 2 : first_half;
-              const int i = in_round ? (j & (RC / 2 - 1)) : i0 + j;
-              float f;
-              asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(-(float)i * g.rope_c));
-              const float ang = pos * f;
-              const float kk = rintf(ang * 0.15915494309189535f);
-              float red = fmaf(-kk, 6.2831854820251465f, ang);
-              red = fmaf(kk, 1.7484556e-7f, red);
-              const float sn = __sinf(red), cs = __cosf(red);
-              const float x = __uint_as_float(rv[j]);
-              const float y = __uint_as_float(in_round ? rv[j ^ (RC / 2)] : rw[j]);
-              acc[j] = fh ? x * cs - y * sn : x * cs + y * sn;
-            }
-          } else {
-            if constexpr (!EARLY) ptx::tmem_ld_wait();
-#pragma unroll
-            for (int j = 0; j < RC; ++j) acc[j] = __uint_as_float(rv[j]);
+          if constexpr (!EARLY) {
+            ptx::tmem_ld_cols<RC>(taddr + c0, rv);
+            ptx::tmem_ld_wait();
           }
+#pragma unroll
+          for (int j = 0; j < RC; ++j) acc[j] = __uint_as_float(rv[j]);
         }
         if (!BARE && g.bias) {
 #pragma unroll
@@ -669,6 +715,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           }
           __syncwarp();
         }
+      }
       }
       // all of this warp's TMEM reads of the buffer have completed (wait::ld above)
       if constexpr (!EARLY) {
@@ -1075,7 +1122,7 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
   if (B.k_stride != 1) return SMARTMEM_ERR_UNSUPPORTED;
   const bool splitk_ok = gemm_splitk_supported(A, B, ep, batch, M, N, K);
   if (ep.rms_gamma) return splitk_ok ? launch_gemm_splitk(A, B, ep, M, N, K, st) : SMARTMEM_ERR_UNSUPPORTED;
-  if (ep.rope_cols > 0 && (N % 256 || ep.rope_cols % 256 || ep.rope_S < 1)) return SMARTMEM_ERR_UNSUPPORTED;
+  if (ep.rope_cols > 0 && (N % 256 || ep.rope_cols % 256 || ep.rope_S < 1 || a_mn || ep.bias || ep.gelu || ep.residual || ep.out2)) return SMARTMEM_ERR_UNSUPPORTED;
   if (ep.rope_cols > 0 && ep.rope_dim != 0 && ep.rope_dim != 32 && ep.rope_dim != 64 && ep.rope_dim != 128) return SMARTMEM_ERR_UNSUPPORTED;
   if (ep.seg_cols > 0) {
     if (ep.seg_cols % 256 || N > 3ll * ep.seg_cols || ep.rowmap || ep.residual || batch != 1) return SMARTMEM_ERR_UNSUPPORTED;

@@ -55,6 +55,14 @@ def test_partial_rotary_layers(B, S, hidden, heads, rot):
     case(32, B, S, hidden, heads, 0, rotary_dim=rot)
 
 
+@pytest.mark.parametrize("B,S,hidden,rot", [(1, 80, 1024, 64), (3, 43, 1024, 0), (1, 300, 2048, 32), (1, 300, 3072, 64), (1, 300, 3072, 0), (2, 260, 3072, 0),
+                                            (4, 130, 3072, 32)])
+def test_rotated_tiles(B, S, hidden, rot):
+    """The QKV product's tiles with rotated columns: 128 columns on one CTA and on a pair, 256 on a pair, whole and as halves (520 rows of 3072);
+    16, 32 and 64 pairs a head, several sequences to a tile, rows past the end."""
+    case(33, B, S, hidden, hidden // 128, 1, rotary_dim=rot, first_rows_allowance=B * S * hidden // 10000 + 2)
+
+
 def test_partial_rotary_layer_full_size():
     """Config 5's shape with rotary_dim 32 (a quarter of the head, as in the Pythia family)."""
     case(5, 1, 2048, 4096, 32, 0, rotary_dim=32, first_rows_allowance=8)
