@@ -1,8 +1,8 @@
 // Causal attention (prefill, head dimension 128) on the tcgen05 tensor cores.
 //
 // One CTA = 128 query positions of one head.  K and V stream through shared memory in tiles of
-// 64 keys (TMA, three stages of keys, two of values); S = Q K^T and O += P V are tcgen05.mma with the accumulators in
-// TMEM (two S buffers, one O: 256 columns); four softmax warps own one query row per thread (the TMEM lane),
+// 64 keys (TMA, three stages of keys and two of values a group); S = Q K^T and O += P V are tcgen05.mma with the accumulators in
+// TMEM (two S buffers and one O a group: 256 columns); the four warps of a softmax group own one query row per thread (the TMEM lane),
 // so row maxima and sums need no shuffles.  P goes back to the tensor core through tensor memory: it is
 // written as bf16 pairs over the S buffer it was computed from and read by the second MMA as its A
 // operand; V is consumed as it lies in memory ([key, d] rows) through the MN-major operand mode, so no
@@ -10,9 +10,10 @@
 // refreshed when it grows by more than 2^8 (then O and the running sum are rescaled), which keeps
 // the TMEM read-modify-write of O off the common path.
 //
-// The 64-key tiles keep a CTA at 112 KB of shared memory and 256 TMEM columns, so TWO CTAs share an
-// SM: while one is in its softmax (which is bound by the exponential unit) the other one's MMAs
-// run, which a single CTA with one softmax group could not overlap.
+// A tile's softmax is a chain of about 1500 cycles for its group, in which the SM is nearly idle.  Where the query tiles fill the chip
+// twice, TWO CTAs of one group share an SM (112 KB of shared memory and 256 TMEM columns each): while one is in its softmax the
+// other one's MMAs run.  Where they do not, a CTA has two groups, which take the key tiles in turn with a running maximum, a sum and
+// an O of their own; the shares of a row meet at the end in the threads that own its lane, so the longest rows take half as long.
 //
 // q, k, v are addressed as TMA boxes inside the buffer the QKV GEMM wrote ([B*S, 3*H*D], head split
 // eliminated) or inside materialised [B, H, S, D] tensors (explicit variant); the output tile is
@@ -28,10 +29,14 @@ namespace {
 constexpr int BQ = 128, BKV = 64, D = 128;
 constexpr int KB = 128 * 64 * 2;                      // one 128 x 64 bf16 block (Q, P)
 constexpr int KBK = BKV * 64 * 2;                     // one 64 x 64 bf16 block (K, V)
-constexpr uint32_t TM_S = 0, TM_O = 128, TMEM_COLS = 256;   // two S buffers of 64 columns, O of 128: two CTAs share an SM's 512
-constexpr int KSTAGES = 3, N_BARS = 1 + 2 * KSTAGES + 4 + 4 + 4;
-constexpr uint32_t SMEM_BYTES = 2 * KB + (2 * KSTAGES + 4) * KBK + N_BARS * 8 + 16;
-constexpr int kThreads = 192;
+// G softmax groups: key tile j belongs to group j % G, which has two S buffers of 64 columns and an O of 128
+template <int G>
+struct Sizes {
+  static constexpr int NS = 2 * G, KSTAGES = 3 * G, VSTAGES = 2 * G, THREADS = 64 + 128 * G;
+  static constexpr uint32_t TM_S = 0, TM_O = NS * BKV, TMEM_COLS = 256 * G;
+  static constexpr int N_BARS = 1 + 2 * KSTAGES + 2 * VSTAGES + 3 * NS + G + 1;
+  static constexpr uint32_t SMEM = 2 * KB + 2 * (KSTAGES + VSTAGES) * KBK + N_BARS * 8 + 16 + (G > 1 ? G * BQ * 8 : 0);
+};
 constexpr float kRescaleThreshold = 8.0f;             // log2 units
 
 struct TcAttnArgs {
@@ -57,22 +62,27 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   return y;
 }
 
-__global__ void __launch_bounds__(kThreads, 2)
+template <int G>
+__global__ void __launch_bounds__(Sizes<G>::THREADS, 3 - G)
 causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                       const __grid_constant__ CUtensorMap tmV, const __grid_constant__ TcAttnArgs g) {
+  using Z = Sizes<G>;
+  constexpr int KSTAGES = Z::KSTAGES, VSTAGES = Z::VSTAGES, NS = Z::NS;
+  constexpr uint32_t TM_S = Z::TM_S, TM_O = Z::TM_O, TMEM_COLS = Z::TMEM_COLS;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const uint32_t pad = (1024u - (ptx::smem_u32(smem_raw) & 1023u)) & 1023u;
   uint8_t* smem = smem_raw + pad;
   uint8_t* sQ = smem;                                  // [2 k-blocks][16 KB]
-  uint8_t* sK = sQ + 2 * KB;                           // [3 stages][2 k-blocks][8 KB]
-  uint8_t* sV = sK + 2 * KSTAGES * KBK;                // [2 stages][2 d-chunks][8 KB]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(sV + 4 * KBK);
-  uint64_t *q_full = bars, *k_full = bars + 1, *k_empty = k_full + KSTAGES, *v_full = k_empty + KSTAGES, *v_empty = v_full + 2;
-  uint64_t *s_full = v_empty + 2, *s_empty = s_full + 2, *p_full = s_empty + 2, *p_empty = p_full + 2, *o_done = p_empty + 1;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + N_BARS);
+  uint8_t* sK = sQ + 2 * KB;                           // [stages][2 k-blocks][8 KB]
+  uint8_t* sV = sK + 2 * KSTAGES * KBK;                // [stages][2 d-chunks][8 KB]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sV + 2 * VSTAGES * KBK);
+  uint64_t *q_full = bars, *k_full = bars + 1, *k_empty = k_full + KSTAGES, *v_full = k_empty + KSTAGES, *v_empty = v_full + VSTAGES;
+  uint64_t *s_full = v_empty + VSTAGES, *s_empty = s_full + NS, *p_full = s_empty + NS, *p_empty = p_full + NS, *o_done = p_empty + G;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + Z::N_BARS);
   int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
+  float2* ml_s = reinterpret_cast<float2*>(tmem_slot + 4);      // (G > 1) [G][128]: a row's maximum and sum over its group's keys
 
-  if (pad + SMEM_BYTES > g.smem_bytes) {
+  if (pad + Z::SMEM > g.smem_bytes) {
     if (threadIdx.x == 0) atomicExch(g.status, (int)SMARTMEM_ERR_UNSUPPORTED);
     return;
   }
@@ -91,16 +101,18 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       ptx::mbar_init(&k_full[i], 1);
       ptx::mbar_init(&k_empty[i], 1);
     }
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < VSTAGES; ++i) {
       ptx::mbar_init(&v_full[i], 1);
       ptx::mbar_init(&v_empty[i], 1);
+    }
+    for (int i = 0; i < NS; ++i) {
       ptx::mbar_init(&s_full[i], 1);
-      ptx::mbar_init(&s_empty[i], 1);                 // P(j) lives in S buffer j & 1: freed by the commit of P V (j)
+      ptx::mbar_init(&s_empty[i], 1);                 // P(j) lives in S buffer j % NS: freed by the commit of P V (j)
     }
     // (a barrier per S buffer: the softmax may be two tiles ahead of P V, and with one for both the issuing warp, held up for that long by a
     // slow read in its wait, found the phase that it waited for already followed by another and waited for good)
-    for (int i = 0; i < 2; ++i) ptx::mbar_init(&p_full[i], 4);
-    ptx::mbar_init(p_empty, 1);
+    for (int i = 0; i < NS; ++i) ptx::mbar_init(&p_full[i], 4);
+    for (int i = 0; i < G; ++i) ptx::mbar_init(&p_empty[i], 1);
     ptx::mbar_init(o_done, 1);
     *abort_flag = 0;
     ptx::fence_barrier_init();
@@ -143,8 +155,8 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         if (++ks == KSTAGES) { ks = 0; kph ^= 1; }
       }
       if (i >= 0) {
-        const int s = i & 1;
-        ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(&v_empty[s], ((i >> 1) & 1) ^ 1, abort_flag, g.status) ? 1 : 0) != 0;
+        const int s = i % VSTAGES;
+        ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(&v_empty[s], ((i / VSTAGES) & 1) ^ 1, abort_flag, g.status) ? 1 : 0) != 0;
         if (!ok) break;
         if (ptx::elect_one()) {
           ptx::mbar_expect_tx(&v_full[s], 2 * KBK);
@@ -162,8 +174,8 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       bool ok = __all_sync(0xFFFFFFFFu, ptx::mbar_wait(q_full, 0, abort_flag, g.status) ? 1 : 0) != 0;
       uint32_t kst = 0, kph = 0;
       auto issue_s = [&](int j) {
-        const int s = j & 1;
-        const uint32_t ph = (j >> 1) & 1;
+        const int s = j % NS;
+        const uint32_t ph = (j / NS) & 1;
         ok = ok && ptx::mbar_wait(&s_empty[s], ph ^ 1, abort_flag, g.status);
         ok = ok && ptx::mbar_wait(&k_full[kst], kph, abort_flag, g.status);
         ok = __all_sync(0xFFFFFFFFu, ok ? 1 : 0) != 0;
@@ -185,9 +197,10 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         if (++kst == KSTAGES) { kst = 0; kph ^= 1; }
       };
       auto issue_pv = [&](int j) {
-        const int s = j & 1;
-        ok = ok && ptx::mbar_wait(&p_full[s], (j >> 1) & 1, abort_flag, g.status);
-        ok = ok && ptx::mbar_wait(&v_full[s], (j >> 1) & 1, abort_flag, g.status);
+        static_assert(NS == VSTAGES, "one index for both");
+        const int s = j % NS;
+        ok = ok && ptx::mbar_wait(&p_full[s], (j / NS) & 1, abort_flag, g.status);
+        ok = ok && ptx::mbar_wait(&v_full[s], (j / NS) & 1, abort_flag, g.status);
         ok = __all_sync(0xFFFFFFFFu, ok ? 1 : 0) != 0;
         if (!ok) return;
         ptx::tc_fence_after();
@@ -197,16 +210,16 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         if (ptx::elect_one()) {
 #pragma unroll
           for (int ks = 0; ks < BKV / 16; ++ks)        // 16 keys per step: P +8 packed columns, V +16 rows of 128 bytes; the two 64-wide d-chunks are KBK apart
-            ptx::tc_mma_bf16_ta(tmem_base + TM_O, pa + 8 * ks, vd + (2048 >> 4) * ks, idesc_pv, (j | ks) ? 1u : 0u);
+            ptx::tc_mma_bf16_ta(tmem_base + TM_O + (j % G) * D, pa + 8 * ks, vd + (2048 >> 4) * ks, idesc_pv, (j >= G || ks) ? 1u : 0u);
           ptx::tc_commit(&v_empty[s]);
           ptx::tc_commit(&s_empty[s]);
-          ptx::tc_commit(p_empty);
+          ptx::tc_commit(&p_empty[j % G]);
         }
         __syncwarp();
       };
-      issue_s(0);
+      for (int j = 0; j < G && j < n_kv && ok; ++j) issue_s(j);
       for (int j = 0; j < n_kv && ok; ++j) {
-        if (j + 1 < n_kv) issue_s(j + 1);
+        if (j + G < n_kv) issue_s(j + G);
         issue_pv(j);
       }
       if (ok && ptx::elect_one()) ptx::tc_commit(o_done);
@@ -216,11 +229,12 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     const int r = q * 32 + lane;                       // query row inside the tile
     const int qi = qt * BQ + r;                        // position
     const uint32_t lane_addr = (uint32_t)(q * 32) << 16;
+    const int gi = G > 1 ? (warp - 2) >> 2 : 0;
     float m_used = -INFINITY, l = 0.f;
     bool ok = true;
-    for (int j = 0; j < n_kv && ok; ++j) {
-      const int sb = j & 1;
-      ok = ptx::mbar_wait(&s_full[sb], (j >> 1) & 1, abort_flag, g.status);
+    for (int j = gi, turn = 0; j < n_kv && ok; j += G, ++turn) {
+      const int sb = j % NS;
+      ok = ptx::mbar_wait(&s_full[sb], (j / NS) & 1, abort_flag, g.status);
       if (!ok) break;
       ptx::tc_fence_after();
       const uint32_t ts = tmem_base + TM_S + sb * BKV + lane_addr;
@@ -248,11 +262,13 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         corr = ex2(m_used - mx);                       // 0 on the first tile
         l *= corr;
         m_used = mx;
-        rescale = j > 0;
+        rescale = turn > 0;
       }
+      // (the second group's first tile can lie past the row's position as a whole: its probabilities are 2^-inf then)
+      const float nm = G > 1 && m_used == -INFINITY ? 0.f : -m_used;
       // p = 2^(s - m), packed to bf16 for the second MMA
       uint32_t pk[BKV / 2];
-      const ptx::f32x2 sc2 = ptx::pack2(g.scale_log2, g.scale_log2), nm2 = ptx::pack2(-m_used, -m_used);
+      const ptx::f32x2 sc2 = ptx::pack2(g.scale_log2, g.scale_log2), nm2 = ptx::pack2(nm, nm);
       ptx::f32x2 l2[2] = {ptx::pack2(0.f, 0.f), ptx::pack2(0.f, 0.f)};
 #pragma unroll
       for (int c = 0; c < BKV; c += 2) {
@@ -269,10 +285,10 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       }
       if (__any_sync(0xFFFFFFFFu, rescale)) {
         // O is rescaled in place: the previous P V, which accumulates into it, must have completed
-        ok = ptx::mbar_wait(p_empty, (j & 1) ^ 1, abort_flag, g.status);
+        ok = ptx::mbar_wait(&p_empty[gi], (turn & 1) ^ 1, abort_flag, g.status);
         if (!ok) break;
         ptx::tc_fence_after();
-        const uint32_t to = tmem_base + TM_O + lane_addr;
+        const uint32_t to = tmem_base + TM_O + gi * D + lane_addr;
 #pragma unroll 1
         for (int ch = 0; ch < 4; ++ch) {
           uint32_t ro[32];
@@ -292,17 +308,37 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       __syncwarp();
       if (lane == 0) ptx::mbar_arrive(&p_full[sb]);
     }
+    // the groups' shares of a row meet: O = (O0 w0 + O1 w1) / (l0 w0 + l1 w1), w = 2^(m - max m), each group storing half of the columns
+    float w0 = 1.f, w1 = 0.f, lsum = l;
+    if constexpr (G > 1) {
+      ml_s[gi * BQ + r] = make_float2(m_used, l);
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      const float2 a = ml_s[r], c = ml_s[BQ + r];
+      const float mt = fmaxf(a.x, c.x);
+      w0 = ex2(a.x - mt);
+      w1 = ex2(c.x - mt);
+      lsum = a.y * w0 + c.y * w1;
+    }
     if (ok) ok = ptx::mbar_wait(o_done, 0, abort_flag, g.status);
     if (ok) {
       ptx::tc_fence_after();
-      const float inv = 1.f / l;
+      const float inv = 1.f / lsum;
       const bool wide_store = (reinterpret_cast<uintptr_t>(g.out) & 31) == 0 && g.o_sn % 16 == 0 && g.o_sh % 16 == 0 && g.o_st % 16 == 0;
       __nv_bfloat16* orow = g.out + (long long)b * g.o_sn + (long long)h * g.o_sh + (long long)qi * g.o_st;
       const uint32_t to = tmem_base + TM_O + lane_addr;
 #pragma unroll 1
-      for (int ch = 0; ch < 4; ++ch) {
+      for (int ch = gi * (4 / G); ch < (gi + 1) * (4 / G); ++ch) {
         uint32_t rv[32];
         ptx::tmem_ld32(to + ch * 32, rv);
+        if constexpr (G > 1) {
+          if (n_kv > 1) {                                // (with one tile the second group has no O)
+            uint32_t rw[32];
+            ptx::tmem_ld32(to + D + ch * 32, rw);
+            ptx::tmem_ld_wait();
+#pragma unroll
+            for (int c = 0; c < 32; ++c) rv[c] = __float_as_uint(__uint_as_float(rv[c]) * w0 + __uint_as_float(rw[c]) * w1);
+          }
+        }
         ptx::tmem_ld_wait();
         if (qi < g.S && wide_store) {                    // whole 32-byte sectors per store
 #pragma unroll
@@ -384,15 +420,21 @@ int launch_causal_attention_tc(const CausalAttnArgs& a, cudaStream_t st) {
   g.scale_log2 = a.scale * 1.4426950408889634f;
   g.status = device_status_ptr();
   if (!g.status) return SMARTMEM_ERR_CUDA;
-  // 112 KB of tiles: two CTAs per SM only fit without a spare kilobyte of alignment slack (the kernel
-  // reports a misaligned base instead of overrunning)
-  const size_t smem = SMEM_BYTES;
-  g.smem_bytes = (uint32_t)smem;
-  if (ensure_max_dynamic_smem((const void*)causal_attn_tc_kernel, (int)smem, 100) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   const long long ctas = (long long)g.n_qt * B * H;
   if (ctas >= (1ll << 31)) return SMARTMEM_ERR_UNSUPPORTED;
+  // Two softmax groups on an SM's one CTA, or two CTAs of one group each: the first where every CTA has an SM to itself, or nearly so and
+  // the longest rows decide.  Us of a layer, one group -> two: 48 CTAs (2 x 333, hidden 1024) 23.9 -> 21.6, 96 (2 x 333, 2048) 37.8 -> 35.5, (1 x 1500,
+  // 1024) 42.5 -> 37.4, 128 (1 x 2048, 1024) 50.9 -> 46.6, (1 x 512, 4096) 94.1 -> 90.5; 192 (1 x 1500, 2048) 75.1 -> 68.1, 256 (1 x 2048, 2048) 91.6 -> 89.5,
+  // but 192 (4 x 333, 2048) 54.7 -> 55.7, 256 (4 x 512, 2048) 69.7 -> 71.5, 384 (1 x 1500, 4096) 187 -> 194, 512 (1 x 2048, 4096) 289 -> 307.
+  const bool two = S > BKV && (ctas <= tc_sm_count() || (ctas <= 2 * tc_sm_count() && g.n_qt >= 10));
+  // 112 KB of tiles: two CTAs per SM only fit without a spare kilobyte of alignment slack (the kernel
+  // reports a misaligned base instead of overrunning)
+  const size_t smem = two ? Sizes<2>::SMEM : Sizes<1>::SMEM;
+  g.smem_bytes = (uint32_t)smem;
+  auto* kern = two ? causal_attn_tc_kernel<2> : causal_attn_tc_kernel<1>;
+  if (ensure_max_dynamic_smem((const void*)kern, (int)smem, 100) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   profile_tick("causal_attention_tc", st);
-  launch_pdl(causal_attn_tc_kernel, dim3((unsigned)ctas), dim3(kThreads), smem, st, tq, tk, tv, g);
+  launch_pdl(kern, dim3((unsigned)ctas), dim3(two ? Sizes<2>::THREADS : Sizes<1>::THREADS), smem, st, tq, tk, tv, g);
   count_launch();
   return cudaGetLastError() == cudaSuccess ? SMARTMEM_OK : SMARTMEM_ERR_CUDA;
 }
