@@ -34,46 +34,92 @@ namespace {
 constexpr int kThreads = 256;                          // of the MLP half
 constexpr int kMaxCluster = 8;
 
-// acc(i, j) = sum_k A[r0 + i][k] W[c0 + j * cs][k], rows and columns clamped to M and N (what lies beyond is not used); K a multiple of 4.
-template <int TM, int TN>
-__device__ __forceinline__ void tile_dot(const float* A, int pa, const float* W, int pw, int M, int N, int K, int r0, int c0, int cs, float (&acc)[TM][TN]) {
+// A product's outputs, mt x nt tiles of TM x TN: a warp takes eight row tiles by four column tiles, a thread the rows tm + i mt and the
+// columns tn + j nt of its tile, so that a warp's reads of either operand are eight or four neighbouring rows: one pass over the banks each.
+// With the lanes along the columns a read of W was up to four passes: [2,21,14,32] in 7 x 7, heads of 16, 8.8 us -> 8.4 this way, [4,16,16,64] in 8 x 8 with
+// its MLP half 32 -> 22.8.  Larger tiles leave too few warps to hide the reads: 8 x 4 and 4 x 4 in place of 4 x 4 and 2 x 4 were a tenth slower.
+struct WarpTile {
+  int tm, tn;
+  bool in;
+  __device__ __forceinline__ WarpTile(int w, int mt, int nt) {
+    const int wr = (mt + 7) >> 3, wc = w / wr, lane = threadIdx.x & 31;
+    tm = (w - wc * wr) * 8 + (lane & 7);
+    tn = wc * 4 + (lane >> 3);
+    in = tm < mt && tn < nt;
+  }
+};
+// warps a product takes
+__device__ __forceinline__ int warp_tiles(int mt, int nt) { return ((mt + 7) >> 3) * ((nt + 3) >> 2); }
+
+// acc(i, j) = sum_k A[r0 + i rs][k] W[c0 + j cs][k], rows and columns clamped to M and N (what lies beyond is not used); K a multiple of 4.
+// Even and odd k are summed apart, as the two halves of packed multiply-adds, where the registers allow it.
+template <int TM, int TN, bool PACKED = (TM * TN <= 8)>
+__device__ __forceinline__ void tile_dot(const float* A, int pa, const float* W, int pw, int M, int N, int K, int r0, int rs, int c0, int cs, float (&acc)[TM][TN]) {
   const float* a[TM];
   const float* w[TN];
 #pragma unroll
-  for (int i = 0; i < TM; ++i) a[i] = A + min(r0 + i, M - 1) * pa;
+  for (int i = 0; i < TM; ++i) a[i] = A + min(r0 + i * rs, M - 1) * pa;
 #pragma unroll
-  for (int j = 0; j < TN; ++j) w[j] = W + min(c0 + j * cs, N - 1) * pw;        // (neighbouring lanes on neighbouring rows)
-#pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
-#pragma unroll (TM * TN > 8 ? 1 : 2)
-  for (int k = 0; k < K; k += 4) {
-    float4 av[TM], wv[TN];
-#pragma unroll
-    for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const float4*>(a[i] + k);
-#pragma unroll
-    for (int j = 0; j < TN; ++j) wv[j] = *reinterpret_cast<const float4*>(w[j] + k);
+  for (int j = 0; j < TN; ++j) w[j] = W + min(c0 + j * cs, N - 1) * pw;
+  if constexpr (PACKED) {
+    ptx::f32x2 s[TM][TN];
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
-      for (int j = 0; j < TN; ++j)
-        acc[i][j] = fmaf(av[i].w, wv[j].w, fmaf(av[i].z, wv[j].z, fmaf(av[i].y, wv[j].y, fmaf(av[i].x, wv[j].x, acc[i][j]))));
+      for (int j = 0; j < TN; ++j) s[i][j] = 0ull;
+#pragma unroll 2
+    for (int k = 0; k < K; k += 4) {
+      ulonglong2 av[TM], wv[TN];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const ulonglong2*>(a[i] + k);
+#pragma unroll
+      for (int j = 0; j < TN; ++j) wv[j] = *reinterpret_cast<const ulonglong2*>(w[j] + k);
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j) s[i][j] = ptx::fma2(av[i].y, wv[j].y, ptx::fma2(av[i].x, wv[j].x, s[i][j]));
+    }
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        float lo, hi;
+        ptx::unpack2(s[i][j], lo, hi);
+        acc[i][j] = lo + hi;
+      }
+  } else {
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+#pragma unroll 1
+    for (int k = 0; k < K; k += 4) {
+      float4 av[TM], wv[TN];
+#pragma unroll
+      for (int i = 0; i < TM; ++i) av[i] = *reinterpret_cast<const float4*>(a[i] + k);
+#pragma unroll
+      for (int j = 0; j < TN; ++j) wv[j] = *reinterpret_cast<const float4*>(w[j] + k);
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
+#pragma unroll
+        for (int j = 0; j < TN; ++j)
+          acc[i][j] = fmaf(av[i].w, wv[j].w, fmaf(av[i].z, wv[j].z, fmaf(av[i].y, wv[j].y, fmaf(av[i].x, wv[j].x, acc[i][j]))));
+    }
   }
 }
 // out(r, c) = sum_k A[r][k] W[c][k] for r < M, c < N; epi(r, c, value)
 template <int TM, int TN, typename Epi>
 __device__ __forceinline__ void tile_gemm(const float* A, int pa, const float* W, int pw, int M, int N, int K, Epi epi) {
-  const int mt = (M + TM - 1) / TM, nt = (N + TN - 1) / TN;
-  for (int idx = threadIdx.x; idx < mt * nt; idx += kThreads) {
-    const int tm = idx / nt, tn = idx - tm * nt;
+  const int mt = (M + TM - 1) / TM, nt = (N + TN - 1) / TN, n = warp_tiles(mt, nt);
+  for (int w = threadIdx.x >> 5; w < n; w += kThreads / 32) {
+    const WarpTile t(w, mt, nt);
     float acc[TM][TN];
-    tile_dot<TM, TN>(A, pa, W, pw, M, N, K, tm * TM, tn, nt, acc);
+    tile_dot<TM, TN>(A, pa, W, pw, M, N, K, t.tm, mt, t.tn, nt, acc);
 #pragma unroll
     for (int i = 0; i < TM; ++i)
 #pragma unroll
       for (int j = 0; j < TN; ++j)
-        if (tm * TM + i < M && tn + j * nt < N) epi(tm * TM + i, tn + j * nt, acc[i][j]);
+        if (t.in && t.tm + i * mt < M && t.tn + j * nt < N) epi(t.tm + i * mt, t.tn + j * nt, acc[i][j]);
   }
 }
 
@@ -135,28 +181,29 @@ struct AttnF32Args {
 };
 
 // q, k and v of one head: a TM x TN tile a thread
-template <int TM, int TN>
+template <int TM, int TN, bool PACKED>
 __device__ __forceinline__ void qkv_phase(const AttnF32Args& g, const float* xs, int pc, const float* wq, const float* bq, float* q, float* k, float* vt, int pd) {
-  const int d = g.d, T = g.T, nt = 3 * d / TN;
-  const int tm = (int)threadIdx.x / nt, tn = (int)threadIdx.x - tm * nt;
-  if (tm * TM >= T) return;
+  const int d = g.d, T = g.T, mt = (T + TM - 1) / TM, nt = 3 * d / TN;
+  const WarpTile t((int)threadIdx.x >> 5, mt, nt);
+  if (!t.in) return;
   float acc[TM][TN];
-  tile_dot<TM, TN>(xs, pc, wq, pc, T, 3 * d, g.C, tm * TM, tn, nt, acc);
+  tile_dot<TM, TN, PACKED>(xs, pc, wq, pc, T, 3 * d, g.C, t.tm, mt, t.tn, nt, acc);
 #pragma unroll
   for (int j = 0; j < TN; ++j) {
-    const int c = tn + j * nt, which = c < d ? 0 : c < 2 * d ? 1 : 2, e = c - which * d;
+    const int c = t.tn + j * nt, which = c < d ? 0 : c < 2 * d ? 1 : 2, e = c - which * d;
     const float b = bq[c], sc = which == 0 ? g.scale : 1.0f;
-    float* dst = which == 0 ? q + tm * TM * pd + e : which == 1 ? k + tm * TM * pd + e : vt + e * g.tp + tm * TM;
-    const int step = which == 2 ? 1 : pd;
+    float* dst = which == 0 ? q + t.tm * pd + e : which == 1 ? k + t.tm * pd + e : vt + e * g.tp + t.tm;
+    const int step = (which == 2 ? 1 : pd) * mt;
 #pragma unroll
     for (int i = 0; i < TM; ++i)
-      if (tm * TM + i < T) dst[i * step] = (acc[i][j] + b) * sc;
+      if (t.tm + i * mt < T) dst[i * step] = (acc[i][j] + b) * sc;
   }
 }
 
-// THREADS: 256 up to 32 tokens, else 512: one output tile a thread in every phase.
-template <int THREADS>
-__global__ void __launch_bounds__(THREADS, THREADS == 256 ? 3 : 2) swin_attn_f32_kernel(const __grid_constant__ AttnF32Args g) {
+// THREADS: 256 up to 32 tokens, else 512: one output tile a thread in every phase.  ALONE: no more CTAs than SMs, so a thread may have all
+// the registers it can use.
+template <int THREADS, bool ALONE>
+__global__ void __launch_bounds__(THREADS, ALONE ? 1 : THREADS == 256 ? 3 : 2) swin_attn_f32_kernel(const __grid_constant__ AttnF32Args g) {
   extern __shared__ __align__(16) float sm[];
   const int C = g.C, d = g.d, T = g.T, pc = C + 4, pd = d + 4, tp = g.tp;
   float* xs = sm;                                      // [T][C]: the normalised rows, later every head's output
@@ -216,27 +263,27 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 3 : 2) swin_attn_f32
   norm_rows<THREADS, 8>(xs, pc, T, C, lng, lnb, g.eps);
   ptx::cp_async_wait<0>();
   __syncthreads();
-  // the smallest tile that gives no thread two (T at most 64 and d 16 or 32: at most 192 and 384 of the largest)
+  // the smallest tile that gives no warp two (T at most 64 and d 16 or 32: at most 6 and 12 of the largest)
   const int t2 = (T + 1) / 2;
-  if (t2 * (3 * d / 2) <= THREADS) qkv_phase<2, 2>(g, xs, pc, wq, bq, q, k, vt, pd);
-  else if (t2 * (3 * d / 4) <= THREADS) qkv_phase<2, 4>(g, xs, pc, wq, bq, q, k, vt, pd);
-  else qkv_phase<4, 4>(g, xs, pc, wq, bq, q, k, vt, pd);
+  if (warp_tiles(t2, 3 * d / 2) <= THREADS / 32) qkv_phase<2, 2, true>(g, xs, pc, wq, bq, q, k, vt, pd);
+  else if (warp_tiles(t2, 3 * d / 4) <= THREADS / 32) qkv_phase<2, 4, true>(g, xs, pc, wq, bq, q, k, vt, pd);
+  else qkv_phase<4, 4, ALONE>(g, xs, pc, wq, bq, q, k, vt, pd);
   __syncthreads();
   {
     const int nk = (T + 3) / 4;
-    const int tm = tid / nk, tn = tid - tm * nk;
-    if (tm * 2 < T) {
+    const WarpTile t(tid >> 5, t2, nk);
+    if (t.in) {
       float acc[2][4];
-      tile_dot<2, 4>(q, pd, k, pd, T, T, d, tm * 2, tn, nk, acc);
-      const int i0 = tm * 2, i1 = min(i0 + 1, T - 1), mid = (g.ws - 1) * 2 * g.ws;
+      tile_dot<2, 4>(q, pd, k, pd, T, T, d, t.tm, t2, t.tn, nk, acc);
+      const int i0 = t.tm, i1 = min(i0 + t2, T - 1), mid = (g.ws - 1) * 2 * g.ws;
       const int c0 = code[i0] + mid, c1 = code[i1] + mid, l0 = label[i0], l1 = label[i1];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int col = tn + j * nk;
+        const int col = t.tn + j * nk;
         if (col < T) {
           const int cc = code[col], lc = label[col];
           P[i0 * tp + col] = acc[0][j] + tab[c0 - cc] - (l0 != lc ? 100.f : 0.f);
-          if (i0 + 1 < T) P[i1 * tp + col] = acc[1][j] + tab[c1 - cc] - (l1 != lc ? 100.f : 0.f);
+          if (i0 + t2 < T) P[i1 * tp + col] = acc[1][j] + tab[c1 - cc] - (l1 != lc ? 100.f : 0.f);
         }
       }
     }
@@ -268,14 +315,15 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 3 : 2) swin_attn_f32
   __syncthreads();
   // o of this head goes straight into every CTA's row buffer: column h d + c of all of them.  A thread has the same two rows and two
   // columns of it and of the projection.
-  const int tm = tid / (d / 2), c0 = tid - tm * (d / 2), c1 = c0 + d / 2, r0 = tm * 2;
-  const bool in0 = r0 < T, in1 = r0 + 1 < T;
+  const WarpTile t(tid >> 5, t2, d / 2);
+  const int c0 = t.tn, c1 = c0 + d / 2, r0 = t.tm, r1 = r0 + t2;
+  const bool in0 = t.in, in1 = t.in && r1 < T;
   float acc[2][2], res[2][2] = {};
-  const long long o0 = in0 ? offs[r0] + h * d : 0, o1 = in1 ? offs[r0 + 1] + h * d : 0;
+  const long long o0 = in0 ? offs[r0] + h * d : 0, o1 = in1 ? offs[r1] + h * d : 0;
   if (in0) { res[0][0] = g.x[o0 + c0]; res[0][1] = g.x[o0 + c1]; }
   if (in1) { res[1][0] = g.x[o1 + c0]; res[1][1] = g.x[o1 + c1]; }
   if (g.heads > 1) ptx::cluster_arrive();              // (everyone has read its normalised rows)
-  if (in0) tile_dot<2, 2>(P, tp, vt, tp, T, d, (T + 3) & ~3, r0, c0, d / 2, acc);
+  if (in0) tile_dot<2, 2>(P, tp, vt, tp, T, d, (T + 3) & ~3, r0, t2, c0, d / 2, acc);
   if (g.heads > 1) ptx::cluster_wait();
   if (in0) {
     const uint32_t xa = ptx::smem_u32(xs), o = (uint32_t)(r0 * pc + h * d + c0) * 4u;
@@ -285,14 +333,14 @@ __global__ void __launch_bounds__(THREADS, THREADS == 256 ? 3 : 2) swin_attn_f32
       ptx::st_cluster_f32(peer, acc[0][0]);
       ptx::st_cluster_f32(peer + d * 2, acc[0][1]);
       if (in1) {
-        ptx::st_cluster_f32(peer + pc * 4, acc[1][0]);
-        ptx::st_cluster_f32(peer + pc * 4 + d * 2, acc[1][1]);
+        ptx::st_cluster_f32(peer + t2 * pc * 4, acc[1][0]);
+        ptx::st_cluster_f32(peer + t2 * pc * 4 + d * 2, acc[1][1]);
       }
     }
   }
   if (g.heads > 1) { __syncwarp(); ptx::cluster_sync(); } else __syncthreads();
   if (in0) {
-    tile_dot<2, 2>(xs, pc, wp, pc, T, d, C, r0, c0, d / 2, acc);
+    tile_dot<2, 2>(xs, pc, wp, pc, T, d, C, r0, t2, c0, d / 2, acc);
     g.y[o0 + c0] = acc[0][0] + bp[c0] + res[0][0];
     g.y[o0 + c1] = acc[0][1] + bp[c1] + res[0][1];
     if (in1) {
@@ -420,7 +468,9 @@ int launch_swin_attn_f32(const smartmem_swin_params_t& p, const DevMap& rowmap, 
   const long long ctas = (long long)p.B * g.win_per_img * p.heads;
   if (ctas >= (1ll << 31) || (long long)p.B * p.H * p.W >= (1ll << 31)) return SMARTMEM_ERR_UNSUPPORTED;
   const size_t smem = attn_f32_smem(g.C, g.d, g.T, g.ws);
-  auto kernel = g.T <= 32 ? swin_attn_f32_kernel<256> : swin_attn_f32_kernel<512>;
+  const bool alone = ctas <= tc_sm_count();
+  auto kernel = g.T <= 32 ? (alone ? swin_attn_f32_kernel<256, true> : swin_attn_f32_kernel<256, false>)
+                          : (alone ? swin_attn_f32_kernel<512, true> : swin_attn_f32_kernel<512, false>);
   if (ensure_max_dynamic_smem((const void*)kernel, (int)kMaxSmem) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   profile_tick("swin_attn_f32", st);
   if (launch_pdl_cluster(kernel, dim3((unsigned)ctas), dim3(g.T <= 32 ? 256 : 512), smem, st, (unsigned)p.heads, g) != cudaSuccess) return SMARTMEM_ERR_CUDA;
