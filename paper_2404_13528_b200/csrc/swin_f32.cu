@@ -9,6 +9,8 @@
 //   * attention: a window per cluster, a head per CTA.  Every CTA gathers and normalises the window's rows (redundantly: they
 //     are few), computes q, k, v of its head, the scores, softmax and P v; the heads' outputs are exchanged through
 //     distributed shared memory and every CTA projects onto its share of the output columns, adds the residual and scatters.
+//     With few windows the tokens are shared out as well: a CTA normalises its own, writes their keys and values into the memory
+//     of the others of its head, and goes on with its own queries.
 //   * MLP: sixteen rows per cluster, a slice of the hidden features per CTA; the partial results of fc2 are added through
 //     distributed shared memory in the order of the CTAs.
 // Operands lie in shared memory with rows of K + 4 floats (an odd number of 16-byte vectors: eight lanes on eight rows hit
@@ -174,6 +176,7 @@ struct AttnF32Args {
   const float *x, *ln_g, *ln_b, *w_qkv, *b_qkv, *table, *w_proj, *b_proj;
   float* y;
   int C, heads, d, T, ws, shift, H, W, nWw, win_per_img;
+  int parts, part_rows;                                // CTAs of a window and head, and the tokens of each (the last one has the rest)
   float eps, scale;
   FastDiv fd_vpr, fd_d, fd_ws;                         // vectors of a row, head dimension, window
   int tp;                                              // pitch of P and of v transposed: T rounded up to an odd number of vectors
@@ -181,28 +184,41 @@ struct AttnF32Args {
 };
 
 // q, k and v of one head: a TM x TN tile a thread
-template <int TM, int TN, bool PACKED>
-__device__ __forceinline__ void qkv_phase(const AttnF32Args& g, const float* xs, int pc, const float* wq, const float* bq, float* q, float* k, float* vt, int pd) {
-  const int d = g.d, T = g.T, mt = (T + TM - 1) / TM, nt = 3 * d / TN;
+template <int TM, int TN, bool PACKED, bool PARTS>
+__device__ __forceinline__ void qkv_phase(const AttnF32Args& g, const float* xs, int pc, const float* wq, const float* bq, float* q, float* k, float* vt, int pd,
+                                          int row0, int rows, int h) {
+  const int d = g.d, mt = (rows + TM - 1) / TM, nt = 3 * d / TN;
   const WarpTile t((int)threadIdx.x >> 5, mt, nt);
-  if (!t.in) return;
   float acc[TM][TN];
-  tile_dot<TM, TN, PACKED>(xs, pc, wq, pc, T, 3 * d, g.C, t.tm, mt, t.tn, nt, acc);
+  if (t.in) tile_dot<TM, TN, PACKED>(xs, pc, wq, pc, rows, 3 * d, g.C, t.tm, mt, t.tn, nt, acc);
+  if (PARTS) ptx::cluster_wait();                      // (every part has zeroed its v)
+  if (!t.in) return;
 #pragma unroll
   for (int j = 0; j < TN; ++j) {
     const int c = t.tn + j * nt, which = c < d ? 0 : c < 2 * d ? 1 : 2, e = c - which * d;
     const float b = bq[c], sc = which == 0 ? g.scale : 1.0f;
-    float* dst = which == 0 ? q + t.tm * pd + e : which == 1 ? k + t.tm * pd + e : vt + e * g.tp + t.tm;
+    float* dst = which == 0 ? q + t.tm * pd + e : which == 1 ? k + (row0 + t.tm) * pd + e : vt + e * g.tp + row0 + t.tm;
     const int step = (which == 2 ? 1 : pd) * mt;
+    if (!PARTS || which == 0) {
 #pragma unroll
-    for (int i = 0; i < TM; ++i)
-      if (t.tm + i * mt < T) dst[i * step] = (acc[i][j] + b) * sc;
+      for (int i = 0; i < TM; ++i)
+        if (t.tm + i * mt < rows) dst[i * step] = (acc[i][j] + b) * sc;
+    } else {                                           // keys and values: into every part's memory
+#pragma unroll 1
+      for (int z = 0; z < g.parts; ++z) {
+        const uint32_t peer = ptx::mapa(ptx::smem_u32(dst), (uint32_t)(z * g.heads + h));
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+          if (t.tm + i * mt < rows) ptx::st_cluster_f32(peer + (uint32_t)(i * step) * 4u, acc[i][j] + b);
+      }
+    }
   }
 }
 
 // THREADS: 256 up to 32 tokens, else 512: one output tile a thread in every phase.  ALONE: no more CTAs than SMs, so a thread may have all
 // the registers it can use.
-template <int THREADS, bool ALONE>
+// PARTS: the tokens of a window are shared out as well.
+template <int THREADS, bool ALONE, bool PARTS>
 __global__ void __launch_bounds__(THREADS, ALONE ? 1 : THREADS == 256 ? 3 : 2) swin_attn_f32_kernel(const __grid_constant__ AttnF32Args g) {
   extern __shared__ __align__(16) float sm[];
   const int C = g.C, d = g.d, T = g.T, pc = C + 4, pd = d + 4, tp = g.tp;
@@ -222,8 +238,10 @@ __global__ void __launch_bounds__(THREADS, ALONE ? 1 : THREADS == 256 ? 3 : 2) s
   long long* offs = reinterpret_cast<long long*>(tab + ((nt + 3) & ~3));
   int* code = reinterpret_cast<int*>(offs + T);        // a token's place in the bias table (differences index it) and its region
   int* label = code + T;
-  const int h = g.heads > 1 ? (int)ptx::cluster_ctarank() : 0;
-  const int n = (int)blockIdx.x / g.heads;             // window
+  const int ctas = PARTS ? g.heads * g.parts : g.heads, cta = ctas > 1 ? (int)ptx::cluster_ctarank() : 0;
+  const int z = PARTS ? cta / g.heads : 0, h = cta - z * g.heads;
+  const int row0 = PARTS ? z * g.part_rows : 0, rows = PARTS ? min(g.part_rows, T - row0) : T;      // this CTA's tokens
+  const int n = (int)blockIdx.x / ctas;                // window
   const int tid = threadIdx.x;
 
   // The head's weights as far as L2: they may still be written by the kernel before this one.  (A line per 32 floats of a head's rows,
@@ -240,11 +258,12 @@ __global__ void __launch_bounds__(THREADS, ALONE ? 1 : THREADS == 256 ? 3 : 2) s
     label[tid] = g.shift > 0 ? region_label2(ty, tx, g.ws, wy, wx, g.H, g.W, g.shift) : 0;
   }
   for (int i = tid; i < d * tp; i += THREADS) vt[i] = 0.f;
-  for (int i = tid; i < T * tp; i += THREADS) P[i] = 0.f;
+  for (int i = tid; i < rows * tp; i += THREADS) P[i] = 0.f;
+  if (PARTS) ptx::cluster_arrive();
   __syncthreads();
   pdl_wait();
   pdl_launch_dependents();
-  load_rows<THREADS>(xs, pc, T, g.fd_vpr, [&](int r) { return g.x + offs[r]; });
+  load_rows<THREADS>(xs, pc, rows, g.fd_vpr, [&](int r) { return g.x + offs[row0 + r]; });
   for (int i = tid; i < C / 2; i += THREADS)
     ptx::cp_async16(lng + i * 4, (i < C / 4 ? g.ln_g : g.ln_b - C) + i * 4);
   ptx::cp_async_commit();
@@ -260,37 +279,37 @@ __global__ void __launch_bounds__(THREADS, ALONE ? 1 : THREADS == 256 ? 3 : 2) s
   }
   ptx::cp_async_wait<1>();
   __syncthreads();
-  norm_rows<THREADS, 8>(xs, pc, T, C, lng, lnb, g.eps);
+  norm_rows<THREADS, 8>(xs, pc, rows, C, lng, lnb, g.eps);
   ptx::cp_async_wait<0>();
   __syncthreads();
   // the smallest tile that gives no warp two (T at most 64 and d 16 or 32: at most 6 and 12 of the largest)
-  const int t2 = (T + 1) / 2;
-  if (warp_tiles(t2, 3 * d / 2) <= THREADS / 32) qkv_phase<2, 2, true>(g, xs, pc, wq, bq, q, k, vt, pd);
-  else if (warp_tiles(t2, 3 * d / 4) <= THREADS / 32) qkv_phase<2, 4, true>(g, xs, pc, wq, bq, q, k, vt, pd);
-  else qkv_phase<4, 4, ALONE>(g, xs, pc, wq, bq, q, k, vt, pd);
-  __syncthreads();
+  const int t2 = (rows + 1) / 2;
+  if (warp_tiles(t2, 3 * d / 2) <= THREADS / 32) qkv_phase<2, 2, true, PARTS>(g, xs, pc, wq, bq, q, k, vt, pd, row0, rows, h);
+  else if (warp_tiles(t2, 3 * d / 4) <= THREADS / 32) qkv_phase<2, 4, true, PARTS>(g, xs, pc, wq, bq, q, k, vt, pd, row0, rows, h);
+  else qkv_phase<4, 4, ALONE, PARTS>(g, xs, pc, wq, bq, q, k, vt, pd, row0, rows, h);
+  if (PARTS) { __syncwarp(); ptx::cluster_sync(); } else __syncthreads();
   {
     const int nk = (T + 3) / 4;
     const WarpTile t(tid >> 5, t2, nk);
     if (t.in) {
       float acc[2][4];
-      tile_dot<2, 4>(q, pd, k, pd, T, T, d, t.tm, t2, t.tn, nk, acc);
-      const int i0 = t.tm, i1 = min(i0 + t2, T - 1), mid = (g.ws - 1) * 2 * g.ws;
-      const int c0 = code[i0] + mid, c1 = code[i1] + mid, l0 = label[i0], l1 = label[i1];
+      tile_dot<2, 4>(q, pd, k, pd, rows, T, d, t.tm, t2, t.tn, nk, acc);
+      const int i0 = t.tm, i1 = min(i0 + t2, rows - 1), mid = (g.ws - 1) * 2 * g.ws;
+      const int c0 = code[row0 + i0] + mid, c1 = code[row0 + i1] + mid, l0 = label[row0 + i0], l1 = label[row0 + i1];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int col = t.tn + j * nk;
         if (col < T) {
           const int cc = code[col], lc = label[col];
           P[i0 * tp + col] = acc[0][j] + tab[c0 - cc] - (l0 != lc ? 100.f : 0.f);
-          if (i0 + t2 < T) P[i1 * tp + col] = acc[1][j] + tab[c1 - cc] - (l1 != lc ? 100.f : 0.f);
+          if (i0 + t2 < rows) P[i1 * tp + col] = acc[1][j] + tab[c1 - cc] - (l1 != lc ? 100.f : 0.f);
         }
       }
     }
   }
   __syncthreads();
   {                                                    // softmax: eight lanes per row, eight keys per lane
-    const int r = min(tid >> 3, T - 1), l = tid & 7;
+    const int r = min(tid >> 3, rows - 1), l = tid & 7;
     float* p = P + r * tp;
     float v[8], m = -INFINITY;
 #pragma unroll
@@ -307,7 +326,7 @@ __global__ void __launch_bounds__(THREADS, ALONE ? 1 : THREADS == 256 ? 3 : 2) s
       s += v[j];
     }
     const float inv = 1.0f / lanes_sum<8>(s);
-    if ((tid >> 3) < T)
+    if ((tid >> 3) < rows)
 #pragma unroll
       for (int j = 0; j < 8; ++j)
         if (l + 8 * j < T) p[l + 8 * j] = v[j] * inv;
@@ -317,19 +336,20 @@ __global__ void __launch_bounds__(THREADS, ALONE ? 1 : THREADS == 256 ? 3 : 2) s
   // columns of it and of the projection.
   const WarpTile t(tid >> 5, t2, d / 2);
   const int c0 = t.tn, c1 = c0 + d / 2, r0 = t.tm, r1 = r0 + t2;
-  const bool in0 = t.in, in1 = t.in && r1 < T;
+  const bool in0 = t.in, in1 = t.in && r1 < rows;
   float acc[2][2], res[2][2] = {};
-  const long long o0 = in0 ? offs[r0] + h * d : 0, o1 = in1 ? offs[r1] + h * d : 0;
+  const long long o0 = in0 ? offs[row0 + r0] + h * d : 0, o1 = in1 ? offs[row0 + r1] + h * d : 0;
   if (in0) { res[0][0] = g.x[o0 + c0]; res[0][1] = g.x[o0 + c1]; }
   if (in1) { res[1][0] = g.x[o1 + c0]; res[1][1] = g.x[o1 + c1]; }
-  if (g.heads > 1) ptx::cluster_arrive();              // (everyone has read its normalised rows)
-  if (in0) tile_dot<2, 2>(P, tp, vt, tp, T, d, (T + 3) & ~3, r0, t2, c0, d / 2, acc);
-  if (g.heads > 1) ptx::cluster_wait();
+  const bool meet = g.heads > 1 && !PARTS;       // everyone has read its normalised rows (where parts met after q, k and v, it has)
+  if (meet) ptx::cluster_arrive();
+  if (in0) tile_dot<2, 2>(P, tp, vt, tp, rows, d, (T + 3) & ~3, r0, t2, c0, d / 2, acc);
+  if (meet) ptx::cluster_wait();
   if (in0) {
     const uint32_t xa = ptx::smem_u32(xs), o = (uint32_t)(r0 * pc + h * d + c0) * 4u;
 #pragma unroll 1
     for (int r = 0; r < g.heads; ++r) {
-      const uint32_t peer = (g.heads > 1 ? ptx::mapa(xa, (uint32_t)r) : xa) + o;
+      const uint32_t peer = (g.heads > 1 ? ptx::mapa(xa, (uint32_t)(z * g.heads + r)) : xa) + o;
       ptx::st_cluster_f32(peer, acc[0][0]);
       ptx::st_cluster_f32(peer + d * 2, acc[0][1]);
       if (in1) {
@@ -340,7 +360,7 @@ __global__ void __launch_bounds__(THREADS, ALONE ? 1 : THREADS == 256 ? 3 : 2) s
   }
   if (g.heads > 1) { __syncwarp(); ptx::cluster_sync(); } else __syncthreads();
   if (in0) {
-    tile_dot<2, 2>(xs, pc, wp, pc, T, d, C, r0, t2, c0, d / 2, acc);
+    tile_dot<2, 2>(xs, pc, wp, pc, rows, d, C, r0, t2, c0, d / 2, acc);
     g.y[o0 + c0] = acc[0][0] + bp[c0] + res[0][0];
     g.y[o0 + c1] = acc[0][1] + bp[c1] + res[0][1];
     if (in1) {
@@ -465,15 +485,27 @@ int launch_swin_attn_f32(const smartmem_swin_params_t& p, const DevMap& rowmap, 
   g.fd_d = make_fastdiv((uint32_t)g.d);
   g.fd_ws = make_fastdiv((uint32_t)g.ws);
   g.rowmap = rowmap;
-  const long long ctas = (long long)p.B * g.win_per_img * p.heads;
+  long long ctas = (long long)p.B * g.win_per_img * p.heads;
+  // Few windows of more than 32 tokens: two or four CTAs share a window and head.  Us, one -> two -> four: 2 CTAs ([1,7,7,64], heads of 32) 13.4 ->
+  // 10.2 -> 8.8, 8 ([2,14,14,32]) 10.3 -> 8.3 -> 7.3, 27 ([3,21,21,32]) 10.3 -> 8.3 -> 8.6, 54 ([3,21,21,64]) 13.5 -> 11.7 -> 13.8; 81 ([3,21,21,96]) 17.2 ->
+  // 20.3; heads of 16 27 ([3,21,7,48]) 9.7 -> 7.9, 36 ([3,21,14,32] with its MLP half) 13.2 -> 13.6; windows of 16 tokens are alike to 24 CTAs and lose
+  // beyond.
+  g.parts = 1;
+  if (g.T > 32) {
+    if (4 * p.heads <= kMaxCluster && 4 * ctas <= tc_sm_count() / 2) g.parts = 4;
+    else if (2 * p.heads <= kMaxCluster && 2 * ctas <= (g.d == 32 ? tc_cluster_ctas(2 * p.heads) : tc_sm_count() * 2 / 5)) g.parts = 2;
+  }
+  g.part_rows = (g.T + g.parts - 1) / g.parts;
+  ctas *= g.parts;
   if (ctas >= (1ll << 31) || (long long)p.B * p.H * p.W >= (1ll << 31)) return SMARTMEM_ERR_UNSUPPORTED;
   const size_t smem = attn_f32_smem(g.C, g.d, g.T, g.ws);
   const bool alone = ctas <= tc_sm_count();
-  auto kernel = g.T <= 32 ? (alone ? swin_attn_f32_kernel<256, true> : swin_attn_f32_kernel<256, false>)
-                          : (alone ? swin_attn_f32_kernel<512, true> : swin_attn_f32_kernel<512, false>);
+  auto kernel = g.T <= 32 ? (alone ? swin_attn_f32_kernel<256, true, false> : swin_attn_f32_kernel<256, false, false>)
+                : g.parts > 1 ? swin_attn_f32_kernel<512, true, true>
+                              : (alone ? swin_attn_f32_kernel<512, true, false> : swin_attn_f32_kernel<512, false, false>);
   if (ensure_max_dynamic_smem((const void*)kernel, (int)kMaxSmem) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   profile_tick("swin_attn_f32", st);
-  if (launch_pdl_cluster(kernel, dim3((unsigned)ctas), dim3(g.T <= 32 ? 256 : 512), smem, st, (unsigned)p.heads, g) != cudaSuccess) return SMARTMEM_ERR_CUDA;
+  if (launch_pdl_cluster(kernel, dim3((unsigned)ctas), dim3(g.T <= 32 ? 256 : 512), smem, st, (unsigned)(p.heads * g.parts), g) != cudaSuccess) return SMARTMEM_ERR_CUDA;
   count_launch();
   return SMARTMEM_OK;
 }
@@ -487,11 +519,15 @@ int launch_swin_mlp_f32(const smartmem_swin_params_t& p, const void* x, void* y,
   g.M = (int)M; g.C = p.C; g.hidden = p.C * p.mlp_ratio; g.eps = p.ln_eps;
   g.splits = mlp_f32_splits(g.C, g.hidden);
   if (g.splits == 0) return SMARTMEM_ERR_UNSUPPORTED;
+  // Few rows: twice the slices, half of the products a CTA (us of a block, four -> eight: 144 rows of 96 17.1 -> 15.9, 144 of 64 13.3 -> 12.2; 196 of 96
+  // 19.9 -> 20.4, 1323 of 64 21.0 -> 25.7).
+  const long long groups = (M + kMlpRows - 1) / kMlpRows;
+  if (g.splits == 4 && g.hidden % (4 * kMaxCluster) == 0 && groups * kMaxCluster <= tc_sm_count() / 2) g.splits = kMaxCluster;
   g.slice = g.hidden / g.splits;
   g.fd_vpr = make_fastdiv((uint32_t)g.C / 4);
   g.fd_vps = make_fastdiv((uint32_t)g.slice / 4);
   g.fd_C = make_fastdiv((uint32_t)g.C);
-  const long long ctas = (M + kMlpRows - 1) / kMlpRows * g.splits;
+  const long long ctas = groups * g.splits;
   if (ctas >= (1ll << 31)) return SMARTMEM_ERR_UNSUPPORTED;
   const size_t smem = mlp_f32_smem(g.C, g.slice);
   if (ensure_max_dynamic_smem((const void*)swin_mlp_f32_kernel, (int)kMaxSmem) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
