@@ -368,12 +368,23 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   }
 }
 
+// Rows of a row tile: at most 256, at most 15 of them padding.  Where the columns are few, as many row tiles as clusters of eight find room
+// for, one CTA per SM: a CTA's share of the exchange shrinks with its tile and nothing else is long (134 x 2048 -> 512: 6.8 us in one row
+// tile, 5.3 in three; 200 x 1536 -> 384 8.0, 5.2 in five; 100 x 1024 -> 256 5.6, 4.4 in four).  Not with few rows of a large weight, which every
+// row tile reads (33 x 3072 -> 768 5.4, 5.8 in two), and beyond eight only for a reduction that is worth it (480 x 768 -> 8 5.1 in fifteen).
+int row_tile(long long M, long long N, long long K) {
+  long long room = tc_cluster_ctas(kMaxSplits) / kMaxSplits / ((N + BN_W - 1) / BN_W);
+  if (M <= 64 && N * K > (1ll << 21)) room = 1;
+  if (K < 1024 && room > 8) room = 8;
+  const long long need = (M + 255) / 256, tiles = room > need ? room : need;
+  return (int)(((M + tiles - 1) / tiles + 15) / 16 * 16);
+}
+
 // Sizes of a launch; returns the bytes of shared memory, 0 if a CTA's part does not fit (with RMSNorm: gamma of its K range lies beside
 // the rings).
 size_t plan_launch(long long M, long long N, long long K, bool norm, SplitArgs& g) {
-  // row tiles of at most 256 rows and at most 15 rows of padding each
-  g.tiles_m = (int)((M + 255) / 256);
-  g.NB = (int)(((M + g.tiles_m - 1) / g.tiles_m + 15) / 16 * 16);
+  g.NB = row_tile(M, N, K);
+  g.tiles_m = (int)((M + g.NB - 1) / g.NB);
   if (norm && g.NB > kMaxNormRows) return 0;
   g.nkb = (int)(K / BK);
   const long long tiles = (N + BN_W - 1) / BN_W * g.tiles_m;
@@ -427,7 +438,7 @@ bool gemm_splitk_supported(const TcOperand& X, const TcOperand& W, const TcEpilo
 }
 
 // Microseconds, fitted to measurements: a fixed part, the exchange of the partial sums (distributed shared memory moves about
-// 14 bytes per clock and SM, which is what ends the range at 128 rows), and the stream of W.  Below 32 rows the tiled kernel's estimate
+// 14 bytes per clock and SM, which is what ends the range at 128 rows where the columns leave room for one row tile only), and the stream of W.  Below 32 rows the tiled kernel's estimate
 // does not hold (its copies of a mostly empty A tile are slower than full ones), so the line is drawn by measurement, tiled -> this one:
 // a long reduction, 2 rows, N = 4096: K = 512 5.1 -> 4.9, 1024 7.7 -> 5.5, 4096 23.6 -> 10.0; 31 rows, N = 512: K = 512 4.4 -> 4.6, 1024
 // 5.9 -> 4.8.  A shorter one only where there are tiles enough for every SM and W is not yet all of the cost: 2 rows, K = 256, N = 1024
@@ -436,6 +447,11 @@ bool gemm_splitk_supported(const TcOperand& X, const TcOperand& W, const TcEpilo
 double gemm_splitk_us(long long M, long long N, long long K) {
   const double nb = (double)((M + 15) / 16 * 16);
   if (M < 32) return K >= (M > 16 ? 768 : 512) || (K >= 256 && N * K >= (1ll << 23) && N < 65536) ? 0.0 : 1e30;
+  // Few columns, in several row tiles: bound by the exchange (4.35 us at tiles of 32 rows and K = 768, 5.3 at 48 and 2048, 7.2 at 112 and 2048; the tiled
+  // kernel 4.8, 8.7 and 8.7), but drawn by whole blocks of 7 x 7 windows, in which the tiled kernel overlaps more of what it follows: 245 rows of 256
+  // channels 20.0 -> 18.7 us, 294 of 384 26.3 -> 25.5, 343 26.3 -> 26.4, 245 of 512 30.5 -> 28.8, 294 30.5 -> 30.4, 343 30.6 -> 31.2.
+  const int tile = row_tile(M, N, K);
+  if (tile < M && M <= 1024 && (N + BN_W - 1) / BN_W * ((M + tile - 1) / tile) <= 24) return 2.96 + 0.04 * tile + 0.00045 * (double)K;
   return M > 128 ? 1e30 : 3.0 + 0.018 * nb + (double)N * (double)K * 2.0 / 6.2e6 * (1.0 + nb / 260.0);
 }
 

@@ -6,6 +6,7 @@ from paper_2404_13528_b200 import synth
 from tests.gpu_util import assert_close_bf16, to_dev, to_host_f64
 from tests.test_gpu_chains import run_plan
 from tests.test_gpu_decode import check_case
+from tests.test_gpu_swin import case as block
 
 pytestmark = pytest.mark.gpu
 
@@ -21,6 +22,9 @@ pytestmark = pytest.mark.gpu
     (16, 136, 448), (17, 136, 704),  # a k-block fewer: the tiled kernel
     (17, 128, 768), (31, 264, 1088),
     (3, 32776, 256), (31, 65528, 256),   # four k-blocks, a large W: no split
+    (129, 512, 2048), (256, 512, 2048), (200, 384, 1536), (160, 768, 3072),  # several row tiles, the last one short
+    (300, 72, 2048), (1024, 256, 4096),  # ten and seven row tiles
+    (64, 768, 3072), (65, 768, 3072),    # a large W: one row tile, two
 ])
 def test_few_row_linear(M, N, K):
     x = synth.normal(401, 0, (M, K), dtype="bf16")
@@ -28,6 +32,12 @@ def test_few_row_linear(M, N, K):
     out = run_plan([sm.make_op(sm.OP_LINEAR, side_input=(1, 0))], [sm.make_desc((M, K)), sm.make_desc((N, K))], sm.ELIMINATE,
                    [to_dev(x), to_dev(w)], (M, N))
     assert_close_bf16(to_host_f64(out), synth.to_f64(x) @ synth.to_f64(w).T, f"{M} x {N} x {K}")
+
+
+@pytest.mark.parametrize("B,C,heads,window", [(4, 384, 12, 7), (5, 256, 8, 7), (3, 512, 16, 8)])
+def test_block_of_few_rows(B, C, heads, window):
+    """Bias and residual of a block's second MLP product in several row tiles."""
+    block(57, B=B, H=window, W=window, C=C, heads=heads, window=window, shift=2, mlp_ratio=4, dtype="bf16")
 
 
 @pytest.mark.parametrize("B,pos,hidden,heads", [
