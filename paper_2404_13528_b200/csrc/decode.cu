@@ -285,9 +285,11 @@ int launch_decode_attention(DecodeAttnArgs a, int B, cudaStream_t st) {
   if (rc != SMARTMEM_OK) return rc;
   a.status = device_status_ptr();
   if (!a.status) return SMARTMEM_ERR_CUDA;
-  // Shares per (sequence, head): whichever reads the cache fastest.  A stage takes 32 KB / 6.5 TB/s times the number of CTAs
-  // at work, but no less than the 0.54 us in which one CTA takes it in; a
-  // wave (of clusters) and a merge across CTAs cost about 1 us each.
+  // Shares per (sequence, head): whichever reads the cache fastest.  A stage takes one CTA 0.54 us by latency and 32 KB / 6.5 TB/s times the CTAs
+  // at work by bandwidth, and where the two are near one another it takes their root sum of squares (with the larger of them 128 CTAs, one per
+  // SM, looked as good as 256: 8 x 7386 positions of 16 heads 101 us in one share, 86 in two; 4 x 2011 29.9 in two, 26.9 in four; 3 x 849 of
+  // 32 heads 41.2 in one, 36.8 in two).  A wave (of clusters) costs about 2 us and a merge across CTAs 1.  Over 120 steps of 1 to 62 sequences this
+  // choice is 0.1 % from the best of all eight on average, 5 % at most.
   // (Two CTAs per SM; with 480 or 2048 sequence-heads more than one share is slower, with 16 eight are best.)
   const int units = B * a.heads;
   double best = 0.0;
@@ -295,9 +297,9 @@ int launch_decode_attention(DecodeAttnArgs a, int B, cudaStream_t st) {
   for (int s = 1; s <= DEC_MAX_SPLIT; ++s) {
     const long long ctas = (long long)units * s, slots = 2ll * tc_cluster_ctas(s), full = ctas / slots, tail = ctas % slots;
     const double stages = ((a.S + s - 1) / s + DEC_STEP - 1) / DEC_STEP;
-    auto wave = [&](long long n) { const double t = n * 0.00504; return n ? stages * (t > 0.54 ? t : 0.54) + 1.0 : 0.0; };
+    auto wave = [&](long long n) { const double t = n * 0.00504; return n ? stages * sqrt(0.54 * 0.54 + t * t) + 2.0 : 0.0; };
     const double t = full * wave(slots) + wave(tail) - (s == 1 ? 0.8 * full : -1.0);
-    if (s == 1 || t < best * 0.98) { best = t; a.split = s; }
+    if (s == 1 || t < best) { best = t; a.split = s; }
   }
   constexpr size_t smem = 128 + DEC_STAGES * DEC_STAGE_BYTES;
   if (ensure_max_dynamic_smem((const void*)decode_attn_kernel, (int)smem, 100) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
