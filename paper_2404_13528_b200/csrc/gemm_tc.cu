@@ -1165,7 +1165,8 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
       if (ep.seg_cols > 0 && ep.seg_cols % o.bn) continue;
       if (B.n_row_atoms > 1 && B.row_extent[B.n_row_atoms - 1] % o.bn) continue;
       const long long tiles = (o.pair ? (tiles_m1 + 1) / 2 : tiles_m1) * ((N + o.bn - 1) / o.bn), slots = tc_sm_count() / (o.pair ? 2 : 1);
-      const double kbs = nkb * o.per_kb, wave = kbs + o.wave > o.wave_min ? kbs + o.wave : o.wave_min;
+      // (64-wide tiles fall behind on long reductions: 161 x 4096 -> 4096 16.4 us on 128 CTAs, 14.9 on as many in 128-wide pairs)
+      const double kbs = nkb * o.per_kb + (o.bn == 64 && nkb > 32 ? (nkb - 32) * 0.035 : 0.0), wave = kbs + o.wave > o.wave_min ? kbs + o.wave : o.wave_min;
       double t = o.fixed + kbs + (double)((tiles + slots - 1) / slots - 1) * wave;
       const bool tail = o.pair && o.bn == 256 && tail_halves(tiles, slots);
       if (tail) t -= 0.44 * wave;
