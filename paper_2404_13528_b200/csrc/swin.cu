@@ -122,7 +122,7 @@ Layout ws_layout(const smartmem_swin_params_t& p, int mode, bool compact) {
   memset(&L, 0, sizeof(L));
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off += bytes; return o; };
-  if (!t.fuse_attn) {
+  if (!t.fuse_attn || t.attn_cluster) {            // (what a caller is asked for does not depend on the choice between the kernels of a wide block)
     if (!t.fuse_ln1) L.xn = take(MC);
     L.qkv = take(3 * MC);
     L.ao = take(MC);
