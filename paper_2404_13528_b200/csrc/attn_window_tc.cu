@@ -1,8 +1,8 @@
 // Window attention (head dimension 32, T = ws*ws <= 64) on the tcgen05 tensor cores.
 //
-// Two windows of one head share a 128-row MMA tile: S = [Q0; Q1] [K0; K1]^T is computed as one
-// 128 x 128 x 32 product (only its two diagonal 64 x 64 blocks are used) and O = P [V0; V1] as one
-// 128 x 32 x 128 product with a block-diagonal P, so each window only sees its own keys.  The tensor
+// Two windows of one head share a 128-row MMA tile: the rows of [Q0; Q1] meet K0 in one 128 x 64 x 32 product that writes lanes 0-63
+// of the accumulator only and K1 in another that writes lanes 64-127 (the lane mask of tcgen05.mma), and O = P V likewise, so each
+// window only sees its own keys and a score row is 64 columns.  The tensor
 // core has time to spare here; what the layout buys is that every query row belongs to exactly one
 // thread (its TMEM lane): bias, mask, maximum, exponentials and the row sum need no shuffles, no
 // fragment bookkeeping and no shared-memory fragment loads, which is what bounded the warp-MMA
@@ -10,22 +10,25 @@
 //
 // q, k, v are TMA boxes of 64 tokens x 32 features x 2 windows inside the [M, 3C] buffer of the QKV GEMM (head
 // split, K transpose eliminated); operands that TMA cannot address (the materialised K^T of the
-// explicit variant) are loaded by four helper warps into the same swizzled layout.  V is used as it
+// explicit variant) are loaded by four helper warps into the same swizzled layout, in a variant of the kernel with two
+// softmax groups.  V is used as it
 // lies ([key, d] rows) through the MN-major operand mode.  Results are stored as whole 64-byte rows
 // at column h*32 of [M, C] (head merge eliminated) or into [nW, nH, T, d].
 //
 // Persistent CTAs keep one head (its relative-position bias is expanded once into a [T, T] table of
-// bf16 pairs in shared memory, read with 16-byte loads) and stream window pairs through a 6-stage
-// ring.  Two softmax groups of four warps alternate over the units, each with its own S and O buffers
+// bf16 pairs in shared memory, read with 16-byte loads) and stream window pairs through an 8-stage
+// ring.  Four softmax groups of four warps take turns over the units, each with its own S and O buffers
 // and its own P region in TMEM (P is written there as bf16 pairs and read by the second MMA as its
-// A operand: it never touches shared memory).  S and P V have an issuing thread each: the S issuer runs ahead as far
+// A operand: it never touches shared memory): 128 columns a group.  S and P V have an issuing thread each: the S issuer runs ahead as far
 // as the S buffers and the ring allow, so a group finds its next score tile waiting when it has
 // written P.  The seam mask of shifted blocks is a 64-bit key mask per row, computed arithmetically
 // (a key is in another region iff it lies on the other side of the wrap line) and only for windows
 // in the last window row or column.
 //
-// What bounds it (measured with clock stamps at every hand-off): the softmax groups, at about 1700 cycles
-// per window pair; the tensor pipe is busy for about 500 of them.
+// What bounds it: a group's chain of tensor-memory load, 56 exponentials, tensor-memory store and the previous unit's output, about 3400
+// cycles a window pair.  With two groups that was 1700 cycles a pair; with four a block of 64 x 14 x 14 x 512 went from 100.6 us to 98.4,
+// 32 x 28 x 28 x 192 from 73.1 to 70.8 (the kernel 20.5 -> 18.4, event-separated; in a first version, whose block-diagonal P and 128-column
+// scores left tensor memory for two groups, a third spilled).
 #include "attn.cuh"
 #include "gemm_tc.cuh"
 #include "ptx.cuh"

@@ -294,8 +294,9 @@ int launch_decode_attention(DecodeAttnArgs a, int B, cudaStream_t st) {
   const int units = B * a.heads;
   double best = 0.0;
   a.split = 1;
+  const ClusterCtas fit = tc_cluster_ctas_all();
   for (int s = 1; s <= DEC_MAX_SPLIT; ++s) {
-    const long long ctas = (long long)units * s, slots = 2ll * tc_cluster_ctas(s), full = ctas / slots, tail = ctas % slots;
+    const long long ctas = (long long)units * s, slots = 2ll * fit.n[s], full = ctas / slots, tail = ctas % slots;
     const double stages = ((a.S + s - 1) / s + DEC_STEP - 1) / DEC_STEP;
     auto wave = [&](long long n) { const double t = n * 0.00504; return n ? stages * sqrt(0.54 * 0.54 + t * t) + 2.0 : 0.0; };
     const double t = full * wave(slots) + wave(tail) - (s == 1 ? 0.8 * full : -1.0);

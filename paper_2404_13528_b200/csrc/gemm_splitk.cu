@@ -372,8 +372,8 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
 // for, one CTA per SM: a CTA's share of the exchange shrinks with its tile and nothing else is long (134 x 2048 -> 512: 6.8 us in one row
 // tile, 5.3 in three; 200 x 1536 -> 384 8.0, 5.2 in five; 100 x 1024 -> 256 5.6, 4.4 in four).  Not with few rows of a large weight, which every
 // row tile reads (33 x 3072 -> 768 5.4, 5.8 in two), and beyond eight only for a reduction that is worth it (480 x 768 -> 8 5.1 in fifteen).
-int row_tile(long long M, long long N, long long K) {
-  long long room = tc_cluster_ctas(kMaxSplits) / kMaxSplits / ((N + BN_W - 1) / BN_W);
+int row_tile(long long M, long long N, long long K, const ClusterCtas& fit) {
+  long long room = fit.n[kMaxSplits] / kMaxSplits / ((N + BN_W - 1) / BN_W);
   if (M <= 64 && N * K > (1ll << 21)) room = 1;
   if (K < 1024 && room > 8) room = 8;
   const long long need = (M + 255) / 256, tiles = room > need ? room : need;
@@ -383,7 +383,8 @@ int row_tile(long long M, long long N, long long K) {
 // Sizes of a launch; returns the bytes of shared memory, 0 if a CTA's part does not fit (with RMSNorm: gamma of its K range lies beside
 // the rings).
 size_t plan_launch(long long M, long long N, long long K, bool norm, SplitArgs& g) {
-  g.NB = row_tile(M, N, K);
+  const ClusterCtas fit = tc_cluster_ctas_all();
+  g.NB = row_tile(M, N, K, fit);
   g.tiles_m = (int)((M + g.NB - 1) / g.NB);
   if (norm && g.NB > kMaxNormRows) return 0;
   g.nkb = (int)(K / BK);
@@ -395,7 +396,7 @@ size_t plan_launch(long long M, long long N, long long K, bool norm, SplitArgs& 
   const int per_sm = g.NB <= 64 ? 2 : 1;
   int splits = 1;
   for (int s = 2; s <= kMaxSplits && s <= g.nkb; ++s)
-    if (tiles * s <= (long long)per_sm * tc_cluster_ctas(s)) splits = s;
+    if (tiles * s <= (long long)per_sm * fit.n[s]) splits = s;
   g.splits = splits;
   const int nk_max = (g.nkb + splits - 1) / splits;
   const uint32_t gamma_bytes = norm ? (uint32_t)(nk_max * BK * 2) : 0u;
@@ -450,8 +451,9 @@ double gemm_splitk_us(long long M, long long N, long long K) {
   // Few columns, in several row tiles: bound by the exchange (4.35 us at tiles of 32 rows and K = 768, 5.3 at 48 and 2048, 7.2 at 112 and 2048; the tiled
   // kernel 4.8, 8.7 and 8.7), but drawn by whole blocks of 7 x 7 windows, in which the tiled kernel overlaps more of what it follows: 245 rows of 256
   // channels 20.0 -> 18.7 us, 294 of 384 26.3 -> 25.5, 343 26.3 -> 26.4, 245 of 512 30.5 -> 28.8, 294 30.5 -> 30.4, 343 30.6 -> 31.2.
-  const int tile = row_tile(M, N, K);
-  if (tile < M && M <= 1024 && (N + BN_W - 1) / BN_W * ((M + tile - 1) / tile) <= 24) return 2.96 + 0.04 * tile + 0.00045 * (double)K;
+  if (M > 1024) return 1e30;
+  const int tile = row_tile(M, N, K, tc_cluster_ctas_all());
+  if (tile < M && (N + BN_W - 1) / BN_W * ((M + tile - 1) / tile) <= 24) return 2.96 + 0.04 * tile + 0.00045 * (double)K;
   return M > 128 ? 1e30 : 3.0 + 0.018 * nb + (double)N * (double)K * 2.0 / 6.2e6 * (1.0 + nb / 260.0);
 }
 

@@ -1065,6 +1065,24 @@ int tc_cluster_ctas(int size) {
   return known = clusters * size;
 }
 
+ClusterCtas tc_cluster_ctas_all() {
+  static_assert(kMaxClusterSize == kMaxCluster, "one table");
+  static thread_local int table_dev = -1;
+  static thread_local ClusterCtas table;
+  int dev = -1;
+  if (cudaGetDevice(&dev) == cudaSuccess && dev == table_dev) return table;
+  ClusterCtas t;
+  t.n[0] = 0;
+  for (int s = 1; s <= kMaxCluster; ++s) t.n[s] = tc_cluster_ctas(s);
+  if (dev < 0 || dev >= kMaxDevices) return t;
+  std::lock_guard<std::mutex> lk(g_cluster_mu);
+  for (int s = 1; s <= kMaxCluster; ++s)
+    if (g_cluster_ctas[dev][s] == 0) return t;           // (a guess: asked again next time)
+  table = t;
+  table_dev = dev;
+  return t;
+}
+
 int tc_operand_from_map(const smartmem_index_map_t& m, int n_batch_atoms, int n_row_atoms, const void* ptr,
                         TcOperand* op) {
   if (m.klass == 3 || m.n_rolls > 0) return SMARTMEM_ERR_UNSUPPORTED;

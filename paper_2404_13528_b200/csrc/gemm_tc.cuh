@@ -87,6 +87,10 @@ int tc_encode_2d_plain(const void* ptr, long long inner, long long outer, long l
 int tc_sm_count();
 // SMs of the current device that clusters of `size` (1..8) CTAs, one per SM, fill: a cluster must find its CTAs inside one GPC.
 int tc_cluster_ctas(int size);
+// The same for all sizes at once (a rule that compares them asks once per call: eight questions are 0.3 us of the host's time).
+constexpr int kMaxClusterSize = 8;
+struct ClusterCtas { int n[kMaxClusterSize + 1]; };
+ClusterCtas tc_cluster_ctas_all();
 
 // Fused MLP half of a block: out = A + GELU(LN(A) W1^T + b1) W2^T + b2 with the hidden activation and the
 // normalised rows kept on chip.  A [M, C], W1 [hidden, C], W2 [C, hidden], C in {64, 96}, hidden a multiple
