@@ -69,7 +69,7 @@ struct Plan {
   static constexpr int off_offs = off_ln + (2 * 64 * NV + W_ROWS + P_ROWS) * 2;
   static constexpr int off_tyx = off_offs + 128 * 8;
   static constexpr int off_code = off_tyx + TP * 4 + 16;                     // a token's place in the bias table: differences index it
-  static constexpr int off_red = off_code + TP * 4;                         // row sums of the two halves of the keys
+  static constexpr int off_red = off_code + TP * 4;                         // row maxima, then row sums, of the two halves of the keys
   static constexpr int off_bars = off_red + HP * 2 * 128 * 4;
   static constexpr int bytes = 1024 + off_bars + 36 * 8;
   static_assert(bytes <= 227 * 1024, "shared memory");
@@ -100,7 +100,7 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
   int* tyx = reinterpret_cast<int*>(smem + L::off_tyx);                     // [64]: ty << 8 | tx
   uint32_t* kmask = reinterpret_cast<uint32_t*>(tyx + TP);
   int* code = reinterpret_cast<int*>(smem + L::off_code);
-  float* sums = reinterpret_cast<float*>(smem + L::off_red);                // [head][half][128]
+  float* red = reinterpret_cast<float*>(smem + L::off_red);                 // [head][half][128]
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::off_bars);
   uint64_t *w_full = bars, *w_empty = bars + 4, *a_ready = bars + 8, *qkv_full = bars + 9, *qk_ready = bars + 10, *v_ready = bars + 12, *s_full = bars + 14,
            *p_full = bars + 16, *o_full = bars + 18, *o_ready = bars + 20, *a_free = bars + 21, *wp_early = bars + 22, *wp_late = bars + 23, *y_full = bars + 24,
@@ -452,11 +452,13 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
       }
 #pragma unroll
       for (int c = 0; c < 32; ++c) mx4[c & 3] = fmaxf(mx4[c & 3], sc[c]);
-      float *sum_h = sums + hh * 256 + r, *max_h = reinterpret_cast<float*>(sA + rank * kLnBlockBytes) + hh * 256 + r;   // (O comes there later)
+      // The two threads of a row exchange their maxima and then their sums, in memory that no other head writes.  A thread's sum goes to
+      // where its partner's maximum was, which it alone has read.
+      float* red_h = red + hh * 256 + r;
       const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-      max_h[part * 128] = mx;
+      red_h[part * 128] = mx;
       asm volatile("bar.sync %0, 64;" ::"r"(2 + hh * 4 + q) : "memory");
-      const float nmx = -fmaxf(mx, max_h[(1 - part) * 128]) * LOG2E;
+      const float nmx = -fmaxf(mx, red_h[(1 - part) * 128]) * LOG2E;
       float sum4[4] = {0.f, 0.f, 0.f, 0.f};
       uint32_t pk[16], zero[16];
 #pragma unroll
@@ -478,7 +480,7 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
         }
       }
       const float sum = (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
-      sum_h[part * 128] = sum;
+      red_h[(1 - part) * 128] = sum;
       ptx::tmem_st16(mine + w * 32 + part * 16, pk);
       ptx::tmem_st_wait();
       ptx::tc_fence_before();
@@ -488,11 +490,12 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
         res[0] = *reinterpret_cast<const uint4*>(g.x + off + col);
         res[1] = *reinterpret_cast<const uint4*>(g.x + off + col + 8);
       }
+      wait(&p_full[hh]);                               // (complete by now: orders the partner's sum before the read below)
       wait(&o_full[hh]);
       if (ok) {
         // O of this head: columns 32 hh of the CTA's block of the projection's operand, half of them a thread
         ptx::tc_fence_after();
-        const float inv = 1.f / (sum_h[0] + sum_h[128]);
+        const float inv = 1.f / (red_h[0] + red_h[128]);
         uint32_t v[16];
         ptx::tmem_ld16(mine + 64 + part * 16, v);
         ptx::tmem_ld_wait();

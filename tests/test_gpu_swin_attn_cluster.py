@@ -1,10 +1,25 @@
 """The wide attention half over a cluster, at the edges of its range: every cluster size, windows of fewer and of 64 tokens, an odd number of
 windows (half a unit), one window, seams in both directions, and the sizes on both sides of the rule that takes it."""
 import pytest
+import torch
 
-from tests.test_gpu_swin import case
+from paper_2404_13528_b200 import binding as sm
+from paper_2404_13528_b200 import synth
+from tests.gpu_util import check_status, stream, to_dev
+from tests.test_gpu_swin import PARAM_NAMES, case
 
 pytestmark = pytest.mark.gpu
+
+
+def device_block(config_id, B, H, W, C, window, shift):
+    """An attention half's parameter block and input; the tensors that it points into come along."""
+    dev = {k: to_dev(v) for k, v in synth.swin_inputs(config_id, B, H, W, C, C // 32, window, 0, "bf16").items()}
+    p = sm.SwinParams()
+    p.dtype, p.B, p.H, p.W, p.C, p.heads, p.window, p.shift, p.mlp_ratio, p.ln_eps = sm.BF16, B, H, W, C, C // 32, window, shift, 0, 1e-5
+    for name in PARAM_NAMES:
+        if name in dev:
+            setattr(p, name, dev[name].data_ptr())
+    return p, dev["x"], dev
 
 
 @pytest.mark.parametrize("C", [128, 192, 256, 384, 512])
@@ -16,3 +31,26 @@ def test_attention_half(C, B, H, W, window, shift):
 @pytest.mark.parametrize("C,B,H,W", [(192, 5, 28, 28), (128, 9, 28, 28), (256, 4, 28, 21), (384, 11, 14, 14), (512, 15, 14, 7), (512, 16, 14, 7)])
 def test_one_wave_and_beyond(C, B, H, W):
     case(900 + C, B=B, H=H, W=W, C=C, heads=C // 32, window=7, shift=3, mlp_ratio=4, dtype="bf16", images=[0, B - 1])
+
+
+@pytest.mark.parametrize("C,B,H,W", [(128, 9, 28, 28), (192, 5, 28, 28), (256, 4, 28, 21), (384, 11, 14, 14), (512, 15, 14, 7)])
+def test_every_call_gives_the_same_bits(C, B, H, W):
+    """Full waves, call after call while copies on another stream hold up loads: the heads of a CTA and the two threads of a row share memory,
+    and no result may depend on which of them is late."""
+    p, x, keep = device_block(950 + C, B, H, W, C, 7, 3)
+    n = sm.smartmem_swin_block_workspace_bytes(p, sm.ELIMINATE)
+    ws = torch.empty(n, dtype=torch.uint8, device="cuda")
+    outs = [torch.full_like(x, float("nan")) for _ in range(100)]
+    a, b = torch.empty(2, 64 << 20, dtype=torch.uint8, device="cuda")
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        for _ in range(40):
+            b.copy_(a)
+    for y in outs:
+        sm.smartmem_swin_block(p, x.data_ptr(), y.data_ptr(), ws.data_ptr(), n, sm.ELIMINATE, stream())
+    torch.cuda.synchronize()
+    check_status()
+    assert torch.isfinite(outs[0].float()).all()
+    for y in outs[1:]:
+        assert torch.equal(y, outs[0])
