@@ -173,6 +173,14 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
   ptx::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
+  // Unwinding: whatever is in flight gets a fixed time to land.  The two warps below see to the copies and products that they have issued and,
+  // the second one, to those that come in: no CTA of the cluster leaves before both of them have arrived.
+  auto settle = [] {
+    const unsigned long long t0 = ptx::globaltimer();
+    while (ptx::globaltimer() - t0 < 100000ull) {
+    }
+  };
+
   // the projection takes the blocks of its operand in the order in which they come: its own, then those of the CTAs before it
   auto ring_block = [&](int t) { return t <= rank ? rank - t : rank - t + NV; };
 
@@ -217,11 +225,7 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
       ptx::bulk_copy_cluster(ptx::mapa(ptx::smem_u32(sA + rank * kLnBlockBytes), to), sA + rank * kLnBlockBytes, kLnBlockBytes, ptx::mapa(ptx::smem_u32(&o_in[lane]), to));
     }
     __syncwarp();
-    if (!ok) {                                         // unwinding: whatever is in flight gets a fixed time to land
-      const unsigned long long t0 = ptx::globaltimer();
-      while (ptx::globaltimer() - t0 < 100000ull) {
-      }
-    }
+    if (!ok) settle();
     ptx::cluster_arrive_relaxed();
   } else if (warp == kWorkers + 1) {
     // ---- products (the whole warp walks, an elected lane issues) ------------------------------------------------------
@@ -291,6 +295,8 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
       }
       __syncwarp();
     }
+    wait(y_full, 0);
+    if (!ok) settle();
     ptx::cluster_arrive_relaxed();                     // (what the others sent is here; each thread arrives when it is done with the others)
   } else {
     bool ok = true;
@@ -425,13 +431,14 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
       if (wy == g.nWh - 1) diff |= kmask[part] ^ ((tyx[i] >> 8) >= ws - g.shift ? 0xFFFFFFFFu : 0u);
       if (wx == g.nWw - 1) diff |= kmask[2 + part] ^ ((tyx[i] & 255) >= ws - g.shift ? 0xFFFFFFFFu : 0u);
     }
+    float sc[32], mx = -INFINITY;
+    float* red_h = red + hh * 256 + r;
     wait(&s_full[hh]);
     if (ok) {
       ptx::tc_fence_after();
       uint32_t rv[32];
       ptx::tmem_ld32(tmem_base + lane_addr + TM_S + hh * 128 + w * 64 + part * 32, rv);
       ptx::tmem_ld_wait();
-      float sc[32];
       float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
       const uint32_t* brow = bias_t + (hh * TP + i) * BIAS_ROW + part * 16;
 #pragma unroll
@@ -452,12 +459,13 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
       }
 #pragma unroll
       for (int c = 0; c < 32; ++c) mx4[c & 3] = fmaxf(mx4[c & 3], sc[c]);
-      // The two threads of a row exchange their maxima and then their sums, in memory that no other head writes.  A thread's sum goes to
-      // where its partner's maximum was, which it alone has read.
-      float* red_h = red + hh * 256 + r;
-      const float mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
+      mx = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
       red_h[part * 128] = mx;
-      asm volatile("bar.sync %0, 64;" ::"r"(2 + hh * 4 + q) : "memory");
+    }
+    // The two threads of a row exchange their maxima and then their sums, in memory that no other head writes.  A thread's sum goes to
+    // where its partner's maximum was, which it alone has read.  (Every warp comes to the barrier: one of the two may have given up waiting.)
+    asm volatile("bar.sync %0, 64;" ::"r"(2 + hh * 4 + q) : "memory");
+    if (ok) {
       const float nmx = -fmaxf(mx, red_h[(1 - part) * 128]) * LOG2E;
       float sum4[4] = {0.f, 0.f, 0.f, 0.f};
       uint32_t pk[16], zero[16];
