@@ -7,8 +7,9 @@
 // two heads:
 //   * every CTA gathers and normalises all rows of the unit (from L2: cheaper than exchanging them) straight into the QKV operand,
 //     which meets its 192 rows of the QKV weights (32 of q, k and v of two heads) as they come in;
-//   * per head, two windows share a product S = [Q0; Q1] [K0; K1]^T of which the diagonal blocks are used, a thread has a row of the
-//     softmax, P stays in tensor memory as the operand of O = P [V0; V1] (as in attn_window_tc.cu, and with the same roundings);
+//   * per head, the 128 rows of two windows meet K0 and K1 in products that write the lanes of their own window only (so nothing of one
+//     window, an infinity least of all, reaches the other), two threads have a row of the softmax, and P stays in tensor memory as the
+//     operand of O = P V, lane by lane alike (as in attn_window_tc.cu, and with the same roundings);
 //   * a CTA's O is one 64-column block of the projection's operand: it goes to every other CTA of the cluster as one bulk copy between
 //     shared memories, into the memory of the normalised rows, and every CTA projects onto its 64 output columns, adds bias and residual
 //     and scatters its 128-byte pieces of the rows through the map.
@@ -38,8 +39,9 @@ constexpr int W_ROWS = HP * 3 * D, W_STAGE = W_ROWS * 128;        // a k-block o
 constexpr int P_ROWS = HP * D, P_BLOCK = P_ROWS * 128;            // a k-block of its rows of the projection's: 8 KB
 constexpr int OP_BYTES = 128 * 64, OPS_BYTES = HP * 3 * OP_BYTES; // q, k, v of a head: 128 rows x 64 bytes each
 constexpr int BIAS_ROW = 36;                           // 32-bit words per row of a bias table (attn_window_tc.cu)
-// tensor memory: q, k, v of head h at 96 h, then P (64 columns) and O (32) in their place; S; the projection
-constexpr uint32_t TM_S = 192, TM_Y = 448, TMEM_COLS = 512;
+// tensor memory: q, k, v of head h at 96 h, then P (32 columns: 64 keys as bf16 pairs) and O (32) in the place of q and v; S (64 a head);
+// the projection
+constexpr uint32_t TM_S = 192, TM_Y = 320, TMEM_COLS = 512;
 
 struct AttnClusterArgs {
   const __nv_bfloat16 *x, *ln_g, *ln_b, *b_qkv, *b_proj;
@@ -232,7 +234,7 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
     const uint32_t a0 = ptx::smem_u32(sA), r0 = ptx::smem_u32(ring), ops0 = ptx::smem_u32(ops), wp0 = ptx::smem_u32(wp);
     bool ok = true;
     auto wait = [&](uint64_t* b, uint32_t ph) { ok = ok && __all_sync(0xFFFFFFFFu, ptx::mbar_wait<true>(b, ph, abort_flag, g.status) ? 1 : 0) != 0; };
-    constexpr uint32_t idesc_qkv = ptx::make_idesc_bf16(128, W_ROWS, false, false), idesc_s = ptx::make_idesc_bf16(128, 128, false, false),
+    constexpr uint32_t idesc_qkv = ptx::make_idesc_bf16(128, W_ROWS, false, false), idesc_s = ptx::make_idesc_bf16(128, TP, false, false),
                        idesc_pv = ptx::make_idesc_bf16(128, D, false, true), idesc_y = ptx::make_idesc_bf16(128, P_ROWS, false, false);
     wait(a_ready, 0);
 #pragma unroll 1
@@ -257,8 +259,11 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
       ptx::tc_fence_after();
       const uint64_t qd = desc_sw64(ops0 + h * 3 * OP_BYTES), kd = desc_sw64(ops0 + (h * 3 + 1) * OP_BYTES);
       if (ptx::elect_one()) {
-        ptx::tc_mma_bf16(tmem_base + TM_S + h * 128, qd, kd, idesc_s, 0u);
-        ptx::tc_mma_bf16(tmem_base + TM_S + h * 128, qd + 2, kd + 2, idesc_s, 1u);
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {               // 16 features per step: +32 bytes; steps 2-3: the second window's keys, +4096 bytes
+          const uint32_t first = ks < 2 ? 0u : ~0u;
+          ptx::tc_mma_bf16_lanes(tmem_base + TM_S + h * TP, qd + 2 * (ks & 1), kd + 2 * (ks & 1) + (ks >> 1) * (4096 >> 4), idesc_s, ks & 1, first, ~first);
+        }
         ptx::tc_commit(&s_full[h]);
       }
       __syncwarp();
@@ -272,8 +277,10 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
       const uint64_t vd = desc_sw64(ops0 + (h * 3 + 2) * OP_BYTES);
       if (ptx::elect_one()) {
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks)                 // 16 keys per step: P +8 packed columns, V +1024 bytes
-          ptx::tc_mma_bf16_ta(tmem_base + h * 96 + 64, tmem_base + h * 96 + 8 * ks, vd + ks * (1024 >> 4), idesc_pv, ks ? 1u : 0u);
+        for (int ks = 0; ks < 8; ++ks) {               // 16 keys per step: P +8 packed columns, V +1024 bytes; steps 4-7: the second window
+          const uint32_t first = ks < 4 ? 0u : ~0u;
+          ptx::tc_mma_bf16_ta_lanes(tmem_base + h * 96 + 64, tmem_base + h * 96 + 8 * (ks & 3), vd + ks * (1024 >> 4), idesc_pv, (ks & 3) ? 1u : 0u, first, ~first);
+        }
         ptx::tc_commit(&o_full[h]);
       }
       __syncwarp();
@@ -437,7 +444,7 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
     if (ok) {
       ptx::tc_fence_after();
       uint32_t rv[32];
-      ptx::tmem_ld32(tmem_base + lane_addr + TM_S + hh * 128 + w * 64 + part * 32, rv);
+      ptx::tmem_ld32(tmem_base + lane_addr + TM_S + hh * TP + part * 32, rv);
       ptx::tmem_ld_wait();
       float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
       const uint32_t* brow = bias_t + (hh * TP + i) * BIAS_ROW + part * 16;
@@ -468,10 +475,7 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
     if (ok) {
       const float nmx = -fmaxf(mx, red_h[(1 - part) * 128]) * LOG2E;
       float sum4[4] = {0.f, 0.f, 0.f, 0.f};
-      uint32_t pk[16], zero[16];
-#pragma unroll
-      for (int c = 0; c < 16; ++c) zero[c] = 0u;       // block-diagonal P: the other window's keys contribute nothing to this row
-      ptx::tmem_st16(mine + (1 - w) * 32 + part * 16, zero);
+      uint32_t pk[16];
 #pragma unroll
       for (int c8 = 0; c8 < 4; ++c8) {
         if (part * 32 + c8 * 8 < T) {                  // (uniform)
@@ -489,7 +493,7 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
       }
       const float sum = (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
       red_h[(1 - part) * 128] = sum;
-      ptx::tmem_st16(mine + w * 32 + part * 16, pk);
+      ptx::tmem_st16(mine + part * 16, pk);
       ptx::tmem_st_wait();
       ptx::tc_fence_before();
       __syncwarp();
