@@ -17,11 +17,11 @@
 //   acc  = [X | e] [Wq_h; Wk_h; Wv_h | f]^T    128 x 96 x (C + 16)  tcgen05; X = the RAW rows (bf16) in shared memory
 //   q,k,v = rstd acc                           LayerNorm applied algebraically (below); q goes back to tensor memory as
 //                                              bf16 pairs, k and v to shared memory in operand layout
-//   S    = [q0 0; 0 q1] [k0 | k1]^T            128 x 64 x 64: the two windows' keys are stacked along the reduction
-//                                              dimension and each query row carries zeros in the other window's half,
-//                                              so a row's 64 scores are its own window's; q is read from tensor memory
+//   S    = q0 k0^T over q1 k1^T                two products of 128 x 64 x 32 that write the lanes of one window each, so a
+//                                              row's 64 scores are its own window's and nothing of one window, an infinity
+//                                              least of all, reaches the other; q is read from tensor memory
 //   P    = softmax(scale S + bias + mask)      one query row per thread (= its TMEM lane); P stored as bf16 pairs
-//   O    = [P0 0; 0 P1] [v0; v1]               128 x 32 x 128, P read from tensor memory, V as it lies (MN-major)
+//   O    = P0 v0 over P1 v1                    likewise, 128 x 32 x 64 each; P read from tensor memory, V as it lies (MN-major)
 //   Ob   = bf16(O / rowsum)                    back into tensor memory as packed pairs
 //   Y   += Ob Wp[:, 32 h : 32 h + 32]^T        128 x C x 32: the head merge is the accumulation over heads
 //
@@ -494,27 +494,23 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
             *reinterpret_cast<uint4*>(slot_base + kv * KBT + sw64_off(r, c)) =
                 make_uint4(o16[c * 4], o16[c * 4 + 1], o16[c * 4 + 2], o16[c * 4 + 3]);
         }
-        // q as the S product's A operand: 64 bf16 = 32 packed columns over the accumulator's last 32 (v has been read): this
-        // window's half carries q, the other half zeros (the two windows' keys are stacked along the reduction dimension)
-        ptx::tmem_st16(tb + 64 + w * 16, q16);
-#pragma unroll
-        for (int c = 0; c < 16; ++c) q16[c] = 0u;
-        ptx::tmem_st16(tb + 64 + (1 - w) * 16, q16);
+        // q as the S product's A operand: 32 bf16 = 16 packed columns over the accumulator's last 32 (v has been read)
+        ptx::tmem_st16(tb + 64, q16);
         ptx::tmem_st_wait();
         ptx::fence_proxy_async();                      // generic-proxy writes -> visible to the MMAs
         ptx::tc_fence_before();
       }
       if (__any_sync(0xFFFFFFFFu, group_sync())) break;
       if (q == 0 && ptx::elect_one()) {
-        // S = [q0 0; 0 q1] [k0 | k1]^T: four k16 steps, the first two over window 0's keys, the last two over window 1's
+        // S: two k16 steps over window 0's keys, which write lanes 0-63, and two over window 1's for the rest
         ptx::tc_fence_after();
         const uint32_t idesc = ptx::make_idesc_bf16(BM, 64, false, false);
         const uint32_t d = tb - lane_addr, qa = d + 64;
         const uint64_t kd0 = desc_sw64(ptx::smem_u32(slot_base)), kd1 = desc_sw64(ptx::smem_u32(slot_base) + 64 * 64);
-        ptx::tc_mma_bf16_ta(d, qa, kd0, idesc, 0u);
-        ptx::tc_mma_bf16_ta(d, qa + 8, kd0 + 2, idesc, 1u);
-        ptx::tc_mma_bf16_ta(d, qa + 16, kd1, idesc, 1u);
-        ptx::tc_mma_bf16_ta(d, qa + 24, kd1 + 2, idesc, 1u);
+        ptx::tc_mma_bf16_ta_lanes(d, qa, kd0, idesc, 0u, 0u, ~0u);
+        ptx::tc_mma_bf16_ta_lanes(d, qa + 8, kd0 + 2, idesc, 1u, 0u, ~0u);
+        ptx::tc_mma_bf16_ta_lanes(d, qa, kd1, idesc, 0u, ~0u, 0u);
+        ptx::tc_mma_bf16_ta_lanes(d, qa + 8, kd1 + 2, idesc, 1u, ~0u, 0u);
         ptx::tc_commit(&s_full[gi]);
       }
       // -- seam mask of this row's window (shifted blocks: windows in the last window row or column) --
@@ -585,26 +581,24 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
         ptx::unpack2(sum2[0], s0, s1);
         ptx::unpack2(sum2[1], s2, s3);
         inv = 1.f / ((s0 + s1) + (s2 + s3));
-        // P row (bf16 pairs) over the score columns: this window's keys at packed columns 32 w .. 32 w + 31, zeros for the
-        // other window's keys (block-diagonal P against the stacked values)
-        ptx::tmem_st32(tb + w * 32, pk);
-#pragma unroll
-        for (int c = 0; c < 32; ++c) pk[c] = 0u;
-        ptx::tmem_st32(tb + (1 - w) * 32, pk);
+        // P row (bf16 pairs) over the first half of the score columns
+        ptx::tmem_st32(tb, pk);
         ptx::tmem_st_wait();
         ptx::tc_fence_before();
       }
       if (__any_sync(0xFFFFFFFFu, group_sync())) break;
       if (q == 0 && ptx::elect_one()) {
-        // O = P [v0; v1] over the columns q has left: P from tensor memory, V as it lies (MN-major B operand); 16 keys per
-        // step: P +8 packed columns, V +16 rows = 1024 bytes
+        // O = P V over the columns q has left: P from tensor memory, V as it lies (MN-major B operand); 16 keys per step: P +8
+        // packed columns, V +16 rows = 1024 bytes; steps 4-7: the second window
         ptx::tc_fence_after();
         const uint32_t idesc = ptx::make_idesc_bf16(BM, D, false, true);
         const uint64_t vd = desc_sw64(ptx::smem_u32(slot_base) + KBT);
         const uint32_t pa = tb - lane_addr, od = pa + 64;
-        ptx::tc_mma_bf16_ta(od, pa, vd, idesc, 0u);
 #pragma unroll
-        for (int ks = 1; ks < 8; ++ks) ptx::tc_mma_bf16_ta(od, pa + 8 * ks, vd + ks * (1024 >> 4), idesc, 1u);
+        for (int ks = 0; ks < 8; ++ks) {
+          const uint32_t first = ks < 4 ? 0u : ~0u;
+          ptx::tc_mma_bf16_ta_lanes(od, pa + 8 * (ks & 3), vd + ks * (1024 >> 4), idesc, (ks & 3) ? 1u : 0u, first, ~first);
+        }
         ptx::tc_commit(&o_full[gi]);
       }
       // -- O row: normalise, bf16 pairs, back into tensor memory as the projection's A operand --

@@ -24,6 +24,7 @@ def other_windows(B, H, W, window, shift, token):
 
 
 @pytest.mark.parametrize("B,H,W,C,heads,window,shift,mlp_ratio", [
+    (2, 14, 14, 64, 2, 7, 3, 4), (3, 14, 7, 96, 3, 7, 0, 0), (1, 16, 16, 96, 3, 8, 4, 4),       # narrow: the fused attention half
     (3, 14, 7, 128, 4, 7, 0, 4), (1, 14, 21, 192, 6, 7, 3, 0), (2, 16, 16, 256, 8, 8, 4, 0),    # wide, few windows: over a cluster
     (3, 14, 7, 384, 12, 7, 3, 0), (5, 7, 7, 512, 16, 7, 0, 0), (7, 7, 7, 512, 16, 7, 3, 0),
     (2, 8, 8, 32, 2, 4, 2, 0), (1, 14, 14, 48, 3, 7, 3, 0),                                     # heads of 16
