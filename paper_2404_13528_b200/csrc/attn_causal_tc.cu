@@ -42,7 +42,7 @@ constexpr float kRescaleThreshold = 8.0f;             // log2 units
 struct TcAttnArgs {
   int S, heads, batch, n_qt;
   int q_col0, k_col0, v_col0, col_per_head;           // TMA column of (operand, head): col0 + h * col_per_head
-  long long row_per_batch, row_per_head;              // TMA row of (b, h, t): b * row_per_batch + h * row_per_head + t
+  int plane_per_batch, plane_per_head;                // a plane of the TMA maps holds S rows: b * plane_per_batch + h * plane_per_head
   __nv_bfloat16* out;
   long long o_sn, o_sh, o_st;
   float scale_log2;
@@ -93,7 +93,7 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
   const int bh = (int)(blockIdx.x % bh_count);
   const int b = bh / g.heads, h = bh - b * g.heads;
   const int n_kv = min(2 * (qt + 1), (g.S + BKV - 1) / BKV);   // 64-key blocks up to and including the diagonal
-  const long long row_base = (long long)b * g.row_per_batch + (long long)h * g.row_per_head;
+  const int plane = b * g.plane_per_batch + h * g.plane_per_head;
 
   if (threadIdx.x == 0) {
     ptx::mbar_init(q_full, 1);
@@ -138,7 +138,7 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
     const int qc = (g.q_col0 + h * g.col_per_head) / 64, kc = (g.k_col0 + h * g.col_per_head) / 64, vc = (g.v_col0 + h * g.col_per_head) / 64;
     if (ptx::elect_one()) {
       ptx::mbar_expect_tx(q_full, 2 * KB);
-      ptx::tma_load_3d(sQ, &tmQ, q_full, 0, (int)(row_base + qt * BQ), qc);
+      ptx::tma_load_4d(sQ, &tmQ, q_full, 0, qt * BQ, qc, plane);
     }
     __syncwarp();
     bool ok = true;
@@ -149,7 +149,7 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         if (!ok) break;
         if (ptx::elect_one()) {
           ptx::mbar_expect_tx(&k_full[ks], 2 * KBK);
-          ptx::tma_load_3d(sK + ks * 2 * KBK, &tmK, &k_full[ks], 0, (int)(row_base + (long long)(i + 1) * BKV), kc);
+          ptx::tma_load_4d(sK + ks * 2 * KBK, &tmK, &k_full[ks], 0, (i + 1) * BKV, kc, plane);
         }
         __syncwarp();
         if (++ks == KSTAGES) { ks = 0; kph ^= 1; }
@@ -160,7 +160,7 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         if (!ok) break;
         if (ptx::elect_one()) {
           ptx::mbar_expect_tx(&v_full[s], 2 * KBK);
-          ptx::tma_load_3d(sV + s * 2 * KBK, &tmV, &v_full[s], 0, (int)(row_base + (long long)i * BKV), vc);
+          ptx::tma_load_4d(sV + s * 2 * KBK, &tmV, &v_full[s], 0, i * BKV, vc, plane);
         }
         __syncwarp();
       }
@@ -388,27 +388,28 @@ int launch_causal_attention_tc(const CausalAttnArgs& a, cudaStream_t st) {
                            a.q.sn == S * st_ && a.k.sn == S * st_ && a.v.sn == S * st_ && st_ % 8 == 0;
   const bool head_major = a.q.st == D && a.k.st == D && a.v.st == D && a.q.sh == S * D && a.k.sh == S * D &&
                           a.v.sh == S * D && a.q.sn == H * S * D && a.k.sn == H * S * D && a.v.sn == H * S * D;
+  // Rows past a sequence's end are a plane's end, which reads as zeros: they meet probabilities of zero, and the next sequence's values, which
+  // need not be finite, would make NaN of them.
+  const int qbox[4] = {64, BQ, 2, 1}, kbox[4] = {64, BKV, 2, 1};
   if (interleaved) {
     // one [B*S, row pitch] matrix holds q, k and v side by side; columns are offsets from q
     const long long kcol = ((const char*)a.k.ptr - (const char*)a.q.ptr) / 2, vcol = ((const char*)a.v.ptr - (const char*)a.q.ptr) / 2;
     if (kcol < 0 || vcol < 0 || kcol + H * D > st_ || vcol + H * D > st_) return SMARTMEM_ERR_UNSUPPORTED;
     if (kcol % 64 || vcol % 64) return SMARTMEM_ERR_UNSUPPORTED;
-    // [64 columns][row][chunk of 64 columns]: both chunks of a head in one copy
-    const long long dims[3] = {64, B * S, st_ / 64}, strides[2] = {st_, 64};
-    const int qbox[3] = {64, BQ, 2}, kbox[3] = {64, BKV, 2};
-    if ((rc = tc_encode_nd_sw128(a.q.ptr, 3, dims, strides, qbox, &tq)) != SMARTMEM_OK) return rc;
-    if ((rc = tc_encode_nd_sw128(a.q.ptr, 3, dims, strides, kbox, &tk)) != SMARTMEM_OK) return rc;   // same buffer, 64-row boxes
+    // [64 columns][row][chunk of 64 columns][sequence]: both chunks of a head in one copy
+    const long long dims[4] = {64, S, st_ / 64, B}, strides[3] = {st_, 64, S * st_};
+    if ((rc = tc_encode_nd_sw128(a.q.ptr, 4, dims, strides, qbox, &tq)) != SMARTMEM_OK) return rc;
+    if ((rc = tc_encode_nd_sw128(a.q.ptr, 4, dims, strides, kbox, &tk)) != SMARTMEM_OK) return rc;   // same buffer, 64-row boxes
     tv = tk;
     g.q_col0 = 0; g.k_col0 = (int)kcol; g.v_col0 = (int)vcol; g.col_per_head = D;
-    g.row_per_batch = S; g.row_per_head = 0;
+    g.plane_per_batch = 1; g.plane_per_head = 0;
   } else if (head_major) {
-    const long long dims[3] = {64, B * H * S, 2}, strides[2] = {D, 64};
-    const int qbox[3] = {64, BQ, 2}, kbox[3] = {64, BKV, 2};
-    if ((rc = tc_encode_nd_sw128(a.q.ptr, 3, dims, strides, qbox, &tq)) != SMARTMEM_OK) return rc;
-    if ((rc = tc_encode_nd_sw128(a.k.ptr, 3, dims, strides, kbox, &tk)) != SMARTMEM_OK) return rc;
-    if ((rc = tc_encode_nd_sw128(a.v.ptr, 3, dims, strides, kbox, &tv)) != SMARTMEM_OK) return rc;
+    const long long dims[4] = {64, S, 2, B * H}, strides[3] = {D, 64, S * D};
+    if ((rc = tc_encode_nd_sw128(a.q.ptr, 4, dims, strides, qbox, &tq)) != SMARTMEM_OK) return rc;
+    if ((rc = tc_encode_nd_sw128(a.k.ptr, 4, dims, strides, kbox, &tk)) != SMARTMEM_OK) return rc;
+    if ((rc = tc_encode_nd_sw128(a.v.ptr, 4, dims, strides, kbox, &tv)) != SMARTMEM_OK) return rc;
     g.col_per_head = 0;
-    g.row_per_batch = H * S; g.row_per_head = S;
+    g.plane_per_batch = (int)H; g.plane_per_head = 1;
   } else {
     return SMARTMEM_ERR_UNSUPPORTED;
   }

@@ -1,12 +1,13 @@
-"""What is not finite stays where it belongs: a token that is infinite makes its own window's outputs not finite, and no other element
-changes by a bit.  Two windows share a tile of the tensor core, where a probability of zero times the other window's infinite value would be
-NaN."""
+"""What is not finite stays where it belongs: a token that is infinite makes its own window's outputs (its own sequence's in a decoder
+layer) not finite, and no other element changes by a bit.  Two windows, or the rows on both sides of a sequence's end, share a tile of the
+tensor core, where a probability of zero times another window's infinite value would be NaN."""
 import pytest
 import torch
 
 from paper_2404_13528_b200 import binding as sm
 from paper_2404_13528_b200 import synth
 from tests.gpu_util import to_dev
+from tests.test_gpu_llama import run_layer
 from tests.test_gpu_swin import run_block
 
 pytestmark = pytest.mark.gpu
@@ -43,3 +44,19 @@ def test_windows(B, H, W, C, heads, window, shift, mlp_ratio, mode):
         mask = other_windows(B, H, W, window, shift, token)
         assert torch.equal(y[mask], clean[mask]), f"token {token} reached another window"
         assert not torch.isfinite(y[~mask].float()).any()
+
+
+@pytest.mark.parametrize("B,S,hidden", [(2, 40, 256), (3, 100, 256), (2, 129, 512), (4, 333, 1024), (3, 1290, 256), (24, 200, 512)])
+@pytest.mark.parametrize("mode", [sm.ELIMINATE, sm.EXPLICIT])
+def test_sequences(B, S, hidden, mode):
+    dev = {k: to_dev(v) for k, v in synth.attn_layer_inputs(611, S, hidden, B=B).items()}
+    cfg = dict(B=B, S=S, hidden=hidden, heads=hidden // 128, add_residual=0, mode=mode)
+    clean = run_layer(dev, **cfg)
+    assert torch.isfinite(clean.float()).all()
+    for b in (0, B - 1):
+        x = dev["x"].clone()
+        x[b, 0, 5] = float("inf")
+        y = run_layer(dict(dev, x=x), **cfg)
+        others = [i for i in range(B) if i != b]
+        assert torch.equal(y[others], clean[others]), f"sequence {b} reached another one"
+        assert not torch.isfinite(y[b, 0].float()).any()
