@@ -61,6 +61,12 @@ struct GemmArgs {
   DevMap rowmap;
 };
 
+// The two-stage kernel's staging tiles, either as boxes (two of 64 KB) or as rows of 512 bytes, the two tiles' side by side and eight rows
+// shifted against one another by 16 bytes (eight threads on eight rows then write distinct banks).
+constexpr int kStageBoxBytes = 4 * 32 * 512, kStageBytes = 16 * (8 * 1024 + 112);
+static_assert(kStageBytes >= 2 * kStageBoxBytes, "room for either form");
+__device__ __forceinline__ uint32_t stage_row_off(int row, uint32_t tile) { return (uint32_t)(row * 1024 + (row >> 3) * 112 + (row & 7) * 16) + tile * 512u; }
+
 // Tile -> TMA coordinates of an operand: row origin inside the innermost row atom and the digits
 // of the outer row atoms / batch atoms (every tensor map is padded to rank 5, so all five
 // coordinates always exist and stay in registers).
@@ -145,7 +151,8 @@ constexpr int kThreads = 64 + 32 * kEpiWarps + 32;      // + a second TMA produc
 // back before any arithmetic -- for short reductions, where a tile's products take no longer than its epilogue -- and its rows
 // leave as 32 x 32 TMA boxes, or as 32-byte vectors through the row map, without staging a tile.  On single CTAs (us):
 // M = 50 176, N = 384, K = 128 16.4 -> 11.1, M = 12 544, N = 768, K = 192 9.5 -> 7.1.
-template <int BN, int STAGES, bool A_MN, bool PAIR, bool LEAN>
+// ROWS: the two-stage kernel's tiles leave a row of 512 bytes at a time instead of in boxes (store_rows).
+template <int BN, int STAGES, bool A_MN, bool PAIR, bool LEAN, bool ROWS>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmC, const __grid_constant__ GemmArgs g,
@@ -170,10 +177,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   // lean epilogue: a 32 x 32 output box per epilogue warp (64-byte rows, 64-byte swizzle), right behind the ring
   constexpr int CBOX_BYTES = 32 * 64;
   uint8_t* cstage = sB + STAGES * B_STAGE_BYTES;
-  // two-stage kernel: two staging tiles of 128 x 256, each four lane quadrants of four 32 x 64 boxes (128-byte rows and swizzle)
+  // two-stage kernel: two staging tiles of 128 x 256, each four lane quadrants of four 32 x 64 boxes (128-byte rows and swizzle) or of 32 rows
   constexpr bool QTMA = STAGES == 2;
-  constexpr int QTILE_BYTES = 4 * 32 * 512;
-  uint64_t* full = reinterpret_cast<uint64_t*>(cstage + (LEAN ? kEpiWarps * CBOX_BYTES : QTMA ? 2 * QTILE_BYTES : 0));
+  uint64_t* full = reinterpret_cast<uint64_t*>(cstage + (LEAN ? kEpiWarps * CBOX_BYTES : QTMA ? kStageBytes : 0));
   uint64_t* empty = full + STAGES;
   uint64_t* tmem_full = empty + STAGES;                      // [2]
   uint64_t* tmem_empty = tmem_full + 2;                      // [2]
@@ -211,7 +217,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if constexpr (HALVES) {
       if (hv.wide_tiles < tiles) ptx::prefetch_tensormap(&hv.map);
     }
-    if (QTMA || (LEAN && g.tma_out)) ptx::prefetch_tensormap(&tmC);
+    if ((QTMA && !ROWS) || (LEAN && g.tma_out)) ptx::prefetch_tensormap(&tmC);
   }
   if (warp == 1) {
     if constexpr (PAIR) ptx::tmem_alloc_pair(tmem_slot, TMEM_COLS);
@@ -528,10 +534,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if (!ok) break;
       ptx::tc_fence_after();
       const uint32_t taddr = tmem_base + buf * ACC_COLS + ((uint32_t)(q * 32) << 16);
-      uint8_t* qtile = cstage + (it & 1) * QTILE_BYTES + q * (QTILE_BYTES / 4);
+      uint8_t* qtile = cstage + (it & 1) * kStageBoxBytes + q * (kStageBoxBytes / 4);
+      uint8_t* qline = cstage + stage_row_off(q * 32 + lane, it & 1);
       if constexpr (QTMA) {
-        // the boxes that left this staging tile two tiles ago have been read
-        if (lane == 0) ptx::bulk_wait_group_read<1>();
+        // what left this staging tile two tiles ago has been read
+        if (lane < 8) ptx::bulk_wait_group_read<1>();
         asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory");
       }
       if constexpr (QSTAGE && QBULK) {
@@ -698,7 +705,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             }
           } else if constexpr (QTMA) {
             const int c = c0 + v * 8;
-            *reinterpret_cast<uint4*>(qtile + (c >> 6) * 4096 + lane * 128 + ((((c & 63) >> 3) ^ (lane & 7)) << 4)) = pk;
+            *reinterpret_cast<uint4*>(ROWS ? qline + c * 2 : qtile + (c >> 6) * 4096 + lane * 128 + ((((c & 63) >> 3) ^ (lane & 7)) << 4)) = pk;
           } else if constexpr (QSTAGE) *reinterpret_cast<uint4*>(qstage + lane * QROW + (c0 + v * 8) * 2) = pk;
           else *reinterpret_cast<uint4*>(stage + lane * STG_ROW + v * 16) = pk;
         }
@@ -733,7 +740,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // 62.8 in a long one.
         ptx::fence_proxy_async();
         asm volatile("bar.sync %0, 128;" ::"r"(1 + q) : "memory");
-        if (lane == 0) {                                     // (the lane that waits for its boxes: groups are a thread's own)
+        if constexpr (ROWS) {                                // (the lanes that wait for their copies: groups are a thread's own)
+          if (lane < 8) {
+            const int tr = q * 32 + grp * 8 + lane, orow = (int)tile_m * BM + tr;
+            if (orow < g.M)
+              ptx::bulk_store(g.out + (long long)batch * g.out_batch_stride + (long long)orow * g.ldc + n0, cstage + stage_row_off(tr, it & 1),
+                              (uint32_t)min(g.N - n0, BN) * 2u);
+            ptx::bulk_commit_group();
+          }
+        } else if (lane == 0) {
           if ((int)tile_m * BM + q * 32 < g.M && n0 + grp * 64 < g.N)
             ptx::tma_store_3d(&tmC, qtile + grp * 4096, n0 + grp * 64, (int)tile_m * BM + q * 32, (int)batch);
           ptx::bulk_commit_group();
@@ -940,13 +955,13 @@ int sm_count() {
   return n;
 }
 
-template <int BN, int STAGES, bool A_MN, bool PAIR = false, bool LEAN = false>
+template <int BN, int STAGES, bool A_MN, bool PAIR = false, bool LEAN = false, bool ROWS = false>
 int launch_t(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc, const Halves<true>& halves, const GemmArgs& g, cudaStream_t st) {
   constexpr bool QST = !PAIR && !(BN == 256 && STAGES == 4);
   constexpr int RCc = !QST ? 16 : ((BN / 4) > 32 ? 32 : (BN / 4));
   constexpr size_t smem = 1024 + STAGES * (A_STAGE_BYTES + (PAIR ? BN / 2 : BN) * BK * 2) + (2 * STAGES + 4) * 8 + 16 +
-                          (LEAN ? kEpiWarps * 32 * 64 : PAIR ? 0 : STAGES == 2 ? 2 * 4 * 32 * 512 : !QST ? kEpiWarps * 32 * (RCc * 2 + 16) : 4 * 32 * (BN * 2 + 16));   // pairs store from registers
-  if (ensure_max_dynamic_smem((const void*)gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN>, (int)smem) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
+                          (LEAN ? kEpiWarps * 32 * 64 : PAIR ? 0 : STAGES == 2 ? kStageBytes : !QST ? kEpiWarps * 32 * (RCc * 2 + 16) : 4 * 32 * (BN * 2 + 16));   // pairs store from registers
+  if (ensure_max_dynamic_smem((const void*)gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN, ROWS>, (int)smem) != SMARTMEM_OK) return SMARTMEM_ERR_CUDA;
   profile_tick("gemm_tc", st);
   long long tiles = (long long)g.tiles_n * g.tiles_m * g.batch;
   Halves<PAIR && BN == 256> hv;
@@ -958,10 +973,10 @@ int launch_t(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& tc
     // one cluster of two CTAs per tile of 256 rows; the two CTAs of a cluster are neighbours in blockIdx.x
     const long long pairs = sm_count() / 2;
     const unsigned grid = (unsigned)(2 * (tiles < pairs ? tiles : pairs));
-    launch_pdl_cluster(gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN>, dim3(grid), dim3(kThreads), smem, st, 2u, ta, tb, tc, g, hv);
+    launch_pdl_cluster(gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN, ROWS>, dim3(grid), dim3(kThreads), smem, st, 2u, ta, tb, tc, g, hv);
   } else {
     const unsigned grid = (unsigned)(tiles < sm_count() ? tiles : sm_count());
-    launch_pdl(gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN>, dim3(grid), dim3(kThreads), smem, st, ta, tb, tc, g, hv);
+    launch_pdl(gemm_tc_kernel<BN, STAGES, A_MN, PAIR, LEAN, ROWS>, dim3(grid), dim3(kThreads), smem, st, ta, tb, tc, g, hv);
   }
   count_launch();
   return cudaGetLastError() == cudaSuccess ? SMARTMEM_OK : SMARTMEM_ERR_CUDA;
@@ -1127,6 +1142,19 @@ TcOperand tc_operand_plain(const void* ptr, long long rows, long long K, long lo
 // 153.7; M = 12544, K = 512, N = 2048 (392) 24.2 -> 23.1; M = 20000, K = 512, N = 1024 21.3 -> 20.0.
 static bool tail_halves(long long tiles, long long pairs) { return tiles > pairs && tiles % pairs != 0 && 2 * (tiles % pairs) <= pairs; }
 
+// Whether the two-stage kernel's output leaves as rows of 512 bytes or as boxes of 32 x 64.  A box's rows of 128 bytes touch two lines each where
+// the output's rows are not whole lines, and where those are not whole sectors of 32 bytes either, L2 holds half-written sectors until the
+// neighbouring box comes: boxes then lose as soon as the stores are what a tile takes, that is where the tiles are full or the output is larger
+// than L2.  Us, boxes -> rows, K = 64, B x heads x S: 128 x 1000 59.6 -> 54.7, 128 x 968 60.7 -> 52.4, 128 x 776 44.2 -> 42.4, 32 x 1288 30.6 -> 29.2,
+// 30 x 1000 16.5 -> 16.1; but 128 x 616 24.9 -> 25.4, 30 x 712 9.9 -> 11.0, and in whole sectors 128 x 992 48.5 -> 53.4, 30 x 1024 15.2 -> 16.8.
+// Two k-blocks (K = 128) keep the ring of two stages from running ahead, and rows, which are one copy where boxes are two lines a row, are the better
+// from four tiles an SM on: 128 x 1000 78.1 -> 71.5, 128 x 1024 75.1 -> 71.7, 33 x 768 14.9 -> 14.3; 30 x 512 6.8 -> 7.4, 30 x 648 12.4 -> 12.5.
+static bool store_rows(long long tiles, long long batch, long long M, long long N, int nkb) {
+  if (nkb == 2) return tiles >= 4ll * tc_sm_count();
+  const double bytes = 2.0 * (double)(batch * M) * (double)N;
+  return N % 16 != 0 && bytes / ((double)tiles * kStageBoxBytes) + bytes / 4e8 > 1.02;
+}
+
 int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep, long long batch, long long M,
                    long long N, long long K, cudaStream_t st) {
   if (M < 1 || N < 1 || K < 1 || batch < 1 ||  M >= (1ll << 31) || N >= (1ll << 31))
@@ -1288,6 +1316,7 @@ int launch_gemm_tc(const TcOperand& A, const TcOperand& B, const TcEpilogue& ep,
     const uint64_t dims[3] = {(uint64_t)N, (uint64_t)M, (uint64_t)batch};
     const uint64_t strides[2] = {(uint64_t)ep.ldc * 2, (uint64_t)(batch > 1 ? ep.out_batch_stride : ep.ldc * M) * 2};
     const uint32_t box[3] = {64, 32, 1};
+    if (store_rows(all_tiles, batch, M, N, nkb)) return launch_t<256, 2, false, false, false, true>(ta, tb, tc, hv, g, st);
     if (encode_cached(ep.out, 3, dims, strides, box, &tc) == SMARTMEM_OK) return launch_t<256, 2, false>(ta, tb, tc, hv, g, st);
     stages = 3;
   }

@@ -31,6 +31,7 @@ def test_ragged_channels_last_copies_bit_exact(B, C, H, W):
     (20, 200, 8, 64),         # one 256-wide tile per 128 rows, clipped at row and column 200
     (40, 136, 4, 32), (10, 264, 16, 128),   # the shortest reduction; two k-blocks, eight columns in the second tile
     (8, 192, 10, 64), (8, 288, 9, 32), (3, 480, 9, 128), (4, 576, 8, 64),   # 96-wide tiles where they fill the columns, 256-wide for 480
+    (6, 504, 8, 64), (37, 200, 8, 128), (20, 264, 5, 128),   # the tiles' rows stored one by one: a last tile of 248 columns, of 72 rows, of 8 by 8
 ])
 def test_batched_scores_clipped_tiles(B, S, H, D):
     q = synth.normal(502, 0, (B, S, H * D), dtype="bf16")
