@@ -61,3 +61,13 @@ def assert_close_f32(got: np.ndarray, ref: np.ndarray, what: str = ""):
 def check_status():
     st = sm.smartmem_last_device_status(stream())
     assert st == sm.OK, f"device status {st}: {sm.smartmem_status_string(st)}"
+
+
+def launched(call):
+    """The labels of the kernels that call() launches, in order."""
+    sm.smartmem_profile_begin()
+    try:
+        call()
+    finally:
+        kernels = sm.smartmem_profile_end(stream())
+    return [label for label, _ in kernels]

@@ -4,7 +4,7 @@ import pytest
 import torch
 
 from paper_2404_13528_b200 import binding as sm
-from tests.gpu_util import check_status, stream
+from tests.gpu_util import check_status, launched, stream
 
 pytestmark = pytest.mark.gpu
 
@@ -36,6 +36,11 @@ def bf16(seed, *shape, std=1.0, mean=0.0, dtype=torch.bfloat16):
 def transposer(rows, cols, dtype=sm.BF16):
     """[cols, rows] -> [rows, cols] as a copy."""
     return Chain([sm.make_op(sm.OP_TRANSPOSE, perm=(1, 0)), sm.make_op(sm.OP_COPY)], [(cols, rows)], dtype=dtype)
+
+
+def roller(n, dtype=sm.BF16):
+    """[n] -> [n], rotated, as a copy."""
+    return Chain([sm.make_op(sm.OP_ROLL, shift=5, axis=0), sm.make_op(sm.OP_COPY)], [(n,)], dtype=dtype)
 
 
 def compare(sources, make, use, out_like):
@@ -97,7 +102,7 @@ def test_weights_then_patch_merging(C, which):
     if which == "w":
         make, target, sources = transposer(N, K), w, [bf16(54 + i, K, N, std=0.05) for i in range(3)]
     else:
-        make, target = Chain([sm.make_op(sm.OP_ROLL, shift=5, axis=0), sm.make_op(sm.OP_COPY)], [(K,)]), g
+        make, target = roller(K), g
         sources = [bf16(57 + i, K, std=0.1, mean=1.0) for i in range(3)]
     compare(sources, lambda s: make([s], target), lambda out: chain([x, g, b, w], out),
             torch.empty(B, H * W // 4, N, dtype=torch.bfloat16, device="cuda"))
@@ -118,16 +123,40 @@ def test_weights_then_decode_step(B):
             torch.empty_like(x))
 
 
-@pytest.mark.parametrize("which,dtype,C,head_dim,H,half", [
-    ("w_qkv", sm.BF16, 192, 32, 14, -1),     # norm + QKV in one kernel
-    ("w_qkv", sm.BF16, 512, 32, 14, -1),     # kernel by kernel
-    ("w_qkv", sm.F32, 32, 16, 8, -1),
-    ("w_fc1", sm.BF16, 192, 32, 14, 1), ("w_fc1", sm.BF16, 256, 32, 14, 1), ("w_fc1", sm.F32, 32, 16, 8, 1),   # the MLP half on its own
-    ("w_fc1", sm.BF16, 128, 32, 49, 1),      # the same over a cluster
+@pytest.mark.parametrize("which", ["rms_g", "w_qkv", "x"])
+@pytest.mark.parametrize("B,S,hidden", [(1, 20, 512), (2, 32, 3072)])
+def test_operands_then_decoder_layer_of_few_rows(B, S, hidden, which):
+    """RMSNorm is part of the QKV product, which is the call's first kernel."""
+    par = dict(x=bf16(90, B * S, hidden), rms_g=bf16(91, hidden, std=0.1, mean=1.0), w_qkv=bf16(92, 3 * hidden, hidden, std=0.05),
+               w_o=bf16(93, hidden, hidden, std=0.05))
+    p = sm.AttnParams()
+    p.dtype, p.B, p.S, p.hidden, p.heads, p.head_dim, p.causal, p.rms_eps, p.rope_theta = sm.BF16, B, S, hidden, hidden // 128, 128, 1, 1e-5, 10000.0
+    p.rms_g, p.w_qkv, p.w_o = par["rms_g"].data_ptr(), par["w_qkv"].data_ptr(), par["w_o"].data_ptr()
+    n = sm.smartmem_attn_layer_workspace_bytes(p, sm.ELIMINATE)
+    ws = torch.empty(n, dtype=torch.uint8, device="cuda")
+    target, std = par[which], 0.05 if which == "w_qkv" else 1.0
+
+    def use(out):
+        sm.smartmem_attn_layer(p, par["x"].data_ptr(), out.data_ptr(), ws.data_ptr(), n, sm.ELIMINATE, stream())
+
+    assert launched(lambda: use(torch.empty_like(par["x"])))[0] == "gemm_splitk"
+    make = roller(target.numel()) if target.dim() == 1 else transposer(*target.shape)
+    compare([bf16(94 + i, *reversed(target.shape), std=std) for i in range(3)], lambda s: make([s], target), use, torch.empty_like(par["x"]))
+
+
+@pytest.mark.parametrize("which,dtype,C,head_dim,H,half,first", [
+    ("w_qkv", sm.BF16, 192, 32, 14, -1, "swin_attn_cluster"), ("w_proj", sm.BF16, 192, 32, 14, -1, "swin_attn_cluster"),
+    ("b_qkv", sm.BF16, 192, 32, 14, -1, "swin_attn_cluster"), ("rel_bias_table", sm.BF16, 192, 32, 14, -1, "swin_attn_cluster"),
+    ("w_qkv", sm.BF16, 192, 32, 77, -1, "gemm_ln_wave"),       # norm + QKV in one kernel: more windows than one wave of clusters
+    ("w_qkv", sm.BF16, 512, 32, 14, -1, "layernorm"),          # kernel by kernel
+    ("w_qkv", sm.F32, 32, 16, 8, -1, "swin_attn_f32"),
+    ("w_fc1", sm.BF16, 192, 32, 14, 1, "gemm_ln_wave"), ("w_fc1", sm.BF16, 256, 32, 14, 1, "gemm_ln_wave"),   # the MLP half on its own
+    ("w_fc1", sm.F32, 32, 16, 8, 1, "swin_mlp_f32"),
+    ("w_fc1", sm.BF16, 128, 32, 49, 1, "mlp_cluster"),         # the same over a cluster
 ])
-def test_weights_then_block(which, dtype, C, head_dim, H, half):
+def test_weights_then_block(which, dtype, C, head_dim, H, half, first):
     td = torch.float32 if dtype == sm.F32 else torch.bfloat16
-    ws_, heads, rows = (4 if H == 8 else 7), C // head_dim, 3 * C if which == "w_qkv" else 4 * C
+    ws_, heads = (4 if H == 8 else 7), C // head_dim
     par = dict(ln1_g=bf16(70, C, std=0.1, mean=1.0, dtype=td), ln1_b=bf16(71, C, std=0.1, dtype=td), w_qkv=bf16(72, 3 * C, C, std=0.05, dtype=td),
                b_qkv=bf16(73, 3 * C, std=0.05, dtype=td), rel_bias_table=bf16(74, (2 * ws_ - 1) ** 2, heads, std=0.1, dtype=td),
                w_proj=bf16(75, C, C, std=0.05, dtype=td), b_proj=bf16(76, C, std=0.05, dtype=td), ln2_g=bf16(77, C, std=0.1, mean=1.0, dtype=td),
@@ -140,7 +169,9 @@ def test_weights_then_block(which, dtype, C, head_dim, H, half):
     x = bf16(83, 1, H, H, C, dtype=td)
     n = sm.smartmem_swin_block_workspace_bytes(p, sm.ELIMINATE)
     ws = torch.empty(n, dtype=torch.uint8, device="cuda")
-    make = transposer(rows, C, dtype)
+    target = par[which]
+    flat = target.dim() == 1 or which == "rel_bias_table"
+    make = roller(target.numel(), dtype) if flat else transposer(*target.shape, dtype)
 
     def use(out):
         if half < 0:
@@ -148,4 +179,6 @@ def test_weights_then_block(which, dtype, C, head_dim, H, half):
         else:
             sm.smartmem_swin_block_half(p, x.data_ptr(), out.data_ptr(), ws.data_ptr(), n, sm.ELIMINATE, half, stream())
 
-    compare([bf16(84 + i, C, rows, std=0.05, dtype=td) for i in range(3)], lambda s: make([s], par[which]), use, torch.empty_like(x))
+    assert launched(lambda: use(torch.empty_like(x)))[0] == first
+    shape, std = ((target.numel(),), 0.1) if flat else (tuple(reversed(target.shape)), 0.05)
+    compare([bf16(84 + i, *shape, std=std, dtype=td) for i in range(3)], lambda s: make([s], target), use, torch.empty_like(x))
