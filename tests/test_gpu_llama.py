@@ -60,14 +60,14 @@ def test_partial_rotary_layers(B, S, hidden, heads, rot):
 def test_rotated_tiles(B, S, hidden, rot):
     """The QKV product's tiles with rotated columns: 128 columns on one CTA and on a pair, 256 on a pair, whole and as halves (520 rows of 3072);
     16, 32 and 64 pairs a head, several sequences to a tile, rows past the end."""
-    case(33, B, S, hidden, hidden // 128, 1, rotary_dim=rot, first_rows_allowance=B * S * hidden // 10000 + 2)
+    case(33, B, S, hidden, hidden // 128, 1, rotary_dim=rot)
 
 
 @pytest.mark.parametrize("B,S,hidden", [(1, 65, 256), (3, 127, 256), (2, 129, 512), (1, 192, 256), (2, 385, 256), (8, 1290, 256), (40, 200, 256)])
 def test_key_tiles_in_turn(B, S, hidden):
     """Two softmax groups taking the 64-key tiles in turn (rows before the second group's first tile, odd and even numbers of tiles, a second
     wave of CTAs at 8 x 1290), and the one-group kernel with rows to spare (40 x 200)."""
-    case(34, B, S, hidden, hidden // 128, 0, first_rows_allowance=B * S * hidden // 10000 + 2)
+    case(34, B, S, hidden, hidden // 128, 0)
 
 
 def test_partial_rotary_layer_full_size():
