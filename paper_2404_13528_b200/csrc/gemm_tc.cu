@@ -410,9 +410,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     uint32_t it = 0;
     bool ok = true;
     const bool res_wide = (reinterpret_cast<uintptr_t>(g.residual) & 31) == 0;   // (row offsets of a pair's output are multiples of 16 elements)
-    constexpr bool PREFETCH_NEXT = false;                   // (tried: next-tile offset + residual a tile ahead; the extra live registers spill and it is slower)
-    long long off_next = 0;
-    uint4 res_next[VPR];
     const uint32_t tmem_empty0 = PAIR ? ptx::mapa(ptx::smem_u32(tmem_empty), 0) : 0u;   // the even CTA's barriers
     for (uint32_t t = cta_first; t < total_tiles && ok; t += cta_step, ++it) {
       const TileItem item = tile_item<HALVES>(t, g, hv);
@@ -434,10 +431,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const uint32_t b2 = fd_div((uint32_t)row, g.fd_out2_S);
         o2_base = (long long)b2 * g.N * g.fd_out2_S.d + ((uint32_t)row - b2 * g.fd_out2_S.d);
       }
-      // Output offset of this thread's row (through the row map when the store is a scatter).  With
-      // one round per tile the offset and the residual of the NEXT tile were requested during the
-      // previous iteration, so neither the map evaluation nor the gather's latency is on the path
-      // between the accumulator becoming ready and its buffer being handed back.
       // column-segmented output: a tile never straddles segments (seg_cols is a multiple of BN), so
       // the whole tile has one base and one pitch; the base is biased by the segment's first column
       __nv_bfloat16* out_t = g.out;
@@ -447,13 +440,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         out_t = g.seg_out[sg] - (long long)sg * g.seg_cols;
         ld_t = g.seg_ld[sg];
       }
-      long long off;
-      if (PREFETCH_NEXT && it > 0) {
-        off = off_next;
-      } else if (BARE) {
-        off = 0;                                             // (the boxes go by coordinates)
-      } else {
-        off = 0;
+      // Output offset of this thread's row, through the row map where the store is a scatter.  (Requested a tile ahead, with the residual, its
+      // registers spill and the kernel is slower.)
+      long long off = 0;
+      if (!BARE) {                                           // (boxes go by coordinates, rows by their own)
         if (row_ok) off = g.has_rowmap ? devmap_eval_unrolled(g.rowmap, (uint32_t)row) : (long long)row * ld_t;
         off += (long long)batch * g.out_batch_stride;
       }
@@ -480,29 +470,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           if (rrow && row_ok && n0 + c0 + v * 8 + 8 <= g.N) res[v] = *reinterpret_cast<const uint4*>(rrow + n0 + c0 + v * 8);
         }
       };
-      if (PREFETCH_NEXT && it > 0) {
-#pragma unroll
-        for (int v = 0; v < VPR; ++v) res[v] = res_next[v];
-      } else if (!BARE) {
-        fetch_res(col_of(0));                                // in flight while this tile's MMAs still run
-      }
-      if (PREFETCH_NEXT) {                                   // request the next tile's row offset and residual now
-        const uint32_t tn = t + cta_step;
-        if (tn < total_tiles) {
-          const TileIdx nx = split_tile(tn, g.fd_tiles_n, g.fd_tiles_m);
-          const int nrow = nx.tile_m * BM + q * 32 + lane;
-          off_next = 0;
-          if (nrow < g.M) off_next = g.has_rowmap ? devmap_eval_unrolled(g.rowmap, (uint32_t)nrow) : (long long)nrow * g.ldc;
-          off_next += (long long)nx.batch * g.out_batch_stride;
-          const int nn0 = nx.tile_n * BN, c0 = col_of(0);
-#pragma unroll
-          for (int v = 0; v < VPR; ++v) {
-            res_next[v] = make_uint4(0, 0, 0, 0);
-            if (g.residual && nrow < g.M && nn0 + c0 + v * 8 + 8 <= g.N)
-              res_next[v] = *reinterpret_cast<const uint4*>(g.residual + off_next + nn0 + c0 + v * 8);
-          }
-        }
-      }
+      if (!BARE) fetch_res(col_of(0));                       // in flight while this tile's MMAs still run
 
       // Rotated columns: pairs (i, i + R/2) of the first R columns of each 128-wide head (R = 128: the whole head).  A warp takes the 16 pairs
       // i = 16 grp + j of every head of the tile (both halves of a pair, as two blocks of 16 columns), or past R two blocks that stay as they
@@ -613,116 +581,116 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       }
       if (!rope_tile) {
 #pragma unroll
-      for (int rd = 0; rd < ROUNDS; ++rd) {
-        const int c0 = col_of(rd);
-        float acc[RC];
-        uint4 bv[VPR];                                       // this round's bias columns: requested before the wait on tensor memory
-        if (!BARE && g.bias) {
+        for (int rd = 0; rd < ROUNDS; ++rd) {
+          const int c0 = col_of(rd);
+          float acc[RC];
+          uint4 bv[VPR];                                       // this round's bias columns: requested before the wait on tensor memory
+          if (!BARE && g.bias) {
 #pragma unroll
-          for (int v = 0; v < VPR; ++v) {
-            bv[v] = make_uint4(0, 0, 0, 0);
-            if (n0 + c0 + v * 8 + 8 <= g.N) bv[v] = *reinterpret_cast<const uint4*>(g.bias + n0 + c0 + v * 8);
-          }
-        }
-        {
-          uint32_t rv_local[EARLY ? 1 : RC];
-          uint32_t* rv = EARLY ? rall[EARLY ? rd : 0] : rv_local;
-          if constexpr (!EARLY) {
-            ptx::tmem_ld_cols<RC>(taddr + c0, rv);
-            ptx::tmem_ld_wait();
-          }
-#pragma unroll
-          for (int j = 0; j < RC; ++j) acc[j] = __uint_as_float(rv[j]);
-        }
-        if (!BARE && g.bias) {
-#pragma unroll
-          for (int v = 0; v < VPR; ++v) {
-            const uint32_t w[4] = {bv[v].x, bv[v].y, bv[v].z, bv[v].w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const float2 f = bf16x2_to_float2(w[j]);
-              acc[v * 8 + 2 * j] += f.x;
-              acc[v * 8 + 2 * j + 1] += f.y;
+            for (int v = 0; v < VPR; ++v) {
+              bv[v] = make_uint4(0, 0, 0, 0);
+              if (n0 + c0 + v * 8 + 8 <= g.N) bv[v] = *reinterpret_cast<const uint4*>(g.bias + n0 + c0 + v * 8);
             }
           }
-        }
-        if (!BARE && g.gelu) {
-#pragma unroll
-          for (int j = 0; j < RC; ++j) acc[j] = gelu_tanh(acc[j]);
-        }
-        if (!BARE && rrow) {
-#pragma unroll
-          for (int v = 0; v < VPR; ++v) {
-            const uint32_t w[4] = {res[v].x, res[v].y, res[v].z, res[v].w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const float2 f = bf16x2_to_float2(w[j]);
-              acc[v * 8 + 2 * j] += f.x;
-              acc[v * 8 + 2 * j + 1] += f.y;
+          {
+            uint32_t rv_local[EARLY ? 1 : RC];
+            uint32_t* rv = EARLY ? rall[EARLY ? rd : 0] : rv_local;
+            if constexpr (!EARLY) {
+              ptx::tmem_ld_cols<RC>(taddr + c0, rv);
+              ptx::tmem_ld_wait();
             }
+#pragma unroll
+            for (int j = 0; j < RC; ++j) acc[j] = __uint_as_float(rv[j]);
           }
-          if (rd + 1 < ROUNDS) fetch_res(col_of(rd + 1));
-        }
-        if (!LEAN && !BARE && g.out2 && row_ok) {
-          // The redundant copy of a producer with consumers of different reduction dimensions: the same values with the
-          // row's position inside its group as the contiguous dimension.  A warp's 32 rows write 64 contiguous bytes per column.
+          if (!BARE && g.bias) {
 #pragma unroll
-          for (int j = 0; j < RC; ++j)
-            if (n0 + c0 + j < g.N) g.out2[o2_base + (long long)(n0 + c0 + j) * g.fd_out2_S.d] = __float2bfloat16_rn(acc[j]);
-        }
-        uint4 pk_prev = make_uint4(0, 0, 0, 0);
+            for (int v = 0; v < VPR; ++v) {
+              const uint32_t w[4] = {bv[v].x, bv[v].y, bv[v].z, bv[v].w};
 #pragma unroll
-        for (int v = 0; v < VPR; ++v) {
-          uint4 pk;
-          pk.x = float2_to_bf16x2(acc[v * 8 + 0], acc[v * 8 + 1]);
-          pk.y = float2_to_bf16x2(acc[v * 8 + 2], acc[v * 8 + 3]);
-          pk.z = float2_to_bf16x2(acc[v * 8 + 4], acc[v * 8 + 5]);
-          pk.w = float2_to_bf16x2(acc[v * 8 + 6], acc[v * 8 + 7]);
-          if constexpr (DIRECT) {
-            // 64 contiguous bytes of the thread's own row per round, as two 32-byte stores: whole sectors, and the
-            // shared memory (whose bandwidth the operands need) is left to the ring, which gets six stages
-            if (LEAN && g.tma_out) {
-              // lean epilogue: the warp's 32 x 32 box goes through its own 2 KB of shared memory and leaves as one TMA
-              // store -- a row-per-thread store touches 32 lines per instruction, and those stores and the next tile's
-              // operand loads were in each other's way
-              if (v == 0) {
-                if (lane == 0) ptx::bulk_wait_group_read<0>();     // the previous round's box has been read
-                __syncwarp();
+              for (int j = 0; j < 4; ++j) {
+                const float2 f = bf16x2_to_float2(w[j]);
+                acc[v * 8 + 2 * j] += f.x;
+                acc[v * 8 + 2 * j + 1] += f.y;
               }
-              *reinterpret_cast<uint4*>(cstage + e * CBOX_BYTES + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4)) = pk;
-              if (v == VPR - 1) {
-                ptx::fence_proxy_async();
-                __syncwarp();
-                if (lane == 0 && (int)tile_m * BM + q * 32 < g.M) {
-                  ptx::tma_store_2d(&tmC, cstage + e * CBOX_BYTES, n0 + c0, (int)tile_m * BM + q * 32);
-                  ptx::bulk_commit_group();
+            }
+          }
+          if (!BARE && g.gelu) {
+#pragma unroll
+            for (int j = 0; j < RC; ++j) acc[j] = gelu_tanh(acc[j]);
+          }
+          if (!BARE && rrow) {
+#pragma unroll
+            for (int v = 0; v < VPR; ++v) {
+              const uint32_t w[4] = {res[v].x, res[v].y, res[v].z, res[v].w};
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const float2 f = bf16x2_to_float2(w[j]);
+                acc[v * 8 + 2 * j] += f.x;
+                acc[v * 8 + 2 * j + 1] += f.y;
+              }
+            }
+            if (rd + 1 < ROUNDS) fetch_res(col_of(rd + 1));
+          }
+          if (!LEAN && !BARE && g.out2 && row_ok) {
+            // The redundant copy of a producer with consumers of different reduction dimensions: the same values with the
+            // row's position inside its group as the contiguous dimension.  A warp's 32 rows write 64 contiguous bytes per column.
+#pragma unroll
+            for (int j = 0; j < RC; ++j)
+              if (n0 + c0 + j < g.N) g.out2[o2_base + (long long)(n0 + c0 + j) * g.fd_out2_S.d] = __float2bfloat16_rn(acc[j]);
+          }
+          uint4 pk_prev = make_uint4(0, 0, 0, 0);
+#pragma unroll
+          for (int v = 0; v < VPR; ++v) {
+            uint4 pk;
+            pk.x = float2_to_bf16x2(acc[v * 8 + 0], acc[v * 8 + 1]);
+            pk.y = float2_to_bf16x2(acc[v * 8 + 2], acc[v * 8 + 3]);
+            pk.z = float2_to_bf16x2(acc[v * 8 + 4], acc[v * 8 + 5]);
+            pk.w = float2_to_bf16x2(acc[v * 8 + 6], acc[v * 8 + 7]);
+            if constexpr (DIRECT) {
+              // 64 contiguous bytes of the thread's own row per round, as two 32-byte stores: whole sectors, and the
+              // shared memory (whose bandwidth the operands need) is left to the ring, which gets six stages
+              if (LEAN && g.tma_out) {
+                // lean epilogue: the warp's 32 x 32 box goes through its own 2 KB of shared memory and leaves as one TMA
+                // store -- a row-per-thread store touches 32 lines per instruction, and those stores and the next tile's
+                // operand loads were in each other's way
+                if (v == 0) {
+                  if (lane == 0) ptx::bulk_wait_group_read<0>();     // the previous round's box has been read
+                  __syncwarp();
                 }
+                *reinterpret_cast<uint4*>(cstage + e * CBOX_BYTES + lane * 64 + ((v ^ ((lane >> 1) & 3)) << 4)) = pk;
+                if (v == VPR - 1) {
+                  ptx::fence_proxy_async();
+                  __syncwarp();
+                  if (lane == 0 && (int)tile_m * BM + q * 32 < g.M) {
+                    ptx::tma_store_2d(&tmC, cstage + e * CBOX_BYTES, n0 + c0, (int)tile_m * BM + q * 32);
+                    ptx::bulk_commit_group();
+                  }
+                }
+              } else if (v & 1) {
+                if (row_ok && n0 + c0 + v * 8 < g.N) ptx::st_global_v8(out_t + off + n0 + c0 + (v - 1) * 8, pk_prev, pk);
+              } else {
+                pk_prev = pk;
               }
-            } else if (v & 1) {
-              if (row_ok && n0 + c0 + v * 8 < g.N) ptx::st_global_v8(out_t + off + n0 + c0 + (v - 1) * 8, pk_prev, pk);
-            } else {
-              pk_prev = pk;
-            }
-          } else if constexpr (QTMA) {
-            const int c = c0 + v * 8;
-            *reinterpret_cast<uint4*>(ROWS ? qline + c * 2 : qtile + (c >> 6) * 4096 + lane * 128 + ((((c & 63) >> 3) ^ (lane & 7)) << 4)) = pk;
-          } else if constexpr (QSTAGE) *reinterpret_cast<uint4*>(qstage + lane * QROW + (c0 + v * 8) * 2) = pk;
-          else *reinterpret_cast<uint4*>(stage + lane * STG_ROW + v * 16) = pk;
-        }
-        if constexpr (!QSTAGE && !DIRECT) {
-          __syncwarp();
-#pragma unroll
-          for (int i = 0; i < VPR; ++i) {
-            const int v = lane + 32 * i;
-            const int rr = v / VPR, seg = v - rr * VPR;
-            const long long roff = __shfl_sync(0xFFFFFFFFu, off, rr);
-            const int rok = __shfl_sync(0xFFFFFFFFu, (int)row_ok, rr);
-            const uint4 pk = *reinterpret_cast<const uint4*>(stage + rr * STG_ROW + seg * 16);
-            if (rok && n0 + c0 + seg * 8 + 8 <= g.N) *reinterpret_cast<uint4*>(out_t + roff + n0 + c0 + seg * 8) = pk;
+            } else if constexpr (QTMA) {
+              const int c = c0 + v * 8;
+              *reinterpret_cast<uint4*>(ROWS ? qline + c * 2 : qtile + (c >> 6) * 4096 + lane * 128 + ((((c & 63) >> 3) ^ (lane & 7)) << 4)) = pk;
+            } else if constexpr (QSTAGE) *reinterpret_cast<uint4*>(qstage + lane * QROW + (c0 + v * 8) * 2) = pk;
+            else *reinterpret_cast<uint4*>(stage + lane * STG_ROW + v * 16) = pk;
           }
-          __syncwarp();
+          if constexpr (!QSTAGE && !DIRECT) {
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < VPR; ++i) {
+              const int v = lane + 32 * i;
+              const int rr = v / VPR, seg = v - rr * VPR;
+              const long long roff = __shfl_sync(0xFFFFFFFFu, off, rr);
+              const int rok = __shfl_sync(0xFFFFFFFFu, (int)row_ok, rr);
+              const uint4 pk = *reinterpret_cast<const uint4*>(stage + rr * STG_ROW + seg * 16);
+              if (rok && n0 + c0 + seg * 8 + 8 <= g.N) *reinterpret_cast<uint4*>(out_t + roff + n0 + c0 + seg * 8) = pk;
+            }
+            __syncwarp();
+          }
         }
-      }
       }
       // all of this warp's TMEM reads of the buffer have completed (wait::ld above)
       if constexpr (!EARLY) {
