@@ -50,12 +50,6 @@ struct TcAttnArgs {
   int* status;
 };
 
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float y;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
@@ -259,7 +253,7 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       float corr = 1.f;
       bool rescale = false;
       if (mx > m_used + kRescaleThreshold) {           // (first tile: m_used = -inf)
-        corr = ex2(m_used - mx);                       // 0 on the first tile
+        corr = ptx::ex2(m_used - mx);                       // 0 on the first tile
         l *= corr;
         m_used = mx;
         rescale = turn > 0;
@@ -274,7 +268,7 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       for (int c = 0; c < BKV; c += 2) {
         float e0, e1;
         ptx::unpack2(ptx::fma2(ptx::pack2(__uint_as_float(rv[c]), __uint_as_float(rv[c + 1])), sc2, nm2), e0, e1);
-        const float p0 = ex2(e0), p1 = ex2(e1);
+        const float p0 = ptx::ex2(e0), p1 = ptx::ex2(e1);
         l2[(c >> 1) & 1] = ptx::add2(l2[(c >> 1) & 1], ptx::pack2(p0, p1));
         pk[c / 2] = float2_to_bf16x2(p0, p1);
       }
@@ -315,8 +309,8 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
       asm volatile("bar.sync 1, 256;" ::: "memory");
       const float2 a = ml_s[r], c = ml_s[BQ + r];
       const float mt = fmaxf(a.x, c.x);
-      w0 = ex2(a.x - mt);
-      w1 = ex2(c.x - mt);
+      w0 = ptx::ex2(a.x - mt);
+      w1 = ptx::ex2(c.x - mt);
       lsum = a.y * w0 + c.y * w1;
     }
     if (ok) ok = ptx::mbar_wait(o_done, 0, abort_flag, g.status);
@@ -331,13 +325,11 @@ causal_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_cons
         uint32_t rv[32];
         ptx::tmem_ld32(to + ch * 32, rv);
         if constexpr (G > 1) {
-          if (n_kv > 1) {                                // (with one tile the second group has no O)
-            uint32_t rw[32];
-            ptx::tmem_ld32(to + D + ch * 32, rw);
-            ptx::tmem_ld_wait();
+          uint32_t rw[32];
+          ptx::tmem_ld32(to + D + ch * 32, rw);
+          ptx::tmem_ld_wait();
 #pragma unroll
-            for (int c = 0; c < 32; ++c) rv[c] = __float_as_uint(__uint_as_float(rv[c]) * w0 + __uint_as_float(rw[c]) * w1);
-          }
+          for (int c = 0; c < 32; ++c) rv[c] = __float_as_uint(__uint_as_float(rv[c]) * w0 + __uint_as_float(rw[c]) * w1);
         }
         ptx::tmem_ld_wait();
         if (qi < g.S && wide_store) {                    // whole 32-byte sectors per store

@@ -32,6 +32,7 @@
 #include "attn.cuh"
 #include "gemm_tc.cuh"
 #include "ptx.cuh"
+#include "tc_tiles.cuh"
 
 
 namespace smartmem {
@@ -56,23 +57,6 @@ struct WinTcArgs {
   FastDiv fd_T;
   int* status;
 };
-
-// Shared-memory matrix descriptor with 64-byte swizzle (rows of 64 bytes, 8-row groups 512 bytes apart).
-__device__ __forceinline__ uint64_t make_desc_sw64(uint32_t smem_addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-  uint64_t d = 0;
-  d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);
-  d |= (uint64_t)((lbo_bytes >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo_bytes >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)4 << 61;
-  return d;
-}
-
-__device__ __forceinline__ float ex2f(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 
 // KC: key columns a softmax thread works on (56 when the window has at most 56 tokens -- a 7 x 7 window
 // has 49 -- else 64).  Columns [T, 64) of a score row are padding whose probability is zero.
@@ -211,7 +195,7 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
         if (!ok) break;
         ptx::tc_fence_after();
         const uint32_t v0 = ptx::smem_u32(sIn + s * STAGE_BYTES + 2 * OP_BYTES);
-        const uint64_t vd = make_desc_sw64(v0, 16, 512);
+        const uint64_t vd = desc_sw64(v0);
         const uint32_t od = tmem_base + TM_O + ob * D, pa = tmem_base + TM_P + ob * 32;
         if (ptx::elect_one()) {
 #pragma unroll
@@ -241,7 +225,7 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
         if (!ok) break;
         ptx::tc_fence_after();
         const uint32_t q0 = ptx::smem_u32(sIn + s * STAGE_BYTES), k0 = q0 + OP_BYTES;
-        const uint64_t qd = make_desc_sw64(q0, 16, 512), kd = make_desc_sw64(k0, 16, 512);
+        const uint64_t qd = desc_sw64(q0), kd = desc_sw64(k0);
         if (ptx::elect_one()) {
 #pragma unroll
           for (int ks = 0; ks < 4; ++ks) {             // 16 features per step: +32 bytes; steps 2-3: the second window's keys, +4096 bytes
@@ -368,7 +352,7 @@ win_attn_tc_kernel(const __grid_constant__ CUtensorMap tm0, const __grid_constan
       for (int c = KC / 2; c < 32; ++c) pk[c] = 0u;        // padding keys
 #pragma unroll
       for (int c = 0; c < KC; c += 2) {
-        const float p0 = ex2f(fmaf(sc[c], LOG2E, nmx)), p1 = ex2f(fmaf(sc[c + 1], LOG2E, nmx));
+        const float p0 = ptx::ex2(fmaf(sc[c], LOG2E, nmx)), p1 = ptx::ex2(fmaf(sc[c + 1], LOG2E, nmx));
         sum4[c & 2] += p0;
         sum4[(c & 2) + 1] += p1;
         pk[c / 2] = float2_to_bf16x2(p0, p1);

@@ -295,8 +295,8 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     __nv_bfloat16* out = g.seg_cols > 0 ? g.seg_out[sg] - (long long)sg * g.seg_cols : g.out;
     float f0 = 0.f, f1 = 0.f;
     if (rot) {
-      asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(f0) : "f"(-(float)(2 * lane) * g.rope_c));
-      asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(f1) : "f"(-(float)(2 * lane + 1) * g.rope_c));
+      f0 = ptx::ex2(-(float)(2 * lane) * g.rope_c);
+      f1 = ptx::ex2(-(float)(2 * lane + 1) * g.rope_c);
     }
     auto rotate = [](float ang, float& x, float& y) {
       // (reduced mod 2 pi in two steps, then the hardware sine / cosine)

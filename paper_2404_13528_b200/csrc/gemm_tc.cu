@@ -487,8 +487,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           const float pos = (float)(row_ok ? g.rope_pos0 + row % g.rope_S : 0);
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            float f;
-            asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(f) : "f"(-(float)(grp * 16 + j) * g.rope_c));
+            const float f = ptx::ex2(-(float)(grp * 16 + j) * g.rope_c);
             const float ang = pos * f;
             const float kk = rintf(ang * 0.15915494309189535f);
             float red = fmaf(-kk, 6.2831854820251465f, ang);

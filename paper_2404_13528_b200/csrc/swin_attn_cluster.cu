@@ -77,12 +77,6 @@ struct Plan {
   static_assert(bytes <= 227 * 1024, "shared memory");
 };
 
-__device__ __forceinline__ float ex2f(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 template <int NV>
 __global__ void __launch_bounds__(kThreads, 1)
 swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmP, const __grid_constant__ AttnClusterArgs g) {
@@ -481,7 +475,7 @@ swin_attn_cluster_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_c
         if (part * 32 + c8 * 8 < T) {                  // (uniform)
 #pragma unroll
           for (int c = c8 * 8; c < c8 * 8 + 8; c += 2) {
-            const float p0 = ex2f(fmaf(sc[c], LOG2E, nmx)), p1 = ex2f(fmaf(sc[c + 1], LOG2E, nmx));
+            const float p0 = ptx::ex2(fmaf(sc[c], LOG2E, nmx)), p1 = ptx::ex2(fmaf(sc[c + 1], LOG2E, nmx));
             sum4[c & 2] += p0;
             sum4[(c & 2) + 1] += p1;
             pk[c / 2] = float2_to_bf16x2(p0, p1);

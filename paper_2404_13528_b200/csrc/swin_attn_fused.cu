@@ -103,12 +103,6 @@ struct FusedArgs {
   DevMap rowmap;                                    // row n T + i of the windowed view -> element offset of the token in x (and y)
 };
 
-__device__ __forceinline__ float ex2f(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
 template <int NH, int KC>
 __global__ void __launch_bounds__(32 * (10 + 4 * NH), 1)
 swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_constant__ CUtensorMap tmWp,
@@ -573,7 +567,7 @@ swin_attn_fused_kernel(const __grid_constant__ CUtensorMap tmWq, const __grid_co
         for (int c = 0; c < KC; c += 2) {
           float e0, e1;
           ptx::unpack2(ptx::fma2(ptx::pack2(sc[c], sc[c + 1]), log2e2, nmx2), e0, e1);
-          const float p0 = ex2f(e0), p1 = ex2f(e1);
+          const float p0 = ptx::ex2(e0), p1 = ptx::ex2(e1);
           sum2[(c >> 1) & 1] = ptx::add2(sum2[(c >> 1) & 1], ptx::pack2(p0, p1));
           pk[c / 2] = float2_to_bf16x2(p0, p1);
         }
