@@ -368,10 +368,11 @@ gemm_splitk_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
   }
 }
 
-// Rows of a row tile: at most 256, at most 15 of them padding.  Where the columns are few, as many row tiles as clusters of eight find room
-// for, one CTA per SM: a CTA's share of the exchange shrinks with its tile and nothing else is long (134 x 2048 -> 512: 6.8 us in one row
-// tile, 5.3 in three; 200 x 1536 -> 384 8.0, 5.2 in five; 100 x 1024 -> 256 5.6, 4.4 in four).  Not with few rows of a large weight, which every
-// row tile reads (33 x 3072 -> 768 5.4, 5.8 in two), and beyond eight only for a reduction that is worth it (480 x 768 -> 8 5.1 in fifteen).
+// Rows of a row tile: a multiple of 16, at most 256; the tiles are alike, so the last one may be mostly padding (300 rows in ten tiles of
+// 32: 12 of its own).  Where the columns are few, as many row tiles as clusters of eight find room for, one CTA per SM: a CTA's share of
+// the exchange shrinks with its tile and nothing else is long (134 x 2048 -> 512: 6.8 us in one row tile, 5.3 in three; 200 x 1536 -> 384
+// 8.0, 5.2 in five; 100 x 1024 -> 256 5.6, 4.4 in four).  Not with few rows of a large weight, which every row tile reads (33 x 3072 -> 768
+// 5.4, 5.8 in two), and beyond eight only for a reduction that is worth it (480 x 768 -> 8 5.1 in fifteen).
 int row_tile(long long M, long long N, long long K, const ClusterCtas& fit) {
   long long room = fit.n[kMaxSplits] / kMaxSplits / ((N + BN_W - 1) / BN_W);
   if (M <= 64 && N * K > (1ll << 21)) room = 1;

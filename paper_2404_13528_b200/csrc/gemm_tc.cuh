@@ -46,7 +46,7 @@ struct TcEpilogue {
   const void* rms_gamma;
   float rms_eps;
   // Non-zero: nothing in flight writes B -- parameters of a layer call, in a kernel that follows another one of the same call, which has
-  // waited for whatever preceded the call.  The few-row kernel then fetches B before its dependency wait.
+  // waited for whatever preceded the call.  The few-row kernel and the tiled one then fetch B before their dependency wait.
   int b_settled;
 };
 

@@ -1,5 +1,5 @@
 // LayerNorm of 128 rows in registers, written to shared memory as a tcgen05 operand: shared by the kernels that normalise the rows
-// of one tile and multiply them where they are (gemm_ln_wave.cu, gemm_ln_pair.cu, gemm_mlp_cluster.cu).
+// of one tile and multiply them where they are (gemm_ln_wave.cu, gemm_ln_pair.cu, gemm_mlp_cluster.cu, swin_attn_cluster.cu).
 #pragma once
 #include "common.cuh"
 #include "ptx.cuh"

@@ -113,7 +113,8 @@ Path choose_path(const smartmem_swin_params_t& p, int mode, bool compact) {
   return t;
 }
 
-// Only the intermediates the chosen path writes are reserved.
+// Only the intermediates the chosen path writes are reserved; a wide block that takes the cluster kernel reserves those of the kernels it takes
+// with more windows as well.
 Layout ws_layout(const smartmem_swin_params_t& p, int mode, bool compact) {
   const size_t esz = p.dtype == SMARTMEM_F32 ? 4 : 2;
   const size_t MC = al((size_t)p.B * p.H * p.W * p.C * esz);
@@ -122,7 +123,7 @@ Layout ws_layout(const smartmem_swin_params_t& p, int mode, bool compact) {
   memset(&L, 0, sizeof(L));
   size_t off = 0;
   auto take = [&](size_t bytes) { size_t o = off; off += bytes; return o; };
-  if (!t.fuse_attn || t.attn_cluster) {            // (what a caller is asked for does not depend on the choice between the kernels of a wide block)
+  if (!t.fuse_attn || t.attn_cluster) {            // (so that what a caller is asked for does not hang on the choice)
     if (!t.fuse_ln1) L.xn = take(MC);
     L.qkv = take(3 * MC);
     L.ao = take(MC);
